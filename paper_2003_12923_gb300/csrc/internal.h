@@ -35,6 +35,7 @@ struct Gemm64 {
   double *C; int64_t sCm, sCn, sCb;
   int Kin;
   int64_t sAk1, sBk1;
+  int sym;                // C is symmetric (M = N, B(k, n) = A(n, k)): tiles above the diagonal only, mirrored
 };
 void gemm64(const Gemm64 &g, cudaStream_t st);
 
@@ -212,6 +213,9 @@ void launch_couple64(esmp2_handle *h, const double *F, int arrow, const double *
 esmp2_status sigma64_tail(esmp2_handle *h, const double *F, int arrow, const double *x, double *y);
 esmp2_status virtual_contraction(esmp2_handle *h, const double *x, double *y, int mode);
 void contractions64(esmp2_handle *h, const double *F, const double *x, double *y, int stage);
+// P_s = x_s F (first n_one listed slices) and y_s = x_s F + F x_s (the others) in float64, F = Fv (row pitch ldF)
+void virt64_list(esmp2_handle *h, const double *Fv, int ldF, const double *x, double *y, double *P, const int *list,
+                 int n_one, int n_list);
 // dot (optional, couple_dot_parts(h) doubles): per-CTA partials of the weighted <x, y>
 void couple32(esmp2_handle *h, const float *F32, const float *x, float *y, double *dot = nullptr);
 int64_t couple_dot_parts(const esmp2_handle *h);

@@ -17,7 +17,7 @@
 #include "internal.h"
 
 namespace esmp2 {
-void virt64_sym(esmp2_handle *h, const double *F, const double *x, double *y);
+esmp2_status virt64_sym(esmp2_handle *h, const double *F, const double *x, double *y);
 namespace {
 
 template <typename CT>
@@ -565,7 +565,8 @@ esmp2_status profile64(esmp2_handle *h, const double *x, double *y, int reps, do
       if (s) return s;
       combine_sym(h, y);
     } else {
-      virt64_sym(h, h->F, x, y);
+      esmp2_status s = virt64_sym(h, h->F, x, y);
+      if (s) return s;
     }
     cudaEventRecord(ev[1], h->stream);
     contractions64(h, h->F, x, y, 2);
@@ -770,42 +771,13 @@ void singlet_project(esmp2_handle *h, double *v) {
   h->launches += 1;
 }
 
-void virt64_sym(esmp2_handle *h, const double *F, const double *x, double *y) {
-  const int No = h->d.No, Nv = h->d.Nv, N = h->d.N;
-  const int64_t B = h->d.B, NvNv = (int64_t)Nv * Nv;
-  const double *Fv = F + (int64_t)No * N + No;
-  Gemm64 g{};
-  // P = x F for T, X, Y on the slices i < j
-  g.N = Nv; g.K = Nv; g.batch = 1; g.alpha = 1.0; g.beta = 0.0;
-  g.sAm = Nv; g.sAk = 1; g.B = Fv; g.sBk = N; g.sBn = 1; g.sCm = Nv; g.sCn = 1;
-  int nl = 0;
-  for (int blk : {BT, BX, BY})
-    for (int i = 0; i + 1 < No; ++i) {
-      const int64_t r0 = ((int64_t)i * No + i + 1) * Nv;
-      g.M = (int)((int64_t)(No - 1 - i) * Nv);
-      g.A = x + blk * B + r0 * Nv;
-      g.C = h->P64 + blk * B + r0 * Nv;
-      gemm64(g, h->stream);
-      ++nl;
-    }
-  // S and Z: y = x F + F x directly
-  for (int blk : {BS, BZ}) {
-    g = Gemm64{};
-    g.N = Nv; g.K = Nv; g.batch = 1; g.alpha = 1.0; g.beta = 0.0;
-    g.sAm = Nv; g.sAk = 1; g.B = Fv; g.sBk = N; g.sBn = 1; g.sCm = Nv; g.sCn = 1;
-    g.M = (int)((int64_t)No * No * Nv);
-    g.A = x + blk * B; g.C = y + blk * B;
-    gemm64(g, h->stream);
-    g = Gemm64{};
-    g.M = Nv; g.N = Nv; g.K = Nv; g.batch = No * No; g.alpha = 1.0; g.beta = 1.0;
-    g.A = Fv; g.sAm = N; g.sAk = 1; g.sAb = 0;
-    g.B = x + blk * B; g.sBk = Nv; g.sBn = 1; g.sBb = NvNv;
-    g.C = y + blk * B; g.sCm = Nv; g.sCn = 1; g.sCb = NvNv;
-    gemm64(g, h->stream);
-    nl += 2;
-  }
-  h->launches += nl;
+esmp2_status virt64_sym(esmp2_handle *h, const double *F, const double *x, double *y) {
+  // P = x F for T, X, Y on the slices i < j; S and Z: y = x F + F x directly
+  if (esmp2_status s0 = ensure_slist(h)) return s0;
+  const int No = h->d.No, N = h->d.N;
+  virt64_list(h, F + (int64_t)No * N + No, N, x, y, h->P64, h->slist, 3 * (No * (No - 1) / 2), h->nslist);
   combine_sym(h, y);
+  return ESMP2_OK;
 }
 
 // y_ij = P_ij - P_ij^T for the T, X, Y blocks from P (= x F on the slices i < j) in P64
@@ -882,7 +854,8 @@ esmp2_status sigma64_F(esmp2_handle *h, const double *F, int arrow, const double
     combine_sym(h, y);
     if (s_sym) combine_s(h, y);
   } else {
-    virt64_sym(h, F, x, y);
+    esmp2_status s = virt64_sym(h, F, x, y);
+    if (s) return s;
   }
   if (!arrow) contractions64(h, F, x, y, 2);
   if (couplings || !arrow) {
