@@ -12,6 +12,7 @@
 //   dE2_S: the S-space sum -b_I^2 / D_I differentiated in b_I (integrals) and D_I (diagonal F).
 // Conventions: dF is the derivative of E2 evaluated on (F + F^T)/2 (so dF is symmetric) and
 // dOVOV[i][a][j][b] the derivative of E2 evaluated on the (ia)<->(jb) symmetrised block.
+#include <algorithm>
 #include <cmath>
 #include <vector>
 
@@ -249,62 +250,175 @@ __device__ void flush_diag(const SG &g, double *sdiag) {
     if (sdiag[k] != 0.0) atomicAdd(&g.Gdiag[k], sdiag[k]);
 }
 
-// same enumeration as the energy kernels (sector A: up-up-up, B: up pair + down-down, C: down pair only)
-__global__ void kg_s_a(SG g) {
-  extern __shared__ double sdiag[];
-  for (int k = threadIdx.x; k <= g.c.N; k += blockDim.x) sdiag[k] = 0.0;
+// S-space derivative, the triples with exactly one transition pair (the energy's k_e2s_ab and
+// k_e2s_cm enumerate the same ones): b_I is lambda_u times one antisymmetrised integral, so a
+// thread that owns the integral sums over the pair u itself, adds its own two (ov|ov) elements
+// without atomics (no other thread writes them) and keeps the diagonal sums in registers and
+// private shared-memory slots.  One triple at a time with nine scattered float64 atomics each took
+// 17.5 ms at No=12 Nv=120, this form 1.0 ms.
+constexpr int kST = 128;   // threads of the S-space gradient kernels
+
+// shared memory: lu2[No], du[No], sdiag[N + 1], private per-u sums [No][kST]
+size_t sgrad_smem(int No, int Nv) { return sizeof(double) * (size_t)(2 * No + No + Nv + 1 + No * kST); }
+struct SSh {
+  double *lu2, *du, *sdiag, *su;
+};
+__device__ __forceinline__ SSh s_shared(const SG &g, double *sm) {
+  const int No = g.c.No, N = g.c.N;
+  SSh s{sm, sm + No, sm + 2 * No, sm + 2 * No + N + 1};
+  for (int u = threadIdx.x; u < No; u += blockDim.x) {
+    s.lu2[u] = g.c.lam[u] * g.c.lam[u];
+    s.du[u] = g.c.F[(int64_t)(No + u) * N + No + u] - g.c.F[(int64_t)u * N + u];
+  }
+  for (int k = threadIdx.x; k <= N; k += blockDim.x) s.sdiag[k] = 0.0;
+  for (int k = threadIdx.x; k < No * kST; k += blockDim.x) s.su[k] = 0.0;
   __syncthreads();
-  const int No = g.c.No, Nv = g.c.Nv;
-  const int64_t blk = blockIdx.x;
-  const int u = (int)(blk / ((int64_t)No * No)), j = (int)((blk / No) % No), k = (int)(blk % No);
-  if (u >= 1 && j < k && j != u && k != u) {
-    for (int b = threadIdx.x; b < Nv; b += blockDim.x) {
-      if (b == u) continue;
-      for (int cc = b + 1; cc < Nv; ++cc) {
-        if (cc == u) continue;
-        const bool pj = (b == j || cc == j), pk = (b == k || cc == k);
-        if ((pj && j < u) || (pk && k < u)) continue;
-        if ((pj && j == 0) || (pk && k == 0)) continue;
-        const int ho[3] = {u, j, k}, hs[3] = {0, 0, 0}, po[3] = {u, b, cc}, ps[3] = {0, 0, 0};
-        g.triple(ho, hs, po, ps, sdiag);
-      }
+  return s;
+}
+// per-u sums of the CTA into sdiag (u' particle, u hole), then everything to the gradient
+__device__ __forceinline__ void s_flush(const SG &g, const SSh &s) {
+  __syncthreads();
+  const int No = g.c.No, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  for (int u = warp; u < No; u += kST / 32) {
+    double v = 0.0;
+    for (int t = lane; t < kST; t += 32) v += s.su[u * kST + t];
+    v = warp_sum(v);
+    if (lane == 0 && v != 0.0) {
+      atomicAdd(&s.sdiag[No + u], v);
+      atomicAdd(&s.sdiag[u], -v);
+      atomicAdd(&s.sdiag[g.c.N], v);
     }
   }
-  flush_diag(g, sdiag);
+  flush_diag(g, s.sdiag);
 }
 
-__global__ void kg_s_b(SG g) {
-  extern __shared__ double sdiag[];
-  for (int k = threadIdx.x; k <= g.c.N; k += blockDim.x) sdiag[k] = 0.0;
-  __syncthreads();
-  const int No = g.c.No, Nv = g.c.Nv;
-  const int64_t blk = blockIdx.x;
-  const int u = (int)(blk / ((int64_t)No * No)), j = (int)((blk / No) % No), k = (int)(blk % No);
-  if (u >= 1 && j < k) {
-    for (int b = threadIdx.x; b < Nv; b += blockDim.x)
-      for (int cc = b + 1; cc < Nv; ++cc) {
-        if ((j == 0 || k == 0) && (b == 0 || cc == 0)) continue;
-        const int ho[3] = {u, j, k}, hs[3] = {0, 1, 1}, po[3] = {u, b, cc}, ps[3] = {0, 1, 1};
-        g.triple(ho, hs, po, ps, sdiag);
+// sectors A and B: block = (pair j < k, one of nchunk strided ranges of c), threads over b < c
+__global__ void __launch_bounds__(kST) kg_s_ab(SG g, int nchunk) {
+  extern __shared__ double sm[];
+  const int No = g.c.No, Nv = g.c.Nv, N = g.c.N;
+  const SSh s = s_shared(g, sm);
+  const int chunk = blockIdx.x % nchunk;
+  int kk = blockIdx.x / nchunk, j = 0;
+  while (kk >= No - 1 - j) { kk -= No - 1 - j; ++j; }
+  const int k = j + 1 + kk;
+  const double base = -g.c.F[(int64_t)j * N + j] - g.c.F[(int64_t)k * N + k] - g.c.omega;
+  double *su = s.su + threadIdx.x;
+  double jk = 0.0;
+  for (int b0 = 0; b0 < Nv; b0 += kST) {
+    const int b = b0 + threadIdx.x;
+    const double eb = b < Nv ? base + g.c.F[(int64_t)(No + b) * N + No + b] : 0.0;
+    double gb = 0.0;
+    for (int cc = 1 + chunk; cc < Nv; cc += nchunk) {
+      if (cc <= b0 || cc == j || cc == k) continue;   // uniform over the CTA
+      double gd = 0.0;
+      if (b < cc && b != j && b != k) {
+        const int64_t i1 = g.c.ov(k, cc, j, b), i2 = g.c.ov(j, cc, k, b);
+        const double dg = g.c.ovov[i1] - g.c.ovov[i2], e = eb + g.c.F[(int64_t)(No + cc) * N + No + cc];
+        double q1 = 0.0;
+        for (int u = 1; u < No; ++u) {
+          const double m = (u != j && u != k && u != b && u != cc) ? 2.0 : 1.0;   // sectors A and B, or B alone
+          const double r = 1.0 / (s.du[u] + e), q = m * s.lu2[u] * r, d = 2.0 * dg * dg * q * r;
+          q1 += q;
+          su[u * kST] += d;
+          gd += d;
+        }
+        g.Gov[i1] -= 4.0 * dg * q1;
+        g.Gov[i2] += 4.0 * dg * q1;
       }
+      gb += gd;
+      gd = warp_sum(gd);
+      if ((threadIdx.x & 31) == 0 && gd != 0.0) atomicAdd(&s.sdiag[No + cc], gd);
+    }
+    if (b < Nv && gb != 0.0) atomicAdd(&s.sdiag[No + b], gb);
+    jk += gb;
   }
-  flush_diag(g, sdiag);
+  jk = warp_sum(jk);
+  if ((threadIdx.x & 31) == 0) {
+    atomicAdd(&s.sdiag[j], -jk);
+    atomicAdd(&s.sdiag[k], -jk);
+  }
+  s_flush(g, s);
 }
 
-__global__ void kg_s_c(SG g) {
+// sector C: block = (i, k, one of nchunk strided ranges of a), threads over c
+__global__ void __launch_bounds__(kST) kg_s_cm(SG g, int nchunk) {
+  extern __shared__ double sm[];
+  const int No = g.c.No, Nv = g.c.Nv, N = g.c.N;
+  const SSh s = s_shared(g, sm);
+  const int chunk = blockIdx.x % nchunk, ik = blockIdx.x / nchunk, i = ik / No, k = ik % No;
+  const double base = -g.c.F[(int64_t)i * N + i] - g.c.F[(int64_t)k * N + k] - g.c.omega;
+  double *su = s.su + threadIdx.x;
+  double sik = 0.0;
+  for (int c0 = 0; c0 < Nv; c0 += kST) {
+    const int cc = c0 + threadIdx.x;
+    const bool on = cc < Nv && cc != k;
+    const double ec = cc < Nv ? base + g.c.F[(int64_t)(No + cc) * N + No + cc] : 0.0;
+    double gc = 0.0;
+    for (int a = chunk; a < Nv; a += nchunk) {
+      if (a == i) continue;
+      double gd = 0.0;
+      if (on) {
+        const int64_t i1 = g.c.ov(i, a, k, cc);
+        const double gv = g.c.ovov[i1], e = ec + g.c.F[(int64_t)(No + a) * N + No + a];
+        double q1 = 0.0;
+        for (int u = 1; u < No; ++u) {
+          if (u == k || u == cc) continue;
+          const double r = 1.0 / (s.du[u] + e), q = s.lu2[u] * r, d = 2.0 * gv * gv * q * r;
+          q1 += q;
+          su[u * kST] += d;
+          gd += d;
+        }
+        g.Gov[i1] -= 4.0 * gv * q1;
+      }
+      gc += gd;
+      gd = warp_sum(gd);
+      if ((threadIdx.x & 31) == 0 && gd != 0.0) atomicAdd(&s.sdiag[No + a], gd);
+    }
+    if (on) atomicAdd(&s.sdiag[No + cc], gc);
+    sik += gc;
+  }
+  sik = warp_sum(sik);
+  if ((threadIdx.x & 31) == 0) {
+    atomicAdd(&s.sdiag[i], -sik);
+    atomicAdd(&s.sdiag[k], -sik);
+  }
+  s_flush(g, s);
+}
+
+// the triples that hold a second transition pair (few), one at a time (the energy's k_e2s_gen
+// enumerates the same ones): block = (u, x, y) for the three sectors' index pairs
+__global__ void __launch_bounds__(kST) kg_s_gen(SG g) {
   extern __shared__ double sdiag[];
   for (int k = threadIdx.x; k <= g.c.N; k += blockDim.x) sdiag[k] = 0.0;
   __syncthreads();
   const int No = g.c.No, Nv = g.c.Nv;
   const int64_t blk = blockIdx.x;
-  const int u = (int)(blk / ((int64_t)No * No)), i = (int)((blk / No) % No), k = (int)(blk % No);
-  if (u >= 1 && k != u) {
-    for (int a = threadIdx.x; a < Nv; a += blockDim.x) {
-      if (a == i) continue;
-      for (int cc = 0; cc < Nv; ++cc) {
-        if (cc == u) continue;
-        if (cc == k && (k < u || k == 0)) continue;
-        const int ho[3] = {i, u, k}, hs[3] = {0, 1, 1}, po[3] = {a, u, cc}, ps[3] = {0, 1, 1};
+  const int u = (int)(blk / ((int64_t)No * No)), x = (int)((blk / No) % No), y = (int)(blk % No);
+  if (u >= 1) {
+    const int j = x, k = y;
+    if (j < k) {
+      for (int e = threadIdx.x; e < 2 * Nv; e += blockDim.x) {
+        const int xx = e < Nv ? j : k, yy = e % Nv;
+        if (yy == xx || ((yy == j || yy == k) && xx != j)) continue;  // the pair (j, k) once
+        const int b = min(xx, yy), cc = max(xx, yy);
+        if (j != u && k != u && b != u && cc != u) {   // sector A
+          const bool pj = (b == j || cc == j), pk = (b == k || cc == k);
+          if (!((pj && j < u) || (pk && k < u)) && !((pj && j == 0) || (pk && k == 0))) {
+            const int ho[3] = {u, j, k}, hs[3] = {0, 0, 0}, po[3] = {u, b, cc}, ps[3] = {0, 0, 0};
+            g.triple(ho, hs, po, ps, sdiag);
+          }
+        }
+        if (!((j == 0 || k == 0) && (b == 0 || cc == 0))) {   // sector B
+          const int ho[3] = {u, j, k}, hs[3] = {0, 1, 1}, po[3] = {u, b, cc}, ps[3] = {0, 1, 1};
+          g.triple(ho, hs, po, ps, sdiag);
+        }
+      }
+    }
+    const int i = x;
+    if (k != u && k >= u && k != 0) {   // sector C: the down particle c == k
+      for (int a = threadIdx.x; a < Nv; a += blockDim.x) {
+        if (a == i) continue;
+        const int ho[3] = {i, u, k}, hs[3] = {0, 1, 1}, po[3] = {a, u, k}, ps[3] = {0, 1, 1};
         g.triple(ho, hs, po, ps, sdiag);
       }
     }
@@ -356,13 +470,13 @@ static void densities(esmp2_handle *h, const double *x, double *Gf) {
     const double *X = x + blk * B;
     Gemm64 g{};
     // virtual: sum over rows (s,a) of X[s][a][p] X[s][a][q]
-    g.M = Nv; g.N = Nv; g.K = No * No * Nv; g.batch = 1; g.alpha = W[blk]; g.beta = 1.0;
+    g.M = Nv; g.N = Nv; g.K = No * No * Nv; g.batch = 1; g.alpha = W[blk]; g.beta = 1.0; g.sym = 1;
     g.A = X; g.sAm = 1; g.sAk = Nv; g.B = X; g.sBk = Nv; g.sBn = 1;
     g.C = Gf + (int64_t)No * N + No; g.sCm = N; g.sCn = 1;
     gemm64(g, h->stream);
     // virtual: sum over (s,b) of X[s][p][b] X[s][q][b]
     g = Gemm64{};
-    g.M = Nv; g.N = Nv; g.K = No * No * Nv; g.batch = 1; g.alpha = W[blk]; g.beta = 1.0;
+    g.M = Nv; g.N = Nv; g.K = No * No * Nv; g.batch = 1; g.alpha = W[blk]; g.beta = 1.0; g.sym = 1;
     g.Kin = Nv;
     g.A = X; g.sAm = Nv; g.sAk = 1; g.sAk1 = NvNv;
     g.B = X; g.sBk = 1; g.sBk1 = NvNv; g.sBn = Nv;
@@ -370,12 +484,12 @@ static void densities(esmp2_handle *h, const double *x, double *Gf) {
     gemm64(g, h->stream);
     // occupied: -(sum over (j,ab) of X[l][j][ab] X[i][j][ab]) - (sum over (i',ab) of X[i'][l][ab] X[i'][i][ab])
     g = Gemm64{};
-    g.M = No; g.N = No; g.K = (int)((int64_t)No * NvNv); g.batch = 1; g.alpha = -W[blk]; g.beta = 1.0;
+    g.M = No; g.N = No; g.K = (int)((int64_t)No * NvNv); g.batch = 1; g.alpha = -W[blk]; g.beta = 1.0; g.sym = 1;
     g.A = X; g.sAm = (int64_t)No * NvNv; g.sAk = 1; g.B = X; g.sBk = 1; g.sBn = (int64_t)No * NvNv;
     g.C = Gf; g.sCm = N; g.sCn = 1;
     gemm64(g, h->stream);
     g = Gemm64{};
-    g.M = No; g.N = No; g.K = (int)((int64_t)No * NvNv); g.batch = 1; g.alpha = -W[blk]; g.beta = 1.0;
+    g.M = No; g.N = No; g.K = (int)((int64_t)No * NvNv); g.batch = 1; g.alpha = -W[blk]; g.beta = 1.0; g.sym = 1;
     g.Kin = (int)NvNv;
     g.A = X; g.sAm = NvNv; g.sAk = 1; g.sAk1 = (int64_t)No * NvNv;
     g.B = X; g.sBk = 1; g.sBk1 = (int64_t)No * NvNv; g.sBn = NvNv;
@@ -418,11 +532,16 @@ esmp2_status gradient(esmp2_handle *h, double *dF_host, double *dOVOV_host, int 
   }
   double *Gf = nullptr, *Gov = nullptr, *acc = nullptr, *T1 = nullptr, *T2 = nullptr, *Gd = nullptr;
   cudaError_t ce = cudaSuccess;
-  auto A = [&](double **p, size_t cnt) { if (ce == cudaSuccess) ce = cudaMalloc(p, sizeof(double) * cnt); };
+  auto A = [&](double **p, size_t cnt) { if (ce == cudaSuccess) ce = dmalloc(reinterpret_cast<void **>(p), sizeof(double) * cnt, st); };
   A(&Gf, (size_t)N * N); A(&Gov, (size_t)nov); A(&acc, 4); A(&T1, (size_t)std::max<int64_t>((int64_t)N * N, nov));
   A(&T2, (size_t)std::max<int64_t>((int64_t)N * N, nov)); A(&Gd, (size_t)N + 1);
+  double *Ut_d = nullptr, *Wvt_d = nullptr;
+  A(&Ut_d, (size_t)No * No); A(&Wvt_d, (size_t)Nv * Nv);
+  auto release = [&]() {
+    for (double *p : {Gf, Gov, acc, T1, T2, Gd, Ut_d, Wvt_d}) dfree(p, st);
+  };
   if (ce != cudaSuccess) {
-    cudaFree(Gf); cudaFree(Gov); cudaFree(acc); cudaFree(T1); cudaFree(T2); cudaFree(Gd);
+    release();
     return check_cuda(h, ce, "gradient workspace");
   }
   cudaMemsetAsync(Gf, 0, sizeof(double) * N * N, st);
@@ -443,11 +562,21 @@ esmp2_status gradient(esmp2_handle *h, double *dF_host, double *dOVOV_host, int 
   kg_finish_scalars<<<1, 32, 0, st>>>(c, acc, Gf);
   SG sg;
   sg.c = c; sg.Gov = Gov; sg.Gdiag = Gd;
-  const int nb = No * No * No;
-  const size_t shm = sizeof(double) * (N + 1);
-  kg_s_a<<<nb, 128, shm, st>>>(sg);
-  kg_s_b<<<nb, 128, shm, st>>>(sg);
-  kg_s_c<<<nb, 128, shm, st>>>(sg);
+  if (No > 1) {   // sums over the small pairs u >= 1
+    const int npair = No * (No - 1) / 2, chAB = (int)std::max<int64_t>(1, std::min<int64_t>(Nv / 8, cdiv(1216, npair))),
+              chC = (int)std::max<int64_t>(1, std::min<int64_t>(Nv / 8, cdiv(1216, No * No)));
+    const size_t shm = sgrad_smem(No, Nv);
+    const int lim = (int)sgrad_smem(64, 4096);   // the largest sizes of the library: one limit for every call
+    cudaError_t ea = smem_limit_once(reinterpret_cast<const void *>(kg_s_ab), lim);
+    if (ea == cudaSuccess) ea = smem_limit_once(reinterpret_cast<const void *>(kg_s_cm), lim);
+    if (ea != cudaSuccess) {
+      release();
+      return check_cuda(h, ea, "gradient shared-memory limit");
+    }
+    kg_s_ab<<<npair * chAB, kST, shm, st>>>(sg, chAB);
+    kg_s_cm<<<No * No * chC, kST, shm, st>>>(sg, chC);
+    kg_s_gen<<<No * No * No, kST, sizeof(double) * (N + 1), st>>>(sg);
+  }
   kg_s_finish<<<(unsigned)cdiv(N, 128), 128, 0, st>>>(c, Gd, Gf);
   h->launches += 13;
   // dF = W sym(Gf) W^T
@@ -461,9 +590,6 @@ esmp2_status gradient(esmp2_handle *h, double *dF_host, double *dOVOV_host, int 
   if (dF_host) cudaMemcpyAsync(dF_host, T1, sizeof(double) * N * N, cudaMemcpyDeviceToHost, st);
   // dOVOV: symmetrise, then rotate every index back (in[i'] -> sum_i' U[i][i'] in[i'])
   kg_sym_ov<<<1216, 256, 0, st>>>(Gov, T1, No, Nv);
-  double *Ut_d = nullptr, *Wvt_d = nullptr;
-  cudaMalloc(&Ut_d, sizeof(double) * No * No);
-  cudaMalloc(&Wvt_d, sizeof(double) * Nv * Nv);
   kg_transpose<<<64, 256, 0, st>>>(h->U, Ut_d, No);
   kg_transpose<<<256, 256, 0, st>>>(h->Wv, Wvt_d, Nv);
   const int dims[4] = {No, Nv, No, Nv};
@@ -477,7 +603,7 @@ esmp2_status gradient(esmp2_handle *h, double *dF_host, double *dOVOV_host, int 
   h->launches += 10;
   if (dOVOV_host) cudaMemcpyAsync(dOVOV_host, src, sizeof(double) * nov, cudaMemcpyDeviceToHost, st);
   ce = cudaStreamSynchronize(st);
-  cudaFree(Gf); cudaFree(Gov); cudaFree(acc); cudaFree(T1); cudaFree(T2); cudaFree(Gd); cudaFree(Ut_d); cudaFree(Wvt_d);
+  release();
   if (ce == cudaSuccess) ce = cudaGetLastError();
   return check_cuda(h, ce, "gradient");
 }
