@@ -114,7 +114,7 @@ struct esmp2_handle {
   float arrow_w[64] = {};   // host copy of F32[l][0] (1 <= l < No) and F32[l][No] (l < No)
   bool arrow_w_ready = false;
   __half *dinv32 = nullptr; // Jacobi preconditioner in that basis (n halves)
-  double *P64 = nullptr;    // x F for the T, S, X, Y blocks (float64 sigma workspace, 4 blocks)
+  double *P64 = nullptr;    // products of the virtual-index pass (float64 sigma workspace, n)
   double *red = nullptr;    // reduction partials
   double *red_out = nullptr;// reduction results (device)
   double *hred = nullptr;   // pinned host copy of reduction results
@@ -165,11 +165,14 @@ struct esmp2_handle {
   bool x_zero = true;       // s64.x is known to be zero (its sigma is zero, no build needed)
   bool r_true = false;      // s64.r holds the true residual -b - A x of s64.x (same basis)
   // float64-accurate virtual-index terms from exact bf16 digit products (tcgen05)
-  void *xdig = nullptr;     // digit planes of x [levels-1][5 No^2][Nv][Nvp] bf16
+  void *xdig = nullptr;     // digit planes of the stacked rows [levels-1][jobs][Nv][Nvp] bf16
+  size_t xdig_bytes = 0;
   void *Fdig = nullptr;     // digit planes of F_vv [levels-1][Nv][Nvp] bf16
   int *es = nullptr;        // per-slice exponents (5 No^2) and that of F_vv (last entry)
   int *slist = nullptr;     // slices of the symmetric form (T, X, Y with i < j; all S, Z)
   int nslist = 0, eF = 0;
+  int *jobs[3] = {};        // job lists of the contraction forms sym = 0, 1, 2 (in slist's allocation)
+  int njobs[3] = {};
   void *Rdig = nullptr;     // digit planes of W_v^T (integral transforms on the tensor cores)
   int eR = 0;
   int last_precision = 0;   // precision of the last solve (the energy's sigma follows it)
@@ -250,11 +253,13 @@ void antisym_project(esmp2_handle *h, double *v);
 void singlet_project(esmp2_handle *h, double *v);
 void combine_sym(esmp2_handle *h, double *y);
 void combine_s(esmp2_handle *h, double *y);
+constexpr int kDigitPlanes = 9;   // digit planes kept of the right operands
 constexpr int kFp64TcLevels = 10;  // digit levels of the float64-exact tensor-core contraction
 int split_levels_for(double tol);
 bool split_supported(const esmp2_handle *h, int levels);
 esmp2_status ensure_split(esmp2_handle *h);
 esmp2_status ensure_slist(esmp2_handle *h);
+esmp2_status ensure_p64(esmp2_handle *h);
 esmp2_status virt_split(esmp2_handle *h, const double *x, double *y, double *p64, int sym, int levels);
 esmp2_status xwv_split(esmp2_handle *h, const double *X, int64_t rows, double *Y);
 esmp2_status xwm_split(esmp2_handle *h, const double *X, int64_t rows, double *Y, const double *M, void **dig,
@@ -290,6 +295,10 @@ cudaError_t smem_limit_once(const void *func, int bytes);
 // rejects the description.
 bool tma_map_2d(CUtensorMap *m, const void *base, bool f32, uint64_t inner, uint64_t outer, uint64_t row_bytes,
                 uint32_t box_inner, uint32_t box_outer, int swizzle_bytes);
+
+// Tensor map of bf16 elements of `rank` <= 3 dims (innermost first), swizzle of 128 or 64 bytes, zero fill.
+bool tma_map_bf16(CUtensorMap *m, const void *base, int rank, const uint64_t *dims, const uint64_t *strides_bytes,
+                  const uint32_t *box, int swizzle_bytes);
 
 // Output options of the virtual-index GEMM (vgemm.cu): transposed rows stored as bf16 into
 // PT16 (instead of float32 into PT), optionally scaled by the reduced-cost-basis inverse

@@ -559,7 +559,7 @@ esmp2_status profile64(esmp2_handle *h, const double *x, double *y, int reps, do
   double acc[5] = {0, 0, 0, 0, 0};
   for (int r = 0; r < reps; ++r) {
     cudaEventRecord(ev[0], h->stream);
-    if (!h->P64) dmalloc(reinterpret_cast<void **>(&h->P64), sizeof(double) * 4 * (size_t)h->d.B, h->stream);
+    if (esmp2_status s0 = ensure_p64(h)) return s0;
     if (tc_levels) {
       esmp2_status s = virt_split(h, x, y, h->P64, 1, tc_levels);
       if (s) return s;
@@ -780,6 +780,13 @@ esmp2_status virt64_sym(esmp2_handle *h, const double *F, const double *x, doubl
   return ESMP2_OK;
 }
 
+esmp2_status ensure_p64(esmp2_handle *h) {
+  if (h->P64) return ESMP2_OK;
+  cudaError_t e = dmalloc(reinterpret_cast<void **>(&h->P64), sizeof(double) * (size_t)h->d.n, h->stream);
+  if (e != cudaSuccess) h->P64 = nullptr;
+  return e == cudaSuccess ? ESMP2_OK : check_cuda(h, e, "sigma64 workspace");
+}
+
 // y_ij = P_ij - P_ij^T for the T, X, Y blocks from P (= x F on the slices i < j) in P64
 void combine_sym(esmp2_handle *h, double *y) {
   const int No = h->d.No, Nv = h->d.Nv, tiles = (Nv + 31) / 32;
@@ -844,10 +851,7 @@ void couple_f32_into(esmp2_handle *h, const double *x, double *y) {
 // coupling pass).
 esmp2_status sigma64_F(esmp2_handle *h, const double *F, int arrow, const double *x, double *y, int tc_levels,
                        int couplings, bool s_sym) {
-  if (!h->P64) {
-    cudaError_t e = dmalloc(reinterpret_cast<void **>(&h->P64), sizeof(double) * 4 * (size_t)h->d.B, h->stream);
-    if (e != cudaSuccess) return check_cuda(h, e, "sigma64 workspace");
-  }
+  if (esmp2_status s0 = ensure_p64(h)) return s0;
   if (tc_levels) {
     esmp2_status s = virt_split(h, x, y, h->P64, s_sym ? 2 : 1, tc_levels);
     if (s) return s;
