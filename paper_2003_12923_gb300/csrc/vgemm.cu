@@ -216,46 +216,47 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       // the column tile's F panel, once
       mbar_expect_tx(&pbar, chunk_bytes * (uint32_t)g.nk);
       for (int kc = 0; kc < g.nk; ++kc) tma_2d(panel + kc * chunk_bytes, &tF, &pbar, kc * BK, b0);
-      int64_t it = 0;
+      // ring positions as running counters: this thread and the MMA issuer are serial chains, and a
+      // 64-bit division per chunk by the (runtime) ring length was the longest link in both
+      int st = 0;
+      uint32_t ph = 1, laps = 0;   // parity of the next wait on an empty slot
       for (int64_t m = gi; m < g.m_tiles && ok; m += group) {
-        for (int kc = 0; kc < g.nk; ++kc, ++it) {
-          const int st = (int)(it % STAGES);
-          const uint32_t rnd = (uint32_t)(it / STAGES);
-          if (!mbar_wait(&empty[st], (rnd & 1) ^ 1)) { ok = false; break; }
+        for (int kc = 0; kc < g.nk; ++kc) {
+          if (!mbar_wait(&empty[st], ph)) { ok = false; break; }
           mbar_expect_tx(&full[st], (uint32_t)A_STAGE);
           tma_2d(ring + st * A_STAGE, &tA, &full[st], kc * BK, (int)(m * BM));
+          if (++st == STAGES) { st = 0; ph ^= 1; laps = 1; }
         }
       }
       if (!ok) atomicExch(&fail, 1);
-      // wait (bounded) until no copy of this CTA is still in flight
+      // wait (bounded) until no copy of this CTA is still in flight: slots before st belong to the
+      // current lap (parity ph ^ 1 of their full barrier), the others to the one before
       mbar_wait(&pbar, 0, 100000000ull);
-      for (int64_t j = it > STAGES ? it - STAGES : 0; j < it; ++j)
-        mbar_wait(&full[j % STAGES], (uint32_t)((j / STAGES) & 1), 100000000ull);
+      for (int j = 0; j < STAGES; ++j)
+        if (j < st) mbar_wait(&full[j], ph ^ 1, 100000000ull);
+        else if (laps) mbar_wait(&full[j], ph, 100000000ull);
     }
   } else if (warp == 1) {
     if (lane == 0) {  // ------------------------------------------------ MMA issuer
       bool ok = mbar_wait(&pbar, 0);
       tc_after();
       const uint32_t id = idesc<TF32>(BM, nmma);
-      const uint32_t pan = smem_u32(panel), rg = smem_u32(ring);
-      int64_t it = 0;
-      int lt = 0;
+      const uint64_t pan = sdesc64(smem_u32(panel)), rg = sdesc64(smem_u32(ring));
+      int st = 0, lt = 0;
+      uint32_t ph = 0;
       for (int64_t m = gi; m < g.m_tiles && ok; m += group, ++lt) {
         const int ab = lt & 1;
         const uint32_t ar = (uint32_t)(lt >> 1);
         if (!mbar_wait(&acc_empty[ab], (ar & 1) ^ 1)) { ok = false; break; }
         tc_after();
         const uint32_t d = tmem + (uint32_t)(ab * 256);
-        for (int kc = 0; kc < g.nk; ++kc, ++it) {
-          const int st = (int)(it % STAGES);
-          const uint32_t rnd = (uint32_t)(it / STAGES);
-          if (!mbar_wait(&full[st], rnd & 1)) { ok = false; break; }
-          tc_after();
-          const int ksteps = min(BK / KMMA, (g.Nv - kc * BK + KMMA - 1) / KMMA);   // skip K steps past Nv
-          for (int k = 0; k < ksteps; ++k)
-            umma<TF32>(d, sdesc64(rg + st * A_STAGE + 32 * k), sdesc64(pan + kc * chunk_bytes + 32 * k), id,
-                       (kc > 0 || k > 0) ? 1u : 0u);
+        for (int kc = 0; kc < g.nk; ++kc) {
+          if (!mbar_wait(&full[st], ph)) { ok = false; break; }
+          const uint64_t a = rg + (uint64_t)(st * (A_STAGE / 16)), b = pan + (uint64_t)(kc * (chunk_bytes / 16));
+          umma<TF32>(d, a, b, id, kc > 0 ? 1u : 0u);
+          if (g.Nv - kc * BK > KMMA) umma<TF32>(d, a + 2, b + 2, id, 1u);   // skip the K step past Nv
           umma_commit(&empty[st]);
+          if (++st == STAGES) { st = 0; ph ^= 1; }
         }
         if (!ok) break;
         umma_commit(&acc_full[ab]);
