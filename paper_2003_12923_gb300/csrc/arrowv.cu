@@ -34,16 +34,6 @@ __global__ void k_to_f32(const double *src, float *dst, int64_t n) {
     dst[e] = (float)src[e];
 }
 
-// A (m x m) = the virtual block of F without t' (rows and columns 1 .. Nv-1); V = I
-__global__ void k_vblock(const double *F, int N, int No, int m, double *A, double *V) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < (int64_t)m * m;
-       e += (int64_t)gridDim.x * blockDim.x) {
-    const int i = (int)(e / m), j = (int)(e % m);
-    A[e] = F[(int64_t)(No + 1 + i) * N + No + 1 + j];
-    V[e] = i == j ? 1.0 : 0.0;
-  }
-}
-
 // One round r of the one-sided (Hestenes) Jacobi method on the symmetric positive definite
 // m x m matrix held as the rows of B: the disjoint pairs (p, q) of the round-robin ordering of
 // n = m (+1 if m is odd) indices, one CTA each, rotate rows p and q of B (B <- G^T B) until
@@ -291,7 +281,15 @@ esmp2_status ensure_vrot(esmp2_handle *h, bool exact) {
     A(reinterpret_cast<void **>(&h->jflag), sizeof(unsigned) * 4);
     if (e != cudaSuccess) return check_cuda(h, e, "virtual rotation buffers");
     if (m >= 1) {
-      k_vblock<<<256, 256, 0, st>>>(h->Fsemi, N, No, m, h->jB, h->jJ);
+      // B = Jt A from the complement of t' next to the input orbitals (2 sweeps to 1e-2 at No=30
+      // Nv=400 from there, 8 from the identity in the TOP basis)
+      complement_basis(h, h->Wv, Nv, h->jJ);
+      Gemm64 g{};
+      g.alpha = 1.0; g.beta = 0.0; g.batch = 1; g.M = m; g.N = m; g.K = m;
+      g.A = h->jJ; g.sAm = m; g.sAk = 1;
+      g.B = h->Fsemi + (int64_t)(No + 1) * N + No + 1; g.sBk = N; g.sBn = 1;
+      g.C = h->jB; g.sCm = m; g.sCn = 1;
+      gemm64(g, st);
       h->launches += 1;
     }
   }
@@ -303,7 +301,7 @@ esmp2_status ensure_vrot(esmp2_handle *h, bool exact) {
     release();
     return check_cuda(h, e, "virtual rotation buffers");
   }
-  // eigenvectors of F_vv without t' (one-sided Jacobi on the rows of B = A, Jt = I)
+  // eigenvectors of F_vv without t' (one-sided Jacobi on the rows of B = Jt A)
   if (m >= 1) {
     const int n2 = (m + (m & 1)) / 2, rounds = m + (m & 1) - 1;
     const unsigned grid = (unsigned)n2;

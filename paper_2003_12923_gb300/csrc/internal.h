@@ -273,7 +273,8 @@ void virt_arrow64(esmp2_handle *h, const double *x, double *y);
 void rotate_occ(esmp2_handle *h, const double *in, double *out, double *tmp, bool to_semi);
 void mode_product_small(const double *in, double *out, int64_t P, int K, int64_t Q, const double *R,
                         cudaStream_t st);
-void eigvecs_block(esmp2_handle *h, const double *F, int off, int m, double *V, double *work);
+esmp2_status eigvecs_occ(esmp2_handle *h, double *Vt);
+void complement_basis(esmp2_handle *h, const double *W, int n, double *J0);
 inline int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }
 
 // Device memory owned by handles: stream-ordered allocations from the device's default

@@ -35,15 +35,15 @@ __global__ void k_f32_to_f64(const float *src, double *dst, int64_t n) {
     dst[e] = (double)src[e];
 }
 
-// R = diag(1, V) (No x No) and its transpose; W2 = diag(R, I_Nv) (N x N)
-__global__ void k_build_rot(const double *V, int No, int Nv, double *R, double *Rt, double *W2) {
+// R = diag(1, V) (No x No; the rows of Vt are the columns of V) and its transpose; W2 = diag(R, I_Nv) (N x N)
+__global__ void k_build_rot(const double *Vt, int No, int Nv, double *R, double *Rt, double *W2) {
   const int N = No + Nv, m = No - 1;
   for (int e = blockIdx.x * blockDim.x + threadIdx.x; e < N * N; e += gridDim.x * blockDim.x) {
     const int p = e / N, q = e % N;
     double v = 0.0;
     if (p < No && q < No) {
       if (p == 0 || q == 0) v = (p == q) ? 1.0 : 0.0;
-      else v = V[(p - 1) * m + (q - 1)];
+      else v = Vt[(q - 1) * m + (p - 1)];
       R[p * No + q] = v;
       Rt[q * No + p] = v;
     } else if (p == q) {
@@ -196,17 +196,19 @@ esmp2_status ensure_mixed(esmp2_handle *h, bool semi) {
     A(reinterpret_cast<void **>(&c.G), sizeof(float) * oN); A(reinterpret_cast<void **>(&c.H), sizeof(float) * oN);
     A(reinterpret_cast<void **>(&c.CYZ), sizeof(float) * oN);
   }
-  double *V = nullptr, *work = nullptr, *W2 = nullptr, *T1 = nullptr;
+  double *V = nullptr, *W2 = nullptr, *T1 = nullptr;
   A(reinterpret_cast<void **>(&V), sizeof(double) * std::max(1, m * m));
-  A(reinterpret_cast<void **>(&work), sizeof(double) * (3 * std::max(1, m * m) + std::max(1, m)));
   A(reinterpret_cast<void **>(&W2), sizeof(double) * (size_t)N * N);
   A(reinterpret_cast<void **>(&T1), sizeof(double) * (size_t)N * N);
   if (e != cudaSuccess) {
-    dfree(V, h->stream); dfree(work, h->stream); dfree(W2, h->stream); dfree(T1, h->stream);
+    dfree(V, h->stream); dfree(W2, h->stream); dfree(T1, h->stream);
     return check_cuda(h, e, "mixed set-up");
   }
   debug_phase(h, "  mixed: allocations");
-  if (m >= 1) eigvecs_block(h, h->F, 1, m, V, work);
+  if (m >= 1 && (s = eigvecs_occ(h, V))) {
+    dfree(V, h->stream); dfree(W2, h->stream); dfree(T1, h->stream);
+    return s;
+  }
   k_build_rot<<<64, 256, 0, h->stream>>>(V, No, Nv, h->Rocc, h->Rocct, W2);
   Gemm64 g{};
   g.alpha = 1.0; g.beta = 0.0; g.batch = 1; g.M = N; g.N = N; g.K = N;
@@ -225,7 +227,7 @@ esmp2_status ensure_mixed(esmp2_handle *h, bool semi) {
     e = cudaMemcpyAsync(rows.data(), h->Fsemi, sizeof(double) * rows.size(), cudaMemcpyDeviceToHost, h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     if (e != cudaSuccess) {
-      dfree(V, h->stream); dfree(work, h->stream); dfree(W2, h->stream); dfree(T1, h->stream);
+      dfree(V, h->stream); dfree(W2, h->stream); dfree(T1, h->stream);
       return check_cuda(h, e, "mixed set-up");
     }
     for (int l = 0; l < 32; ++l) {
@@ -234,7 +236,7 @@ esmp2_status ensure_mixed(esmp2_handle *h, bool semi) {
     }
     h->arrow_w_ready = true;
   }
-  dfree(V, h->stream); dfree(work, h->stream); dfree(W2, h->stream); dfree(T1, h->stream);
+  dfree(V, h->stream); dfree(W2, h->stream); dfree(T1, h->stream);
   h->mixed_ready = true;
   return check_cuda(h, cudaGetLastError(), "mixed set-up");
 }

@@ -40,18 +40,19 @@ __global__ void k_normalise(const double *Cin, double *C, int n) {
   for (int k = threadIdx.x; k < n; k += blockDim.x) C[k] = Cin[k] * scale;
 }
 
-// One-sided Jacobi SVD of C (No x Nv, No <= 64): rotate the rows of B = C with an
+// One-sided Jacobi SVD of C (No x Nv, No <= 64): rotate the rows of B = J^T C with an
 // orthogonal J until they are mutually orthogonal; then C = J diag(|B_k|) (B_k/|B_k|).
-// One warp per row pair, pairs of a round disjoint (round-robin ordering).
+// One warp per row pair, pairs of a round disjoint (round-robin ordering).  On entry Jt holds the
+// eigenvectors of C C^T as rows and B = Jt C: the rows are orthogonal up to the rounding of C C^T, so
+// the sweeps (float64 on one SM: 15 pairs of 400 elements take its pipe 10 us a round) only clean up.
 // Outputs: U (No x No), lam (No), V into columns 0..No-1 of Wv (Nv x Nv).
-__global__ void __launch_bounds__(1024) k_jacobi_svd(const double *C, double *B, double *J, double *U,
+__global__ void __launch_bounds__(1024) k_jacobi_svd(const double *C, double *B, const double *Jt, double *J, double *U,
                                                      double *lam, double *Wv, int No, int Nv) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
   __shared__ int rotated;
   __shared__ int perm[64];
   __shared__ double nrm[64];
-  for (int k = threadIdx.x; k < No * Nv; k += blockDim.x) B[k] = C[k];
-  for (int k = threadIdx.x; k < No * No; k += blockDim.x) J[k] = (k / No == k % No) ? 1.0 : 0.0;
+  for (int k = threadIdx.x; k < No * No; k += blockDim.x) J[k] = Jt[(k % No) * No + k / No];
   __syncthreads();
   const int n = (No & 1) ? No + 1 : No;  // padded with a dummy row when No is odd
   for (int sweep = 0; sweep < 60; ++sweep) {
@@ -112,63 +113,169 @@ __global__ void __launch_bounds__(1024) k_jacobi_svd(const double *C, double *B,
   }
   __syncthreads();
   const double lmax = nrm[perm[0]];
-  // V columns, sign convention, u_k = C v_k / lambda_k.  Done by warp 0 in order so that
-  // columns with a vanishing singular value can be completed against earlier ones.
+  // V columns, sign convention, u_k = C v_k / lambda_k: a warp per column with a singular value
+  // that is not negligible; then warp 0 completes the others (the last ones) in order
+  auto finish = [&](int kk, bool live, double l) {   // column kk of Wv holds v_k up to its sign
+    double best = -1.0;
+    int bi = 0x7fffffff;
+    for (int a = lane; a < Nv; a += 32) {   // argmax |v| (first occurrence)
+      const double v = fabs(Wv[a * Nv + kk]);
+      if (v > best) { best = v; bi = a; }
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+      const double ob = __shfl_xor_sync(0xffffffffu, best, off);
+      const int oi = __shfl_xor_sync(0xffffffffu, bi, off);
+      if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
+    }
+    if (bi >= Nv) bi = 0;   // NaN input
+    const double sg = Wv[bi * Nv + kk] < 0 ? -1.0 : 1.0;
+    __syncwarp();
+    for (int a = lane; a < Nv; a += 32) Wv[a * Nv + kk] *= sg;
+    __syncwarp();
+    for (int i = 0; i < No; ++i) {
+      double u = sg * J[i * No + perm[kk]];
+      if (live) {
+        u = 0.0;
+        for (int a = lane; a < Nv; a += 32) u += C[i * Nv + a] * Wv[a * Nv + kk];
+        u = warp_sum(u) / l;
+      }
+      if (lane == 0) U[i * No + kk] = u;
+    }
+    if (lane == 0) lam[kk] = live ? l : 0.0;
+  };
+  auto is_live = [&](double l) { return l > 1e-12 * lmax && l > 1e-300; };
+  for (int kk = warp; kk < No; kk += nw) {
+    const int o = perm[kk];
+    const double l = nrm[o];
+    if (!is_live(l)) continue;
+    for (int a = lane; a < Nv; a += 32) Wv[a * Nv + kk] = B[o * Nv + a] / l;
+    __syncwarp();
+    finish(kk, true, l);
+  }
+  __syncthreads();
   if (warp == 0) {
     for (int kk = 0; kk < No; ++kk) {
-      const int o = perm[kk];
-      const double l = nrm[o];
-      const bool live = l > 1e-12 * lmax && l > 1e-300;
-      if (live) {
-        for (int a = lane; a < Nv; a += 32) Wv[a * Nv + kk] = B[o * Nv + a] / l;
-      } else {  // Gram-Schmidt completion with the first unit vector that survives
-        for (int m = 0; m < Nv; ++m) {
-          double nn = 0.0;
-          for (int a = lane; a < Nv; a += 32) {
-            double v = (a == m) ? 1.0 : 0.0;
-            for (int prev = 0; prev < kk; ++prev) v -= Wv[m * Nv + prev] * Wv[a * Nv + prev];
-            Wv[a * Nv + kk] = v;
-            nn += v * v;
-          }
-          nn = warp_sum(nn);
-          if (nn > 0.25) {
-            const double inv = 1.0 / sqrt(nn);
-            for (int a = lane; a < Nv; a += 32) Wv[a * Nv + kk] *= inv;
-            break;
-          }
+      if (is_live(nrm[perm[kk]])) continue;
+      for (int m = 0; m < Nv; ++m) {   // Gram-Schmidt completion with the first unit vector that survives
+        double nn = 0.0;
+        for (int a = lane; a < Nv; a += 32) {
+          double v = (a == m) ? 1.0 : 0.0;
+          for (int prev = 0; prev < kk; ++prev) v -= Wv[m * Nv + prev] * Wv[a * Nv + prev];
+          Wv[a * Nv + kk] = v;
+          nn += v * v;
+        }
+        nn = warp_sum(nn);
+        if (nn > 0.25) {
+          const double inv = 1.0 / sqrt(nn);
+          for (int a = lane; a < Nv; a += 32) Wv[a * Nv + kk] *= inv;
+          break;
         }
       }
       __syncwarp();
-      // argmax |v| (first occurrence)
-      double best = -1.0;
-      int bi = 0x7fffffff;
-      for (int a = lane; a < Nv; a += 32) {
-        const double v = fabs(Wv[a * Nv + kk]);
-        if (v > best) { best = v; bi = a; }
-      }
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) {
-        const double ob = __shfl_xor_sync(0xffffffffu, best, off);
-        const int oi = __shfl_xor_sync(0xffffffffu, bi, off);
-        if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
-      }
-      const double sg = Wv[bi * Nv + kk] < 0 ? -1.0 : 1.0;
-      for (int a = lane; a < Nv; a += 32) Wv[a * Nv + kk] *= sg;
-      __syncwarp();
-      for (int i = lane; i < No; i += 32) {
-        double u;
-        if (live) {
-          u = 0.0;
-          for (int a = 0; a < Nv; ++a) u += C[i * Nv + a] * Wv[a * Nv + kk];
-          u /= l;
-        } else {
-          u = sg * J[i * No + o];
-        }
-        U[i * No + kk] = u;
-      }
-      if (lane == 0) lam[kk] = live ? l : 0.0;
+      finish(kk, false, 0.0);
       __syncwarp();
     }
+  }
+}
+
+// Eigenvectors (rows of Vt) of a symmetric matrix A (m x m <= 64 x 64, row pitch ldA, positive
+// semi-definite, or any when shifted: A + (1 + largest absolute row sum) I has the same
+// eigenvectors): one-sided Jacobi on the rows of B = Vt A held in shared memory, a warp per pair.
+// A round is bound by its dependency chain (three reductions, one rotation).
+__global__ void __launch_bounds__(1024) k_eig_small(const double *A, int64_t ldA, int m, int shifted, double *Vt) {
+  extern __shared__ double sm_eig[];
+  double *B = sm_eig, *J = sm_eig + m * m;
+  __shared__ double red[32];
+  __shared__ int rotated;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  double shift = 0.0;
+  if (shifted) {
+    double mx = 0.0;
+    for (int p = warp; p < m; p += nw) {
+      double r = 0.0;
+      for (int q = lane; q < m; q += 32) r += fabs(A[p * ldA + q]);
+      mx = fmax(mx, warp_sum(r));
+    }
+    if (lane == 0) red[warp] = mx;
+    __syncthreads();
+    for (int w = 0; w < nw; ++w) shift = fmax(shift, red[w]);
+    shift += 1.0;
+  }
+  for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
+    const int p = e / m, q = e % m;
+    J[e] = p == q ? 1.0 : 0.0;
+    B[e] = A[p * ldA + q] + (p == q ? shift : 0.0);
+  }
+  __syncthreads();
+  const int n = m + (m & 1);
+  for (int sweep = 0; sweep < 60; ++sweep) {
+    if (threadIdx.x == 0) rotated = 0;
+    __syncthreads();
+    for (int r = 0; r < n - 1; ++r) {
+      for (int pi = warp; pi < n / 2; pi += nw) {
+        int p, q;
+        if (pi == 0) { p = 0; q = 1 + (r % (n - 1)); }
+        else { p = 1 + ((pi + r) % (n - 1)); q = 1 + ((n - 1 - pi + r) % (n - 1)); }
+        if (p > q) { const int t = p; p = q; q = t; }
+        if (q >= m) continue;
+        double *bp = B + p * m, *bq = B + q * m, *jp = J + p * m, *jq = J + q * m;
+        double al = 0.0, be = 0.0, ga = 0.0;
+        for (int k = lane; k < m; k += 32) {
+          const double x = bp[k], y = bq[k];
+          al += x * x; be += y * y; ga += x * y;
+        }
+        al = warp_sum(al); be = warp_sum(be); ga = warp_sum(ga);
+        if (al <= 1e-300 || be <= 1e-300 || fabs(ga) <= 1e-15 * sqrt(al * be)) continue;
+        const double zeta = (be - al) / (2.0 * ga);
+        const double t = (zeta >= 0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
+        const double c = 1.0 / sqrt(1.0 + t * t), s = c * t;
+        for (int k = lane; k < m; k += 32) {
+          const double x = bp[k], y = bq[k], u = jp[k], v = jq[k];
+          bp[k] = c * x - s * y;
+          bq[k] = s * x + c * y;
+          jp[k] = c * u - s * v;
+          jq[k] = s * u + c * v;
+        }
+        if (lane == 0) rotated = 1;
+      }
+      __syncthreads();
+    }
+    const int any = rotated;
+    __syncthreads();
+    if (!any) break;
+  }
+  for (int e = threadIdx.x; e < m * m; e += blockDim.x) Vt[e] = J[e];
+}
+
+// An orthonormal basis of the complement of orbital 0 of the orthogonal W (n x n, its columns the
+// rotated orbitals in the input basis), in the coordinates of the columns 1 .. n-1: the rows
+// j != k of H W without column 0, H the Householder reflector that takes column 0 to the input
+// orbital k of its largest component.  It is as close to the input orbitals as the complement
+// allows, where the Fock matrix is usually close to diagonal, so Jacobi starts from it.
+__global__ void k_complement(const double *W, int n, double *J0) {
+  __shared__ int k_sh;
+  if (threadIdx.x < 32) {
+    double best = -1.0;
+    int bi = 0x7fffffff;
+    for (int a = threadIdx.x; a < n; a += 32) {
+      const double v = fabs(W[(int64_t)a * n]);
+      if (v > best) { best = v; bi = a; }
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+      const double ob = __shfl_xor_sync(0xffffffffu, best, off);
+      const int oi = __shfl_xor_sync(0xffffffffu, bi, off);
+      if (ob > best || (ob == best && oi < bi)) { best = ob; bi = oi; }
+    }
+    if (threadIdx.x == 0) k_sh = bi < n ? bi : 0;   // (0: NaN input)
+  }
+  __syncthreads();
+  const int k = k_sh, m = n - 1;
+  const double vk = W[(int64_t)k * n], f = (vk >= 0.0 ? -1.0 : 1.0) / (1.0 + fabs(vk));
+  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < (int64_t)m * m; e += (int64_t)gridDim.x * blockDim.x) {
+    const int jr = (int)(e / m), b = (int)(e % m) + 1, j = jr < k ? jr : jr + 1;
+    J0[e] = W[(int64_t)j * n + b] + f * W[(int64_t)j * n] * W[(int64_t)k * n + b];
   }
 }
 
@@ -365,39 +472,26 @@ __global__ void __launch_bounds__(256) k_rhs(const double *lam, const double *f0
 #undef F0
 }
 
-// Eigenvectors of a symmetric m x m block M of F (rows/cols off..off+m-1): one-sided
-// Jacobi SVD of M + shift I, with the shift (1 + largest absolute row sum) making it
-// positive definite so that its singular vectors are its eigenvectors.
-__global__ void k_shifted_block(const double *F, int N, int off, int m, double *M) {
-  __shared__ double shift;
-  if (threadIdx.x == 0) {
-    double mx = 0.0;
-    for (int p = 0; p < m; ++p) {
-      double r = 0.0;
-      for (int q = 0; q < m; ++q) r += fabs(F[(int64_t)(off + p) * N + off + q]);
-      mx = fmax(mx, r);
-    }
-    shift = 1.0 + mx;
-  }
-  __syncthreads();
-  for (int e = threadIdx.x; e < m * m; e += blockDim.x) {
-    const int p = e / m, q = e % m;
-    M[e] = F[(int64_t)(off + p) * N + off + q] + (p == q ? shift : 0.0);
-  }
-}
-
 }  // namespace
 
-void eigvecs_block(esmp2_handle *h, const double *F, int off, int m, double *V, double *work) {
-  // work: 3 m^2 + m doubles
-  double *M = work, *B = work + m * m, *J = work + 2 * m * m, *lam = work + 3 * m * m;
-  double *Vt = nullptr;
-  cudaMalloc(&Vt, sizeof(double) * m * m);
-  k_shifted_block<<<1, 256, 0, h->stream>>>(F, h->d.N, off, m, M);
-  k_jacobi_svd<<<1, 1024, 0, h->stream>>>(M, B, J, V, lam, Vt, m, m);
-  h->launches += 2;
-  cudaStreamSynchronize(h->stream);
-  cudaFree(Vt);
+static esmp2_status eig_small(esmp2_handle *h, const double *A, int64_t ldA, int m, int shifted, double *Vt) {
+  const int lim = (int)(sizeof(double) * 2 * 64 * 64);
+  if (cudaError_t e = smem_limit_once(reinterpret_cast<const void *>(k_eig_small), lim)) return check_cuda(h, e, "k_eig_small shared-memory limit");
+  k_eig_small<<<1, 1024, sizeof(double) * 2 * (size_t)m * m, h->stream>>>(A, ldA, m, shifted, Vt);
+  h->launches += 1;
+  return ESMP2_OK;
+}
+
+// rows of J0 ((n-1) x (n-1)): start of the Jacobi rotations in the complement of orbital 0 of W (n x n)
+void complement_basis(esmp2_handle *h, const double *W, int n, double *J0) {
+  k_complement<<<(unsigned)std::min<int64_t>(cdiv((int64_t)(n - 1) * (n - 1), 256), 304), 256, 0, h->stream>>>(W, n, J0);
+  h->launches += 1;
+}
+
+// eigenvectors (rows of Vt) of F_oo without t (from the identity: the columns of U that belong to
+// tiny singular values are orthogonal only to rounding over that value, W_v's always to rounding)
+esmp2_status eigvecs_occ(esmp2_handle *h, double *Vt) {
+  return eig_small(h, h->F + h->d.N + 1, h->d.N, h->d.No - 1, 1, Vt);
 }
 
 esmp2_status check_cuda(esmp2_handle *h, cudaError_t e, const char *what) {
@@ -409,29 +503,37 @@ esmp2_status check_cuda(esmp2_handle *h, cudaError_t e, const char *what) {
 esmp2_status setup_top_basis(esmp2_handle *h) {
   const int No = h->d.No, Nv = h->d.Nv, N = h->d.N;
   cudaStream_t st = h->stream;
-  double *work = nullptr, *Jm = nullptr, *A = nullptr, *R = nullptr, *ww = nullptr, *E = nullptr, *T1 = nullptr;
-  const size_t wbytes = sizeof(double) * (size_t)No * Nv;
-  cudaError_t ce = cudaSuccess;
-  if ((ce = cudaMalloc(&work, wbytes)) != cudaSuccess) return check_cuda(h, ce, "setup alloc");
-  cudaMalloc(&Jm, sizeof(double) * No * No);
-  cudaMalloc(&A, wbytes);
-  cudaMalloc(&R, wbytes);
-  cudaMalloc(&ww, sizeof(double) * No);
-  cudaMalloc(&E, sizeof(double) * (size_t)(Nv - No + 1) * Nv);
-  cudaMalloc(&T1, sizeof(double) * (size_t)N * N);
-  ce = cudaGetLastError();
+  // one pooled workspace: B, A, R (No x Nv each), the Gram matrix, its eigenvectors and J (No x No
+  // each), the reflector norms, AVO scratch, and W^T F's intermediate
+  const size_t nC = (size_t)No * Nv, nO = (size_t)No * No, nE = (size_t)(Nv - No + 1) * Nv, nF = (size_t)N * N;
+  double *ws = nullptr;
+  cudaError_t ce = dmalloc(reinterpret_cast<void **>(&ws), sizeof(double) * (3 * nC + 3 * nO + No + nE + nF), st);
   if (ce != cudaSuccess) return check_cuda(h, ce, "setup alloc");
+  double *work = ws, *A = work + nC, *R = A + nC, *Gm = R + nC, *Jt = Gm + nO, *Jm = Jt + nO, *ww = Jm + nO, *E = ww + No, *T1 = E + nE;
 
   k_normalise<<<1, 1024, 0, st>>>(h->C, h->C, No * Nv);
-  k_jacobi_svd<<<1, 1024, 0, st>>>(h->C, work, Jm, h->U, h->lam, h->Wv, No, Nv);
+  Gemm64 g{};
+  g.alpha = 1.0; g.beta = 0.0; g.batch = 1;
+  g.M = No; g.N = No; g.K = Nv; g.sym = 1;   // C C^T
+  g.A = h->C; g.sAm = Nv; g.sAk = 1;
+  g.B = h->C; g.sBk = 1; g.sBn = Nv;
+  g.C = Gm; g.sCm = No; g.sCn = 1;
+  gemm64(g, st);
+  esmp2_status se = eig_small(h, Gm, No, No, 0, Jt);
+  if (se) { dfree(ws, st); return se; }
+  g.N = Nv; g.K = No; g.sym = 0;             // B = Jt C
+  g.A = Jt; g.sAm = No; g.sAk = 1;
+  g.B = h->C; g.sBk = Nv; g.sBn = 1;
+  g.C = work; g.sCm = Nv; g.sCn = 1;
+  gemm64(g, st);
+  h->launches += 2;
+  k_jacobi_svd<<<1, 1024, 0, st>>>(h->C, work, Jt, Jm, h->U, h->lam, h->Wv, No, Nv);
   k_householder<<<1, 1024, 0, st>>>(h->Wv, A, R, ww, No, Nv);
   const int navo = Nv - No;
   if (navo > 0) k_avo<<<(unsigned)cdiv((int64_t)navo * 32, 256), 256, 0, st>>>(R, ww, E, h->Wv, No, Nv);
   k_assemble_W<<<256, 256, 0, st>>>(h->U, h->Wv, h->W, No, Nv);
   h->launches += 4 + (navo > 0);
   // F_TOP = W^T F W
-  Gemm64 g{};
-  g.alpha = 1.0; g.beta = 0.0; g.batch = 1;
   g.M = N; g.N = N; g.K = N;
   g.A = h->F; g.sAm = N; g.sAk = 1;   // h->F holds the input F here
   g.B = h->W; g.sBk = N; g.sBn = 1;
@@ -444,12 +546,11 @@ esmp2_status setup_top_basis(esmp2_handle *h) {
   k_scalars<<<1, 32, 0, st>>>(h->F, h->lam, h->scal, No, Nv);
   h->launches += 3;
   ce = cudaGetLastError();
-  cudaStreamSynchronize(st);
-  double sc[2];
-  cudaMemcpy(sc, h->scal, sizeof(sc), cudaMemcpyDeviceToHost);
-  h->omega = sc[0];
-  h->E0 = sc[1];
-  cudaFree(work); cudaFree(Jm); cudaFree(A); cudaFree(R); cudaFree(ww); cudaFree(E); cudaFree(T1);
+  dfree(ws, st);
+  if (ce == cudaSuccess) ce = cudaMemcpyAsync(h->hred, h->scal, sizeof(double) * 2, cudaMemcpyDeviceToHost, st);
+  if (ce == cudaSuccess) ce = cudaStreamSynchronize(st);
+  h->omega = h->hred[0];
+  h->E0 = h->hred[1];
   if (ce == cudaSuccess) ce = cudaGetLastError();
   return check_cuda(h, ce, "TOP basis");
 }
