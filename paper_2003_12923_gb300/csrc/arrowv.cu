@@ -462,6 +462,17 @@ esmp2_status x_to_basis(esmp2_handle *h, int target) {
   return check_cuda(h, cudaGetLastError(), "x_to_basis");
 }
 
+// row sums of every slice and column sums of the Z slices (what the symmetric residual needs)
+void virt_arrow_sums(esmp2_handle *h, const double *x) {
+  const int No = h->d.No, Nv = h->d.Nv;
+  const int64_t NN = (int64_t)No * No, S = 5 * NN;
+  KScope ks(h->stream, ESMP2_KT_CONTRACTION, alg_virtual_flops(No, Nv), 6.0 * (double)h->d.n);
+  k_rowsum64<<<1216, 256, 0, h->stream>>>(x, h->Farr, No, Nv, S * Nv, h->rho64);
+  k_colsum64<<<(unsigned)std::min<int64_t>(cdiv(NN * Nv, 256), 4864), 256, 0, h->stream>>>(x + BZ * h->d.B, h->Farr, No, Nv, NN,
+                                                                                         h->kap64 + BZ * NN * Nv);
+  h->launches += 2;
+}
+
 void virt_arrow64(esmp2_handle *h, const double *x, double *y) {
   const int No = h->d.No, Nv = h->d.Nv;
   const int64_t S = 5LL * No * No;

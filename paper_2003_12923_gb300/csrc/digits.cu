@@ -609,8 +609,8 @@ esmp2_status ensure_split(esmp2_handle *h) {
 // sym = 2: as sym = 1, and the S slices (S_ij^ab = S_ji^ba exactly) also take only x F into
 // p64: F x_ij = (x_ji F)^T, so the caller forms y_ij = P_ij + P_ji^T.
 // sym = 0: every slice takes both terms into y (any input).
-// p64: a full block vector (5 blocks).
-esmp2_status virt_split(esmp2_handle *h, const double *x, double *y, double *p64, int sym, int levels) {
+// p64: a full block vector (5 blocks).  join = false: F x stays in p64 (the caller adds it).
+esmp2_status virt_split(esmp2_handle *h, const double *x, double *y, double *p64, int sym, int levels, bool join) {
   if (!split_supported(h, levels)) { h->err = "digit-split contraction not exact for this Nv"; return ESMP2_ERR_UNSUPPORTED; }
   esmp2_status s = ensure_split(h);
   if (s) return s;
@@ -632,6 +632,7 @@ esmp2_status virt_split(esmp2_handle *h, const double *x, double *y, double *p64
   const double per_pair = 2.0 * njobs * (double)Nv * Nv * Nv;
   if ((s = run_digits(h, x, h->jobs[sym], nplain, njobs, h->Fdig, g, levels, sym ? alg_virtual_flops(No, Nv) : per_pair, per_pair)))
     return s;
+  if (!join) return check_cuda(h, cudaGetLastError(), "virt_split");
   const int64_t B = h->d.B;
   if (sym == 0) dg::k_add64<<<2432, 256, 0, h->stream>>>(p64, y, 5 * B);
   else {

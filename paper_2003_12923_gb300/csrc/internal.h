@@ -5,6 +5,7 @@
 #include <cuda_runtime.h>
 #include <cstdint>
 #include <string>
+#include <type_traits>
 
 #include "../../include/esmp2.h"
 
@@ -112,7 +113,7 @@ struct esmp2_handle {
   esmp2::CouplingsT<float> cp32{};
   float *F32 = nullptr;     // float copy of Fsemi (inner solve)
   float arrow_w[64] = {};   // host copy of F32[l][0] (1 <= l < No) and F32[l][No] (l < No)
-  bool arrow_w_ready = false;
+  double arrow_w64[64] = {}; // the same in float64
   __half *dinv32 = nullptr; // Jacobi preconditioner in that basis (n halves)
   double *P64 = nullptr;    // products of the virtual-index pass (float64 sigma workspace, n)
   double *red = nullptr;    // reduction partials
@@ -164,6 +165,7 @@ struct esmp2_handle {
   cudaEvent_t ovvv_ready = nullptr;  // create: the OVVV input copy (side stream) has landed
   bool x_zero = true;       // s64.x is known to be zero (its sigma is zero, no build needed)
   bool r_true = false;      // s64.r holds the true residual -b - A x of s64.x (same basis)
+  bool r_sym = false;       // ... on the independent slices only (residual_sym)
   // float64-accurate virtual-index terms from exact bf16 digit products (tcgen05)
   void *xdig = nullptr;     // digit planes of the stacked rows [levels-1][jobs][Nv][Nvp] bf16
   size_t xdig_bytes = 0;
@@ -210,7 +212,6 @@ esmp2_status sigma64(esmp2_handle *h, const double *x, double *y, int tc_levels 
 // digit-level virtual pass then contracts the S slices with F_vv from one side only
 esmp2_status sigma64_F(esmp2_handle *h, const double *F, int arrow, const double *x, double *y, int tc_levels = 0,
                        int couplings = 1, bool s_sym = false);
-void couple_f32_into(esmp2_handle *h, const double *x, double *y);
 void launch_intermediates64(esmp2_handle *h, const double *F, int arrow, const double *x);
 void launch_couple64(esmp2_handle *h, const double *F, int arrow, const double *x, double *y);
 esmp2_status sigma64_tail(esmp2_handle *h, const double *F, int arrow, const double *x, double *y);
@@ -260,7 +261,13 @@ bool split_supported(const esmp2_handle *h, int levels);
 esmp2_status ensure_split(esmp2_handle *h);
 esmp2_status ensure_slist(esmp2_handle *h);
 esmp2_status ensure_p64(esmp2_handle *h);
-esmp2_status virt_split(esmp2_handle *h, const double *x, double *y, double *p64, int sym, int levels);
+esmp2_status virt_split(esmp2_handle *h, const double *x, double *y, double *p64, int sym, int levels, bool join = true);
+// float64 residual of the refinement on the independent slices (resid.cu)
+int residual_parts();
+esmp2_status residual_sym(esmp2_handle *h, const double *x, const double *b, double *r, int levels);
+int hyll_parts();
+void hylleraas_sym(esmp2_handle *h, const double *b, const double *x, const double *r);
+void virt_arrow_sums(esmp2_handle *h, const double *x);
 esmp2_status xwv_split(esmp2_handle *h, const double *X, int64_t rows, double *Y);
 esmp2_status xwm_split(esmp2_handle *h, const double *X, int64_t rows, double *Y, const double *M, void **dig,
                        int *eM, int eslot);

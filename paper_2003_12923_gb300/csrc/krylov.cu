@@ -720,7 +720,7 @@ esmp2_status solve64(esmp2_handle *h, double tol, int maxit, esmp2_solve_info *i
   double *x = h->s64.x, *r = h->s64.r, *p = h->s64.p, *q = h->s64.q;
   cudaStream_t st = h->stream;
   h->last_precision = virt_tc ? ESMP2_FP64_TC : ESMP2_FP64;
-  h->r_true = false;
+  h->r_true = h->r_sym = false;
   const int lv = virt_tc ? kFp64TcLevels : 0;
   antisym_project(h, x);
   esmp2_status s = ESMP2_OK;
@@ -795,7 +795,11 @@ esmp2_status energy(esmp2_handle *h, esmp2_energy_parts *parts) {
   esmp2_status s = ESMP2_OK;
   if (h->r_true) {
     // the solve ended on a true residual r = -b - A x of this x: A x = -b - r, no sigma build
-    k_hylleraas<<<kRedBlocks, kRedThreads, 0, st>>>(vctx(h, F), bb, h->s64.x, h->s64.r, 1, h->red);
+    if (h->r_sym) hylleraas_sym(h, bb, h->s64.x, h->s64.r);
+    else {
+      k_hylleraas<<<kRedBlocks, kRedThreads, 0, st>>>(vctx(h, F), bb, h->s64.x, h->s64.r, 1, h->red);
+      h->launches += 1;
+    }
   } else {
     // after a tensor-core solve the Hylleraas sigma uses the float64-exact digit levels
     const int lv = (h->last_precision != ESMP2_FP64 && split_supported(h, kFp64TcLevels)) ? kFp64TcLevels : 0;
@@ -803,9 +807,10 @@ esmp2_status energy(esmp2_handle *h, esmp2_energy_parts *parts) {
     else s = sigma64_F(h, F, basis, h->s64.x, h->s64.q, lv);
     if (s) return s;
     k_hylleraas<<<kRedBlocks, kRedThreads, 0, st>>>(vctx(h, F), bb, h->s64.x, h->s64.q, 0, h->red);
+    h->launches += 1;
   }
-  k_finalize<<<1, 256, 0, st>>>(h->red, kRedBlocks, 10, h->red_out, 3);
-  h->launches += 2;
+  k_finalize<<<1, 256, 0, st>>>(h->red, h->r_true && h->r_sym ? hyll_parts() : kRedBlocks, 10, h->red_out, 3);
+  h->launches += 1;
   double sl[32];
   if ((s = read_slots(h, sl, 32))) return s;
   double e_blk[5];
@@ -878,7 +883,7 @@ esmp2_status solve_minres(esmp2_handle *h, double tol, int maxit, esmp2_solve_in
     return ESMP2_ERR_STATE;
   }
   h->last_precision = ESMP2_REDUCED_MINRES;
-  h->r_true = false;
+  h->r_true = h->r_sym = false;
   double sl[32], relres = 1.0, bn = -1.0;
   int iters = 0, nsig = 0, restarts = 0;
   esmp2_status result = ESMP2_ERR_NOT_CONVERGED;
@@ -1075,25 +1080,28 @@ esmp2_status solve_mixed(esmp2_handle *h, double tol, int maxit, esmp2_solve_inf
     int lv_k = lv;
     if (lv && rho_next > 1e1 * tol) lv_k = std::min(lv, split_levels_for(rho_next));
     const bool cold = outer == 0 && h->x_zero;  // cold start: the first true residual is -b
-    bool approx = false;   // formed with reduced accuracy (relative to itself only)
-    if (cold) {
-      lv_k = lv;
+    bool approx = false;   // formed with fewer digit levels (accurate relative to itself only)
+    if (cold) lv_k = lv;
+    else approx = lv_k < lv;
+    // x holds the singlet symmetries exactly (the packed accumulation keeps them bit for bit, the
+    // full-storage path projects x after each step), so the packed solve forms the residual on the
+    // independent amplitudes in one pass; the first one also takes <b, b>
+    h->r_sym = packed && !cold && bb >= 0.0;
+    if (h->r_sym) {
+      if ((s = residual_sym(h, x, bsel, r, lv_k))) return s;
+      k_finalize<<<1, 256, 0, st>>>(h->red, residual_parts(), 1, h->red_out, 3);
+      h->launches += 1;
     } else {
-      // far from the tolerance the coupling pass runs in float32 (its ~1e-7 relative error
-      // is a small fraction of the residual it feeds), next to reduced digit levels
-      const bool c32 = (arrowv || lv_k < lv) && rho_next >= 1e-5;
-      if (arrowv) s = sigma64_arrow(h, x, q, c32 ? 0 : 1);
-      // x holds the singlet symmetries exactly (the packed accumulation keeps them bit for
-      // bit, the full-storage path projects x after each step)
-      else s = sigma64_F(h, h->Fsemi, 1, x, q, lv_k, c32 ? 0 : 1, true);
-      if (s) return s;
-      if (c32) couple_f32_into(h, x, q);
-      approx = c32 || lv_k < lv;
-      ++nsig64;
+      if (!cold) {
+        if (arrowv) s = sigma64_arrow(h, x, q);
+        else s = sigma64_F(h, h->Fsemi, 1, x, q, lv_k, 1, true);
+        if (s) return s;
+      }
+      k_residual<<<kRedBlocks, kRedThreads, 0, st>>>(c, bsel, cold ? nullptr : q, r, h->red, bb < 0.0 ? 1 : 0);
+      k_finalize<<<1, 256, 0, st>>>(h->red, kRedBlocks, 2, h->red_out, 3);
+      h->launches += 2;
     }
-    k_residual<<<kRedBlocks, kRedThreads, 0, st>>>(c, bsel, cold ? nullptr : q, r, h->red, bb < 0.0 ? 1 : 0);
-    k_finalize<<<1, 256, 0, st>>>(h->red, kRedBlocks, 2, h->red_out, 3);
-    h->launches += 2;
+    if (!cold) ++nsig64;
     if ((s = read_slots(h, sl, 32))) return s;
     if (bb < 0.0) bb = sl[9];
     const double rn = std::sqrt(sl[8]), bn = std::sqrt(bb);
@@ -1112,7 +1120,7 @@ esmp2_status solve_mixed(esmp2_handle *h, double tol, int maxit, esmp2_solve_inf
     // projects z = M^-1 r onto the singlet subspace itself, so every search direction and d
     // have the symmetries exactly whatever rounding-level asymmetry r carries; r is then
     // read as it is.
-    if (!rj) singlet_project(h, r);
+    if (!rj && !h->r_sym) singlet_project(h, r);   // residual_sym writes the symmetries exactly
     if (rj) {
       if ((s = packed_rj_init(h, r, kRedBlocks))) return s;
     } else {

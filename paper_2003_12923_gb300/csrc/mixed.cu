@@ -148,28 +148,34 @@ void rotate_occ(esmp2_handle *h, const double *in, double *out, double *tmp, boo
   h->launches += 2;
 }
 
-static esmp2_status alloc_mixed_buffers(esmp2_handle *h) {
-  if (h->xlp) return ESMP2_OK;
+// device flag and the float64 arrow sums (every mixed solve); with `operand` the bf16 copies and
+// the float32 product of a full-storage vector (the tensor-core contraction of such a vector: No > 32 and
+// the API-level contraction)
+static esmp2_status alloc_mixed_buffers(esmp2_handle *h, bool operand) {
   const int No = h->d.No, Nv = h->d.Nv, Nvp = (Nv + 7) & ~7;
-  const size_t n = (size_t)h->d.n;
   cudaError_t e = cudaSuccess;
   auto A = [&](void **p, size_t bytes) {
     if (e == cudaSuccess) e = dmalloc(p, bytes ? bytes : 1, h->stream);
   };
-  A(&h->xlp, sizeof(__nv_bfloat16) * (size_t)5 * No * No * Nv * Nvp);
-  A(&h->Fvlp, sizeof(__nv_bfloat16) * (size_t)Nv * Nvp);
-  A(reinterpret_cast<void **>(&h->ylp), sizeof(float) * n);
-  if (!h->dflag) A(reinterpret_cast<void **>(&h->dflag), sizeof(int));
-  A(reinterpret_cast<void **>(&h->cp.OC1), sizeof(double) * (size_t)5 * No * Nv * Nv);
-  A(reinterpret_cast<void **>(&h->cp.OC2), sizeof(double) * (size_t)5 * No * Nv * Nv);
+  if (!h->dflag) {
+    A(reinterpret_cast<void **>(&h->dflag), sizeof(int));
+    if (e == cudaSuccess) cudaMemsetAsync(h->dflag, 0, sizeof(int), h->stream);
+  }
+  if (!h->cp.OC1) A(reinterpret_cast<void **>(&h->cp.OC1), sizeof(double) * (size_t)5 * No * Nv * Nv);
+  if (!h->cp.OC2) A(reinterpret_cast<void **>(&h->cp.OC2), sizeof(double) * (size_t)5 * No * Nv * Nv);
+  if (operand && !h->ylp) {
+    A(&h->xlp, sizeof(__nv_bfloat16) * (size_t)5 * No * No * Nv * Nvp);
+    A(&h->Fvlp, sizeof(__nv_bfloat16) * (size_t)Nv * Nvp);
+    A(reinterpret_cast<void **>(&h->ylp), sizeof(float) * (size_t)h->d.n);
+    if (e == cudaSuccess) fvv_bf16(h, h->F, h->Fvlp);  // the virtual block is the same in both bases
+  }
   if (e != cudaSuccess) return check_cuda(h, e, "mixed buffers");
-  cudaMemsetAsync(h->dflag, 0, sizeof(int), h->stream);
-  fvv_bf16(h, h->F, h->Fvlp);  // the virtual block is the same in both bases
   return check_cuda(h, cudaGetLastError(), "mixed buffers");
 }
 
 esmp2_status ensure_mixed(esmp2_handle *h, bool semi) {
-  esmp2_status s = alloc_mixed_buffers(h);
+  const bool full = h->d.No > 32;   // inner vectors in full storage (the packed solve has its own)
+  esmp2_status s = alloc_mixed_buffers(h, full || !semi);
   if (s || !semi || h->mixed_ready) return s;
   const int No = h->d.No, Nv = h->d.Nv, N = h->d.N, m = No - 1;
   const size_t n = (size_t)h->d.n;
@@ -181,12 +187,13 @@ esmp2_status ensure_mixed(esmp2_handle *h, bool semi) {
   A(reinterpret_cast<void **>(&h->Rocct), sizeof(double) * No * No);
   A(reinterpret_cast<void **>(&h->Fsemi), sizeof(double) * (size_t)N * N);
   A(reinterpret_cast<void **>(&h->bsemi), sizeof(double) * n);
-  A(reinterpret_cast<void **>(&h->r32), sizeof(float) * n);
-  A(reinterpret_cast<void **>(&h->p32), sizeof(float) * n);
-  A(reinterpret_cast<void **>(&h->q32), sizeof(float) * n);
-  A(reinterpret_cast<void **>(&h->x32), sizeof(float) * n);
   A(reinterpret_cast<void **>(&h->F32), sizeof(float) * (size_t)N * N);
-  {
+  if (full) {
+    A(reinterpret_cast<void **>(&h->r32), sizeof(float) * n);
+    A(reinterpret_cast<void **>(&h->p32), sizeof(float) * n);
+    A(reinterpret_cast<void **>(&h->q32), sizeof(float) * n);
+    A(reinterpret_cast<void **>(&h->x32), sizeof(float) * n);
+
     const size_t ooN = (size_t)No * No * Nv, oNN = (size_t)No * Nv * Nv, oN = (size_t)No * Nv;
     auto &c = h->cp32;
     A(reinterpret_cast<void **>(&c.VX), sizeof(float) * ooN); A(reinterpret_cast<void **>(&c.GP), sizeof(float) * ooN);
@@ -233,8 +240,9 @@ esmp2_status ensure_mixed(esmp2_handle *h, bool semi) {
     for (int l = 0; l < 32; ++l) {
       h->arrow_w[l] = (l >= 1 && l < No) ? (float)rows[(size_t)l * N] : 0.f;
       h->arrow_w[32 + l] = l < No ? (float)rows[(size_t)l * N + No] : 0.f;
+      h->arrow_w64[l] = (l >= 1 && l < No) ? rows[(size_t)l * N] : 0.0;
+      h->arrow_w64[32 + l] = l < No ? rows[(size_t)l * N + No] : 0.0;
     }
-    h->arrow_w_ready = true;
   }
   dfree(V, h->stream); dfree(W2, h->stream); dfree(T1, h->stream);
   h->mixed_ready = true;

@@ -156,79 +156,16 @@ __global__ void k_inter_d(CtxT<CT> c, const T *x, CouplingsT<CT> cp) {
   }
 }
 
-// (b) in one pass for the arrow form (No <= 32): a thread owns one (blk, a, b) and reads
-// the block's No x No occupied matrix at that (a, b) once; its row sums give OC2 (and OZ
-// on Z), its column sums OC1 (and OX on X), the column sums held in registers.  The
-// weights F_l0 (l >= 1) and F_l,t' travel as launch parameters, so the unrolled sums take
-// them as constant operands instead of registers or shared-memory loads.
-// BLK < 0: grid.y runs over T, S, Y (no OX/OZ terms); else the one block BLK.
-struct ArrowW {
-  float fl[32];  // F_l0 for 1 <= l < No, else 0
-  float fk[32];  // F_l,t' for l < No, else 0
-};
-template <int BLK, typename T, typename CT>
-__global__ void __launch_bounds__(128, 4) k_inter_b1(CtxT<CT> c, const T *__restrict__ x, CouplingsT<CT> cp,
-                                                     const ArrowW w) {
-  const int No = c.No;
-  const int blk = BLK >= 0 ? BLK : (blockIdx.y == 0 ? BT : (blockIdx.y == 1 ? BS : BY));
-  const int64_t NvNv = (int64_t)c.Nv * c.Nv, n = (int64_t)No * NvNv;
-  const T *xb = x + blk * c.B;
-  CT *oc1 = cp.OC1 + blk * n, *oc2 = cp.OC2 + blk * n;
-  for (int64_t ab = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; ab < NvNv; ab += (int64_t)gridDim.x * blockDim.x) {
-    CT o1[32];
-    CT ox[BLK == BX ? 32 : 1];
-#pragma unroll
-    for (int m = 0; m < 32; ++m) o1[m] = CT(0);
-#pragma unroll
-    for (int m = 0; m < (BLK == BX ? 32 : 1); ++m) ox[m] = CT(0);
-    for (int l = 0; l < No; ++l) {
-      const T *row = xb + (int64_t)l * n + ab;
-      const CT fll = w.fl[l], fkl = w.fk[l];
-      CT r2 = CT(0), rz = CT(0);
-#pragma unroll
-      for (int m = 0; m < 32; ++m) {
-        if (m < No) {
-          const CT v = (CT)row[(int64_t)m * NvNv];
-          o1[m] += fll * v;
-          r2 += w.fl[m] * v;
-          if constexpr (BLK == BX) ox[m] += fkl * v;
-          if constexpr (BLK == BZ) rz += w.fk[m] * v;
-        }
-      }
-      oc2[(int64_t)l * NvNv + ab] = r2;
-      if constexpr (BLK == BZ) cp.OZ[(int64_t)l * NvNv + ab] = rz;
-    }
-#pragma unroll
-    for (int m = 0; m < 32; ++m) {
-      if (m < No) {
-        oc1[(int64_t)m * NvNv + ab] = o1[m];
-        if constexpr (BLK == BX) cp.OX[(int64_t)m * NvNv + ab] = ox[m];
-      }
-    }
-  }
-}
-
 template <typename T, typename CT>
 void launch_inter(esmp2_handle *h, const CtxT<CT> &c, const T *x, const CouplingsT<CT> &cp) {
   k_inter_a<T, CT><<<1216, 256, 0, h->stream>>>(c, x, cp);
-  bool one_pass = false;
-  if constexpr (sizeof(CT) == 4) one_pass = c.arrow && c.No <= 32 && h->arrow_w_ready;
-  if (one_pass) {
-    if constexpr (sizeof(CT) == 4) {
-      ArrowW w;
-      for (int l = 0; l < 32; ++l) { w.fl[l] = h->arrow_w[l]; w.fk[l] = h->arrow_w[32 + l]; }
-      const unsigned gx = (unsigned)std::min<int64_t>(cdiv((int64_t)c.Nv * c.Nv, 128), 8192);
-      k_inter_b1<-1, T, CT><<<dim3(gx, 3), 128, 0, h->stream>>>(c, x, cp, w);
-      k_inter_b1<BX, T, CT><<<gx, 128, 0, h->stream>>>(c, x, cp, w);
-      k_inter_b1<BZ, T, CT><<<gx, 128, 0, h->stream>>>(c, x, cp, w);
-      h->launches += 2;
-    }
-  } else {
+  if (c.arrow != 2) {   // 2: the sums over an occupied index come from the caller
     k_inter_b<T, CT><<<1216, 256, 0, h->stream>>>(c, x, cp);
+    h->launches += 1;
   }
   k_inter_c<T, CT><<<1216, 256, 0, h->stream>>>(c, x, cp);
   k_inter_d<T, CT><<<(unsigned)cdiv(3LL * c.No * c.Nv, 256), 256, 0, h->stream>>>(c, x, cp);
-  h->launches += 4;
+  h->launches += 3;
 }
 
 // Vector loads/stores of VW consecutive elements (16 bytes when VW * sizeof(T) == 16); the
@@ -801,45 +738,6 @@ void combine_s(esmp2_handle *h, double *y) {
   const int64_t nblocks = (int64_t)No * No * tiles * tiles;
   k_combine_s<<<(unsigned)nblocks, 256, 0, h->stream>>>(No, Nv, h->P64, y);
   h->launches += 1;
-}
-
-namespace {
-__global__ void k_round_f32(const double *src, float *dst, int64_t n) {
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x)
-    dst[e] = (float)src[e];
-}
-// y += (double) y32 on amplitude slots, y = 0 on the others; a warp per row (block, i, j, a)
-__global__ void k_add_f32_masked(const float *src, double *dst, int No, int Nv) {
-  const int64_t rows = 5LL * No * No * Nv;
-  const int lane = threadIdx.x & 31;
-  for (int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5; r < rows;
-       r += ((int64_t)gridDim.x * blockDim.x) >> 5) {
-    const int a = (int)(r % Nv);
-    int64_t f = r / Nv;
-    const int j = (int)(f % No);
-    f /= No;
-    const int i = (int)(f % No), blk = (int)(f / No);
-    for (int b = lane; b < Nv; b += 32) {
-      const int64_t e = r * Nv + b;
-      dst[e] = valid_elem(blk, i, j, a, b) ? dst[e] + (double)src[e] : 0.0;
-    }
-  }
-}
-}  // namespace
-
-// Couplings, shifts, arrow terms and masks of y = A x in float32, added to the float64 y
-// (semicanonical-occupied basis): x rounded to float into the inner p buffer, the inner
-// coupling pass on it into the inner q buffer, the result added in float64 and the
-// non-amplitude slots cleared.  For the intermediate true residuals of the refinement,
-// which need A x to about 1e-7 of |A x| only; the float64 coupling pass runs at the
-// float64 rate.
-void couple_f32_into(esmp2_handle *h, const double *x, double *y) {
-  const int64_t n = h->d.n;
-  k_round_f32<<<1216, 256, 0, h->stream>>>(x, h->p32, n);
-  cudaMemsetAsync(h->q32, 0, sizeof(float) * (size_t)n, h->stream);
-  couple32(h, h->arrowv ? h->F32arr : h->F32, h->p32, h->q32);
-  k_add_f32_masked<<<1216, 256, 0, h->stream>>>(h->q32, y, h->d.No, h->d.Nv);
-  h->launches += 2;
 }
 
 // float64 sigma with an arbitrary orthonormal-basis Fock matrix F (t = occupied 0, t' =
