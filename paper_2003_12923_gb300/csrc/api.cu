@@ -296,7 +296,7 @@ esmp2_status esmp2_get_solution(esmp2_handle *h, double *x) {
       if (esmp2_status s = rotate_virt(h, src, x, h->s64.p, false)) return s;
       src = x;
     }
-    rotate_occ(h, src, x, h->s64.p, false);
+    if (esmp2_status s = rotate_occ(h, src, x, h->s64.p, false)) return s;
   }
   return check_cuda(h, cudaGetLastError(), "get_solution");
 }

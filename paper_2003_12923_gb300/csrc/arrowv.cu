@@ -446,12 +446,12 @@ esmp2_status x_to_basis(esmp2_handle *h, int target) {
     h->x_basis = 1;
   }
   if (target == 0 && h->x_basis == 1) {
-    rotate_occ(h, x, x, tmp, false);
+    if ((s = rotate_occ(h, x, x, tmp, false))) return s;
     h->x_basis = 0;
   }
   if (target >= 1 && h->x_basis == 0) {
     if ((s = ensure_mixed(h, true))) return s;
-    rotate_occ(h, x, x, tmp, true);
+    if ((s = rotate_occ(h, x, x, tmp, true))) return s;
     h->x_basis = 1;
   }
   if (target == 2 && h->x_basis == 1) {

@@ -1,0 +1,76 @@
+// Digit split of a float64 element and the integer join of the level sums (digits.cu, narrow.cu).
+#pragma once
+#include <cstdint>
+
+namespace esmp2 {
+
+// V 2^e as float64, V rounded to 53 bits; integer operations only
+__device__ __forceinline__ double scale_i64(long long V, int e) {
+  if (V == 0) return 0.0;
+  unsigned long long u = V < 0 ? 0ull - (unsigned long long)V : (unsigned long long)V;
+  const int lz = __clzll((long long)u);
+  u <<= lz;
+  const unsigned long long m = (u >> 11) + ((u >> 10) & 1);   // in [2^52, 2^53]
+  const int eb = 1023 + 63 - lz + e;                          // biased exponent of the leading bit
+  unsigned long long bits = ((unsigned long long)(eb - 1) << 52) + m;
+  if (eb <= 0) bits = 0;
+  if (eb >= 2047) bits = 0x7FF0000000000000ull;
+  if (V < 0) bits |= 0x8000000000000000ull;
+  return __longlong_as_double((long long)bits);
+}
+
+// Digits of one element.  The magnitude is split, U = |Z| + sum_k 32 64^k over the lower P - 1 digits, so
+// that digit p >= 2 of |Z| is field - 32 and digit 1 the rest; the sign goes to every digit, so -v has
+// the negated digits and its products (with the dropped pairs of low weight) are exactly the
+// negated ones.  |Z| by shifts of the significand (round half up): float64 arithmetic would cost two
+// operations of its slow pipe.
+template <int P>
+__device__ __forceinline__ long long digit_word(double v, int es) {
+  constexpr long long bias = (((1ll << (6 * (P - 1))) - 1) / 63) * 32;
+  const unsigned long long u = (unsigned long long)__double_as_longlong(v);
+  const int ef = (int)(u >> 52) & 0x7FF;
+  const int sh = 1075 - ef + es - 6 * P;   // >= 0 for every finite |v| < 2^(es - 1)
+  unsigned long long m = (u & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull;
+  if (sh > 0) m = sh < 55 && ef != 0 ? ((m >> (sh - 1)) + 1) >> 1 : 0;
+  if (ef == 0x7FF) m = 1ull << (6 * P - 1);   // an infinity or NaN saturates
+  return (long long)m + bias;
+}
+// digit p (1-based) of the magnitude as the high half of its float32 (a bf16)
+template <int P>
+__device__ __forceinline__ uint32_t digit_bits(long long U, int p) {
+  const int sh = 6 * (P - p);
+  if (p == 1) return __float_as_uint(__uint_as_float(0x4B400000u + (uint32_t)(int)(U >> sh)) - 12582912.0f);
+  return __float_as_uint(__uint_as_float(0x4B400000u | ((uint32_t)(U >> sh) & 63u)) - 12582944.0f);
+}
+// the signs of two elements as they stand in a packed pair of bf16 digits
+__device__ __forceinline__ uint32_t sign_pair(double v0, double v1) {
+  return ((uint32_t)__double2hiint(v0) >> 16 & 0x8000u) | ((uint32_t)__double2hiint(v1) & 0x80000000u);
+}
+// digit p of two elements, packed
+template <int P>
+__device__ __forceinline__ uint32_t digit_pair(long long U0, long long U1, uint32_t sg, int p) {
+  return __byte_perm(digit_bits<P>(U0, p), digit_bits<P>(U1, p), 0x7632) ^ sg;
+}
+// Integer-valued accumulators v[0 .. NL-1] (levels 2 .. NL + 1 of one element) joined at the weight of
+// the last one, for NL <= 8: sum_l v[l] 64^(NL-1-l).  SMALL: every |v| < 2^22, so that the integer is
+// read off the bits of v + 1.5 2^23 (two full-rate operations; conversions run at an eighth of the rate);
+// else |v| < 2^23, converted.
+template <int NL, bool SMALL>
+__device__ __forceinline__ long long join_levels(const float (&v)[NL]) {
+  constexpr uint32_t C = 0x4B400000u;   // bits of 1.5 2^23
+  auto bits = [&](int l) -> uint32_t {
+    return SMALL ? __float_as_uint(v[l] + 12582912.0f) : (uint32_t)__float2int_rn(v[l]);
+  };
+  auto pair = [&](int l) -> int {       // two levels fit 32 bits
+    return (int)(bits(l) * 64u + bits(l + 1) - (SMALL ? C * 65u : 0u));
+  };
+  long long V = pair(0);
+#pragma unroll
+  for (int l = 2; l + 1 < NL; l += 2) V = V * 4096 + pair(l);
+  if constexpr (NL & 1) V = V * 64 + (int)(bits(NL - 1) - (SMALL ? C : 0u));
+  return V;
+}
+// v / 64 rounded half away from zero (odd in v)
+__device__ __forceinline__ int round64(int v) { return (v + 31 + (v >= 0 ? 1 : 0)) >> 6; }
+
+}  // namespace esmp2

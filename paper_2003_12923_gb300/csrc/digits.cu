@@ -3,9 +3,9 @@
 // GB300's float64 pipe (two multiply-adds per clock and SM) out of the inner loop.
 //
 // Digits (Ozaki-type splitting): with 2^e the smallest power of two above 2 max |x_s|, z = x / 2^e
-// lies in (-1/2, 1/2); Z = round(z 64^P) is an integer of magnitude <= 2^(6P-1) and its balanced
-// base-64 digits Z = sum_{p=1..P} d_p 64^(P-p), d_p in [-32, 31] (d_1 in [-32, 32]), give z to
-// within 64^-P / 2.  Every digit is exact in bf16, every product of two an integer of magnitude
+// lies in (-1/2, 1/2); Z = round(z 64^P) is an integer of magnitude <= 2^(6P-1) and the balanced
+// base-64 digits of |Z|, Z = +-sum_{p=1..P} d_p 64^(P-p), d_p in [-32, 31] (d_1 in [0, 32]), give z
+// to within 64^-P / 2.  Every digit is exact in bf16, every product of two an integer of magnitude
 // <= 2^10.  Level L = p + q collects the digit pairs of one weight in one fp32 accumulator: a sum
 // over K = Nv of at most L - 1 pairs stays below 2^24 whenever Nv (L - 1) 2^10 < 2^24, so the
 // tensor cores add exactly.  The levels 2 .. Lmax are joined as integers and rounded to float64
@@ -19,6 +19,7 @@
 #include <algorithm>
 #include <cmath>
 
+#include "digit_split.h"
 #include "internal.h"
 #include "tc_ptx.h"
 
@@ -71,22 +72,7 @@ struct Args {
   int *err;
 };
 
-// V 2^e as float64, V rounded to 53 bits; integer operations only
-__device__ __forceinline__ double scale_i64(long long V, int e) {
-  if (V == 0) return 0.0;
-  unsigned long long u = V < 0 ? 0ull - (unsigned long long)V : (unsigned long long)V;
-  const int lz = __clzll((long long)u);
-  u <<= lz;
-  const unsigned long long m = (u >> 11) + ((u >> 10) & 1);   // in [2^52, 2^53]
-  const int eb = 1023 + 63 - lz + e;                          // biased exponent of the leading bit
-  unsigned long long bits = ((unsigned long long)(eb - 1) << 52) + m;
-  if (eb <= 0) bits = 0;
-  if (eb >= 2047) bits = 0x7FF0000000000000ull;
-  if (V < 0) bits |= 0x8000000000000000ull;
-  return __longlong_as_double((long long)bits);
-}
-
-template <int NLEV>
+template <int NLEV, bool SMALL>   // SMALL: every level sum is below 2^22
 __global__ void __launch_bounds__(NTHREADS, 1)
     k_levels(const __grid_constant__ CUtensorMap tA, const __grid_constant__ CUtensorMap tF,
              const __grid_constant__ Args g) {
@@ -219,18 +205,14 @@ __global__ void __launch_bounds__(NTHREADS, 1)
         tmem_wait();
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
-          int iv[NLEV];
-#pragma unroll
-          for (int l = 0; l < NLEV; ++l) {
-            keep(r[l][c]);
-            iv[l] = __float2int_rn(__uint_as_float(r[l][c]));   // |.| < 2^23: two levels fit an int32
-          }
           constexpr int NI = NLEV < 8 ? NLEV : 8;
-          long long v = iv[0] * 64 + iv[1];
+          float f[NI];
 #pragma unroll
-          for (int l = 2; l + 1 < NI; l += 2) v = v * 4096 + (iv[l] * 64 + iv[l + 1]);
-          if constexpr (NI & 1) v = v * 64 + iv[NI - 1];
-          if constexpr (NLEV > 8) v += (iv[8] + 32) >> 6;
+          for (int l = 0; l < NLEV; ++l) keep(r[l][c]);
+#pragma unroll
+          for (int l = 0; l < NI; ++l) f[l] = __uint_as_float(r[l][c]);
+          long long v = join_levels<NI, SMALL>(f);
+          if constexpr (NLEV > 8) v += round64(__float2int_rn(__uint_as_float(r[8][c])));
           V[c8 * 8 + c] = v;
         }
       }
@@ -338,29 +320,6 @@ __global__ void __launch_bounds__(256) k_slice_exp(const double *x, int n /* Nv^
   }
 }
 
-// Digits of one element as packed fields: U = Z + sum_k 32 64^k over the lower P - 1 digits, so that
-// digit p >= 2 is field - 32 and digit 1 the (signed) rest.  Z by shifts of the significand
-// (round half away from zero): float64 arithmetic would cost two operations of its slow pipe.
-template <int P>
-__device__ __forceinline__ long long digit_word(double v, int es) {
-  constexpr long long bias = (((1ll << (6 * (P - 1))) - 1) / 63) * 32;
-  const unsigned long long u = (unsigned long long)__double_as_longlong(v);
-  const int ef = (int)(u >> 52) & 0x7FF;
-  const int sh = 1075 - ef + es - 6 * P;   // >= 0 for every finite |v| < 2^(es - 1)
-  unsigned long long m = (u & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull;
-  if (sh > 0) m = sh < 55 && ef != 0 ? ((m >> (sh - 1)) + 1) >> 1 : 0;
-  if (ef == 0x7FF) m = 1ull << (6 * P - 1);   // an infinity or NaN saturates
-  const long long Z = (long long)u < 0 ? -(long long)m : (long long)m;
-  return Z + bias;
-}
-// digit p (1-based) as the high half of its float32 (a bf16)
-template <int P>
-__device__ __forceinline__ uint32_t digit_bits(long long U, int p) {
-  const int sh = 6 * (P - p);
-  if (p == 1) return __float_as_uint(__uint_as_float(0x4B400000u + (uint32_t)(int)(U >> sh)) - 12582912.0f);
-  return __float_as_uint(__uint_as_float(0x4B400000u | ((uint32_t)(U >> sh) & 63u)) - 12582944.0f);
-}
-
 // Digit planes of the stacked rows, out[p][job Nv + a][c] (row pitch Nvp, pad columns zero): plain
 // jobs row by row, a warp per row and two columns per lane (one 128-byte line per plane and warp).
 template <int P>
@@ -385,10 +344,10 @@ __global__ void __launch_bounds__(256) k_digits(const double *x, int Nv, int Nvp
         if (c + 1 < Nv) v.y = src[c + 1];
       }
       const long long U0 = digit_word<P>(v.x, e), U1 = digit_word<P>(v.y, e);
+      const uint32_t sg = sign_pair(v.x, v.y);
 #pragma unroll
       for (int p = 1; p <= P; ++p)
-        *reinterpret_cast<uint32_t *>(dst + (p - 1) * plane + c) =
-            __byte_perm(digit_bits<P>(U0, p), digit_bits<P>(U1, p), 0x7632);
+        *reinterpret_cast<uint32_t *>(dst + (p - 1) * plane + c) = digit_pair<P>(U0, U1, sg, p);
     }
   }
 }
@@ -413,11 +372,11 @@ __global__ void __launch_bounds__(256) k_digits_t(const double *x, int Nv, int N
     if (c0 + c >= Nvp) continue;
     for (int q = w; q < 32 && a0 + q < Nv; q += 8) {
       const long long U0 = digit_word<P>(t[c][q], e), U1 = digit_word<P>(t[c + 1][q], e);
+      const uint32_t sg = sign_pair(t[c][q], t[c + 1][q]);
       __nv_bfloat16 *dst = out + ((int64_t)job * Nv + a0 + q) * Nvp + c0 + c;
 #pragma unroll
       for (int p = 1; p <= P; ++p)
-        *reinterpret_cast<uint32_t *>(dst + (p - 1) * plane) =
-            __byte_perm(digit_bits<P>(U0, p), digit_bits<P>(U1, p), 0x7632);
+        *reinterpret_cast<uint32_t *>(dst + (p - 1) * plane) = digit_pair<P>(U0, U1, sg, p);
     }
   }
 }
@@ -480,7 +439,9 @@ const char *launch_levels(cudaStream_t st, const void *xd, int64_t xplane, const
   CUtensorMap mA, mF;
   if (!digit_map(&mA, xd, Nvp, g.R, xplane, NLEV, dg::BM) || !digit_map(&mF, Fd, Nvp, Nv, (int64_t)Nv * Nvp, Fplanes, BN))
     return "tensor map encoding failed";
-  if (smem_limit_once(reinterpret_cast<const void *>(dg::k_levels<NLEV>), smem) != cudaSuccess)
+  const bool small = (int64_t)Nv * NLEV * 1024 < (1 << 22);
+  const void *fn = small ? reinterpret_cast<const void *>(dg::k_levels<NLEV, true>) : reinterpret_cast<const void *>(dg::k_levels<NLEV, false>);
+  if (smem_limit_once(fn, smem) != cudaSuccess)
     return "cannot raise the shared-memory limit of the digit-level kernel";
   g.n_tiles = (Nv + BN - 1) / BN;
   g.nk = (Nv + dg::BK - 1) / dg::BK;
@@ -488,7 +449,9 @@ const char *launch_levels(cudaStream_t st, const void *xd, int64_t xplane, const
   int dev = 0, sms = 148;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  dg::k_levels<NLEV><<<(unsigned)std::min<int64_t>(g.tiles, sms), dg::NTHREADS, smem, st>>>(mA, mF, g);
+  const unsigned grid = (unsigned)std::min<int64_t>(g.tiles, sms);
+  if (small) dg::k_levels<NLEV, true><<<grid, dg::NTHREADS, smem, st>>>(mA, mF, g);
+  else dg::k_levels<NLEV, false><<<grid, dg::NTHREADS, smem, st>>>(mA, mF, g);
   return nullptr;
 }
 
@@ -556,6 +519,20 @@ bool split_supported(const esmp2_handle *h, int levels) {
   return 2LL * h->d.Nv * (levels - 1) * 1024 < (1LL << 24);
 }
 
+// binary exponents of n contiguous Nv x Nv slices
+void slice_exponents(esmp2_handle *h, const double *x, int n, int *es) {
+  dg::k_slice_exp<<<n, 256, 0, h->stream>>>(x, h->d.Nv * h->d.Nv, es, nullptr);
+  h->launches += 1;
+}
+
+// device error flag of the bounded waits
+esmp2_status ensure_dflag(esmp2_handle *h) {
+  if (h->dflag) return ESMP2_OK;
+  cudaError_t e = dmalloc(reinterpret_cast<void **>(&h->dflag), sizeof(int), h->stream);
+  if (e != cudaSuccess) { h->dflag = nullptr; return check_cuda(h, e, "device flag"); }
+  return check_cuda(h, cudaMemsetAsync(h->dflag, 0, sizeof(int), h->stream), "device flag");
+}
+
 // plain slices of the symmetric forms (T, X, Y with i < j, all of S and Z)
 esmp2_status ensure_slist(esmp2_handle *h) {
   if (h->slist) return ESMP2_OK;
@@ -588,11 +565,7 @@ esmp2_status ensure_split(esmp2_handle *h) {
     h->Fdig = nullptr; h->es = nullptr;
     return check_cuda(h, e, "split workspace");
   }
-  if (!h->dflag) {
-    if ((e = dmalloc(reinterpret_cast<void **>(&h->dflag), sizeof(int), h->stream)) != cudaSuccess)
-      return check_cuda(h, e, "split workspace");
-    cudaMemsetAsync(h->dflag, 0, sizeof(int), h->stream);
-  }
+  if (esmp2_status s0 = ensure_dflag(h)) return s0;
   // digits of F_vv (the same block in the TOP and the semicanonical-occupied basis); the
   // leading digits do not depend on how many are kept
   const double *Fv = h->F + (int64_t)No * N + No;
@@ -643,22 +616,9 @@ esmp2_status virt_split(esmp2_handle *h, const double *x, double *y, double *p64
   return check_cuda(h, cudaGetLastError(), "virt_split");
 }
 
-// Y = X M (rows x Nv times an Nv x Nv matrix M, rows a multiple of Nv) in float64 accuracy from
-// exact digit products on the tensor cores (ten levels): the right-factor form of the orbital
-// rotations (M = W_v for the integral transforms, the virtual rotation of the reduced-cost
-// basis).  X is read as rows/Nv slices of Nv x Nv.  The digit planes of M^T (row b' holds column
-// b' of M, the K-major right operand) are built on first use into *dig with the power-of-two
-// scale in es[eslot] (device) and *eM (host).
-esmp2_status xwm_split(esmp2_handle *h, const double *X, int64_t rows, double *Y, const double *M, void **dig,
-                       int *eM, int eslot) {
-  esmp2_status s = ensure_split(h);
-  if (s) return s;
+// the digit planes of M^T (Nv x Nv), built on first use
+static esmp2_status ensure_matrix_digits(esmp2_handle *h, const double *M, void **dig, int *eM, int eslot) {
   const int No = h->d.No, Nv = h->d.Nv, Nvp = (Nv + 7) & ~7;
-  const int S = (int)(rows / Nv), levels = dg::kMaxLevels;
-  if (rows % Nv != 0 || S > 5 * No * No || (int64_t)(levels - 1) * Nv * 1024 >= (1LL << 24)) {
-    h->err = "xwm_split: unsupported shape";
-    return ESMP2_ERR_UNSUPPORTED;
-  }
   if (!*dig) {
     cudaError_t e = dmalloc(dig, sizeof(__nv_bfloat16) * (size_t)kDigitPlanes * Nv * Nvp, h->stream);
     if (e != cudaSuccess) return check_cuda(h, e, "rotation digits");
@@ -670,6 +630,26 @@ esmp2_status xwm_split(esmp2_handle *h, const double *X, int64_t rows, double *Y
     h->launches += 2;
     if (e != cudaSuccess) return check_cuda(h, e, "rotation digits");
   }
+  return ESMP2_OK;
+}
+
+// Y = X M (rows x Nv times an Nv x Nv matrix M, rows a multiple of Nv) in float64 accuracy from
+// exact digit products on the tensor cores (ten levels): the right-factor form of the orbital
+// rotations (M = W_v for the integral transforms, the virtual rotation of the reduced-cost
+// basis).  X is read as rows/Nv slices of Nv x Nv.  The digit planes of M^T (row b' holds column
+// b' of M, the K-major right operand) are built on first use into *dig with the power-of-two
+// scale in es[eslot] (device) and *eM (host).
+esmp2_status xwm_split(esmp2_handle *h, const double *X, int64_t rows, double *Y, const double *M, void **dig,
+                       int *eM, int eslot) {
+  esmp2_status s = ensure_split(h);
+  if (s) return s;
+  const int No = h->d.No, Nv = h->d.Nv;
+  const int S = (int)(rows / Nv), levels = dg::kMaxLevels;
+  if (rows % Nv != 0 || S > 5 * No * No || (int64_t)(levels - 1) * Nv * 1024 >= (1LL << 24)) {
+    h->err = "xwm_split: unsupported shape";
+    return ESMP2_ERR_UNSUPPORTED;
+  }
+  if ((s = ensure_matrix_digits(h, M, dig, eM, eslot))) return s;
   dg::k_slice_exp<<<S, 256, 0, h->stream>>>(X, Nv * Nv, h->es, nullptr);
   h->launches += 1;
   dg::Args g{};
@@ -681,6 +661,12 @@ esmp2_status xwm_split(esmp2_handle *h, const double *X, int64_t rows, double *Y
   g.err = h->dflag;
   const double fl = 2.0 * (double)rows * Nv * Nv;   // one float64-accurate rotation
   return run_digits(h, X, nullptr, S, S, *dig, g, levels, fl, fl);
+}
+
+// digit planes of W_v^T
+esmp2_status ensure_wv_digits(esmp2_handle *h) {
+  if (esmp2_status s = ensure_split(h)) return s;
+  return ensure_matrix_digits(h, h->Wv, &h->Rdig, &h->eR, 1);
 }
 
 esmp2_status xwv_split(esmp2_handle *h, const double *X, int64_t rows, double *Y) {

@@ -1528,7 +1528,7 @@ esmp2_status profile_packed(esmp2_handle *h, const double *x, int reps, double *
 // full-storage float64 in the TOP basis), through the working basis of the inner solve.
 esmp2_status sigma_mixed_packed(esmp2_handle *h, const double *x, double *y) {
   double *t1 = h->s64.w ? h->s64.w : h->s64.p;
-  rotate_occ(h, x, y, t1, true);                 // y: x in the working basis
+  if (esmp2_status s = rotate_occ(h, x, y, t1, true)) return s;   // y: x in the working basis
   if (h->arrowv) {
     if (esmp2_status s = ensure_arrow(h)) return s;
     if (esmp2_status s = rotate_virt(h, y, y, t1, true)) return s;
@@ -1541,7 +1541,7 @@ esmp2_status sigma_mixed_packed(esmp2_handle *h, const double *x, double *y) {
   h->launches += 1;
   if (h->arrowv)
     if (esmp2_status s = rotate_virt(h, y, y, t1, false)) return s;
-  rotate_occ(h, y, y, t1, false);
+  if (esmp2_status s = rotate_occ(h, y, y, t1, false)) return s;
   // the rotation back mixes slices: the non-amplitude slots (i == j of T, X, Y, ...) carry
   // rounding-level values, cleared here
   kp_mask64<<<2432, 128, 0, h->stream>>>(h->d.No, h->d.Nv, y);

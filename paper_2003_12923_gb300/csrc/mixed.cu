@@ -53,99 +53,19 @@ __global__ void k_build_rot(const double *Vt, int No, int Nv, double *R, double 
   }
 }
 
-// out[p][k'][q] = sum_k R[k][k'] in[p][k][q] for K <= 32 in double-float arithmetic: every
-// float64 operand is split into two floats (hi + lo); products are formed with the exact
-// product error (fma) and summed with Knuth's two-sum, so the float32 pipes do the work at
-// about 2^-46 relative accuracy; the float64 result is hi + lo.  The orbital rotations have
-// only No multiply-adds per element, which on GB300 would otherwise be float64-bound.
-constexpr int kDfK = 32;
-
-__global__ void __launch_bounds__(256) k_mode_df(const double *in, double *out, int64_t P, int K, int64_t Q,
-                                                 const double *R) {
-  __shared__ float2 R2[kDfK * kDfK];      // (hi, lo) pairs: one 8-byte broadcast load per product
-  for (int e = threadIdx.x; e < K * K; e += blockDim.x) {
-    const double r = R[e];
-    const float hi = (float)r;
-    R2[e] = make_float2(hi, (float)(r - (double)hi));
-  }
-  __syncthreads();
-  const int64_t n = P * Q;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t p = e / Q, q = e % Q;
-    const double *src = in + p * K * Q + q;
-    double *dst = out + p * K * Q + q;
-    float xh[kDfK], xl[kDfK];
-#pragma unroll
-    for (int k = 0; k < kDfK; ++k) {
-      if (k < K) {
-        const double v = src[k * Q];
-        xh[k] = (float)v;
-        xl[k] = (float)(v - (double)xh[k]);
-      }
-    }
-    for (int k2 = 0; k2 < K; k2 += 4) {
-      float sh[4] = {0.f, 0.f, 0.f, 0.f}, sl[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-      for (int k = 0; k < kDfK; ++k) {
-        if (k < K) {
-#pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            if (k2 + c < K) {   // exact leading product, two-sum; renormalised once at the end
-              const float2 r = R2[k * K + k2 + c];
-              const float ph = r.x * xh[k];
-              const float pe = fmaf(r.x, xh[k], -ph) + fmaf(r.x, xl[k], r.y * xh[k]);
-              const float t = sh[c] + ph;
-              const float bv = t - sh[c];
-              sl[c] += ((sh[c] - (t - bv)) + (ph - bv)) + pe;
-              sh[c] = t;
-            }
-          }
-        }
-      }
-#pragma unroll
-      for (int c = 0; c < 4; ++c)
-        if (k2 + c < K) dst[(k2 + c) * Q] = (double)sh[c] + (double)sl[c];
-    }
-  }
-}
-
 }  // namespace
 
-// out[p][k'][q] = sum_k R[k][k'] in[p][k][q] (R: K x K, row pitch K) in double-float
-// arithmetic when K <= 32, else as a float64 GEMM.
-void mode_product_small(const double *in, double *out, int64_t P, int K, int64_t Q, const double *R,
-                        cudaStream_t st) {
-  if (K <= kDfK) {
-    k_mode_df<<<1216, 256, 0, st>>>(in, out, P, K, Q, R);
-    return;
-  }
-  Gemm64 g{};
-  g.alpha = 1.0; g.beta = 0.0;
-  g.M = K; g.N = (int)Q; g.K = K; g.batch = (int)P;
-  g.A = R; g.sAm = 1; g.sAk = K; g.sAb = 0;
-  g.B = in; g.sBk = Q; g.sBn = 1; g.sBb = (int64_t)K * Q;
-  g.C = out; g.sCm = Q; g.sCn = 1; g.sCb = (int64_t)K * Q;
-  gemm64(g, st);
-}
-
 // in/out: block vectors; new occupied index i' = sum_i R[i][i'] (old i) (to_semi), or back.
-void rotate_occ(esmp2_handle *h, const double *in, double *out, double *tmp, bool to_semi) {
+esmp2_status rotate_occ(esmp2_handle *h, const double *in, double *out, double *tmp, bool to_semi) {
   const int No = h->d.No, Nv = h->d.Nv;
   if (No == 1) {
     if (in != out) cudaMemcpyAsync(out, in, sizeof(double) * h->d.n, cudaMemcpyDeviceToDevice, h->stream);
-    return;
+    return ESMP2_OK;
   }
-  const int dims[4] = {5, No, No, Nv * Nv};
   const double *R = to_semi ? h->Rocc : h->Rocct;
-  if (No <= kDfK) {
-    const int64_t NvNv = (int64_t)Nv * Nv;
-    k_mode_df<<<1216, 256, 0, h->stream>>>(in, tmp, 5, No, (int64_t)No * NvNv, R);
-    k_mode_df<<<1216, 256, 0, h->stream>>>(tmp, out, 5LL * No, No, NvNv, R);
-  } else {
-    mode_product(in, tmp, dims, 1, R, No, No, h->stream);
-    mode_product(tmp, out, dims, 2, R, No, No, h->stream);
-  }
-  h->launches += 2;
+  const int64_t NvNv = (int64_t)Nv * Nv;
+  esmp2_status s = mode_product_small(h, in, tmp, 5, No, (int64_t)No * NvNv, R);
+  return s ? s : mode_product_small(h, tmp, out, 5LL * No, No, NvNv, R);
 }
 
 // device flag and the float64 arrow sums (every mixed solve); with `operand` the bf16 copies and
@@ -157,10 +77,7 @@ static esmp2_status alloc_mixed_buffers(esmp2_handle *h, bool operand) {
   auto A = [&](void **p, size_t bytes) {
     if (e == cudaSuccess) e = dmalloc(p, bytes ? bytes : 1, h->stream);
   };
-  if (!h->dflag) {
-    A(reinterpret_cast<void **>(&h->dflag), sizeof(int));
-    if (e == cudaSuccess) cudaMemsetAsync(h->dflag, 0, sizeof(int), h->stream);
-  }
+  if (esmp2_status s = ensure_dflag(h)) return s;
   if (!h->cp.OC1) A(reinterpret_cast<void **>(&h->cp.OC1), sizeof(double) * (size_t)5 * No * Nv * Nv);
   if (!h->cp.OC2) A(reinterpret_cast<void **>(&h->cp.OC2), sizeof(double) * (size_t)5 * No * Nv * Nv);
   if (operand && !h->ylp) {
@@ -225,7 +142,10 @@ esmp2_status ensure_mixed(esmp2_handle *h, bool semi) {
   gemm64(g, h->stream);
   h->launches += 3;
   debug_phase(h, "  mixed: basis (eigenvectors, F)");
-  rotate_occ(h, h->b, h->bsemi, h->s64.w ? h->s64.w : h->s64.p, true);
+  if ((s = rotate_occ(h, h->b, h->bsemi, h->s64.w ? h->s64.w : h->s64.p, true))) {
+    dfree(V, h->stream); dfree(W2, h->stream); dfree(T1, h->stream);
+    return s;
+  }
   debug_phase(h, "  mixed: rhs rotation");
   k_f64_to_f32<<<64, 256, 0, h->stream>>>(h->Fsemi, h->F32, (int64_t)N * N);
   h->launches += 1;

@@ -1,0 +1,401 @@
+// Products with a narrow right factor (at most 32 columns) in float64 accuracy on the tensor cores:
+// the rotations of an occupied index (K = No <= 32) and the contraction of the last OVVV index with
+// the TOP virtuals (K = Nv, No columns), steps a1 of the transforms and the basis changes of the solves.
+//
+// Both have only No multiply-adds per element, too few to hide double-float arithmetic on the float32
+// pipes (13 operations per multiply-add bound them) and far too many for the float64 pipe.  Here the
+// operand is split into eight exact bf16 digit planes (digits.cu) on its way through shared memory,
+// tcgen05 forms the level sums (levels 2 .. 9, exact in fp32; 2^-48 of the row's largest element), and the levels are joined as integers
+// and rounded once: one read and one write of HBM, no digit planes in memory.  @KNAR@
+//
+// A tile is 128 result rows; persistent CTAs of 20 warps:
+//   warps 0, 1   MMA issuer; TMA of the right factor's digit chunks (OVVV form)
+//   warps 4..11  epilogue (two warps per TMEM lane quarter)
+//   warps 12..19 conversion: float64 from global memory into the eight planes of a 64-byte-swizzled
+//                K-major tile, 16-byte shared-memory stores, the next tile's loads in flight
+// Digit p of the operand meets the digits 1 .. 9 - p of the right factor, stacked along N (their
+// levels are neighbouring accumulators): eight MMAs per K step instead of 36.  Two sets of
+// accumulators (2 x 8 levels x 32 columns fill TMEM): the epilogue of a tile runs beside the next one.
+#include <cuda.h>
+#include <cuda_bf16.h>
+
+#include <algorithm>
+
+#include "internal.h"
+#include "digit_split.h"
+#include "tc_ptx.h"
+
+namespace esmp2 {
+namespace nr {
+
+using namespace ptx;
+
+constexpr int P = 8;                    // digit planes of both operands
+constexpr int BM = 128, BK = 32;
+constexpr int A_PLANE = BM * 64, A_STAGE = P * A_PLANE;   // 64 KB
+// result columns of a tile, 32 or 16 (No <= 16)
+template <int BN> constexpr int b_plane() { return BN * 64; }
+template <int BN> constexpr int smem_bytes() { return 1024 + 2 * A_STAGE + 2 * P * b_plane<BN>(); }
+constexpr int NTHREADS = 640, kConv = 256;
+
+struct Args {
+  const double *in;
+  double *out;
+  int64_t rows, tiles;
+  int K, N, nk;
+  int64_t Q;         // occupied form: row c = p Q + q reads in[(p K + k) Q + q], writes out[(p N + n) Q + q]
+  const double *R;   // occupied form: right factor, K x N row-major
+  const int *es;     // OVVV form: binary exponents, row r belongs to slice r / per
+  int per, eR;
+  int vec;           // OVVV form: 16-byte loads
+  int *err;
+};
+
+// byte offset of 16-byte group c of row r in a K-major tile of 64-byte rows, 64-byte swizzle
+__device__ __forceinline__ uint32_t sw64(int r, int c) { return (uint32_t)(r * 64 + ((c ^ ((r >> 1) & 3)) << 4)); }
+
+// digits of eight consecutive K elements of one row, one 16-byte store per plane
+__device__ __forceinline__ void store_digits(uint8_t *tile, int plane_bytes, int row, int c, const double (&v)[8], int e) {
+  long long U[8];
+#pragma unroll
+  for (int k = 0; k < 8; ++k) U[k] = digit_word<P>(v[k], e);
+  uint32_t sg[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) sg[k] = sign_pair(v[2 * k], v[2 * k + 1]);
+  uint8_t *dst = tile + sw64(row, c);
+#pragma unroll
+  for (int p = 1; p <= P; ++p)
+    *reinterpret_cast<uint4 *>(dst + (p - 1) * plane_bytes) =
+        make_uint4(digit_pair<P>(U[0], U[1], sg[0], p), digit_pair<P>(U[2], U[3], sg[1], p),
+                   digit_pair<P>(U[4], U[5], sg[2], p), digit_pair<P>(U[6], U[7], sg[3], p));
+}
+__device__ __forceinline__ int hi_abs(double v) {   // high word of |v|; infinities and NaN do not take part in a scale
+  const int h = __double2hiint(v) & 0x7FFFFFFF;
+  return h < 0x7FF00000 ? h : 0;
+}
+__device__ __forceinline__ int exp_of(int hi) { return hi >> 20 ? (hi >> 20) - 1021 : 0; }   // as k_slice_exp
+
+// ROW: OVVV form; BN: result columns; SMALL: every level sum below 2^22.  The occupied form with BN = 16
+// has K <= 16: one K step, eight elements per conversion thread.
+template <bool ROW, int BN, bool SMALL>
+__global__ void __launch_bounds__(NTHREADS, 1) k_narrow(const __grid_constant__ CUtensorMap tB, const __grid_constant__ Args g) {
+  constexpr int B_PLANE = b_plane<BN>(), B_STAGE = P * B_PLANE, ACC = 256;   // TMEM columns per accumulator set
+  constexpr int U = ROW || BN == 32 ? 2 : 1;   // K groups of eight per conversion thread
+  extern __shared__ uint8_t smem_raw[];
+  uint8_t *sA = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
+  uint8_t *sB = sA + 2 * A_STAGE;
+  __shared__ uint64_t a_full[2], a_empty[2], b_full[2], acc_full[2], acc_empty[2];
+  __shared__ uint32_t tmem_base;
+  __shared__ int fail, rmax, rexp[8][BM];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (threadIdx.x == 0) {
+    for (int s = 0; s < 2; ++s) { mbar_init(&a_full[s], kConv / 32); mbar_init(&a_empty[s], 1); mbar_init(&b_full[s], 1); mbar_init(&acc_full[s], 1); mbar_init(&acc_empty[s], 8); }
+    fail = 0;
+    rmax = 0;
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  for (int k = threadIdx.x; k < 8 * BM; k += NTHREADS) (&rexp[0][0])[k] = 0;
+  if (warp == 0) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)), "r"(512) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  int eR = g.eR;
+  if constexpr (!ROW) {   // the right factor's digits, row n = column n of R, once per CTA
+    __syncthreads();
+    int m = 0;
+    for (int e = threadIdx.x; e < g.K * g.N; e += NTHREADS) m = max(m, hi_abs(g.R[e]));
+    atomicMax(&rmax, m);
+    __syncthreads();
+    eR = exp_of(rmax);
+    for (int u = threadIdx.x; u < BN * 4; u += NTHREADS) {   // (every K group: unused ones are zero)
+      const int n = u >> 2, c = u & 3;
+      double v[8];
+#pragma unroll
+      for (int k = 0; k < 8; ++k) v[k] = (n < g.N && c * 8 + k < g.K) ? g.R[(c * 8 + k) * g.N + n] : 0.0;
+      store_digits(sB, B_PLANE, n, c, v, eR);
+    }
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  tc_before();
+  __syncthreads();
+  tc_after();
+  const uint32_t tmem = tmem_base;
+
+  if (warp == 0) {
+    if (lane == 0) {  // ------------------------------------------------ MMA issuer
+      int st = 0, ab = 0;
+      uint32_t ph = 0, aph = 1;
+      bool ok = true;
+      const uint64_t dA = sdesc64(smem_u32(sA)), dB = sdesc64(smem_u32(sB));
+      for (int64_t t = blockIdx.x; t < g.tiles && ok; t += gridDim.x) {
+        if (!mbar_wait(&acc_empty[ab], aph)) { ok = false; break; }
+        tc_after();
+        const uint32_t acc = tmem + (uint32_t)(ab * ACC);
+        for (int kc = 0; kc < g.nk; ++kc) {
+          if (!mbar_wait(&a_full[st], ph) || (ROW && !mbar_wait(&b_full[st], ph))) { ok = false; break; }
+          const int ks = g.K - kc * BK > 16 ? 2 : 1;
+          const uint64_t B = dB + (ROW ? (uint64_t)(st * (B_STAGE / 16)) : 0ull);
+          for (int k = 0; k < ks; ++k) {
+#pragma unroll
+            for (int i = 1; i <= P; ++i) {   // operand digit P + 1 - i, right-factor digits 1 .. i
+              const uint64_t A = dA + (uint64_t)(st * (A_STAGE / 16) + (P - i) * (A_PLANE / 16) + 2 * k);
+              const uint32_t d0 = acc + (uint32_t)((P - i) * BN);
+              if (kc == 0 && k == 0) {       // the lowest level of the group is met for the first time
+                umma_bf16(d0, A, B, idesc_bf16(BM, BN), 0u);
+                if (i > 1) umma_bf16(d0 + BN, A, B + B_PLANE / 16, idesc_bf16(BM, (i - 1) * BN), 1u);
+              } else {
+                umma_bf16(d0, A, B + 2 * k, idesc_bf16(BM, i * BN), 1u);
+              }
+            }
+          }
+          umma_commit(&a_empty[st]);
+          st ^= 1;
+          ph ^= (uint32_t)(st == 0);
+        }
+        if (!ok) break;
+        umma_commit(&acc_full[ab]);
+        ab ^= 1;
+        aph ^= (uint32_t)(ab == 0);
+      }
+      if (!ok) atomicExch(&fail, 1);
+    }
+  } else if (warp == 1) {
+    if (ROW && lane == 0) {  // ------------------------------------------ right-factor chunks
+      int st = 0;
+      uint32_t ph = 1;
+      int64_t it = 0;
+      bool ok = true;
+      for (int64_t t = blockIdx.x; t < g.tiles && ok; t += gridDim.x)
+        for (int kc = 0; kc < g.nk; ++kc, ++it) {
+          if (!mbar_wait(&a_empty[st], ph)) { ok = false; break; }
+          mbar_expect_tx(&b_full[st], (uint32_t)B_STAGE);
+#pragma unroll
+          for (int p = 0; p < P; ++p) tma_3d(sB + st * B_STAGE + p * B_PLANE, &tB, &b_full[st], kc * BK, 0, p);
+          st ^= 1;
+          ph ^= (uint32_t)(st == 0);
+        }
+      if (!ok) atomicExch(&fail, 1);
+      for (int64_t j = it > 2 ? it - 2 : 0; j < it; ++j) mbar_wait(&b_full[j & 1], (uint32_t)((j >> 1) & 1), 100000000ull);
+    }
+  } else if (warp >= 12) {  // ------------------------------------------- conversion
+    const int tid = threadIdx.x - 12 * 32;
+    int st = 0, slot = 0;
+    uint32_t ph = 1;
+    double v[U][8];
+    // occupied form: a warp has 16 rows, each half of it one half of K; OVVV form: (row, K group) and row + 64
+    const int orow = (tid >> 5) * 16 + (lane & 15), ohalf = lane >> 4;
+    auto load = [&](int64_t t, int kc) {
+      if constexpr (!ROW) {
+        const int64_t c = t * BM + orow;
+        const int k0 = ohalf * 8 * U;
+        const int64_t p = c < g.rows ? c / g.Q : 0;
+        const double *src = g.in + p * g.K * g.Q + (c - p * g.Q);
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+          for (int k = 0; k < 8; ++k) v[u][k] = (c < g.rows && k0 + 8 * u + k < g.K) ? src[(int64_t)(k0 + 8 * u + k) * g.Q] : 0.0;
+      } else {
+        const int k0 = kc * BK + (tid & 3) * 8;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+          const int64_t r = t * BM + (tid >> 2) + 64 * u;
+          const double *src = g.in + r * g.K + k0;
+          if (g.vec) {
+#pragma unroll
+            for (int k = 0; k < 8; k += 2) {
+              const double2 w = (r < g.rows && k0 + k < g.K) ? *reinterpret_cast<const double2 *>(src + k) : make_double2(0.0, 0.0);
+              v[u][k] = w.x;
+              v[u][k + 1] = w.y;
+            }
+          } else {
+#pragma unroll
+            for (int k = 0; k < 8; ++k) v[u][k] = (r < g.rows && k0 + k < g.K) ? src[k] : 0.0;
+          }
+        }
+      }
+    };
+    bool ok = true;
+    if (blockIdx.x < g.tiles) load(blockIdx.x, 0);
+    for (int64_t t = blockIdx.x; t < g.tiles && ok; t += gridDim.x) {
+      for (int kc = 0; kc < g.nk; ++kc) {
+        double w[U][8];
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+#pragma unroll
+          for (int k = 0; k < 8; ++k) w[u][k] = v[u][k];
+        if (kc + 1 < g.nk) load(t, kc + 1);   // in flight while this chunk is converted
+        else if (t + gridDim.x < g.tiles) load(t + gridDim.x, 0);
+        int e0, e1;
+        if constexpr (!ROW) {   // the row's own scale: the largest of its K elements
+          int m = 0;
+#pragma unroll
+          for (int u = 0; u < U; ++u)
+#pragma unroll
+            for (int k = 0; k < 8; ++k) m = max(m, hi_abs(w[u][k]));
+          m = max(m, __shfl_xor_sync(0xffffffffu, m, 16));
+          e0 = e1 = exp_of(m);
+          // eight slots: this one was last read eight tiles back, and the conversion of the tile
+          // before this one waited for MMAs that came after the epilogue five tiles back
+          if (ohalf == 0) rexp[slot][orow] = m;
+        } else {
+          const int64_t r0 = t * BM + (tid >> 2), r1 = r0 + 64;
+          e0 = r0 < g.rows ? __ldg(g.es + r0 / g.per) : 0;
+          e1 = r1 < g.rows ? __ldg(g.es + r1 / g.per) : 0;
+        }
+        // every warp waits for itself: a wait that runs out ends the conversion for good
+        ok = __all_sync(0xffffffffu, mbar_wait(&a_empty[st], ph));
+        if (!ok) break;
+        uint8_t *tile = sA + st * A_STAGE;
+        if constexpr (!ROW) {
+#pragma unroll
+          for (int u = 0; u < U; ++u) store_digits(tile, A_PLANE, orow, U * ohalf + u, w[u], e0);
+        } else {
+          store_digits(tile, A_PLANE, tid >> 2, tid & 3, w[0], e0);
+          store_digits(tile, A_PLANE, (tid >> 2) + 64, tid & 3, w[U - 1], e1);
+        }
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&a_full[st]);
+        st ^= 1;
+        ph ^= (uint32_t)(st == 0);
+      }
+      slot = (slot + 1) & 7;
+    }
+    if (!ok) atomicExch(&fail, 1);
+  } else if (warp >= 4) {  // -------------------------------------------- epilogue
+    const int quarter = warp & 3, chalf = (warp - 4) >> 2;
+    uint32_t lt = 0;
+    for (int64_t t = blockIdx.x; t < g.tiles; t += gridDim.x, ++lt) {
+      const int ab = (int)(lt & 1);
+      if (!mbar_wait(&acc_full[ab], (lt >> 1) & 1)) { if (lane == 0) atomicExch(&fail, 1); break; }
+      __syncwarp();
+      tc_after();
+      const int row = quarter * 32 + lane;
+      const int64_t r = t * BM + row;
+      const int e = (ROW ? (r < g.rows ? __ldg(g.es + r / g.per) : 0) : exp_of(rexp[lt & 7][row])) + eR - 54;
+      const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(ab * ACC + chalf * (BN / 2));
+      double *dst = nullptr;
+      int64_t pitch = 1;
+      if (r < g.rows) {
+        if constexpr (ROW) {
+          dst = g.out + r * g.N;
+        } else {
+          const int64_t p = r / g.Q;
+          dst = g.out + p * g.N * g.Q + (r - p * g.Q);
+          pitch = g.Q;
+        }
+      }
+#pragma unroll
+      for (int c4 = 0; c4 < BN / 8; ++c4) {
+        uint32_t q[P][4];
+#pragma unroll
+        for (int l = 0; l < P; ++l) tmem_ld4(taddr + (uint32_t)(l * BN + c4 * 4), q[l]);
+        tmem_wait();
+        if (c4 == BN / 8 - 1) {
+          tc_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(&acc_empty[ab]);   // the MMAs of the tile after the next may start
+        }
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          float f[P];
+#pragma unroll
+          for (int l = 0; l < P; ++l) {
+            keep(q[l][c]);
+            f[l] = __uint_as_float(q[l][c]);
+          }
+          const long long V = join_levels<P, SMALL>(f);
+          const int n = chalf * (BN / 2) + c4 * 4 + c;
+          if (dst && n < g.N) dst[n * pitch] = scale_i64(V, e);
+        }
+      }
+      __syncwarp();
+    }
+  }
+  tc_before();
+  __syncthreads();
+  if (warp == 0) {
+    tc_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(512) : "memory");
+  }
+  if (threadIdx.x == 0 && fail) atomicOr(g.err, 1);
+}
+
+template <bool ROW, int BN, bool SMALL>
+esmp2_status launch(esmp2_handle *h, const CUtensorMap &mB, nr::Args &g) {
+  if (g.rows <= 0) return ESMP2_OK;
+  constexpr int smem = smem_bytes<BN>();
+  if (cudaError_t e = smem_limit_once(reinterpret_cast<const void *>(k_narrow<ROW, BN, SMALL>), smem))
+    return check_cuda(h, e, "k_narrow shared-memory limit");
+  g.tiles = cdiv(g.rows, BM);
+  g.nk = (g.K + BK - 1) / BK;
+  g.err = h->dflag;
+  int dev = 0, sms = 148;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  k_narrow<ROW, BN, SMALL><<<(unsigned)std::min<int64_t>(g.tiles, sms), NTHREADS, smem, h->stream>>>(mB, g);
+  h->launches += 1;
+  return check_cuda(h, cudaGetLastError(), "k_narrow");
+}
+
+}  // namespace nr
+
+// out[p][n][q] = sum_k R[k][n] in[p][k][q] (R: K x K, row pitch K): on the tensor cores for K <= 32, else
+// a float64 GEMM.  in and out must not overlap.
+esmp2_status mode_product_small(esmp2_handle *h, const double *in, double *out, int64_t P, int K, int64_t Q, const double *R) {
+  if (K <= nr::BK) {
+    if (esmp2_status s = ensure_dflag(h)) return s;
+    nr::Args g{};
+    g.in = in; g.out = out;
+    g.rows = P * Q;
+    g.K = K; g.N = K; g.Q = Q;
+    g.R = R;
+    return K <= 16 ? nr::launch<false, 16, true>(h, CUtensorMap{}, g) : nr::launch<false, 32, true>(h, CUtensorMap{}, g);
+  }
+  Gemm64 g{};
+  g.alpha = 1.0; g.beta = 0.0;
+  g.M = K; g.N = (int)Q; g.K = K; g.batch = (int)P;
+  g.A = R; g.sAm = 1; g.sAk = K; g.sAb = 0;
+  g.B = in; g.sBk = Q; g.sBn = 1; g.sBb = (int64_t)K * Q;
+  g.C = out; g.sCm = Q; g.sCn = 1; g.sCb = (int64_t)K * Q;
+  gemm64(g, h->stream);
+  h->launches += 1;
+  return ESMP2_OK;
+}
+
+// out[m][n] = sum_k in[m][k] W[k][n], n < N <= 32, for M rows of length Nv (M a multiple of Nv): the first N
+// columns of the matrix whose transposed digit planes are `dig` (exponent eR).  in is read twice, for
+// the power-of-two scale of each Nv x Nv slice and for the product.
+esmp2_status rows_times_narrow(esmp2_handle *h, const double *in, double *out, int64_t M, int N, const void *dig, int eR) {
+  const int Nv = h->d.Nv, Nvp = (Nv + 7) & ~7;
+  if (esmp2_status s = ensure_dflag(h)) return s;
+  int *es = nullptr;
+  cudaError_t e = dmalloc(reinterpret_cast<void **>(&es), sizeof(int) * (size_t)(M / Nv), h->stream);
+  if (e != cudaSuccess) return check_cuda(h, e, "slice exponents");
+  slice_exponents(h, in, (int)(M / Nv), es);
+  CUtensorMap mB;
+  const uint64_t dims[3] = {(uint64_t)Nvp, (uint64_t)Nv, (uint64_t)kDigitPlanes};
+  const uint64_t str[2] = {(uint64_t)Nvp * 2, (uint64_t)Nvp * Nv * 2};
+  const int bn = N <= 16 ? 16 : 32;
+  const uint32_t box[3] = {nr::BK, (uint32_t)bn, 1};
+  if (!tma_map_bf16(&mB, dig, 3, dims, str, box, 64)) {
+    dfree(es, h->stream);
+    h->err = "tensor map encoding failed";
+    return ESMP2_ERR_CUDA;
+  }
+  nr::Args g{};
+  g.in = in; g.out = out;
+  g.rows = M;
+  g.K = Nv; g.N = N; g.Q = 1;
+  g.es = es;
+  g.per = Nv;
+  g.eR = eR;
+  g.vec = (Nv % 2) == 0 && reinterpret_cast<uintptr_t>(in) % 16 == 0;
+  const bool small = (int64_t)Nv * nr::P * 1024 < (1 << 22);
+  const esmp2_status s = bn == 16 ? (small ? nr::launch<true, 16, true>(h, mB, g) : nr::launch<true, 16, false>(h, mB, g))
+                                  : (small ? nr::launch<true, 32, true>(h, mB, g) : nr::launch<true, 32, false>(h, mB, g));
+  dfree(es, h->stream);
+  return s;
+}
+
+}  // namespace esmp2

@@ -583,115 +583,12 @@ void permute4(esmp2_handle *h, const double *in, double *out, const int d[4], in
   h->launches += 1;
 }
 
-// v = hi + lo: hi holds the leading 24 significand bits of v (truncated), lo the remaining
-// 29 bits rounded to float, so |v - hi - lo| <= 2^-48 |v|.  Integer operations only (one
-// integer-to-float conversion): float64 conversions and adds run at the float64 rate,
-// which GB300 keeps at a small fraction of the float32 rate.  |v| < 2^-74 (and zero)
-// gives (0, 0) up to that bound; |v| >= 2^127 takes the float64 route.
-__device__ __forceinline__ float2 split_df(double v) {
-  const unsigned long long u = (unsigned long long)__double_as_longlong(v);
-  const unsigned sign = (unsigned)(u >> 32) & 0x80000000u;
-  const int e = (int)((u >> 52) & 0x7FF);  // biased float64 exponent
-  if (e < 949) return make_float2(0.f, 0.f);
-  if (e > 1150) {
-    const float h = (float)v;
-    return make_float2(h, (float)(v - (double)h));
-  }
-  const unsigned long long m = u & 0xFFFFFFFFFFFFFull;
-  const float hi = __uint_as_float(sign | ((unsigned)(e - 896) << 23) | (unsigned)(m >> 29));
-  // lo = rest * 2^(e - 1075), the power of two a normal float for e >= 949
-  const float scale = __uint_as_float(sign | ((unsigned)(e - 948) << 23));
-  const float lo = __uint2float_rn((unsigned)(m & 0x1FFFFFFFu)) * scale;
-  return make_float2(hi, lo);
-}
-
-// Double-float sum (two floats hi + lo per float64 value): Knuth's two-sum, renormalised.
-__device__ __forceinline__ void df_add(float &sh, float &sl, float bh, float bl) {
-  const float t = sh + bh;
-  const float bv = t - sh;
-  const float err = (sh - (t - bv)) + (bh - bv);
-  const float lo = sl + bl + err;
-  sh = t + lo;
-  sl = lo - (sh - t);
-}
-
-// out[m][n] = sum_k in[m][k] R[k][n] for n < N <= 32 (a tall matrix times a narrow right
-// factor): lane n of a warp owns output column n of kXrRows rows at once, so one shared
-// load of R[k][n] serves kXrRows products and no cross-lane sum is needed.  The rows are
-// staged 32 columns at a time, split into (hi, lo) floats, through a per-warp shared
-// buffer while the next 32 columns are in flight.  Double-float accumulation: exact
-// leading product and two-sum per term, every 32-term chunk added into the running sum
-// with a renormalised double-float add.  The contraction of the last OVVV index with the
-// TOP virtuals (No multiply-adds per input element).
-constexpr int kXrN = 32, kXrRows = 8, kXrWarps = 16;
-size_t xr_df_smem(int K) { return sizeof(float2) * ((size_t)K * kXrN + (size_t)kXrWarps * kXrRows * 32); }
-__global__ void __launch_bounds__(kXrWarps * 32) k_xr_df(const double *__restrict__ in, double *__restrict__ out,
-                                                         int64_t M, int K, int N, const double *__restrict__ R,
-                                                         int64_t ldR) {
-  extern __shared__ float2 sm[];
-  float2 *sR = sm;  // [K][32] (hi, lo), columns >= N zero
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  float2 *sx = sm + (size_t)K * kXrN + warp * (kXrRows * 32);  // this warp's [kXrRows][32]
-  for (int e = threadIdx.x; e < K * kXrN; e += blockDim.x) {
-    const int k = e >> 5, n = e & 31;
-    sR[e] = n < N ? split_df(R[(int64_t)k * ldR + n]) : make_float2(0.f, 0.f);
-  }
-  __syncthreads();
-  const int64_t groups = (M + kXrRows - 1) / kXrRows;
-  for (int64_t g = (int64_t)blockIdx.x * kXrWarps + warp; g < groups; g += (int64_t)gridDim.x * kXrWarps) {
-    const int64_t m0 = g * kXrRows;
-    float sh[kXrRows], sl[kXrRows];
-    double nx[kXrRows];
-#pragma unroll
-    for (int r = 0; r < kXrRows; ++r) {
-      sh[r] = 0.f;
-      sl[r] = 0.f;
-      nx[r] = (m0 + r < M && lane < K) ? in[(m0 + r) * K + lane] : 0.0;
-    }
-    for (int k0 = 0; k0 < K; k0 += 32) {
-      __syncwarp();
-#pragma unroll
-      for (int r = 0; r < kXrRows; ++r) sx[r * 32 + lane] = split_df(nx[r]);
-      __syncwarp();
-      if (k0 + 32 < K) {
-        const int k = k0 + 32 + lane;
-#pragma unroll
-        for (int r = 0; r < kXrRows; ++r) nx[r] = (m0 + r < M && k < K) ? in[(m0 + r) * K + k] : 0.0;
-      }
-      const int kn = min(32, K - k0);
-      float ah[kXrRows], al[kXrRows];
-#pragma unroll
-      for (int r = 0; r < kXrRows; ++r) { ah[r] = 0.f; al[r] = 0.f; }
-#pragma unroll 2
-      for (int kk = 0; kk < kn; ++kk) {
-        const float2 rv = sR[(k0 + kk) * 32 + lane];
-#pragma unroll
-        for (int r = 0; r < kXrRows; ++r) {
-          const float2 xv = sx[r * 32 + kk];  // broadcast
-          const float ph = xv.x * rv.x;
-          const float pe = fmaf(xv.x, rv.x, -ph) + fmaf(xv.x, rv.y, xv.y * rv.x);
-          const float t = ah[r] + ph;
-          const float bv = t - ah[r];
-          al[r] += ((ah[r] - (t - bv)) + (ph - bv)) + pe;
-          ah[r] = t;
-        }
-      }
-#pragma unroll
-      for (int r = 0; r < kXrRows; ++r) df_add(sh[r], sl[r], ah[r], al[r]);
-    }
-    if (lane < N) {
-#pragma unroll
-      for (int r = 0; r < kXrRows; ++r)
-        if (m0 + r < M) out[(m0 + r) * N + lane] = (double)sh[r] + (double)sl[r];
-    }
-  }
-}
 }  // namespace
 
-// The N^5 integral transforms of step a1.  Rotations by the occupied U (No x No) are float64
-// GEMMs; rotations by W_v (Nv x Nv) run as X W_v on the tensor cores from exact digit
-// products (float64 accuracy), after moving the rotated index last.  The contraction of
-// the last OVVV index with the TOP virtuals (Nv -> No columns) stays a float64 GEMM.
+// The N^5 integral transforms of step a1, on the tensor cores from exact digit products (float64
+// accuracy): rotations by the occupied U and the contraction of the last OVVV index with the TOP
+// virtuals (Nv -> No columns) by the narrow-factor kernel (No <= 32, else float64 GEMMs),
+// rotations by W_v (Nv x Nv) as X W_v after moving the rotated index last.
 esmp2_status setup_rhs_from(esmp2_handle *h, const double *ovov_src, double *ovov_in, double *ooov_in,
                             const double *ovvv_src, double *ovvv_in, double *scratch) {
   const int No = h->d.No, Nv = h->d.Nv;
@@ -702,9 +599,8 @@ esmp2_status setup_rhs_from(esmp2_handle *h, const double *ovov_src, double *ovo
   {
     const int dims[4] = {No, Nv, No, Nv};
     if (tc) {
-      mode_product_small(ovov_src, scratch, 1, No, (int64_t)Nv * No * Nv, h->U, st);  // i
-      mode_product_small(scratch, ovov_in, (int64_t)No * Nv, No, Nv, h->U, st);       // j
-      h->launches += 2;
+      if ((s = mode_product_small(h, ovov_src, scratch, 1, No, (int64_t)Nv * No * Nv, h->U))) return s;  // i
+      if ((s = mode_product_small(h, scratch, ovov_in, (int64_t)No * Nv, No, Nv, h->U))) return s;       // j
       if ((s = xwv_split(h, ovov_in, (int64_t)No * Nv * No, scratch))) return s;   // b
       permute4(h, scratch, ovov_in, dims, 0, 2, 3, 1);                              // [i][j][b][a]
       if ((s = xwv_split(h, ovov_in, (int64_t)No * No * Nv, scratch))) return s;   // a
@@ -734,8 +630,7 @@ esmp2_status setup_rhs_from(esmp2_handle *h, const double *ovov_src, double *ovo
         int64_t P = 1, Q = 1;
         for (int k = 0; k < m; ++k) P *= dims[k];
         for (int k = m + 1; k < 4; ++k) Q *= dims[k];
-        mode_product_small(src, dst, P, No, Q, h->U, st);
-        h->launches += 1;
+        if ((s = mode_product_small(h, src, dst, P, No, Q, h->U))) return s;
       } else {
         mode_product(src, dst, dims, m, R[m], K[m], K[m], st);
       }
@@ -747,23 +642,16 @@ esmp2_status setup_rhs_from(esmp2_handle *h, const double *ovov_src, double *ovo
     debug_phase(h, "  ooov transform");
     if (h->ovvv_ready) cudaStreamWaitEvent(st, h->ovvv_ready, 0);   // host OVVV copied on a side stream
     int dims[4] = {No, Nv, Nv, Nv};
-    const size_t smem = xr_df_smem(Nv);
-    if (No <= kXrN && smem <= 220 * 1024) {  // c -> u' (first No columns of Wv)
-      // one limit for every Nv (220 KB): set once per device, never lowered under a running launch
-      if (cudaError_t ea = smem_limit_once(reinterpret_cast<const void *>(k_xr_df), 220 * 1024))
-        return check_cuda(h, ea, "k_xr_df shared-memory limit");
-      const int64_t M = (int64_t)No * Nv * Nv;
-      const unsigned grid = (unsigned)std::min<int64_t>(1216, cdiv(cdiv(M, kXrRows), kXrWarps));
-      k_xr_df<<<grid, kXrWarps * 32, smem, st>>>(ovvv_src, scratch, M, Nv, No, h->Wv, Nv);
-      h->launches += 1;
+    if (No <= 32 && tc) {  // c -> u' (first No columns of Wv)
+      if ((s = ensure_wv_digits(h))) return s;
+      if ((s = rows_times_narrow(h, ovvv_src, scratch, (int64_t)No * Nv * Nv, No, h->Rdig, h->eR))) return s;
     } else {
       mode_product(ovvv_src, scratch, dims, 3, h->Wv, No, Nv, st);
     }
     dims[3] = No;
     debug_phase(h, "  ovvv last index -> u'");
     if (tc) {
-      mode_product_small(scratch, ovvv_in, 1, No, (int64_t)Nv * Nv * No, h->U, st);  // [i][a][b][u]
-      h->launches += 1;
+      if ((s = mode_product_small(h, scratch, ovvv_in, 1, No, (int64_t)Nv * Nv * No, h->U))) return s;  // [i][a][b][u]
       permute4(h, ovvv_in, scratch, dims, 0, 3, 1, 2);                             // [i][u][a][b]
       if ((s = xwv_split(h, scratch, (int64_t)No * No * Nv, ovvv_in))) return s;  // b
       const int d2[4] = {No, No, Nv, Nv};

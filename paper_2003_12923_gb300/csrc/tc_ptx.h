@@ -51,7 +51,13 @@ __device__ __forceinline__ void tma_3d(void *dst, const CUtensorMap *m, uint64_t
 __device__ __forceinline__ void tc_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-// shared-memory descriptor of a K-major operand with 128-byte swizzle: start >> 4, leading byte
+// shared-memory descriptor of a K-major operand with 64-byte swizzle: start >> 4, leading byte
+// offset 16 >> 4 (unused by swizzled K-major layouts), stride of one group of 8 rows of 64 bytes
+// (512 >> 4), descriptor version 1 at bit 46, layout type 4 (64-byte swizzle) at bit 61
+__device__ __forceinline__ uint64_t sdesc64(uint32_t addr) {
+  return (uint64_t)((addr >> 4) & 0x3FFFu) | ((uint64_t)1 << 16) | ((uint64_t)(512 >> 4) << 32) | (1ull << 46) | (4ull << 61);
+}
+// the same with 128-byte rows and swizzle: start >> 4, leading byte
 // offset 16 >> 4 (unused by swizzled K-major layouts), stride of one group of 8 rows of 128 bytes
 // (1024 >> 4), descriptor version 1 at bit 46, layout type 2 (128-byte swizzle) at bit 61
 __device__ __forceinline__ uint64_t sdesc128(uint32_t addr) {
@@ -76,6 +82,11 @@ __device__ __forceinline__ void umma_commit(uint64_t *bar) {
 __device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
   asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_ld4(uint32_t taddr, uint32_t (&r)[4]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x4.b32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
                : "r"(taddr));
 }
 __device__ __forceinline__ void tmem_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
