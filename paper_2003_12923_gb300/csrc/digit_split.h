@@ -35,22 +35,22 @@ __device__ __forceinline__ long long digit_word(double v, int es) {
   if (ef == 0x7FF) m = 1ull << (6 * P - 1);   // an infinity or NaN saturates
   return (long long)m + bias;
 }
-// digit p (1-based) of the magnitude as the high half of its float32 (a bf16)
-template <int P>
-__device__ __forceinline__ uint32_t digit_bits(long long U, int p) {
-  const int sh = 6 * (P - p);
-  if (p == 1) return __float_as_uint(__uint_as_float(0x4B400000u + (uint32_t)(int)(U >> sh)) - 12582912.0f);
-  return __float_as_uint(__uint_as_float(0x4B400000u | ((uint32_t)(U >> sh) & 63u)) - 12582944.0f);
-}
-// the signs of two elements as they stand in a packed pair of bf16 digits
+// The signs of two elements as bf16 factors +-1.0, packed.
 __device__ __forceinline__ uint32_t sign_pair(double v0, double v1) {
-  return ((uint32_t)__double2hiint(v0) >> 16 & 0x8000u) | ((uint32_t)__double2hiint(v1) & 0x80000000u);
+  return (((uint32_t)__double2hiint(v0) >> 16) & 0x8000u) | ((uint32_t)__double2hiint(v1) & 0x80000000u) | 0x3F803F80u;
 }
-// digit p of two elements, packed
+// Digit p (1-based) of two elements as packed bf16: 128 + field is the bf16 with the field in its low
+// mantissa bits, so one packed fused multiply-add gives sign (field - 32) (digit 1: sign field) exactly.
 template <int P>
 __device__ __forceinline__ uint32_t digit_pair(long long U0, long long U1, uint32_t sg, int p) {
-  return __byte_perm(digit_bits<P>(U0, p), digit_bits<P>(U1, p), 0x7632) ^ sg;
+  const int sh = 6 * (P - p);
+  const uint32_t w = (__byte_perm((uint32_t)(U0 >> sh), (uint32_t)(U1 >> sh), 0x5410) & 0x003F003Fu) | 0x43004300u;
+  const uint32_t c = (p == 1 ? 0xC300C300u : 0xC320C320u) ^ (sg & 0x80008000u);   // -128 or -160 times the sign
+  uint32_t r;
+  asm("fma.rn.bf16x2 %0, %1, %2, %3;" : "=r"(r) : "r"(w), "r"(sg), "r"(c));
+  return r;
 }
+
 // Integer-valued accumulators v[0 .. NL-1] (levels 2 .. NL + 1 of one element) joined at the weight of
 // the last one, for NL <= 8: sum_l v[l] 64^(NL-1-l).  SMALL: every |v| < 2^22, so that the integer is
 // read off the bits of v + 1.5 2^23 (two full-rate operations; conversions run at an eighth of the rate);

@@ -8,10 +8,10 @@
 // tcgen05 forms the level sums (levels 2 .. 9, exact in fp32; 2^-48 of the row's largest element), and the levels are joined as integers
 // and rounded once: one read and one write of HBM, no digit planes in memory.  @KNAR@
 //
-// A tile is 128 result rows; persistent CTAs of 20 warps:
+// A tile is 128 result rows; persistent CTAs of 28 warps:
 //   warps 0, 1   MMA issuer; TMA of the right factor's digit chunks (OVVV form)
 //   warps 4..11  epilogue (two warps per TMEM lane quarter)
-//   warps 12..19 conversion: float64 from global memory into the eight planes of a 64-byte-swizzled
+//   warps 12..27 conversion: float64 from global memory into the eight planes of a 64-byte-swizzled
 //                K-major tile, 16-byte shared-memory stores, the next tile's loads in flight
 // Digit p of the operand meets the digits 1 .. 9 - p of the right factor, stacked along N (their
 // levels are neighbouring accumulators): eight MMAs per K step instead of 36.  Two sets of
@@ -36,7 +36,7 @@ constexpr int A_PLANE = BM * 64, A_STAGE = P * A_PLANE;   // 64 KB
 // result columns of a tile, 32 or 16 (No <= 16)
 template <int BN> constexpr int b_plane() { return BN * 64; }
 template <int BN> constexpr int smem_bytes() { return 1024 + 2 * A_STAGE + 2 * P * b_plane<BN>(); }
-constexpr int NTHREADS = 640, kConv = 256;
+constexpr int NTHREADS = 896;
 
 struct Args {
   const double *in;
@@ -75,12 +75,14 @@ __device__ __forceinline__ int hi_abs(double v) {   // high word of |v|; infinit
 }
 __device__ __forceinline__ int exp_of(int hi) { return hi >> 20 ? (hi >> 20) - 1021 : 0; }   // as k_slice_exp
 
-// ROW: OVVV form; BN: result columns; SMALL: every level sum below 2^22.  The occupied form with BN = 16
-// has K <= 16: one K step, eight elements per conversion thread.
+// ROW: OVVV form; BN: result columns; SMALL: every level sum below 2^22.  A conversion thread takes
+// eight K elements of a row; the occupied form with BN = 16 has K <= 16 and half as many of these per
+// tile, so its two halves of the conversion warps take turns.
 template <bool ROW, int BN, bool SMALL>
 __global__ void __launch_bounds__(NTHREADS, 1) k_narrow(const __grid_constant__ CUtensorMap tB, const __grid_constant__ Args g) {
   constexpr int B_PLANE = b_plane<BN>(), B_STAGE = P * B_PLANE, ACC = 256;   // TMEM columns per accumulator set
-  constexpr int U = ROW || BN == 32 ? 2 : 1;   // K groups of eight per conversion thread
+  constexpr bool HALF = !ROW && BN == 16;
+  constexpr int CW = HALF ? 8 : 16;   // conversion warps per chunk
   extern __shared__ uint8_t smem_raw[];
   uint8_t *sA = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint8_t *sB = sA + 2 * A_STAGE;
@@ -89,7 +91,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_narrow(const __grid_constant__ 
   __shared__ int fail, rmax, rexp[8][BM];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
-    for (int s = 0; s < 2; ++s) { mbar_init(&a_full[s], kConv / 32); mbar_init(&a_empty[s], 1); mbar_init(&b_full[s], 1); mbar_init(&acc_full[s], 1); mbar_init(&acc_empty[s], 8); }
+    for (int s = 0; s < 2; ++s) { mbar_init(&a_full[s], CW); mbar_init(&a_empty[s], 1); mbar_init(&b_full[s], 1); mbar_init(&acc_full[s], 1); mbar_init(&acc_empty[s], 8); }
     fail = 0;
     rmax = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -178,88 +180,78 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_narrow(const __grid_constant__ 
       for (int64_t j = it > 2 ? it - 2 : 0; j < it; ++j) mbar_wait(&b_full[j & 1], (uint32_t)((j >> 1) & 1), 100000000ull);
     }
   } else if (warp >= 12) {  // ------------------------------------------- conversion
-    const int tid = threadIdx.x - 12 * 32;
-    int st = 0, slot = 0;
-    uint32_t ph = 1;
-    double v[U][8];
-    // occupied form: a warp has 16 rows, each half of it one half of K; OVVV form: (row, K group) and row + 64
-    const int orow = (tid >> 5) * 16 + (lane & 15), ohalf = lane >> 4;
+    const int cw = warp - 12, grp = HALF ? cw >> 3 : 0;
+    // occupied form: 8 rows by 4 K groups per warp (HALF: 16 by 2), consecutive lanes on consecutive
+    // rows; OVVV form: 8 rows, the 4 K groups of a row on neighbouring lanes
+    const int row = HALF ? (cw & 7) * 16 + (lane & 15) : ROW ? cw * 8 + (lane >> 2) : cw * 8 + (lane & 7);
+    const int kg = HALF ? lane >> 4 : ROW ? lane & 3 : lane >> 3;
+    double v[8];
     auto load = [&](int64_t t, int kc) {
+      const int64_t r = t * BM + row;
       if constexpr (!ROW) {
-        const int64_t c = t * BM + orow;
-        const int k0 = ohalf * 8 * U;
-        const int64_t p = c < g.rows ? c / g.Q : 0;
-        const double *src = g.in + p * g.K * g.Q + (c - p * g.Q);
+        const int64_t p = r < g.rows ? r / g.Q : 0;
+        const double *src = g.in + (p * g.K + kg * 8) * g.Q + (r - p * g.Q);
 #pragma unroll
-        for (int u = 0; u < U; ++u)
-#pragma unroll
-          for (int k = 0; k < 8; ++k) v[u][k] = (c < g.rows && k0 + 8 * u + k < g.K) ? src[(int64_t)(k0 + 8 * u + k) * g.Q] : 0.0;
+        for (int k = 0; k < 8; ++k) v[k] = (r < g.rows && kg * 8 + k < g.K) ? src[(int64_t)k * g.Q] : 0.0;
       } else {
-        const int k0 = kc * BK + (tid & 3) * 8;
+        const int k0 = kc * BK + kg * 8;
+        const double *src = g.in + r * g.K + k0;
+        if (g.vec) {
 #pragma unroll
-        for (int u = 0; u < U; ++u) {
-          const int64_t r = t * BM + (tid >> 2) + 64 * u;
-          const double *src = g.in + r * g.K + k0;
-          if (g.vec) {
-#pragma unroll
-            for (int k = 0; k < 8; k += 2) {
-              const double2 w = (r < g.rows && k0 + k < g.K) ? *reinterpret_cast<const double2 *>(src + k) : make_double2(0.0, 0.0);
-              v[u][k] = w.x;
-              v[u][k + 1] = w.y;
-            }
-          } else {
-#pragma unroll
-            for (int k = 0; k < 8; ++k) v[u][k] = (r < g.rows && k0 + k < g.K) ? src[k] : 0.0;
+          for (int k = 0; k < 8; k += 2) {
+            const double2 w = (r < g.rows && k0 + k < g.K) ? *reinterpret_cast<const double2 *>(src + k) : make_double2(0.0, 0.0);
+            v[k] = w.x;
+            v[k + 1] = w.y;
           }
+        } else {
+#pragma unroll
+          for (int k = 0; k < 8; ++k) v[k] = (r < g.rows && k0 + k < g.K) ? src[k] : 0.0;
         }
       }
     };
+    // HALF: group 0 fills stage 0 with this CTA's even tiles, group 1 stage 1 with its odd ones
+    const int64_t t0 = blockIdx.x + (HALF ? (int64_t)grp * gridDim.x : 0), dt = (HALF ? 2 : 1) * (int64_t)gridDim.x;
+    int st = grp, slot = grp;
+    uint32_t ph = 1;
     bool ok = true;
-    if (blockIdx.x < g.tiles) load(blockIdx.x, 0);
-    for (int64_t t = blockIdx.x; t < g.tiles && ok; t += gridDim.x) {
+    if (t0 < g.tiles) load(t0, 0);
+    for (int64_t t = t0; t < g.tiles && ok; t += dt) {
       for (int kc = 0; kc < g.nk; ++kc) {
-        double w[U][8];
+        double w[8];
 #pragma unroll
-        for (int u = 0; u < U; ++u)
-#pragma unroll
-          for (int k = 0; k < 8; ++k) w[u][k] = v[u][k];
+        for (int k = 0; k < 8; ++k) w[k] = v[k];
         if (kc + 1 < g.nk) load(t, kc + 1);   // in flight while this chunk is converted
-        else if (t + gridDim.x < g.tiles) load(t + gridDim.x, 0);
-        int e0, e1;
+        else if (t + dt < g.tiles) load(t + dt, 0);
+        int e;
         if constexpr (!ROW) {   // the row's own scale: the largest of its K elements
           int m = 0;
 #pragma unroll
-          for (int u = 0; u < U; ++u)
-#pragma unroll
-            for (int k = 0; k < 8; ++k) m = max(m, hi_abs(w[u][k]));
+          for (int k = 0; k < 8; ++k) m = max(m, hi_abs(w[k]));
+          if constexpr (!HALF) m = max(m, __shfl_xor_sync(0xffffffffu, m, 8));
           m = max(m, __shfl_xor_sync(0xffffffffu, m, 16));
-          e0 = e1 = exp_of(m);
-          // eight slots: this one was last read eight tiles back, and the conversion of the tile
-          // before this one waited for MMAs that came after the epilogue five tiles back
-          if (ohalf == 0) rexp[slot][orow] = m;
+          e = exp_of(m);
+          // eight slots: this one was last read eight tiles back, and the conversion of the tile two
+          // before this one waited for MMAs that came after the epilogue six tiles back
+          if (kg == 0) rexp[slot][row] = m;
         } else {
-          const int64_t r0 = t * BM + (tid >> 2), r1 = r0 + 64;
-          e0 = r0 < g.rows ? __ldg(g.es + r0 / g.per) : 0;
-          e1 = r1 < g.rows ? __ldg(g.es + r1 / g.per) : 0;
+          const int64_t r = t * BM + row;
+          e = r < g.rows ? __ldg(g.es + r / g.per) : 0;
         }
         // every warp waits for itself: a wait that runs out ends the conversion for good
         ok = __all_sync(0xffffffffu, mbar_wait(&a_empty[st], ph));
         if (!ok) break;
-        uint8_t *tile = sA + st * A_STAGE;
-        if constexpr (!ROW) {
-#pragma unroll
-          for (int u = 0; u < U; ++u) store_digits(tile, A_PLANE, orow, U * ohalf + u, w[u], e0);
-        } else {
-          store_digits(tile, A_PLANE, tid >> 2, tid & 3, w[0], e0);
-          store_digits(tile, A_PLANE, (tid >> 2) + 64, tid & 3, w[U - 1], e1);
-        }
+        store_digits(sA + st * A_STAGE, A_PLANE, row, kg, w, e);
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncwarp();
         if (lane == 0) mbar_arrive(&a_full[st]);
-        st ^= 1;
-        ph ^= (uint32_t)(st == 0);
+        if constexpr (HALF) {
+          ph ^= 1;
+        } else {
+          st ^= 1;
+          ph ^= (uint32_t)(st == 0);
+        }
       }
-      slot = (slot + 1) & 7;
+      slot = (slot + (HALF ? 2 : 1)) & 7;
     }
     if (!ok) atomicExch(&fail, 1);
   } else if (warp >= 4) {  // -------------------------------------------- epilogue
