@@ -486,12 +486,10 @@ void virt_arrow64(esmp2_handle *h, const double *x, double *y) {
 
 // float64 sigma in the reduced-cost basis: the virtual-index terms element-wise, the
 // occupied-index terms and couplings by the arrow-form coupling pass (Farr).
-esmp2_status sigma64_arrow(esmp2_handle *h, const double *x, double *y, int couplings) {
+esmp2_status sigma64_arrow(esmp2_handle *h, const double *x, double *y) {
   virt_arrow64(h, x, y);
-  if (couplings) {
-    launch_intermediates64(h, h->Farr, 1, x);
-    launch_couple64(h, h->Farr, 1, x, y);
-  }
+  launch_intermediates64(h, h->Farr, 1, x);
+  launch_couple64(h, h->Farr, 1, x, y);
   return check_cuda(h, cudaGetLastError(), "sigma64_arrow");
 }
 

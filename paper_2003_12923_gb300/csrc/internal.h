@@ -211,7 +211,7 @@ esmp2_status sigma64(esmp2_handle *h, const double *x, double *y, int tc_levels 
 // s_sym: x has the spin-flip symmetry of S exactly (S_ij^ab = S_ji^ba bit for bit); the
 // digit-level virtual pass then contracts the S slices with F_vv from one side only
 esmp2_status sigma64_F(esmp2_handle *h, const double *F, int arrow, const double *x, double *y, int tc_levels = 0,
-                       int couplings = 1, bool s_sym = false);
+                       bool s_sym = false);
 void launch_intermediates64(esmp2_handle *h, const double *F, int arrow, const double *x);
 void launch_couple64(esmp2_handle *h, const double *F, int arrow, const double *x, double *y);
 esmp2_status sigma64_tail(esmp2_handle *h, const double *F, int arrow, const double *x, double *y);
@@ -275,7 +275,7 @@ esmp2_status xwm_split(esmp2_handle *h, const double *X, int64_t rows, double *Y
 esmp2_status ensure_arrow(esmp2_handle *h);
 esmp2_status rotate_virt(esmp2_handle *h, const double *in, double *out, double *tmp, bool to_arrow);
 esmp2_status x_to_basis(esmp2_handle *h, int target);
-esmp2_status sigma64_arrow(esmp2_handle *h, const double *x, double *y, int couplings = 1);
+esmp2_status sigma64_arrow(esmp2_handle *h, const double *x, double *y);
 void virt_arrow64(esmp2_handle *h, const double *x, double *y);
 esmp2_status rotate_occ(esmp2_handle *h, const double *in, double *out, double *tmp, bool to_semi);
 esmp2_status mode_product_small(esmp2_handle *h, const double *in, double *out, int64_t P, int K, int64_t Q, const double *R);

@@ -1094,7 +1094,7 @@ esmp2_status solve_mixed(esmp2_handle *h, double tol, int maxit, esmp2_solve_inf
     } else {
       if (!cold) {
         if (arrowv) s = sigma64_arrow(h, x, q);
-        else s = sigma64_F(h, h->Fsemi, 1, x, q, lv_k, 1, true);
+        else s = sigma64_F(h, h->Fsemi, 1, x, q, lv_k, true);
         if (s) return s;
       }
       k_residual<<<kRedBlocks, kRedThreads, 0, st>>>(c, bsel, cold ? nullptr : q, r, h->red, bb < 0.0 ? 1 : 0);
