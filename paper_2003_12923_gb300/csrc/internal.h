@@ -115,6 +115,7 @@ struct esmp2_handle {
   float arrow_w[64] = {};   // host copy of F32[l][0] (1 <= l < No) and F32[l][No] (l < No)
   double arrow_w64[64] = {}; // the same in float64
   __half *dinv32 = nullptr; // Jacobi preconditioner in that basis (n halves)
+  double *dinv64 = nullptr; // Jacobi preconditioner of the float64 solve (n)
   double *P64 = nullptr;    // products of the virtual-index pass (float64 sigma workspace, n)
   double *red = nullptr;    // reduction partials
   double *red_out = nullptr;// reduction results (device)
@@ -207,7 +208,9 @@ namespace esmp2 {
 // kernels.cu
 esmp2_status setup_top_basis(esmp2_handle *h);
 esmp2_status setup_rhs(esmp2_handle *h);
-esmp2_status sigma64(esmp2_handle *h, const double *x, double *y, int tc_levels = 0);
+// s_sym: x has the spin-flip symmetry of S bit for bit, and so has y; for No <= 32 the partials of <x, y>
+// are left in h->red (residual_parts())
+esmp2_status sigma64(esmp2_handle *h, const double *x, double *y, int tc_levels = 0, bool s_sym = false);
 // s_sym: x has the spin-flip symmetry of S exactly (S_ij^ab = S_ji^ba bit for bit); the
 // digit-level virtual pass then contracts the S slices with F_vv from one side only
 esmp2_status sigma64_F(esmp2_handle *h, const double *F, int arrow, const double *x, double *y, int tc_levels = 0,
@@ -264,6 +267,8 @@ esmp2_status ensure_p64(esmp2_handle *h);
 esmp2_status virt_split(esmp2_handle *h, const double *x, double *y, double *p64, int sym, int levels, bool join = true);
 // float64 residual of the refinement on the independent slices (resid.cu)
 int residual_parts();
+esmp2_status sigma_sym_tail(esmp2_handle *h, const double *x, double *y, bool s_sym);
+esmp2_status sigma64_finish(esmp2_handle *h, const double *x, double *y, bool s_sym);
 esmp2_status residual_sym(esmp2_handle *h, const double *x, const double *b, double *r, int levels);
 int hyll_parts();
 void hylleraas_sym(esmp2_handle *h, const double *b, const double *x, const double *r);

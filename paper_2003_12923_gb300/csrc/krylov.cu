@@ -114,18 +114,50 @@ __global__ void k_finalize(const double *red, int nparts, int nq, double *slots,
   }
 }
 
-// r = -b - q; p = M^-1 r; partials <r,M^-1 r>, <r,r>, <b,b>
-__global__ void k_pcg_init(VCtx c, const double *b, const double *q, double *r, double *p, double *red) {
-  double v[3] = {0.0, 0.0, 0.0};
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < 5 * c.B; e += (int64_t)gridDim.x * blockDim.x) {
-    const double ri = -b[e] - q[e], z = c.dinv(e) * ri, w = c.w(e);
-    r[e] = ri;
-    p[e] = z;
-    v[0] += w * ri * z;
-    v[1] += w * ri * ri;
-    v[2] += w * b[e] * b[e];
+// M^-1 = 1 / diag(A), zero on the slots that are not amplitudes; a CTA iteration per row (blk, i, j, a).
+// (F_aa + F_bb) - (F_ii + F_jj): the same rounding for every image of an amplitude.
+__global__ void __launch_bounds__(128) k_dinv64(VCtx c, double *dinv) {
+  const int No = c.No, Nv = c.Nv, N = c.N;
+  const int64_t rows = 5LL * No * No * Nv;
+  const double shift = c.F[(int64_t)No * N + No] - c.F[0];
+  for (int64_t row = blockIdx.x; row < rows; row += gridDim.x) {
+    int64_t f = row;
+    const int a = (int)(f % Nv); f /= Nv;
+    const int j = (int)(f % No); f /= No;
+    const int i = (int)(f % No), blk = (int)(f / No);
+    const double occ = (c.F[(int64_t)i * N + i] + c.F[(int64_t)j * N + j]) + c.omega - (blk >= BX ? shift : 0.0);
+    const double fa = c.F[(int64_t)(No + a) * N + No + a];
+    double *out = dinv + row * Nv;
+    for (int b = threadIdx.x; b < Nv; b += blockDim.x) {
+      bool zero = false;
+      if ((blk == BT || blk == BX || blk == BY) && (i == j || a == b)) zero = true;
+      if (blk == BX && (i == 0 || j == 0 || a == 0 || b == 0)) zero = true;
+      if (blk == BZ && (j == 0 || b == 0 || (i == 0 && a == 0))) zero = true;
+      out[b] = zero ? 0.0 : 1.0 / ((fa + c.F[(int64_t)(No + b) * N + No + b]) - occ);
+    }
   }
-  block_partials<3>(v, red);
+}
+
+__device__ __forceinline__ double blk_weight(int blk) { return blk == 1 ? 1.0 : (blk == 4 ? 2.0 : 0.5); }
+
+// p = M^-1 r; partials <r, M^-1 r>_w, <r, r>_w.  Block by block, weights on the block sums; M^-1 is read
+// (8 bytes) instead of formed (an index decode and a float64 division, some 20 operations of the
+// float64 pipe per element: 72 us against 20 at No=8 Nv=80).
+__global__ void k_pcg_start(VCtx c, const double *dinv, const double *r, double *p, double *red) {
+  double v[2] = {0.0, 0.0};
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x, t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  for (int blk = 0; blk < 5; ++blk) {
+    double s0 = 0.0, s1 = 0.0;
+    for (int64_t e = blk * c.B + t0; e < (blk + 1) * c.B; e += stride) {
+      const double ri = r[e], z = dinv[e] * ri;
+      p[e] = z;
+      s0 = fma(ri, z, s0);
+      s1 = fma(ri, ri, s1);
+    }
+    v[0] += blk_weight(blk) * s0;
+    v[1] += blk_weight(blk) * s1;
+  }
+  block_partials<2>(v, red);
 }
 
 __global__ void k_dot_w(VCtx c, const double *u, const double *v_, double *red) {
@@ -136,26 +168,31 @@ __global__ void k_dot_w(VCtx c, const double *u, const double *v_, double *red) 
 }
 
 // x += alpha p; r -= alpha q; partials <r,M^-1 r>, <r,r>
-__global__ void k_pcg_update(VCtx c, const double *slots, double *x, double *r, const double *p, const double *q,
-                             double *red) {
+__global__ void k_pcg_update(VCtx c, const double *slots, const double *dinv, double *x, double *r, const double *p,
+                             const double *q, double *red) {
   const double alpha = slots[4];
   double v[2] = {0.0, 0.0};
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < 5 * c.B; e += (int64_t)gridDim.x * blockDim.x) {
-    x[e] += alpha * p[e];
-    const double ri = r[e] - alpha * q[e];
-    r[e] = ri;
-    const double w = c.w(e);
-    v[0] += w * ri * c.dinv(e) * ri;
-    v[1] += w * ri * ri;
+  const int64_t stride = (int64_t)gridDim.x * blockDim.x, t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  for (int blk = 0; blk < 5; ++blk) {
+    double s0 = 0.0, s1 = 0.0;
+    for (int64_t e = blk * c.B + t0; e < (blk + 1) * c.B; e += stride) {
+      x[e] = fma(alpha, p[e], x[e]);
+      const double ri = fma(-alpha, q[e], r[e]);
+      r[e] = ri;
+      s0 = fma(ri * dinv[e], ri, s0);
+      s1 = fma(ri, ri, s1);
+    }
+    v[0] += blk_weight(blk) * s0;
+    v[1] += blk_weight(blk) * s1;
   }
   block_partials<2>(v, red);
 }
 
 // p = M^-1 r + beta p
-__global__ void k_pcg_p(VCtx c, const double *slots, const double *r, double *p) {
+__global__ void k_pcg_p(VCtx c, const double *slots, const double *dinv, const double *r, double *p) {
   const double beta = slots[5];
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < 5 * c.B; e += (int64_t)gridDim.x * blockDim.x)
-    p[e] = c.dinv(e) * r[e] + beta * p[e];
+    p[e] = fma(beta, p[e], dinv[e] * r[e]);
 }
 
 // ---- low-precision inner PCG (vectors of type T, float64 reductions)
@@ -680,8 +717,6 @@ __global__ void k_negsum64(const double *b, const double *q, double *out, int64_
 
 }  // namespace
 
-void launch_pcg_init(esmp2_handle *h, const double *b, const double *q, double *r, double *p);
-
 // one quantity's partials summed into the slots with the bookkeeping of `mode` (k_finalize)
 void k_finalize_ext(const double *red, int nparts, double *slots, int mode, cudaStream_t st) {
   k_finalize<<<1, 256, 0, st>>>(red, nparts, 1, slots, mode);
@@ -722,23 +757,38 @@ esmp2_status solve64(esmp2_handle *h, double tol, int maxit, esmp2_solve_info *i
   h->last_precision = virt_tc ? ESMP2_FP64_TC : ESMP2_FP64;
   h->r_true = h->r_sym = false;
   const int lv = virt_tc ? kFp64TcLevels : 0;
-  antisym_project(h, x);
+  // every vector stays on the singlet symmetries bit for bit: x and the first residual are projected,
+  // A keeps them (No <= 32; larger No takes the general sigma and projects p), and M^-1 has them
+  const bool sym = h->d.No <= 32;
   esmp2_status s = ESMP2_OK;
-  int nsig = 0;
-  if (h->x_zero) {  // cold start: A x = 0, the first residual is b
-    cudaMemsetAsync(q, 0, sizeof(double) * h->d.n, st);
-  } else {
-    if ((s = sigma64(h, x, q, lv))) return s;
-    nsig = 1;
+  if (!h->dinv64) {
+    cudaError_t e = dmalloc(reinterpret_cast<void **>(&h->dinv64), sizeof(double) * (size_t)h->d.n, st);
+    if (e != cudaSuccess) return check_cuda(h, e, "preconditioner");
+    k_dinv64<<<2432, 128, 0, st>>>(c, h->dinv64);
+    h->launches += 1;
   }
+  if (!h->x_zero) singlet_project(h, x);
+  int nsig = 0;
+  double sl[32], bnorm = -1.0;
+  // r = -b - A x (projected), p = M^-1 r, the slots rz and rr
+  auto start = [&]() -> esmp2_status {
+    const bool zero = h->x_zero;
+    if (!zero) {
+      if (esmp2_status s2 = sigma64(h, x, q, lv, sym)) return s2;
+      ++nsig;
+    }
+    k_residual<<<kRedBlocks, kRedThreads, 0, st>>>(c, h->b, zero ? nullptr : q, r, h->red, bnorm < 0.0 ? 1 : 0);
+    k_finalize<<<1, 256, 0, st>>>(h->red, kRedBlocks, 2, h->red_out, 3);
+    singlet_project(h, r);
+    k_pcg_start<<<kRedBlocks, kRedThreads, 0, st>>>(c, h->dinv64, r, p, h->red);
+    k_finalize<<<1, 256, 0, st>>>(h->red, kRedBlocks, 2, h->red_out, 0);
+    h->launches += 4;
+    if (esmp2_status s2 = read_slots(h, sl, 32)) return s2;
+    if (bnorm < 0.0) bnorm = std::sqrt(sl[9]);
+    return ESMP2_OK;
+  };
+  if ((s = start())) return s;   // cold start: A x = 0, the first residual is b
   h->x_zero = false;
-  k_pcg_init<<<kRedBlocks, kRedThreads, 0, st>>>(c, h->b, q, r, p, h->red);
-  k_finalize<<<1, 256, 0, st>>>(h->red, kRedBlocks, 3, h->red_out, 0);
-  h->launches += 2;
-  antisym_project(h, p);
-  double sl[32];
-  if ((s = read_slots(h, sl, 32))) return s;
-  const double bnorm = std::sqrt(sl[2]);
   double rr = sl[1];
   int it = 0;
   esmp2_status result = ESMP2_ERR_NOT_CONVERGED;
@@ -746,27 +796,27 @@ esmp2_status solve64(esmp2_handle *h, double tol, int maxit, esmp2_solve_info *i
   if (bnorm == 0.0) { result = ESMP2_OK; h->r_true = true; }
   while (result != ESMP2_OK && it < maxit) {
     if (std::sqrt(rr) <= tol * bnorm) {  // confirm with the true residual
-      if ((s = sigma64(h, x, q, lv))) return s;
-      ++nsig;
-      k_pcg_init<<<kRedBlocks, kRedThreads, 0, st>>>(c, h->b, q, r, p, h->red);
-      k_finalize<<<1, 256, 0, st>>>(h->red, kRedBlocks, 3, h->red_out, 0);
-      h->launches += 2;
-      antisym_project(h, p);
-      if ((s = read_slots(h, sl, 32))) return s;
+      if ((s = start())) return s;
       rr = sl[1];
       relres = std::sqrt(rr) / bnorm;
       if (relres <= tol) { result = ESMP2_OK; h->r_true = true; break; }
     }
-    if ((s = sigma64(h, p, q, lv))) return s;
+    if ((s = sigma64(h, p, q, lv, sym))) return s;
     if (virt_tc && (s = check_device_flag(h))) return s;
     ++nsig;
-    k_dot_w<<<kRedBlocks, kRedThreads, 0, st>>>(c, p, q, h->red);
-    k_finalize<<<1, 256, 0, st>>>(h->red, kRedBlocks, 1, h->red_out, 1);
-    k_pcg_update<<<kRedBlocks, kRedThreads, 0, st>>>(c, h->red_out, x, r, p, q, h->red);
+    if (sym) {   // <p, q> came with the sigma
+      k_finalize<<<1, 256, 0, st>>>(h->red, residual_parts(), 1, h->red_out, 1);
+      h->launches += 1;
+    } else {
+      k_dot_w<<<kRedBlocks, kRedThreads, 0, st>>>(c, p, q, h->red);
+      k_finalize<<<1, 256, 0, st>>>(h->red, kRedBlocks, 1, h->red_out, 1);
+      h->launches += 2;
+    }
+    k_pcg_update<<<kRedBlocks, kRedThreads, 0, st>>>(c, h->red_out, h->dinv64, x, r, p, q, h->red);
     k_finalize<<<1, 256, 0, st>>>(h->red, kRedBlocks, 2, h->red_out, 2);
-    k_pcg_p<<<kRedBlocks, kRedThreads, 0, st>>>(c, h->red_out, r, p);
-    h->launches += 5;
-    antisym_project(h, p);
+    k_pcg_p<<<kRedBlocks, kRedThreads, 0, st>>>(c, h->red_out, h->dinv64, r, p);
+    h->launches += 3;
+    if (!sym) antisym_project(h, p);
     if ((s = read_slots(h, sl, 32))) return s;
     ++it;
     if (!(sl[3] > 0.0)) { h->err = "CG: p.Ap <= 0 (operator not positive definite)"; result = ESMP2_ERR_INDEFINITE; break; }

@@ -1,7 +1,9 @@
-// The float64 true residual r = -b - A x of the mixed-precision refinement in one pass over the
-// amplitudes that are independent under the singlet symmetries (antisymmetric T, X, Y;
-// S_ij^ab = S_ji^ba), in the basis whose occupied orbitals other than t diagonalise F_oo (arrow
-// form of the occupied-index terms), for full-storage float64 vectors and No <= 32.
+// One pass over the amplitudes that are independent under the singlet symmetries (antisymmetric T,
+// X, Y; S_ij^ab = S_ji^ba), full-storage float64 vectors, No <= 32, in two forms:
+//   * the true residual r = -b - A x of the mixed-precision refinement, in the basis whose occupied
+//     orbitals other than t diagonalise F_oo (arrow form of the occupied-index terms);
+//   * SIG: y = A x in the TOP basis after the index contractions (sigma.cu index_terms64), the last
+//     stage of the float64 sigma, with the partials of <x, y>.
 //
 // The general float64 sigma (sigma.cu) combines the virtual-index products, adds the couplings to y
 // element by element on every stored image (four of T, X, Y, two of S) and leaves r to a further
@@ -27,8 +29,9 @@ struct RC {
   const double *F;          // Fock matrix of the working basis, N x N
   double omega;
   const double *x, *b;
-  const double *P;          // x F: T, X, Y (i < j) and S slices; Z: F Z (or nullptr)
-  const double *yz;         // Z F (P != nullptr) or Z F + F Z (Z slices)
+  const double *P;          // x F: T, X, Y (i < j) and S slices
+  const double *Pz;         // Z: F Z (block vector) or nullptr
+  const double *yz;         // Z F (Pz != nullptr) or Z F + F Z (Z slices)
   double *r;
   const double *VX, *WZ, *OC1, *OX, *OZ, *G, *H, *CYZ;
   const double *rho, *kap;  // reduced-cost basis: row sums [5 No^2][Nv], column sums of the Z slices
@@ -65,10 +68,13 @@ __device__ __forceinline__ void cta_items(int64_t items, int64_t &first, int64_t
 
 // T, X, Y: item = (slice i < j, tile pair ta <= tb).  AV (reduced-cost basis): the virtual-index
 // terms x F - (x F)^T element-wise from the arrow form of F_vv.
-template <int BLK, bool AV>
-__global__ void __launch_bounds__(kThreads) kr_anti(const RC c) {
-  __shared__ double Pb[kT][kT + 1];   // the transposed product tile, then -r of the tile
-  const int nt = (c.Nv + kT - 1) / kT, npairs = nt * (nt + 1) / 2, No = c.No, Nv = c.Nv, nh = No * (No - 1) / 2;
+// SIG: the occupied-index terms are in P; y also goes to the slice (j, i), and the slices i = j (zero)
+// are items too.
+typedef double Tile[kT][kT + 1];
+template <int BLK, bool AV, bool SIG>
+__device__ __forceinline__ void kr_anti(const RC &c, Tile &Pb /* the transposed product tile, then -r of the tile */) {
+  const int nt = (c.Nv + kT - 1) / kT, npairs = nt * (nt + 1) / 2, No = c.No, Nv = c.Nv;
+  const int nh = No * (SIG ? No + 1 : No - 1) / 2;
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   int64_t first, last;
   cta_items((int64_t)nh * npairs, first, last);
@@ -77,11 +83,19 @@ __global__ void __launch_bounds__(kThreads) kr_anti(const RC c) {
     int k = (int)(it / npairs), tp = (int)(it % npairs), ta = 0, i = 0;
     while (tp >= nt - ta) { tp -= nt - ta; ++ta; }
     const int tb = ta + tp;
-    while (k >= No - 1 - i) { k -= No - 1 - i; ++i; }
-    const int j = i + 1 + k;
+    while (k >= (SIG ? No : No - 1) - i) { k -= (SIG ? No : No - 1) - i; ++i; }
+    const int j = i + (SIG ? 0 : 1) + k;
     const int64_t so = c.sl(BLK, i, j);
+    if (SIG && i == j) {   // uniform
+      for (int q = ty; q < kT; q += 8) {
+        const int a = ta * kT + q, b = tb * kT + tx, a2 = tb * kT + q, b2 = ta * kT + tx;
+        if (a < Nv && b < Nv) c.r[so + (int64_t)a * Nv + b] = 0.0;
+        if (a2 < Nv && b2 < Nv) c.r[so + (int64_t)a2 * Nv + b2] = 0.0;
+      }
+      continue;
+    }
     const double *x = c.x + so, *P = c.P + so, *bv = c.b + so;
-    double *r = c.r + so;
+    double *r = c.r + so, *rj = c.r + c.sl(BLK, j, i);
     const int b = tb * kT + tx;
     double pa[4], xe[4], bb[4];
     if constexpr (!AV) __syncthreads();   // Pb of the previous item has been read
@@ -91,7 +105,7 @@ __global__ void __launch_bounds__(kThreads) kr_anti(const RC c) {
       const int64_t e = (int64_t)a * Nv + b;
       const bool in = a < Nv && b < Nv;
       xe[rr] = in ? x[e] : 0.0;
-      bb[rr] = in ? bv[e] : 0.0;
+      bb[rr] = !SIG && in ? bv[e] : 0.0;
       if constexpr (!AV) {
         const int a2 = tb * kT + q, b2 = ta * kT + tx;
         pa[rr] = in ? P[e] : 0.0;
@@ -99,7 +113,7 @@ __global__ void __launch_bounds__(kThreads) kr_anti(const RC c) {
       }
     }
     const bool i0 = i == 0;
-    const double cxe = -c.omega + (BLK == BT ? 0.0 : c.v(0, 0) - c.o(0, 0)) - (c.o(i, i) + c.o(j, j));
+    const double cxe = -c.omega + (BLK == BT ? 0.0 : c.v(0, 0) - c.o(0, 0)) - (SIG ? 0.0 : c.o(i, i) + c.o(j, j));
     const double s1 = i0 ? 1.0 : c.o(0, i), s2 = i0 ? 0.0 : c.o(0, j), f00 = c.ov(0, 0), fi0 = c.ov(i, 0), fj0 = c.ov(j, 0);
     const double *t1p = i0 ? c.OC1 + ((int64_t)BLK * No + j) * c.NvNv : c.x + c.sl(BLK, 0, j);
     const double *t2p = c.x + c.sl(BLK, 0, i0 ? j : i);   // x_i0 = -x_0i (not used for i = 0)
@@ -140,8 +154,11 @@ __global__ void __launch_bounds__(kThreads) kr_anti(const RC c) {
       const bool ok = a < Nv && bin && (ta < tb || q < tx) && !(BLK == BX && (i0 || a == 0));   // a < b; X: b >= 1 follows
       if (ok) {
         const int64_t ab = (int64_t)a * Nv + b;
-        double u = cxe * xe[rr] - s1 * t1p[ab];
-        if (!i0) u += s2 * t2p[ab];
+        double u = cxe * xe[rr];
+        if constexpr (!SIG) {
+          u -= s1 * t1p[ab];
+          if (!i0) u += s2 * t2p[ab];
+        }
         if constexpr (AV) {   // X_ba = -X_ab
           u += fvbb * xe[rr];
           if (a == 0) u -= c.rho[(int64_t)(BLK * No * No + i * No + j) * Nv + b];
@@ -164,10 +181,13 @@ __global__ void __launch_bounds__(kThreads) kr_anti(const RC c) {
           u += f00 * A1[ab] + fobj * A2[a] - fobi * A3[a] - c.ov(j, a) * h2 + c.ov(i, a) * h3;
           if (i0 && a == 0) u += r1[b];
         }
-        rv[rr] = -bb[rr] - u;
-        nrm += rv[rr] * rv[rr];
+        rv[rr] = SIG ? u : -bb[rr] - u;
+        nrm += (SIG ? xe[rr] : rv[rr]) * rv[rr];
       }
-      if (a < Nv && bin && (ta < tb || q <= tx)) r[(int64_t)a * Nv + b] = rv[rr];
+      if (a < Nv && bin && (ta < tb || q <= tx)) {
+        r[(int64_t)a * Nv + b] = rv[rr];
+        if (SIG) rj[(int64_t)a * Nv + b] = -rv[rr];
+      }
     }
     __syncthreads();
 #pragma unroll
@@ -176,7 +196,10 @@ __global__ void __launch_bounds__(kThreads) kr_anti(const RC c) {
 #pragma unroll
     for (int rr = 0; rr < 4; ++rr) {   // element (tb*32 + q, ta*32 + tx) = -r(ta*32 + tx, tb*32 + q)
       const int q = ty + 8 * rr, a = tb * kT + q, b2 = ta * kT + tx;
-      if (a < Nv && b2 < Nv && (ta < tb || q > tx)) r[(int64_t)a * Nv + b2] = Pb[tx][q];
+      if (a < Nv && b2 < Nv && (ta < tb || q > tx)) {
+        r[(int64_t)a * Nv + b2] = Pb[tx][q];
+        if (SIG) rj[(int64_t)a * Nv + b2] = -Pb[tx][q];
+      }
     }
     if constexpr (AV) __syncthreads();
   }
@@ -184,9 +207,8 @@ __global__ void __launch_bounds__(kThreads) kr_anti(const RC c) {
 }
 
 // S: item = (slice pair i <= j, tile (ta, tb)); r_ji = r_ij^T
-template <bool AV>
-__global__ void __launch_bounds__(kThreads) kr_s(const RC c) {
-  __shared__ double Pb[kT][kT + 1], Zt[kT][kT + 1], Ot[kT][kT + 1];
+template <bool AV, bool SIG>
+__device__ __forceinline__ void kr_s(const RC &c, Tile &Pb, Tile &Zt, Tile &Ot) {
   const int nt = (c.Nv + kT - 1) / kT, No = c.No, Nv = c.Nv, npair = No * (No + 1) / 2;
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   int64_t first, last;
@@ -212,7 +234,7 @@ __global__ void __launch_bounds__(kThreads) kr_s(const RC c) {
       if (i0) Ot[q][tx] = in ? OZj[e2] : 0.0;
     }
     __syncthreads();
-    const double cxe = -c.omega - (c.o(i, i) + c.o(j, j)), f00 = c.ov(0, 0);
+    const double cxe = -c.omega - (SIG ? 0.0 : c.o(i, i) + c.o(j, j)), f00 = c.ov(0, 0);
     const double s1 = i0 ? 1.0 : c.o(0, i), s2 = j0 ? 1.0 : c.o(0, j);
     const double *t1p = i0 ? c.OC1 + ((int64_t)BS * No + j) * c.NvNv : c.x + c.sl(BS, 0, j);
     const double *t2p = c.x + c.sl(BS, i, 0);   // j = 0 (then i = 0): OC1_0 transposed
@@ -229,9 +251,12 @@ __global__ void __launch_bounds__(kThreads) kr_s(const RC c) {
       if (a < Nv && b < Nv && (!diag || q <= tx)) {
         const int64_t ab = (int64_t)a * Nv + b;
         const double xe = c.x[sij + ab];
-        double u = cxe * xe - s1 * t1p[ab] + f00 * (Zij[ab] + Zt[tx][q]);
-        if (j0) u -= c.OC1[(int64_t)BS * No * c.NvNv + (int64_t)b * Nv + a];   // sum_m F_mt S_0m^ab = sum_m F_mt S_m0^ba
-        else u -= s2 * t2p[ab];
+        double u = cxe * xe + f00 * (Zij[ab] + Zt[tx][q]);
+        if constexpr (!SIG) {
+          u -= s1 * t1p[ab];
+          if (j0) u -= c.OC1[(int64_t)BS * No * c.NvNv + (int64_t)b * Nv + a];   // sum_m F_mt S_0m^ab = sum_m F_mt S_m0^ba
+          else u -= s2 * t2p[ab];
+        }
         if constexpr (AV) {   // S_ji^ba = S_ij^ab
           const double *xs = c.x + sij;
           u += b == 0 ? c.rho[(int64_t)(BS * No * No + i * No + j) * Nv + a] : fvbb * xe + xs[(int64_t)a * Nv] * fv0b;
@@ -249,8 +274,8 @@ __global__ void __launch_bounds__(kThreads) kr_s(const RC c) {
           u -= Ot[tx][q];
           if (a == 0) u += c.H[(int64_t)j * Nv + b];
         }
-        rv[rr] = -c.b[sij + ab] - u;
-        nrm += (diag && q == tx ? 1.0 : 2.0) * rv[rr] * rv[rr];
+        rv[rr] = SIG ? u : -c.b[sij + ab] - u;
+        nrm += (diag && q == tx ? 1.0 : 2.0) * (SIG ? xe : rv[rr]) * rv[rr];
         c.r[sij + ab] = rv[rr];
       }
     }
@@ -268,8 +293,8 @@ __global__ void __launch_bounds__(kThreads) kr_s(const RC c) {
 }
 
 // Z: a warp per row (slice, a), what depends on the row alone taken once
-template <bool AV>
-__global__ void __launch_bounds__(kThreads) kr_z(const RC c) {
+template <bool AV, bool SIG>
+__device__ __forceinline__ void kr_z(const RC &c) {
   const int No = c.No, Nv = c.Nv, lane = threadIdx.x & 31;
   const int64_t rows = (int64_t)No * No * Nv;
   double nrm = 0.0;
@@ -284,13 +309,13 @@ __global__ void __launch_bounds__(kThreads) kr_z(const RC c) {
       continue;
     }
     const double *x = c.x + so, *bv = c.b + so, *yz = c.yz + (int64_t)s * c.NvNv + (int64_t)a * Nv;
-    const double *fz = c.P ? c.P + so : nullptr;
+    const double *fz = c.Pz ? c.Pz + so : nullptr;
     const double *Sij = c.x + c.sl(BS, i, j) + (int64_t)a * Nv, *Si0 = c.x + c.sl(BS, i, 0) + (int64_t)a * Nv;
     const double *T0j = c.x + c.sl(BT, 0, j), *Y0j = c.x + c.sl(BY, 0, j);   // row 0
     const double *t1 = (i0 ? c.OC1 + ((int64_t)BZ * No + j) * c.NvNv : c.x + c.sl(BZ, 0, j)) + (int64_t)a * Nv;
     const double *t2 = c.x + c.sl(BZ, i, 0) + (int64_t)a * Nv;
     const double *F0 = c.F + No, *Fj = c.F + (int64_t)j * c.N + No;
-    const double cxe = -c.omega + (c.v(0, 0) - c.o(0, 0)) - (c.o(i, i) + c.o(j, j)), s1 = i0 ? 1.0 : c.o(0, i), s2 = c.o(0, j);
+    const double cxe = -c.omega + (c.v(0, 0) - c.o(0, 0)) - (SIG ? 0.0 : c.o(i, i) + c.o(j, j)), s1 = i0 ? 1.0 : c.o(0, i), s2 = c.o(0, j);
     const double f00 = c.ov(0, 0), fj0 = c.ov(j, 0), foai = c.ov(i, a), sija0 = Sij[0], si0a0 = Si0[0];
     const double fy = (i0 ? c.v(a, 0) : 0.0) - (a == 0 ? c.o(0, i) : 0.0);
     double xa0 = 0.0, fva = 0.0, fvaa = 0.0;
@@ -305,8 +330,8 @@ __global__ void __launch_bounds__(kThreads) kr_z(const RC c) {
       double rb = 0.0;
       if (b != 0) {
         const double xe = x[b];
-        double u = cxe * xe - s1 * t1[b] - s2 * t2[b] + f00 * Sij[b] - __ldg(F0 + b) * sija0 - fj0 * Si0[b] +
-                   __ldg(Fj + b) * si0a0 + foai * T0j[b];
+        double u = cxe * xe + f00 * Sij[b] - __ldg(F0 + b) * sija0 - fj0 * Si0[b] + __ldg(Fj + b) * si0a0 + foai * T0j[b];
+        if constexpr (!SIG) u -= s1 * t1[b] + s2 * t2[b];
         if (i0 || a == 0) u += fy * Y0j[b];
         if constexpr (AV) {
           u += c.v(b, b) * xe + xa0 * __ldg(Fv0 + b);
@@ -315,13 +340,29 @@ __global__ void __launch_bounds__(kThreads) kr_z(const RC c) {
           u += yz[b];
           if (fz) u += fz[b];
         }
-        rb = -bv[b] - u;
-        nrm += rb * rb;
+        rb = SIG ? u : -bv[b] - u;
+        nrm += (SIG ? xe : rb) * rb;
       }
       r[b] = rb;
     }
   }
   cta_partial(2.0 * nrm, c.red + c.base + blockIdx.x);
+}
+
+// All blocks in one launch (grid.y: T, X, Y, Z, S): the small sizes are bound by their launches.  SIG
+// without the S part: S of an arbitrary input is left to the element-wise pass of sigma.cu.
+template <bool AV, bool SIG>
+__global__ void __launch_bounds__(kThreads) k_sym_pass(const __grid_constant__ RC cin) {
+  __shared__ Tile t[3];
+  RC c = cin;
+  c.base = (int64_t)blockIdx.y * kGrid;
+  switch (blockIdx.y) {
+    case 0: kr_anti<BT, AV, SIG>(c, t[0]); break;
+    case 1: kr_anti<BX, AV, SIG>(c, t[0]); break;
+    case 2: kr_anti<BY, AV, SIG>(c, t[0]); break;
+    case 3: kr_z<AV, SIG>(c); break;
+    default: kr_s<AV, SIG>(c, t[0], t[1], t[2]); break;
+  }
 }
 
 // ---- arrow sums over an occupied index, weights as launch parameters (constant operands)
@@ -332,8 +373,8 @@ struct ArrowW64 {
 // T, X, Y from the slices i < j: OC1[q] = sum_{l>=1} F_lt x_lq (x_lq = -x_ql for l > q), X also OX[q] =
 // sum_l F_l,t' X_lq; one thread per element (a, b)
 template <int BLK>
-__global__ void __launch_bounds__(128) kr_arrow_anti(int No, int64_t NvNv, int64_t B, const double *__restrict__ x, double *oc1,
-                                                     double *ox, const __grid_constant__ ArrowW64 w) {
+__device__ __forceinline__ void kr_arrow_anti(int No, int64_t NvNv, int64_t B, const double *__restrict__ x, double *oc1, double *ox,
+                                              const ArrowW64 &w) {
   constexpr bool WX = BLK == BX;
   const double *xb = x + BLK * B;
   double *o1 = oc1 + (int64_t)BLK * No * NvNv;
@@ -373,8 +414,8 @@ __global__ void __launch_bounds__(128) kr_arrow_anti(int No, int64_t NvNv, int64
 }
 // S, Z: OC1[m] = sum_{l>=1} F_lt x_lm; Z also OZ[l] = sum_m F_m,t' Z_lm
 template <int BLK>
-__global__ void __launch_bounds__(128) kr_arrow_full(int No, int64_t NvNv, int64_t B, const double *__restrict__ x, double *oc1,
-                                                     double *oz, const __grid_constant__ ArrowW64 w) {
+__device__ __forceinline__ void kr_arrow_full(int No, int64_t NvNv, int64_t B, const double *__restrict__ x, double *oc1, double *oz,
+                                              const ArrowW64 &w) {
   const double *xb = x + BLK * B;
   double *o1 = oc1 + (int64_t)BLK * No * NvNv;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < NvNv; e += (int64_t)gridDim.x * blockDim.x) {
@@ -398,6 +439,17 @@ __global__ void __launch_bounds__(128) kr_arrow_full(int No, int64_t NvNv, int64
 #pragma unroll
     for (int m = 0; m < 32; ++m)
       if (m < No) o1[(int64_t)m * NvNv + e] = c1[m];
+  }
+}
+
+__global__ void __launch_bounds__(128) k_arrow_sums(int No, int64_t NvNv, int64_t B, const double *__restrict__ x, double *oc1,
+                                                    double *ox, double *oz, const __grid_constant__ ArrowW64 w) {
+  switch (blockIdx.y) {   // X first: it does the most
+    case 0: kr_arrow_anti<BX>(No, NvNv, B, x, oc1, ox, w); break;
+    case 1: kr_arrow_full<BZ>(No, NvNv, B, x, oc1, oz, w); break;
+    case 2: kr_arrow_full<BS>(No, NvNv, B, x, oc1, oz, w); break;
+    case 3: kr_arrow_anti<BT>(No, NvNv, B, x, oc1, ox, w); break;
+    default: kr_arrow_anti<BY>(No, NvNv, B, x, oc1, ox, w); break;
   }
 }
 
@@ -438,6 +490,20 @@ __global__ void __launch_bounds__(256) kr_hyll(int No, int64_t NvNv, int64_t B, 
 
 }  // namespace
 
+namespace {
+void fill(esmp2_handle *h, RC &c, const double *F, const double *x) {
+  c.No = h->d.No; c.Nv = h->d.Nv; c.N = h->d.N;
+  c.NvNv = (int64_t)h->d.Nv * h->d.Nv;
+  c.B = h->d.B;
+  c.F = F;
+  c.omega = h->omega_op;
+  c.x = x;
+  c.VX = h->cp.VX; c.WZ = h->cp.WZ; c.OC1 = h->cp.OC1; c.OX = h->cp.OX; c.OZ = h->cp.OZ;
+  c.G = h->cp.G; c.H = h->cp.H; c.CYZ = h->cp.CYZ;
+  c.red = h->red;
+}
+}  // namespace
+
 int residual_parts() { return 5 * kGrid; }
 
 // r = -b - A x (the independent slices), partials of <r, r>_w in h->red (residual_parts()); x with the
@@ -463,6 +529,7 @@ esmp2_status residual_sym(esmp2_handle *h, const double *x, const double *b, dou
   } else if (levels) {
     if ((s = virt_split(h, x, q, h->P64, 2, levels, false))) return s;
     c.yz = q + BZ * B;
+    c.Pz = h->P64;
   } else {   // T, X, Y, S one-sided, Z both terms
     virt64_list(h, F + (int64_t)No * N + No, N, x, q, h->P64, h->slist, h->nslist - NN, h->nslist);
     c.yz = q + BZ * B;
@@ -470,41 +537,36 @@ esmp2_status residual_sym(esmp2_handle *h, const double *x, const double *b, dou
   ArrowW64 w;
   for (int l = 0; l < 32; ++l) { w.fl[l] = h->arrow_w64[l]; w.fk[l] = h->arrow_w64[32 + l]; }
   const unsigned ga = (unsigned)std::min<int64_t>(cdiv(NvNv, 128), 4096);
-  kr_arrow_anti<BT><<<ga, 128, 0, st>>>(No, NvNv, B, x, h->cp.OC1, h->cp.OX, w);
-  kr_arrow_anti<BX><<<ga, 128, 0, st>>>(No, NvNv, B, x, h->cp.OC1, h->cp.OX, w);
-  kr_arrow_anti<BY><<<ga, 128, 0, st>>>(No, NvNv, B, x, h->cp.OC1, h->cp.OX, w);
-  kr_arrow_full<BS><<<ga, 128, 0, st>>>(No, NvNv, B, x, h->cp.OC1, h->cp.OZ, w);
-  kr_arrow_full<BZ><<<ga, 128, 0, st>>>(No, NvNv, B, x, h->cp.OC1, h->cp.OZ, w);
+  k_arrow_sums<<<dim3(ga, 5), 128, 0, st>>>(No, NvNv, B, x, h->cp.OC1, h->cp.OX, h->cp.OZ, w);
   launch_intermediates64(h, F, 2, x);
-  c.No = No; c.Nv = Nv; c.N = N; c.NvNv = NvNv; c.B = B;
-  c.F = F;
-  c.omega = h->omega_op;
-  c.x = x; c.b = b; c.r = r;
-  c.VX = h->cp.VX; c.WZ = h->cp.WZ; c.OC1 = h->cp.OC1; c.OX = h->cp.OX; c.OZ = h->cp.OZ;
-  c.G = h->cp.G; c.H = h->cp.H; c.CYZ = h->cp.CYZ;
-  c.red = h->red;
+  fill(h, c, F, x);
+  c.b = b;
+  c.r = r;
   {
     const double bytes = 8.0 * (double)(h->nslist) * NvNv * (av ? 3.0 : 4.0);
     KScope ks(st, ESMP2_KT_COUPLING, bytes, bytes);
-    auto run = [&](auto tag) {
-      constexpr bool AV = decltype(tag)::value;
-      c.base = 0;
-      kr_anti<BT, AV><<<kGrid, kThreads, 0, st>>>(c);
-      c.base = kGrid;
-      kr_anti<BX, AV><<<kGrid, kThreads, 0, st>>>(c);
-      c.base = 2 * kGrid;
-      kr_anti<BY, AV><<<kGrid, kThreads, 0, st>>>(c);
-      c.base = 3 * kGrid;
-      kr_s<AV><<<kGrid, kThreads, 0, st>>>(c);
-      if (!AV && !levels) c.P = nullptr;   // Z: both terms are in yz
-      c.base = 4 * kGrid;
-      kr_z<AV><<<kGrid, kThreads, 0, st>>>(c);
-    };
-    if (av) run(std::true_type{});
-    else run(std::false_type{});
+    if (av) k_sym_pass<true, false><<<dim3(kGrid, 5), kThreads, 0, st>>>(c);
+    else k_sym_pass<false, false><<<dim3(kGrid, 5), kThreads, 0, st>>>(c);
   }
-  h->launches += 10;
+  h->launches += 2;
   return check_cuda(h, cudaGetLastError(), "residual");
+}
+
+// The last stage of the float64 sigma in the TOP basis (No <= 32): y from the products P64 with the
+// occupied sums folded in (T, X, Y; with s_sym also S) and the Z part already in y; the partials of
+// <x, y> over these blocks go to h->red (T, X, Y, Z and, with s_sym, S: residual_parts() in all).
+esmp2_status sigma_sym_tail(esmp2_handle *h, const double *x, double *y, bool s_sym) {
+  RC c{};
+  launch_intermediates64(h, h->F, 0, x);
+  fill(h, c, h->F, x);
+  c.P = h->P64;
+  c.yz = y + BZ * h->d.B;
+  c.r = y;
+  const double bytes = 24.0 * (double)h->d.n * (s_sym ? 1.0 : 0.8);
+  KScope ks(h->stream, ESMP2_KT_COUPLING, bytes, bytes);
+  k_sym_pass<false, true><<<dim3(kGrid, s_sym ? 5 : 4), kThreads, 0, h->stream>>>(c);
+  h->launches += 1;
+  return check_cuda(h, cudaGetLastError(), "sigma64");
 }
 
 // per-block Hylleraas partials (2 x 5 quantities of hyll_parts() CTAs) from the residual of residual_sym

@@ -55,7 +55,7 @@ __device__ __forceinline__ bool valid_elem(int blk, int i, int j, int a, int b) 
 // (a) per (i, j, b): VX[i][j][b] = sum_c Fov[0][c] X[i][j][c][b],
 //                    GP[k][j][b] = sum_c Fov[k][c] (X+Z)[k][j][c][b]
 template <typename T, typename CT>
-__global__ void k_inter_a(CtxT<CT> c, const T *x, CouplingsT<CT> cp) {
+__device__ __forceinline__ void inter_a(const CtxT<CT> &c, const T *x, const CouplingsT<CT> &cp) {
   const int No = c.No, Nv = c.Nv;
   const int64_t n = (int64_t)No * No * Nv;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
@@ -77,7 +77,7 @@ __global__ void k_inter_a(CtxT<CT> c, const T *x, CouplingsT<CT> cp) {
 // (b) per (q, a, b): OX[q][ab] = sum_k Fov[k][0] X[k][q][ab], OZ[q][ab] = sum_k Fov[k][0] Z[q][k][ab];
 //     arrow form: OC1[blk][q][ab] = sum_{l>=1} Foo[l][0] x[blk][l][q][ab], OC2 likewise on the 2nd index
 template <typename T, typename CT>
-__global__ void k_inter_b(CtxT<CT> c, const T *x, CouplingsT<CT> cp) {
+__device__ __forceinline__ void inter_b(const CtxT<CT> &c, const T *x, const CouplingsT<CT> &cp) {
   const int No = c.No, Nv = c.Nv;
   const int64_t NvNv = (int64_t)Nv * Nv, n = (int64_t)No * NvNv;
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
@@ -108,7 +108,7 @@ __global__ void k_inter_b(CtxT<CT> c, const T *x, CouplingsT<CT> cp) {
 // (c) warp per row (i, j, a): WZ[i][j][a] = sum_c Fov[0][c] Z[i][j][a][c],
 //                             HP[i][j][a] = sum_c Fov[j][c] (Y+Z)[i][j][a][c]
 template <typename T, typename CT>
-__global__ void k_inter_c(CtxT<CT> c, const T *x, CouplingsT<CT> cp) {
+__device__ __forceinline__ void inter_c(const CtxT<CT> &c, const T *x, const CouplingsT<CT> &cp) {
   const int No = c.No, Nv = c.Nv, lane = threadIdx.x & 31;
   const int64_t rows = (int64_t)No * No * Nv;
   const int64_t w0 = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
@@ -156,16 +156,18 @@ __global__ void k_inter_d(CtxT<CT> c, const T *x, CouplingsT<CT> cp) {
   }
 }
 
+// (a), (b) and (c) side by side (grid.y), (d) after them; arrow = 2: the sums (b) come from the caller
+template <typename T, typename CT>
+__global__ void __launch_bounds__(256) k_inter_abc(CtxT<CT> c, const T *x, CouplingsT<CT> cp) {
+  if (blockIdx.y == 0) inter_a<T, CT>(c, x, cp);
+  else if (blockIdx.y == 1) inter_c<T, CT>(c, x, cp);
+  else inter_b<T, CT>(c, x, cp);
+}
 template <typename T, typename CT>
 void launch_inter(esmp2_handle *h, const CtxT<CT> &c, const T *x, const CouplingsT<CT> &cp) {
-  k_inter_a<T, CT><<<1216, 256, 0, h->stream>>>(c, x, cp);
-  if (c.arrow != 2) {   // 2: the sums over an occupied index come from the caller
-    k_inter_b<T, CT><<<1216, 256, 0, h->stream>>>(c, x, cp);
-    h->launches += 1;
-  }
-  k_inter_c<T, CT><<<1216, 256, 0, h->stream>>>(c, x, cp);
+  k_inter_abc<T, CT><<<dim3(1216, c.arrow == 2 ? 2 : 3), 256, 0, h->stream>>>(c, x, cp);
   k_inter_d<T, CT><<<(unsigned)cdiv(3LL * c.No * c.Nv, 256), 256, 0, h->stream>>>(c, x, cp);
-  h->launches += 3;
+  h->launches += 2;
 }
 
 // Vector loads/stores of VW consecutive elements (16 bytes when VW * sizeof(T) == 16); the
@@ -411,6 +413,17 @@ void launch_couple(const CtxT<CT> &c, const TX *x, TY *y, const CouplingsT<CT> &
     launch_couple_vw<1>(c, x, y, cp, st);
 }
 
+// the S block alone, float64
+void launch_couple_s(const CtxT<double> &c, const double *x, double *y, const CouplingsT<double> &cp, cudaStream_t st) {
+  const double bytes = 24.0 * (double)c.B;
+  KScope ks(st, ESMP2_KT_COUPLING, bytes, bytes);
+  const dim3 grid((unsigned)((c.Nv + 31) / 32), (unsigned)(c.No * c.No));
+  if (c.Nv % 2 == 0 && (reinterpret_cast<uintptr_t>(x) | reinterpret_cast<uintptr_t>(y)) % 16 == 0)
+    k_couple<BS, 2, double, double, double><<<grid, 256, 0, st>>>(c, x, y, cp);
+  else
+    k_couple<BS, 1, double, double, double><<<grid, 256, 0, st>>>(c, x, y, cp);
+}
+
 }  // namespace
 
 template <typename CT>
@@ -497,12 +510,11 @@ void contractions64(esmp2_handle *h, const double *F, const double *x, double *y
 // No=20 Nv=200 sigma, now 3.4 ms.
 constexpr int kOccW = 16;
 size_t occ_smem(int No) { return sizeof(double) * ((size_t)No * No * kOccW + No * No); }
-template <bool ANTI>
-__global__ void __launch_bounds__(256) k_occ64(int No, int Nv, int N, const double *F, const double *x, double *out,
-                                               const double *add) {
-  extern __shared__ double sm_occ[];
+//   ONE (S with S_ij^ab = S_ji^ba): only sum_l F_li S_lj, taken off P_ij: y_ij = P_ij + P_ji^T.
+template <bool ANTI, bool ONE>
+__device__ __forceinline__ void occ64(int blk, int No, int Nv, int N, const double *F, const double *x, double *out,
+                                      const double *add, double *sm_occ) {
   double *M = sm_occ, *Fs = sm_occ + No * No * kOccW;
-  const int blk = ANTI ? (blockIdx.y == 0 ? BT : blockIdx.y == 1 ? BX : BY) : (blockIdx.y == 0 ? BS : BZ);
   const int64_t NvNv = (int64_t)Nv * Nv, e0 = (int64_t)blockIdx.x * kOccW, base = (int64_t)blk * No * No * NvNv;
   const int w = threadIdx.x & 15, NN = No * No;
   const int64_t e = e0 + w;
@@ -541,7 +553,10 @@ __global__ void __launch_bounds__(256) k_occ64(int No, int Nv, int N, const doub
         const int i = i0 + ii;
         if (i < No) {   // uniform
           const double fi = Fl[i], mi = ANTI ? Ml[i * kOccW] : M[(i * No + l) * kOccW + w];
-          if constexpr (ANTI) {   // x_il = -x_li
+          if constexpr (ONE) {
+            acc[ii][0] = fma(fi, ma, acc[ii][0]);
+            acc[ii][1] = fma(fi, mb, acc[ii][1]);
+          } else if constexpr (ANTI) {   // x_il = -x_li
             acc[ii][0] = fma(fi, ma, fma(-fa, mi, acc[ii][0]));
             acc[ii][1] = fma(fi, mb, fma(-fb, mi, acc[ii][1]));
           } else {
@@ -564,32 +579,55 @@ __global__ void __launch_bounds__(256) k_occ64(int No, int Nv, int N, const doub
   }
 }
 
-// Virtual- and occupied-index terms of y for a dense F_oo: the products, the occupied sums, then
-// y_ij = P_ij - P_ij^T of the T, X, Y blocks (tc_levels: digit levels of the products, 0: float64 GEMMs)
+// grid.y: S, Z, X, T, Y (the larger ones first)
+__global__ void __launch_bounds__(256) k_occ64(int No, int Nv, int N, const double *F, const double *x, double *y, double *P,
+                                               const double *add, int s_sym) {
+  extern __shared__ double sm_occ[];
+  if (blockIdx.y >= 2) {
+    occ64<true, false>(blockIdx.y == 2 ? BX : blockIdx.y == 3 ? BT : BY, No, Nv, N, F, x, P, nullptr, sm_occ);
+  } else if (blockIdx.y == 0 && s_sym) {
+    occ64<false, true>(BS, No, Nv, N, F, x, P, nullptr, sm_occ);
+  } else {
+    occ64<false, false>(blockIdx.y == 0 ? BS : BZ, No, Nv, N, F, x, y, add, sm_occ);
+  }
+}
+
+// Virtual- and occupied-index terms of y for a dense F_oo: the products with the occupied sums folded
+// in (T, X, Y and, with s_sym, S in P64; the others in y), for No <= 32 (larger No: y complete) (tc_levels: digit levels of the products, 0: float64 GEMMs)
 // mid: event recorded between the virtual- and the occupied-index terms
-esmp2_status index_terms64(esmp2_handle *h, const double *F, const double *x, double *y, int tc_levels, cudaEvent_t mid = nullptr) {
+esmp2_status index_terms64(esmp2_handle *h, const double *F, const double *x, double *y, int tc_levels, bool s_sym,
+                           cudaEvent_t mid = nullptr) {
   const int No = h->d.No, Nv = h->d.Nv, N = h->d.N;
   const bool fused = No <= 32;
   esmp2_status s = ensure_p64(h);
   if (!s) s = ensure_slist(h);
   if (s) return s;
-  if (tc_levels) s = virt_split(h, x, y, h->P64, 1, tc_levels, !fused);
-  else virt64_list(h, F + (int64_t)No * N + No, N, x, y, h->P64, h->slist, 3 * (No * (No - 1) / 2), h->nslist);
+  s_sym = s_sym && fused;
+  if (tc_levels) s = virt_split(h, x, y, h->P64, s_sym ? 2 : 1, tc_levels, !fused);
+  else virt64_list(h, F + (int64_t)No * N + No, N, x, y, h->P64, h->slist, h->nslist - (s_sym ? 1 : 2) * No * No, h->nslist);
   if (s) return s;
   if (mid) cudaEventRecord(mid, h->stream);
   if (fused) {
-    const int lim = (int)occ_smem(32);
-    cudaError_t e = smem_limit_once(reinterpret_cast<const void *>(k_occ64<true>), lim);
-    if (e == cudaSuccess) e = smem_limit_once(reinterpret_cast<const void *>(k_occ64<false>), lim);
-    if (e != cudaSuccess) return check_cuda(h, e, "k_occ64 shared-memory limit");
-    const unsigned g = (unsigned)cdiv((int64_t)Nv * Nv, kOccW);
-    if (No > 1) k_occ64<true><<<dim3(g, 3), 256, occ_smem(No), h->stream>>>(No, Nv, N, F, x, h->P64, nullptr);
-    k_occ64<false><<<dim3(g, 2), 256, occ_smem(No), h->stream>>>(No, Nv, N, F, x, y, tc_levels ? h->P64 : nullptr);
-    h->launches += 2;
+    if (cudaError_t e = smem_limit_once(reinterpret_cast<const void *>(k_occ64), (int)occ_smem(32)))
+      return check_cuda(h, e, "k_occ64 shared-memory limit");
+    k_occ64<<<dim3((unsigned)cdiv((int64_t)Nv * Nv, kOccW), No > 1 ? 5 : 2), 256, occ_smem(No), h->stream>>>(
+        No, Nv, N, F, x, y, h->P64, tc_levels ? h->P64 : nullptr, s_sym);
+    h->launches += 1;
+  } else {
+    combine_sym(h, y);
+    contractions64(h, F, x, y, 2);
   }
-  combine_sym(h, y);
-  if (!fused) contractions64(h, F, x, y, 2);
   return check_cuda(h, cudaGetLastError(), "index terms");
+}
+
+// couplings, shift and masks after index_terms64 (TOP basis, No <= 32): the symmetric pass, and the
+// element-wise pass for an S without the spin-flip symmetry
+esmp2_status sigma64_finish(esmp2_handle *h, const double *x, double *y, bool s_sym) {
+  esmp2_status s = sigma_sym_tail(h, x, y, s_sym);
+  if (s || s_sym) return s;
+  launch_couple_s(make_ctx<double>(h, h->F, 0), x, y, h->cp, h->stream);
+  h->launches += 1;
+  return check_cuda(h, cudaGetLastError(), "sigma64");
 }
 
 // Per-stage timing of `reps` float64 sigma builds (CUDA events on the handle's stream):
@@ -601,11 +639,16 @@ esmp2_status profile64(esmp2_handle *h, const double *x, double *y, int reps, do
   double acc[5] = {0, 0, 0, 0, 0};
   for (int r = 0; r < reps; ++r) {
     cudaEventRecord(ev[0], h->stream);
-    if (esmp2_status s = index_terms64(h, h->F, x, y, tc_levels, ev[1])) return s;
+    if (esmp2_status s = index_terms64(h, h->F, x, y, tc_levels, false, ev[1])) return s;
     cudaEventRecord(ev[2], h->stream);
-    launch_intermediates64(h, h->F, 0, x);
-    cudaEventRecord(ev[3], h->stream);
-    launch_couple64(h, h->F, 0, x, y);
+    if (h->d.No > 32) {
+      launch_intermediates64(h, h->F, 0, x);
+      cudaEventRecord(ev[3], h->stream);
+      launch_couple64(h, h->F, 0, x, y);
+    } else {
+      cudaEventRecord(ev[3], h->stream);   // the intermediates are part of the last stage
+      if (esmp2_status s = sigma64_finish(h, x, y, false)) return s;
+    }
     cudaEventRecord(ev[4], h->stream);
     cudaEventSynchronize(ev[4]);
     for (int k = 0; k < 4; ++k) {
@@ -842,8 +885,9 @@ void combine_s(esmp2_handle *h, double *y) {
 // cores, digit levels 2 .. tc_levels (F_vv of the handle); 0: float64 GEMMs with F.
 esmp2_status sigma64_F(esmp2_handle *h, const double *F, int arrow, const double *x, double *y, int tc_levels,
                        bool s_sym) {
-  if (!arrow) {
-    if (esmp2_status s = index_terms64(h, F, x, y, tc_levels)) return s;
+  if (!arrow) {   // F is the handle's
+    if (esmp2_status s = index_terms64(h, F, x, y, tc_levels, s_sym)) return s;
+    if (h->d.No <= 32) return sigma64_finish(h, x, y, s_sym);
   } else {
     if (esmp2_status s0 = ensure_p64(h)) return s0;
     if (tc_levels) {
@@ -861,7 +905,9 @@ esmp2_status sigma64_F(esmp2_handle *h, const double *F, int arrow, const double
   return check_cuda(h, cudaGetLastError(), "sigma64");
 }
 
-esmp2_status sigma64(esmp2_handle *h, const double *x, double *y, int tc_levels) { return sigma64_F(h, h->F, 0, x, y, tc_levels); }
+esmp2_status sigma64(esmp2_handle *h, const double *x, double *y, int tc_levels, bool s_sym) {
+  return sigma64_F(h, h->F, 0, x, y, tc_levels, s_sym);
+}
 
 // parts (2)-(3) only: couplings, shift and masks added to y
 esmp2_status sigma64_tail(esmp2_handle *h, const double *F, int arrow, const double *x, double *y) {
