@@ -111,7 +111,7 @@ esmp2_status esmp2::create_impl(esmp2_handle **out, const esmp2_desc *d, cudaStr
   ALLOC(h->cp.OZ, (size_t)No * Nv * Nv); ALLOC(h->cp.G, nC);
   ALLOC(h->cp.GP, (size_t)No * No * Nv); ALLOC(h->cp.HP, (size_t)No * No * Nv); ALLOC(h->cp.H, nC); ALLOC(h->cp.CYZ, nC);
   {
-    const size_t nred = std::max<size_t>(std::max<size_t>((size_t)16 * 1216, (size_t)No * No * No),
+    const size_t nred = std::max<size_t>(std::max<size_t>((size_t)16 * 1216, (size_t)No * No * No + 8 * (size_t)No * No),
                                          (size_t)couple_dot_parts(h));
     ALLOC(h->red, nred);
   }

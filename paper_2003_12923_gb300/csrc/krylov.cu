@@ -80,37 +80,42 @@ __device__ __forceinline__ void block_partials(double (&v)[NQ], double *red) {
 // Sum the partials of nq quantities in fixed order; mode selects the scalar bookkeeping.
 // slots: 0 rz, 1 rr, 2 bb, 3 pq, 4 alpha, 5 beta, 8.. generic results (slots 4, 5 of a zeroed
 // slot array give alpha = beta = 0)
-__global__ void k_finalize(const double *red, int nparts, int nq, double *slots, int mode) {
-  __shared__ double sh[32];
+// One CTA, every quantity in the same pass: it sits on the critical path of each iteration (a loop per
+// quantity on 256 threads took 7.5 us for 6080 partials).
+__global__ void __launch_bounds__(1024) k_finalize(const double *__restrict__ red, int nparts, int nq, double *slots, int mode) {
+  __shared__ double sh[10][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   for (int q = 0; q < nq; ++q) {
     double s = 0.0;
-    for (int k = threadIdx.x; k < nparts; k += blockDim.x) s += red[(int64_t)q * nparts + k];
+#pragma unroll 6
+    for (int k = threadIdx.x; k < nparts; k += 1024) s += red[(int64_t)q * nparts + k];
     s = warp_sum(s);
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      double t = 0.0;
-      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += sh[w];
-      if (mode == 0) {            // init: rz, rr, bb
-        slots[q] = t;
-      } else if (mode == 1) {     // pq -> alpha (no step along a direction of non-positive curvature)
-        slots[3] = t;
-        slots[4] = t > 0.0 ? slots[0] / t : 0.0;
-      } else if (mode == 2) {     // rz_new, rr -> beta
-        if (q == 0) { slots[5] = t / slots[0]; slots[0] = t; }
-        else slots[1] = t;
-      } else if (mode == 5) {     // rr alone
-        slots[1] = t;
-      } else if (mode == 6) {     // rz_new alone -> beta
-        slots[5] = t / slots[0];
-        slots[0] = t;
-      } else if (mode == 7) {     // rz alone (start)
-        slots[0] = t;
-      } else {                    // generic
-        slots[8 + q] = t;
-      }
-    }
-    __syncthreads();
+    if (lane == 0) sh[q][warp] = s;
+  }
+  __syncthreads();
+  if (warp >= nq) return;
+  const int q = warp;
+  const double t = warp_sum(sh[q][lane]);
+  if (lane != 0) return;
+  if (mode == 0) {            // init: rz, rr, bb
+    slots[q] = t;
+  } else if (mode == 1) {     // pq -> alpha (no step along a direction of non-positive curvature)
+    slots[3] = t;
+    slots[4] = t > 0.0 ? slots[0] / t : 0.0;
+  } else if (mode == 2) {     // rz_new, rr -> beta
+    if (q == 0) { slots[5] = t / slots[0]; slots[0] = t; }
+    else slots[1] = t;
+  } else if (mode == 5) {     // rr alone
+    slots[1] = t;
+  } else if (mode == 6) {     // rz_new alone -> beta
+    slots[5] = t / slots[0];
+    slots[0] = t;
+  } else if (mode == 7) {     // rz alone (start)
+    slots[0] = t;
+  } else if (mode == 8) {     // the S-space energy
+    slots[20] = t;
+  } else {                    // generic
+    slots[8 + q] = t;
   }
 }
 
@@ -138,26 +143,44 @@ __global__ void __launch_bounds__(128) k_dinv64(VCtx c, double *dinv) {
   }
 }
 
+// the same with one grid row per block (grid.y = 5): partials of CTA (x, y) at y gridDim.x + x
+constexpr int kRowCtas = 243;   // 5 x 243 CTAs
+template <int NQ>
+__device__ __forceinline__ void block_partials_rows(double (&v)[NQ], double *red) {
+  __shared__ double sh[NQ][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+  for (int q = 0; q < NQ; ++q) {
+    const double s = warp_sum(v[q]);
+    if (lane == 0) sh[q][warp] = s;
+  }
+  __syncthreads();
+  if (warp == 0) {
+#pragma unroll
+    for (int q = 0; q < NQ; ++q) {
+      double s = lane < (int)(blockDim.x >> 5) ? sh[q][lane] : 0.0;
+      s = warp_sum(s);
+      if (lane == 0) red[((int64_t)q * gridDim.y + blockIdx.y) * gridDim.x + blockIdx.x] = s;
+    }
+  }
+}
+
 __device__ __forceinline__ double blk_weight(int blk) { return blk == 1 ? 1.0 : (blk == 4 ? 2.0 : 0.5); }
 
 // p = M^-1 r; partials <r, M^-1 r>_w, <r, r>_w.  Block by block, weights on the block sums; M^-1 is read
 // (8 bytes) instead of formed (an index decode and a float64 division, some 20 operations of the
 // float64 pipe per element: 72 us against 20 at No=8 Nv=80).
 __global__ void k_pcg_start(VCtx c, const double *dinv, const double *r, double *p, double *red) {
-  double v[2] = {0.0, 0.0};
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x, t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  for (int blk = 0; blk < 5; ++blk) {
-    double s0 = 0.0, s1 = 0.0;
-    for (int64_t e = blk * c.B + t0; e < (blk + 1) * c.B; e += stride) {
-      const double ri = r[e], z = dinv[e] * ri;
-      p[e] = z;
-      s0 = fma(ri, z, s0);
-      s1 = fma(ri, ri, s1);
-    }
-    v[0] += blk_weight(blk) * s0;
-    v[1] += blk_weight(blk) * s1;
+  const int blk = blockIdx.y;
+  double s0 = 0.0, s1 = 0.0;
+  for (int64_t e = blk * c.B + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < (blk + 1) * c.B; e += (int64_t)gridDim.x * blockDim.x) {
+    const double ri = r[e], z = dinv[e] * ri;
+    p[e] = z;
+    s0 = fma(ri, z, s0);
+    s1 = fma(ri, ri, s1);
   }
-  block_partials<2>(v, red);
+  double v[2] = {blk_weight(blk) * s0, blk_weight(blk) * s1};
+  block_partials_rows<2>(v, red);
 }
 
 __global__ void k_dot_w(VCtx c, const double *u, const double *v_, double *red) {
@@ -171,21 +194,19 @@ __global__ void k_dot_w(VCtx c, const double *u, const double *v_, double *red) 
 __global__ void k_pcg_update(VCtx c, const double *slots, const double *dinv, double *x, double *r, const double *p,
                              const double *q, double *red) {
   const double alpha = slots[4];
-  double v[2] = {0.0, 0.0};
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x, t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  for (int blk = 0; blk < 5; ++blk) {
-    double s0 = 0.0, s1 = 0.0;
-    for (int64_t e = blk * c.B + t0; e < (blk + 1) * c.B; e += stride) {
-      x[e] = fma(alpha, p[e], x[e]);
-      const double ri = fma(-alpha, q[e], r[e]);
-      r[e] = ri;
-      s0 = fma(ri * dinv[e], ri, s0);
-      s1 = fma(ri, ri, s1);
-    }
-    v[0] += blk_weight(blk) * s0;
-    v[1] += blk_weight(blk) * s1;
+  const int blk = blockIdx.y;
+  double s0 = 0.0, s1 = 0.0;
+#pragma unroll 2
+  for (int64_t e = blk * c.B + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < (blk + 1) * c.B; e += (int64_t)gridDim.x * blockDim.x) {
+    const double pe = p[e], qe = q[e], xe = x[e], re = r[e], de = dinv[e];
+    x[e] = fma(alpha, pe, xe);
+    const double ri = fma(-alpha, qe, re);
+    r[e] = ri;
+    s0 = fma(ri * de, ri, s0);
+    s1 = fma(ri, ri, s1);
   }
-  block_partials<2>(v, red);
+  double v[2] = {blk_weight(blk) * s0, blk_weight(blk) * s1};
+  block_partials_rows<2>(v, red);
 }
 
 // p = M^-1 r + beta p
@@ -383,26 +404,22 @@ __global__ void k_dinv32(VCtx c, __half *dinv) {
 }
 
 // r = -b - q (fp64 true residual); partials <r,r>, <b,b>
-// r = -b - q (q == nullptr: q = 0); partials <r, r>_w and, with with_b, <b, b>_w.  Block by
-// block (no per-element index arithmetic), weights applied to the block sums: float64 runs
+// r = -b - q (q == nullptr: q = 0); partials <r, r>_w and, with with_b, <b, b>_w.  A grid row
+// per block (no per-element index arithmetic), weights applied to the block sums: float64 runs
 // at a small fraction of the float32 rate on GB300, so the pass keeps to one add and one or
 // two fused multiply-adds per element.
 __global__ void k_residual(VCtx c, const double *b, const double *q, double *r, double *red, int with_b) {
-  double v[2] = {0.0, 0.0};
-  const int64_t stride = (int64_t)gridDim.x * blockDim.x, t0 = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  for (int blk = 0; blk < 5; ++blk) {
-    double s0 = 0.0, s1 = 0.0;
-    for (int64_t e = blk * c.B + t0; e < (blk + 1) * c.B; e += stride) {
-      const double bi = b[e], ri = q ? -bi - q[e] : -bi;
-      r[e] = ri;
-      s0 = fma(ri, ri, s0);
-      if (with_b) s1 = fma(bi, bi, s1);
-    }
-    const double w = blk == 1 ? 1.0 : (blk == 4 ? 2.0 : 0.5);
-    v[0] += w * s0;
-    v[1] += w * s1;
+  const int blk = blockIdx.y;
+  double s0 = 0.0, s1 = 0.0;
+#pragma unroll 2
+  for (int64_t e = blk * c.B + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < (blk + 1) * c.B; e += (int64_t)gridDim.x * blockDim.x) {
+    const double bi = b[e], ri = q ? -bi - q[e] : -bi;
+    r[e] = ri;
+    s0 = fma(ri, ri, s0);
+    if (with_b) s1 = fma(bi, bi, s1);
   }
-  block_partials<2>(v, red);
+  double v[2] = {blk_weight(blk) * s0, blk_weight(blk) * s1};
+  block_partials_rows<2>(v, red);
 }
 
 template <typename T>
@@ -428,6 +445,8 @@ __global__ void k_hylleraas(VCtx c, const double *b, const double *x, const doub
   block_partials<10>(v, red);
 }
 
+// strided ranges of an index pair in the two main sectors of the S-space energy
+constexpr int kE2sAB = 8, kE2sC = 4;
 // ---- S-space energy: E2_S = -sum_{I in S} b_I^2 / D_I, both spin sectors (factor 2).
 struct SCtx {
   int No, Nv, N;
@@ -719,7 +738,7 @@ __global__ void k_negsum64(const double *b, const double *q, double *out, int64_
 
 // one quantity's partials summed into the slots with the bookkeeping of `mode` (k_finalize)
 void k_finalize_ext(const double *red, int nparts, double *slots, int mode, cudaStream_t st) {
-  k_finalize<<<1, 256, 0, st>>>(red, nparts, 1, slots, mode);
+  k_finalize<<<1, 1024, 0, st>>>(red, nparts, 1, slots, mode);
 }
 
 static VCtx vctx(const esmp2_handle *h, const double *F = nullptr) {
@@ -738,7 +757,7 @@ static esmp2_status read_slots(esmp2_handle *h, double *out, int n) {
 
 double dot_w(esmp2_handle *h, const double *u, const double *v) {
   k_dot_w<<<kRedBlocks, kRedThreads, 0, h->stream>>>(vctx(h), u, v, h->red);
-  k_finalize<<<1, 256, 0, h->stream>>>(h->red, kRedBlocks, 1, h->red_out, 3);
+  k_finalize<<<1, 1024, 0, h->stream>>>(h->red, kRedBlocks, 1, h->red_out, 3);
   h->launches += 2;
   double s[32];
   read_slots(h, s, 32);
@@ -777,11 +796,11 @@ esmp2_status solve64(esmp2_handle *h, double tol, int maxit, esmp2_solve_info *i
       if (esmp2_status s2 = sigma64(h, x, q, lv, sym)) return s2;
       ++nsig;
     }
-    k_residual<<<kRedBlocks, kRedThreads, 0, st>>>(c, h->b, zero ? nullptr : q, r, h->red, bnorm < 0.0 ? 1 : 0);
-    k_finalize<<<1, 256, 0, st>>>(h->red, kRedBlocks, 2, h->red_out, 3);
+    k_residual<<<dim3(kRowCtas, 5), kRedThreads, 0, st>>>(c, h->b, zero ? nullptr : q, r, h->red, bnorm < 0.0 ? 1 : 0);
+    k_finalize<<<1, 1024, 0, st>>>(h->red, 5 * kRowCtas, 2, h->red_out, 3);
     singlet_project(h, r);
-    k_pcg_start<<<kRedBlocks, kRedThreads, 0, st>>>(c, h->dinv64, r, p, h->red);
-    k_finalize<<<1, 256, 0, st>>>(h->red, kRedBlocks, 2, h->red_out, 0);
+    k_pcg_start<<<dim3(kRowCtas, 5), kRedThreads, 0, st>>>(c, h->dinv64, r, p, h->red);
+    k_finalize<<<1, 1024, 0, st>>>(h->red, 5 * kRowCtas, 2, h->red_out, 0);
     h->launches += 4;
     if (esmp2_status s2 = read_slots(h, sl, 32)) return s2;
     if (bnorm < 0.0) bnorm = std::sqrt(sl[9]);
@@ -805,15 +824,15 @@ esmp2_status solve64(esmp2_handle *h, double tol, int maxit, esmp2_solve_info *i
     if (virt_tc && (s = check_device_flag(h))) return s;
     ++nsig;
     if (sym) {   // <p, q> came with the sigma
-      k_finalize<<<1, 256, 0, st>>>(h->red, residual_parts(), 1, h->red_out, 1);
+      k_finalize<<<1, 1024, 0, st>>>(h->red, residual_parts(), 1, h->red_out, 1);
       h->launches += 1;
     } else {
       k_dot_w<<<kRedBlocks, kRedThreads, 0, st>>>(c, p, q, h->red);
-      k_finalize<<<1, 256, 0, st>>>(h->red, kRedBlocks, 1, h->red_out, 1);
+      k_finalize<<<1, 1024, 0, st>>>(h->red, kRedBlocks, 1, h->red_out, 1);
       h->launches += 2;
     }
-    k_pcg_update<<<kRedBlocks, kRedThreads, 0, st>>>(c, h->red_out, h->dinv64, x, r, p, q, h->red);
-    k_finalize<<<1, 256, 0, st>>>(h->red, kRedBlocks, 2, h->red_out, 2);
+    k_pcg_update<<<dim3(kRowCtas, 5), kRedThreads, 0, st>>>(c, h->red_out, h->dinv64, x, r, p, q, h->red);
+    k_finalize<<<1, 1024, 0, st>>>(h->red, 5 * kRowCtas, 2, h->red_out, 2);
     k_pcg_p<<<kRedBlocks, kRedThreads, 0, st>>>(c, h->red_out, h->dinv64, r, p);
     h->launches += 3;
     if (!sym) antisym_project(h, p);
@@ -859,43 +878,36 @@ esmp2_status energy(esmp2_handle *h, esmp2_energy_parts *parts) {
     k_hylleraas<<<kRedBlocks, kRedThreads, 0, st>>>(vctx(h, F), bb, h->s64.x, h->s64.q, 0, h->red);
     h->launches += 1;
   }
-  k_finalize<<<1, 256, 0, st>>>(h->red, h->r_true && h->r_sym ? hyll_parts() : kRedBlocks, 10, h->red_out, 3);
+  k_finalize<<<1, 1024, 0, st>>>(h->red, h->r_true && h->r_sym ? hyll_parts() : kRedBlocks, 10, h->red_out, 3);
   h->launches += 1;
-  double sl[32];
-  if ((s = read_slots(h, sl, 32))) return s;
-  double e_blk[5];
-  for (int k = 0; k < 5; ++k) e_blk[k] = kWeights[k] * (2.0 * sl[8 + 2 * k] + sl[9 + 2 * k]);
-  if (!h->e2s_done) {
+  const bool small_pairs = !h->e2s_done;
+  if (small_pairs) {   // the three sectors' partials behind one another, one sum (slot 20)
     const int No = h->d.No;
     SCtx sc;
     sc.No = No; sc.Nv = h->d.Nv; sc.N = h->d.N; sc.F = h->F; sc.lam = h->lam; sc.ovov = h->ovov; sc.omega = h->omega_op;
-    const int nb = No * No * No;
     const int64_t ng = (int64_t)No * h->d.Nv * No * h->d.Nv;
     float2 *gdf = nullptr;
     cudaError_t ce = dmalloc(reinterpret_cast<void **>(&gdf), sizeof(float2) * (size_t)ng, st);
     if (ce != cudaSuccess) return check_cuda(h, ce, "S-space integrals");
     k_ovov_df<<<1216, 256, 0, st>>>(h->ovov, gdf, ng);
-    h->launches += 1;
     SDf gd{gdf};
-    double tot = 0.0;
-    const int npair = No * (No - 1) / 2, chAB = 8, chC = 4;
-    const int grids[3] = {npair * chAB, No * No * chC, nb};
-    for (int sector = 0; sector < 3; ++sector) {
-      if (grids[sector] == 0) continue;
-      {
-        KScope ks(st, ESMP2_KT_E2S, 0.0, 0.0);
-        if (sector == 0) k_e2s_ab<<<grids[0], 128, 0, st>>>(sc, gd, chAB, h->red);
-        else if (sector == 1) k_e2s_cm<<<grids[1], 128, 0, st>>>(sc, gd, chC, h->red);
-        else k_e2s_gen<<<grids[2], 128, 0, st>>>(sc, h->red);
-      }
-      k_finalize<<<1, 256, 0, st>>>(h->red, grids[sector], 1, h->red_out, 3);
-      h->launches += 2;
-      if ((s = read_slots(h, sl, 32))) break;
-      tot += sl[8];
+    const int nAB = No * (No - 1) / 2 * kE2sAB, nC = No * No * kE2sC, nG = No * No * No;
+    {
+      KScope ks(st, ESMP2_KT_E2S, 0.0, 0.0);
+      if (nAB) k_e2s_ab<<<nAB, 128, 0, st>>>(sc, gd, kE2sAB, h->red);
+      k_e2s_cm<<<nC, 128, 0, st>>>(sc, gd, kE2sC, h->red + nAB);
+      k_e2s_gen<<<nG, 128, 0, st>>>(sc, h->red + nAB + nC);
     }
+    k_finalize<<<1, 1024, 0, st>>>(h->red, nAB + nC + nG, 1, h->red_out, 8);
+    h->launches += 4 + (nAB > 0);
     dfree(gdf, st);
-    if (s) return s;
-    h->e2s = tot;
+  }
+  double sl[32];
+  if ((s = read_slots(h, sl, 32))) return s;
+  double e_blk[5];
+  for (int k = 0; k < 5; ++k) e_blk[k] = kWeights[k] * (2.0 * sl[8 + 2 * k] + sl[9 + 2 * k]);
+  if (small_pairs) {
+    h->e2s = sl[20];
     h->e2s_done = true;
   }
   parts->E2_D = e_blk[0] + e_blk[1];
@@ -947,12 +959,12 @@ esmp2_status solve_minres(esmp2_handle *h, double tol, int maxit, esmp2_solve_in
       k_negsum64<<<1216, 256, 0, st>>>(h->barr, q, r2, n);
     }
     k_mr_res<<<kRedBlocks, kRedThreads, 0, st>>>(c, r2, h->red);
-    k_finalize<<<1, 256, 0, st>>>(h->red, kRedBlocks, 2, h->red_out, 3);
+    k_finalize<<<1, 1024, 0, st>>>(h->red, kRedBlocks, 2, h->red_out, 3);
     h->launches += 3;
     if ((s = read_slots(h, sl, 32))) return s;
     if (bn < 0.0) {   // |b|_w
       k_mr_dot<<<kRedBlocks, kRedThreads, 0, st>>>(c, h->barr, h->barr, h->red);
-      k_finalize<<<1, 256, 0, st>>>(h->red, kRedBlocks, 1, h->red_out, 3);
+      k_finalize<<<1, 1024, 0, st>>>(h->red, kRedBlocks, 1, h->red_out, 3);
       h->launches += 2;
       double sb[32];
       if ((s = read_slots(h, sb, 32))) return s;
@@ -984,13 +996,13 @@ esmp2_status solve_minres(esmp2_handle *h, double tol, int maxit, esmp2_solve_in
       if ((s = sigma64_arrow(h, v, q))) return s;   // q = A v
       ++nsig;
       k_mr_dot<<<kRedBlocks, kRedThreads, 0, st>>>(c, v, q, h->red);
-      k_finalize<<<1, 256, 0, st>>>(h->red, kRedBlocks, 1, h->red_out, 3);
+      k_finalize<<<1, 1024, 0, st>>>(h->red, kRedBlocks, 1, h->red_out, 3);
       h->launches += 2;
       if ((s = read_slots(h, sl, 32))) return s;
       const double alpha = sl[8];
       // y = q - (alpha / beta) r2 - (beta / oldb) r1, over r1; then r1 <-> r2
       k_mr_y<<<kRedBlocks, kRedThreads, 0, st>>>(c, q, r2, r1, alpha / beta, oldb > 0.0 ? beta / oldb : 0.0, h->red);
-      k_finalize<<<1, 256, 0, st>>>(h->red, kRedBlocks, 1, h->red_out, 3);
+      k_finalize<<<1, 1024, 0, st>>>(h->red, kRedBlocks, 1, h->red_out, 3);
       h->launches += 2;
       if ((s = read_slots(h, sl, 32))) return s;
       std::swap(r1, r2);   // r2 = y (the new Lanczos residual), r1 = the previous one
@@ -1139,7 +1151,7 @@ esmp2_status solve_mixed(esmp2_handle *h, double tol, int maxit, esmp2_solve_inf
     h->r_sym = packed && !cold && bb >= 0.0;
     if (h->r_sym) {
       if ((s = residual_sym(h, x, bsel, r, lv_k))) return s;
-      k_finalize<<<1, 256, 0, st>>>(h->red, residual_parts(), 1, h->red_out, 3);
+      k_finalize<<<1, 1024, 0, st>>>(h->red, residual_parts(), 1, h->red_out, 3);
       h->launches += 1;
     } else {
       if (!cold) {
@@ -1147,8 +1159,8 @@ esmp2_status solve_mixed(esmp2_handle *h, double tol, int maxit, esmp2_solve_inf
         else s = sigma64_F(h, h->Fsemi, 1, x, q, lv_k, true);
         if (s) return s;
       }
-      k_residual<<<kRedBlocks, kRedThreads, 0, st>>>(c, bsel, cold ? nullptr : q, r, h->red, bb < 0.0 ? 1 : 0);
-      k_finalize<<<1, 256, 0, st>>>(h->red, kRedBlocks, 2, h->red_out, 3);
+      k_residual<<<dim3(kRowCtas, 5), kRedThreads, 0, st>>>(c, bsel, cold ? nullptr : q, r, h->red, bb < 0.0 ? 1 : 0);
+      k_finalize<<<1, 1024, 0, st>>>(h->red, 5 * kRowCtas, 2, h->red_out, 3);
       h->launches += 2;
     }
     if (!cold) ++nsig64;
@@ -1176,7 +1188,7 @@ esmp2_status solve_mixed(esmp2_handle *h, double tol, int maxit, esmp2_solve_inf
     } else {
       if (packed) packed_init(h, r, kRedBlocks);
       else ki_init<<<kRedBlocks, kRedThreads, 0, st>>>(ic, r, r32, p32, d32, h->red);
-      k_finalize<<<1, 256, 0, st>>>(h->red, kRedBlocks, 2, h->red_out, 0);
+      k_finalize<<<1, 1024, 0, st>>>(h->red, kRedBlocks, 2, h->red_out, 0);
       h->launches += packed ? 1 : 2;
     }
     if ((s = read_slots(h, sl, 32))) return s;
@@ -1200,14 +1212,14 @@ esmp2_status solve_mixed(esmp2_handle *h, double tol, int maxit, esmp2_solve_inf
         for (double v : part) fused_pq += v;
         sep_pq = packed_wdot(h, p32, q32);
       }
-      if (packed) k_finalize<<<1, 256, 0, st>>>(h->pdot, h->pdot_n, 1, h->red_out, 1);
-      else k_finalize<<<1, 256, 0, st>>>(h->red, (int)couple_dot_parts(h), 1, h->red_out, 1);
+      if (packed) k_finalize<<<1, 1024, 0, st>>>(h->pdot, h->pdot_n, 1, h->red_out, 1);
+      else k_finalize<<<1, 1024, 0, st>>>(h->red, (int)couple_dot_parts(h), 1, h->red_out, 1);
       h->launches += 1;
       if (rj) {   // r -= alpha q, z = M^-1 r (rotated Jacobi), beta, d and p
         if ((s2 = packed_rj_step(h, kRedBlocks))) return s2;
       } else {
         ki_update<<<kRedBlocks, kRedThreads, 0, st>>>(ic, h->red_out, r32, q32, h->red);
-        k_finalize<<<1, 256, 0, st>>>(h->red, kRedBlocks, 2, h->red_out, 2);
+        k_finalize<<<1, 1024, 0, st>>>(h->red, kRedBlocks, 2, h->red_out, 2);
         ki_p<<<kRedBlocks, kRedThreads, 0, st>>>(ic, h->red_out, r32, p32, d32);
         h->launches += 3;
       }
