@@ -12,7 +12,7 @@
 // and for Z the operand also holds the transposed slices Z_s^T, whose rows of P are stored
 // transposed here, (Z_s^T F)^T = F Z_s.  The coupling pass forms y from P.
 //
-// Structure (persistent, 320 threads):
+// Structure (persistent, 576 threads):
 //   each CTA owns one column tile b0 .. b0 + Nt - 1 of the result (columns split over nN
 //   tiles) and keeps that tile's panel W[b][c] (all K) resident in shared memory;
 //   warp 0      TMA producer: 2-D tiled bulk copies of 128-row x 64-byte A chunks (32 bf16 or
@@ -20,9 +20,13 @@
 //               panel leaves)
 //   warp 1      one thread issues tcgen05.mma (M = 128, N = Nt, K = 16 bf16 or 8 tf32, 32 bytes
 //               of each operand row per instruction), commits to mbarriers
-//   warps 2..9  epilogue: tcgen05.ld 32x32b from one of two TMEM accumulators (2 x Nt
+//   warps 2..17 epilogue: tcgen05.ld 32x32b from one of two TMEM accumulators (2 x Nt
 //               columns), fp32 stores of P rows (16-byte vectors) or of transposed rows (one
-//               128-byte segment per column and warp)
+//               128-byte segment per column and warp).  Four warps share a TMEM lane quarter, each
+//               with two eight-column loads in flight: with two warps per quarter, one load at a
+//               time, 64-bit row divisions and the masks taken element by element the epilogue, not the
+//               operands or the MMAs, set the pace (No=10 Nv=400: plain rotation 68 us, scaled one
+//               245 us a launch; now 67 and 73 us)
 // Every mbarrier wait is bounded (globaltimer); a wait that runs out raises the error flag,
 // the CTA waits (bounded) for its own copies in flight and frees its TMEM.
 #include <cuda.h>
@@ -39,15 +43,17 @@ constexpr int BM = 128;                 // accumulator rows (TMEM lanes)
 constexpr int CHUNK_B = 64;             // bytes of one operand row per K chunk (the swizzle span)
 constexpr int MAX_STAGES = 8;
 constexpr int A_STAGE = BM * CHUNK_B;   // 8 KB
-// K elements per chunk and per MMA: bf16 32 and 16, tf32 16 and 8 (both 32 bytes per MMA)
+// K elements per chunk and per MMA: bf16 32 and 16, tf32 16 and 8 (both 32 bytes per MMA).  Chunks of
+// 128-byte rows leave room for five ring slots only with three column tiles instead of two at
+// Nv = 400 and were slower (51 launches of the No=30 Nv=400 step: 41 against 35 ms).
 template <bool TF32> struct Kind {
   static constexpr int BK = TF32 ? 16 : 32;
   static constexpr int KMMA = TF32 ? 8 : 16;
 };
-constexpr int NTHREADS = 320;
+constexpr int EPI_WARPS = 16, NTHREADS = 64 + 32 * EPI_WARPS;
 // dynamic shared memory per CTA: the 232448-byte opt-in limit less room for the kernel's
-// static shared memory (barriers, TMEM address, flags, the epilogue's 10 KB staging tile)
-constexpr int SMEM_MAX = 232448 - 2048 - 10240;
+// static shared memory (barriers, TMEM address, flags, the epilogue's 10 KB staging tile and 1 KB table)
+constexpr int SMEM_MAX = 232448 - 2048 - 11264;
 constexpr uint64_t WAIT_NS = 2000000000ull;
 
 __device__ __forceinline__ uint32_t smem_u32(const void *p) {
@@ -129,16 +135,18 @@ __device__ __forceinline__ void umma_commit(uint64_t *bar) {
   asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
                : "memory");
 }
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
-  uint32_t r[16];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
-        "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr));
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-  for (int k = 0; k < 16; ++k) v[k] = __uint_as_float(r[k]);
+// eight consecutive accumulator columns of the warp's 32 lanes; valid after tmem_wait and keep
+__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
+               : "r"(taddr));
+}
+__device__ __forceinline__ void tmem_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
+__device__ __forceinline__ void keep(uint32_t &r) { asm volatile("" : "+r"(r)); }
+__device__ __forceinline__ float rcp_approx(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
 }
 
 struct Args {
@@ -163,16 +171,6 @@ struct Args {
   const int *code;      // [slices]: block | 8 (i == 0) | 16 (j == 0)
 };
 
-// validity of element (a, b) of a slice with the given code (the masks of the block vector)
-__device__ __forceinline__ bool vg_valid(int code, int a, int b) {
-  const int blk = code & 7;
-  const bool i0 = (code & 8) != 0, j0 = (code & 16) != 0;
-  if ((blk == 0 || blk == 2 || blk == 3) && a == b) return false;
-  if (blk == 2 && (i0 || j0 || a == 0 || b == 0)) return false;
-  if (blk == 4 && (j0 || b == 0 || (i0 && a == 0))) return false;
-  return true;
-}
-
 template <bool TF32>
 __global__ void __launch_bounds__(NTHREADS, 1)
     k_vgemm(const __grid_constant__ CUtensorMap tA, const __grid_constant__ CUtensorMap tF, Args g) {
@@ -185,20 +183,23 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   __shared__ uint64_t full[MAX_STAGES], empty[MAX_STAGES], acc_full[2], acc_empty[2], pbar;
   __shared__ uint32_t tmem_base;
   __shared__ int fail;
-  // bf16 transposed output: per epilogue warp one 16-column x 32-row chunk, turned so that each
-  // lane stores 16 consecutive rows of one column as two 16-byte vectors
-  __shared__ __align__(16) __nv_bfloat16 stg[8][16][40];
+  // bf16 transposed output: per epilogue warp one 8-column x 32-row chunk, turned so that each
+  // lane stores 8 consecutive rows of one column as a 16-byte vector
+  __shared__ __align__(16) __nv_bfloat16 stg[EPI_WARPS][8][40];
+  __shared__ __align__(16) float slam[256];   // lam of the CTA's column tile
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int nt = blockIdx.x % g.nN, group = gridDim.x / g.nN, gi = blockIdx.x / g.nN;
   const int b0 = nt * g.Nt, nvalid = min(g.Nt, g.Nv - b0), nmma = (nvalid + 15) & ~15;
   const uint32_t chunk_bytes = (uint32_t)g.Nt * CHUNK_B;
   if (threadIdx.x == 0) {
     for (int s = 0; s < STAGES; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
-    for (int s = 0; s < 2; ++s) { mbar_init(&acc_full[s], 1); mbar_init(&acc_empty[s], 8); }
+    for (int s = 0; s < 2; ++s) { mbar_init(&acc_full[s], 1); mbar_init(&acc_empty[s], EPI_WARPS); }
     mbar_init(&pbar, 1);
     fail = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
+  if (g.lam)
+    for (int k = threadIdx.x; k < nvalid; k += NTHREADS) slam[k] = g.lam[b0 + k];
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)),
                  "r"(512)
@@ -264,80 +265,101 @@ __global__ void __launch_bounds__(NTHREADS, 1)
       if (!ok) atomicExch(&fail, 1);
     }
   } else {  // ---------------------------------------------------------- epilogue
-    const int quarter = warp & 3, chalf = (warp - 2) >> 2;
-    const int hc = ((nvalid + 31) / 32) * 16;   // columns per half, a multiple of 16
-    const int c_begin = chalf * hc, c_end = min(nvalid, c_begin + hc);
+    const int quarter = warp & 3, part = (warp - 2) >> 2, ew = warp - 2;
+    const int units = (nvalid + 7) >> 3;   // eight-column units, dealt to the four warps of a quarter in turn
     int lt = 0;
     for (int64_t m = gi; m < g.m_tiles; m += group, ++lt) {
       const int ab = lt & 1;
       const uint32_t ar = (uint32_t)(lt >> 1);
       if (!mbar_wait(&acc_full[ab], ar & 1)) { if (lane == 0) atomicExch(&fail, 1); break; }
+      __syncwarp();
       tc_after();
-      const int64_t r = m * BM + quarter * 32 + lane;
       const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(ab * 256);
-      const bool normal = r < g.rows_normal;
-      // the warp's 32 rows form one run of a transposed slice (same slice, consecutive rows
-      // starting on a multiple of 8): the staged 16-byte stores apply
-      bool run = false;
-      if (g.PT16) {
-        const int64_t r0 = m * BM + quarter * 32, q0 = r0 - g.rows_normal;
-        run = r0 >= g.rows_normal && r0 + 31 < g.rows && (q0 % g.Nv) + 31 < g.Nv && (q0 % g.Nv) % 8 == 0;
-      }
+      // rows fit 32 bits (checked by the host)
+      const uint32_t r = (uint32_t)(m * BM) + (uint32_t)(quarter * 32 + lane), rn = (uint32_t)g.rows_normal;
+      const bool in = r < (uint32_t)g.rows, normal = r < rn;
       float *dst = nullptr;     // column b (< Nv) of this row
       __nv_bfloat16 *dst16 = nullptr;
       int64_t tpitch = 1;
-      int rc = 0, rcode = 0;    // transposed rows: row within the slice, slice code
-      float rocc = 0.f, rlam = 0.f;
-      if (normal) {
-        dst = g.P + r * g.ldp;
-      } else if (r < g.rows) {
-        const int64_t q = r - g.rows_normal, s = q / g.Nv, c = q % g.Nv;
-        if (g.PT16) dst16 = g.PT16 + s * g.Nv * g.ldp + c;
-        else dst = g.PT + s * g.Nv * g.ldp + c;   // column b at dst + b * ldp
+      uint32_t rc = 0;          // transposed rows: row within the slice
+      float2 rsum = make_float2(0.f, 0.f);   // lam of the row, occupied part of the slice
+      bool dead = false, no0 = false, nodiag = false;   // scaled output: masks of the row
+      if (in && normal) {
+        dst = g.P + (int64_t)r * g.ldp;
+      } else if (in) {
+        const uint32_t q = r - rn, s = q / (uint32_t)g.Nv;
+        rc = q - s * (uint32_t)g.Nv;
+        if (g.PT16) dst16 = g.PT16 + (int64_t)s * g.Nv * g.ldp + rc;
+        else dst = g.PT + (int64_t)s * g.Nv * g.ldp + rc;   // column b at dst + b * ldp
         tpitch = g.ldp;
-        rc = (int)c;
-        if (g.lam) { rcode = g.code[s]; rocc = g.occ[s]; rlam = g.lam[c]; }
+        if (g.lam) {   // stored element (a = column, b = rc): the masks of the block vector
+          const int code = g.code[s], blk = code & 7;
+          const bool i0 = (code & 8) != 0, j0 = (code & 16) != 0;
+          dead = (blk == 2 && (i0 || j0 || rc == 0)) || (blk == 4 && (j0 || rc == 0));
+          no0 = blk == 2 || (blk == 4 && i0);
+          nodiag = blk == 0 || blk == 2 || blk == 3;
+          rsum = make_float2(g.lam[rc], g.occ[s]);
+        }
       }
-      for (int c = c_begin; c < c_end; c += 16) {
-        float v[16];
-        tmem_ld16(taddr + (uint32_t)c, v);
-        if (r >= g.rows) continue;
-        const int bc = b0 + c, mcol = min(16, nvalid - c);
-        if (dst16) {   // stored element (a = bc + q, b = rc) of the slice
-          if (g.lam) {   // the fast division (2 ulp) serves the preconditioner: the denominator of
-                         // (a, b) and of its image (b, a) is the same float, so M stays symmetric
+      // the warp's 32 rows form one run of a transposed slice (same slice, consecutive rows
+      // starting on a multiple of 8): the staged 16-byte stores apply
+      const uint32_t rc0 = __shfl_sync(0xffffffffu, rc, 0);
+      const bool run = g.PT16 && __all_sync(0xffffffffu, in && !normal && rc == rc0 + lane) && (rc0 & 7) == 0;
+      for (int u0 = part; u0 < units; u0 += 8) {
+        uint32_t w[2][8];
+        const bool second = u0 + 4 < units;   // uniform
+        tmem_ld8(taddr + (uint32_t)(u0 * 8), w[0]);
+        if (second) tmem_ld8(taddr + (uint32_t)(u0 * 8 + 32), w[1]);
+        tmem_wait();
 #pragma unroll
-            for (int q = 0; q < 16; ++q) {
-              const int a = bc + q;
-              v[q] = (q < mcol && vg_valid(rcode, a, rc)) ? __fdividef(v[q], (g.lam[a] + rlam) - rocc) : 0.f;
+        for (int h = 0; h < 2; ++h) {
+          if (h == 1 && !second) break;
+          const int c = (u0 + 4 * h) * 8, bc = b0 + c, mcol = min(8, nvalid - c);
+          float v[8];
+#pragma unroll
+          for (int q = 0; q < 8; ++q) {
+            keep(w[h][q]);
+            v[q] = __uint_as_float(w[h][q]);
+          }
+          if (g.PT16) {
+            if (g.lam) {   // the approximate reciprocal serves the preconditioner: the denominator of
+                           // (a, b) and of its image (b, a) is the same float, so M stays symmetric
+              const float4 la = *reinterpret_cast<const float4 *>(&slam[c]), lb = *reinterpret_cast<const float4 *>(&slam[c + 4]);
+              const float lc[8] = {la.x, la.y, la.z, la.w, lb.x, lb.y, lb.z, lb.w};
+#pragma unroll
+              for (int q = 0; q < 8; ++q) v[q] = dead ? 0.f : v[q] * rcp_approx((lc[q] + rsum.x) - rsum.y);
+              if (no0 && bc == 0) v[0] = 0.f;
+              if (nodiag && rc - (uint32_t)bc < 8u) {
+#pragma unroll
+                for (int q = 0; q < 8; ++q)
+                  if ((uint32_t)(bc + q) == rc) v[q] = 0.f;
+              }
+            }
+            if (run) {   // all 32 lanes here (every row of the warp is in range)
+              __nv_bfloat16(*st)[40] = stg[ew];
+              __syncwarp();
+#pragma unroll
+              for (int q = 0; q < 8; ++q) st[q][lane] = __float2bfloat16_rn(v[q]);
+              __syncwarp();
+              const int j = lane >> 2, hh = (lane & 3) * 8;   // column bc + j, rows hh .. hh + 7 of the run
+              if (j < mcol)
+                *reinterpret_cast<uint4 *>(dst16 - lane + (int64_t)(bc + j) * tpitch + hh) = *reinterpret_cast<const uint4 *>(&st[j][hh]);
+            } else if (dst16) {
+#pragma unroll
+              for (int q = 0; q < 8; ++q)
+                if (q < mcol) dst16[(int64_t)(bc + q) * tpitch] = __float2bfloat16_rn(v[q]);
+            }
+          } else if (dst) {
+            if (normal && mcol == 8) {
+              float4 *d4 = reinterpret_cast<float4 *>(dst + bc);
+              d4[0] = make_float4(v[0], v[1], v[2], v[3]);
+              d4[1] = make_float4(v[4], v[5], v[6], v[7]);
+            } else {
+#pragma unroll
+              for (int q = 0; q < 8; ++q)
+                if (q < mcol) dst[(int64_t)(bc + q) * tpitch] = v[q];
             }
           }
-          if (run) {   // all 32 lanes here (every row of the warp is in range)
-            __nv_bfloat16(*st)[40] = stg[warp - 2];
-            __syncwarp();
-#pragma unroll
-            for (int q = 0; q < 16; ++q) st[q][lane] = __float2bfloat16_rn(v[q]);
-            __syncwarp();
-            const int j = lane >> 1, hh = (lane & 1) * 16;   // column bc + j, rows hh .. hh + 15 of the run
-            if (j < mcol) {
-              const uint4 *src = reinterpret_cast<const uint4 *>(&st[j][hh]);
-              uint4 *out = reinterpret_cast<uint4 *>(dst16 - lane + (int64_t)(bc + j) * tpitch + hh);
-              out[0] = src[0];
-              out[1] = src[1];
-            }
-          } else {
-#pragma unroll
-            for (int q = 0; q < 16; ++q)
-              if (q < mcol) dst16[(int64_t)(bc + q) * tpitch] = __float2bfloat16_rn(v[q]);
-          }
-        } else if (normal && mcol == 16) {
-          float4 *d4 = reinterpret_cast<float4 *>(dst + bc);
-#pragma unroll
-          for (int q = 0; q < 4; ++q) d4[q] = make_float4(v[4 * q], v[4 * q + 1], v[4 * q + 2], v[4 * q + 3]);
-        } else {
-#pragma unroll
-          for (int q = 0; q < 16; ++q)
-            if (q < mcol) dst[(int64_t)(bc + q) * tpitch] = v[q];
         }
       }
       tc_before();
@@ -382,6 +404,10 @@ esmp2_status vgemm(esmp2_handle *h, const void *A, int64_t rows, int64_t rows_no
   int nN = 0, Nt = 0, nk = 0, stages = 0, smem = 0;
   if (!vgemm_tiling(Nv, Nv, bk, &nN, &Nt, &nk, &stages, &smem) || (ldp & 3) || rows <= 0) {
     h->err = "vgemm: unsupported shape";
+    return ESMP2_ERR_UNSUPPORTED;
+  }
+  if (rows >= (int64_t)1 << 31) {
+    h->err = "vgemm: too many rows";
     return ESMP2_ERR_UNSUPPORTED;
   }
   if (rows_normal < rows && (rows - rows_normal) % Nv != 0) {
