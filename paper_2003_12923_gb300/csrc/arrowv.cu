@@ -25,6 +25,7 @@
 #include <vector>
 
 #include "internal.h"
+#include "jacobi.h"
 
 namespace esmp2 {
 namespace {
@@ -41,28 +42,12 @@ __global__ void k_to_f32(const double *src, float *dst, int64_t n) {
 // At convergence B = Jt A with orthogonal rows, so the rows of Jt are eigenvectors of A^2,
 // hence of A (A positive definite).  Rotation of a pair: alpha = |b_p|^2, beta = |b_q|^2,
 // gamma = b_p . b_q, zeta = (beta - alpha) / (2 gamma), t = sign(zeta) / (|zeta| + sqrt(1 +
-// zeta^2)), c = 1 / sqrt(1 + t^2), s = c t; skipped when |gamma| <= 1e-14 sqrt(alpha beta)
+// zeta^2)), c = 1 / sqrt(1 + t^2), s = c t (jacobi.h); skipped when |gamma| <= 1e-14 sqrt(alpha beta)
 // (the remaining off-diagonal part of R^T A R is then of the order of 1e-14 of its diagonal).
 // Rows are contiguous, so every access is coalesced.  *maxr2 receives the largest
 // gamma^2 / (alpha beta) of the pairs that rotate (as float bits).
-// Newton-Raphson refinements in float64 of float32 seeds: 1/sqrt(x) by y <- y (3 - x y^2) / 2 and
-// 1/x by y <- y (2 - x y), two steps each (quadratic convergence from the seed's 2^-22 to the
-// float64 rounding level); for x in a range where the float32 seed is a normal number
-__device__ __forceinline__ double rsqrt_nr(double x) {
-  double y = (double)rsqrtf((float)x);
-  y = y * (1.5 - 0.5 * x * y * y);
-  y = y * (1.5 - 0.5 * x * y * y);
-  return y;
-}
-__device__ __forceinline__ double rcp_nr(double x) {
-  double y = (double)(1.0f / (float)x);
-  y = y * (2.0 - x * y);
-  y = y * (2.0 - x * y);
-  return y;
-}
-
 constexpr int kJT = 128;                 // threads per pair (one CTA)
-constexpr int kJE = 8;                   // row elements per thread: m <= kJT kJE = 1024
+template <int NE>                        // row elements per thread: m <= kJT NE
 __global__ void __launch_bounds__(kJT) k_jacobi_os_round(double *B, double *Jt, int m, int r, unsigned *maxr2) {
   __shared__ double red[3][kJT / 32];
   const int n = m + (m & 1), pi = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
@@ -79,9 +64,9 @@ __global__ void __launch_bounds__(kJT) k_jacobi_os_round(double *B, double *Jt, 
   double *bp = B + (int64_t)p * m, *bq = B + (int64_t)q * m;
   double *jp = Jt + (int64_t)p * m, *jq = Jt + (int64_t)q * m;
   // every load of the two rows (and of the two rows of Jt) issued before it is used
-  double x[kJE], y[kJE], u[kJE], v[kJE];
+  double x[NE], y[NE], u[NE], v[NE];
 #pragma unroll
-  for (int e = 0; e < kJE; ++e) {
+  for (int e = 0; e < NE; ++e) {
     const int k = tid + e * kJT;
     const bool in = k < m;
     x[e] = in ? bp[k] : 0.0;
@@ -91,54 +76,35 @@ __global__ void __launch_bounds__(kJT) k_jacobi_os_round(double *B, double *Jt, 
   }
   double al = 0.0, be = 0.0, ga = 0.0;
 #pragma unroll
-  for (int e = 0; e < kJE; ++e) {
-    al += x[e] * x[e];
-    be += y[e] * y[e];
-    ga += x[e] * y[e];
+  for (int e = 0; e < NE; ++e) {
+    al = fma(x[e], x[e], al);
+    be = fma(y[e], y[e], be);
+    ga = fma(x[e], y[e], ga);
   }
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    al += __shfl_xor_sync(0xffffffffu, al, o);
-    be += __shfl_xor_sync(0xffffffffu, be, o);
-    ga += __shfl_xor_sync(0xffffffffu, ga, o);
-  }
+  warp_sum3(al, be, ga);
   if (lane == 0) { red[0][warp] = al; red[1][warp] = be; red[2][warp] = ga; }
   __syncthreads();
-  // the rotation from one thread (float64 division and square root are long sequences on
-  // the float64 pipe), broadcast through shared memory
-  __shared__ double cs[2];
-  __shared__ int skip;
-  if (tid == 0) {
-    al = be = ga = 0.0;
-#pragma unroll
-    for (int w = 0; w < kJT / 32; ++w) { al += red[0][w]; be += red[1][w]; ga += red[2][w]; }
-    skip = (al <= 1e-300 || be <= 1e-300 || ga * ga <= 1e-28 * al * be) ? 1 : 0;
-    if (!skip) {
-      // largest gamma^2 / (alpha beta) of the pass (non-negative floats order as their bits)
-      atomicMax(maxr2, __float_as_uint((float)(ga * ga * rcp_nr(al * be))));
-      // t = sign(d) g / (|d| + sqrt(d^2 + g^2)) with d = beta - alpha, g = 2 gamma (the smaller
-      // root of t^2 + 2 zeta t - 1 = 0, zeta = d / g), formed on (d, g) scaled to max 1
-      const double d0 = be - al, g0 = 2.0 * ga;
-      const double sc = rcp_nr(fmax(fabs(d0), fabs(g0)));
-      const double d = d0 * sc, g = g0 * sc, q2 = d * d + g * g;   // q2 in [1, 2]
-      const double rt = q2 * rsqrt_nr(q2);
-      const double t = (d >= 0.0 ? g : -g) * rcp_nr(fabs(d) + rt);
-      const double c0 = rsqrt_nr(1.0 + t * t);
-      cs[0] = c0;
-      cs[1] = c0 * t;
-    }
+  // every warp forms the rotation for itself (its pipe would wait for another one's all the same)
+  al = (red[0][0] + red[0][1]) + (red[0][2] + red[0][3]);
+  be = (red[1][0] + red[1][1]) + (red[1][2] + red[1][3]);
+  ga = (red[2][0] + red[2][1]) + (red[2][2] + red[2][3]);
+  const double ab = al * be, g2 = ga * ga;
+  if (al <= 1e-300 || be <= 1e-300 || g2 <= 1e-28 * ab) return;   // uniform
+  // largest gamma^2 / (alpha beta) of the pass (non-negative floats order as their bits)
+  if (warp == 0) {
+    const double sc = __hiloint2double(0x7FE00000 - (__double2hiint(ab) & 0x7FF00000), 0);   // alpha beta to [1, 2)
+    if (lane == 0) atomicMax(maxr2, __float_as_uint((float)(g2 * sc) / (float)(ab * sc)));
   }
-  __syncthreads();
-  if (skip) return;   // uniform
-  const double c = cs[0], s = cs[1];
+  double c, s;
+  jacobi_rotation(al, be, ga, c, s);
 #pragma unroll
-  for (int e = 0; e < kJE; ++e) {
+  for (int e = 0; e < NE; ++e) {
     const int k = tid + e * kJT;
     if (k < m) {
-      bp[k] = c * x[e] - s * y[e];
-      bq[k] = s * x[e] + c * y[e];
-      jp[k] = c * u[e] - s * v[e];
-      jq[k] = s * u[e] + c * v[e];
+      bp[k] = fma(c, x[e], -s * y[e]);
+      bq[k] = fma(s, x[e], c * y[e]);
+      jp[k] = fma(c, u[e], -s * v[e]);
+      jq[k] = fma(s, u[e], c * v[e]);
     }
   }
 }
@@ -306,6 +272,10 @@ esmp2_status ensure_vrot(esmp2_handle *h, bool exact) {
     const int n2 = (m + (m & 1)) / 2, rounds = m + (m & 1) - 1;
     const unsigned grid = (unsigned)n2;
     unsigned *mr = h->jflag;
+    const void *fn = m <= kJT ? reinterpret_cast<const void *>(k_jacobi_os_round<1>)
+                     : m <= 2 * kJT ? reinterpret_cast<const void *>(k_jacobi_os_round<2>)
+                     : m <= 4 * kJT ? reinterpret_cast<const void *>(k_jacobi_os_round<4>)
+                                    : reinterpret_cast<const void *>(k_jacobi_os_round<8>);
     double *B = h->jB, *J = h->jJ;
     // one sweep as one CUDA graph (a reset of the sweep maximum, then the rounds as dependent
     // kernel nodes), replayed until the sweep's largest gamma^2 / (alpha beta) is below the target
@@ -324,7 +294,7 @@ esmp2_status ensure_vrot(esmp2_handle *h, bool exact) {
         int rr = k % rounds, mm_ = m;
         void *args[] = {&B, &J, &mm_, &rr, &mr};
         cudaKernelNodeParams kp{};
-        kp.func = reinterpret_cast<void *>(k_jacobi_os_round);
+        kp.func = const_cast<void *>(fn);
         kp.gridDim = dim3(grid);
         kp.blockDim = dim3(kJT);
         kp.sharedMemBytes = 0;
@@ -348,7 +318,11 @@ esmp2_status ensure_vrot(esmp2_handle *h, bool exact) {
         if ((e = cudaGraphLaunch(gexec, st)) != cudaSuccess) break;
       } else {
         cudaMemsetAsync(mr, 0, sizeof(unsigned), st);
-        for (int k = 0; k < rounds; ++k) k_jacobi_os_round<<<grid, kJT, 0, st>>>(B, J, m, k, mr);
+        for (int k = 0; k < rounds; ++k) {
+          int rr = k, mm_ = m;
+          void *args[] = {&B, &J, &mm_, &rr, &mr};
+          cudaLaunchKernel(fn, dim3(grid), dim3(kJT), args, 0, st);
+        }
       }
       h->launches += rounds;
       ++sweeps;

@@ -12,6 +12,7 @@
 #include <cmath>
 
 #include "internal.h"
+#include "jacobi.h"
 
 namespace esmp2 {
 namespace {
@@ -70,12 +71,10 @@ __global__ void __launch_bounds__(1024) k_jacobi_svd(const double *C, double *B,
           const double x = B[p * Nv + a], y = B[q * Nv + a];
           al += x * x; be += y * y; ga += x * y;
         }
-        al = warp_sum(al); be = warp_sum(be); ga = warp_sum(ga);
-        if (al <= 1e-300 || be <= 1e-300) continue;
-        if (fabs(ga) <= 1e-15 * sqrt(al * be)) continue;
-        const double zeta = (be - al) / (2.0 * ga);
-        const double t = (zeta >= 0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
-        const double c = 1.0 / sqrt(1.0 + t * t), s = c * t;
+        warp_sum3(al, be, ga);
+        if (al <= 1e-300 || be <= 1e-300 || ga * ga <= 1e-30 * al * be) continue;
+        double c, s;
+        jacobi_rotation(al, be, ga, c, s);
         for (int a = lane; a < Nv; a += 32) {
           const double x = B[p * Nv + a], y = B[q * Nv + a];
           B[p * Nv + a] = c * x - s * y;
@@ -225,11 +224,10 @@ __global__ void __launch_bounds__(1024) k_eig_small(const double *A, int64_t ldA
           const double x = bp[k], y = bq[k];
           al += x * x; be += y * y; ga += x * y;
         }
-        al = warp_sum(al); be = warp_sum(be); ga = warp_sum(ga);
-        if (al <= 1e-300 || be <= 1e-300 || fabs(ga) <= 1e-15 * sqrt(al * be)) continue;
-        const double zeta = (be - al) / (2.0 * ga);
-        const double t = (zeta >= 0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
-        const double c = 1.0 / sqrt(1.0 + t * t), s = c * t;
+        warp_sum3(al, be, ga);
+        if (al <= 1e-300 || be <= 1e-300 || ga * ga <= 1e-30 * al * be) continue;
+        double c, s;
+        jacobi_rotation(al, be, ga, c, s);
         for (int k = lane; k < m; k += 32) {
           const double x = bp[k], y = bq[k], u = jp[k], v = jq[k];
           bp[k] = c * x - s * y;
