@@ -75,6 +75,7 @@ __global__ void __launch_bounds__(NT) gemm64_kernel(Gemm64 g, int mtiles, int nt
   const int mi = max(0, min(4, (g.M - m0 - wm + 3) >> 2)), nj = max(0, min(2, (g.N - n0 - wn + 7) >> 3));
   double acc[4][2] = {};
   double ra[4], rb[4];
+  auto kslice = [&](int gk) { return !g.klist ? gk / g.Kin : gk < kend ? __ldg(g.klist + gk / g.Kin) : 0; };
   auto load = [&](int k0) {
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
@@ -83,13 +84,13 @@ __global__ void __launch_bounds__(NT) gemm64_kernel(Gemm64 g, int mtiles, int nt
       if (a_kfast) { k = idx % BK; m = idx / BK; } else { m = idx % TS; k = idx / TS; }
       int gk = k0 + k;
       int64_t ko = (int64_t)gk * g.sAk;
-      if (g.Kin > 0) ko = (int64_t)(gk / g.Kin) * g.sAk1 + (int64_t)(gk % g.Kin) * g.sAk;
+      if (g.Kin > 0) ko = (int64_t)kslice(gk) * g.sAk1 + (int64_t)(gk % g.Kin) * g.sAk;
       ra[r] = (m0 + m < g.M && gk < kend) ? A[(int64_t)(m0 + m) * g.sAm + ko] : 0.0;
       int n;
       if (b_nfast) { n = idx % TS; k = idx / TS; } else { k = idx % BK; n = idx / BK; }
       gk = k0 + k;
       ko = (int64_t)gk * g.sBk;
-      if (g.Kin > 0) ko = (int64_t)(gk / g.Kin) * g.sBk1 + (int64_t)(gk % g.Kin) * g.sBk;
+      if (g.Kin > 0) ko = (int64_t)kslice(gk) * g.sBk1 + (int64_t)(gk % g.Kin) * g.sBk;
       rb[r] = (n0 + n < g.N && gk < kend) ? B[ko + (int64_t)(n0 + n) * g.sBn] : 0.0;
     }
   };
@@ -128,19 +129,29 @@ __global__ void __launch_bounds__(NT) gemm64_kernel(Gemm64 g, int mtiles, int nt
   }
 }
 
-// C = alpha sum_k part[k] + beta C, the K slices in order
-__global__ void __launch_bounds__(128) gemm64_sum(Gemm64 g, int nsplit, const double *part) {
+// C = alpha sum_k part[k] + beta C, in a fixed order: 32 elements per CTA, eight threads each (a small C
+// comes with many slices, and one thread per element was a chain of up to 900 loads)
+__global__ void __launch_bounds__(256) gemm64_sum(Gemm64 g, int nsplit, const double *part) {
+  __shared__ double sh[8][33];
   const int64_t per = (int64_t)g.batch * g.M * g.N;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < per; e += (int64_t)gridDim.x * blockDim.x) {
-    const int n = (int)(e % g.N);
-    const int64_t f = e / g.N;
-    const int m = (int)(f % g.M);
+  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  for (int64_t e0 = (int64_t)blockIdx.x * 32; e0 < per; e0 += (int64_t)gridDim.x * 32) {
+    const int64_t e = e0 + tx, f = e / g.N;
+    const int n = (int)(e - f * g.N), m = (int)(f % g.M);
     const int64_t src = g.sym && m / TS > n / TS ? e + (int64_t)(n - m) * g.N + (m - n) : e;   // element (n, m)
     double s = 0.0;
-#pragma unroll 8
-    for (int k = 0; k < nsplit; ++k) s += part[k * per + src];
-    double *c = g.C + (f / g.M) * g.sCb + (int64_t)m * g.sCm + (int64_t)n * g.sCn;
-    *c = (g.beta == 0.0) ? g.alpha * s : fma(g.alpha, s, g.beta * *c);
+    if (e < per) {
+#pragma unroll 4
+      for (int k = ty; k < nsplit; k += 8) s += part[k * per + src];
+    }
+    sh[ty][tx] = s;
+    __syncthreads();
+    if (ty == 0 && e < per) {
+      for (int w = 1; w < 8; ++w) s += sh[w][tx];
+      double *c = g.C + (f / g.M) * g.sCb + (int64_t)m * g.sCm + (int64_t)n * g.sCn;
+      *c = (g.beta == 0.0) ? g.alpha * s : fma(g.alpha, s, g.beta * *c);
+    }
+    __syncthreads();
   }
 }
 
@@ -235,7 +246,7 @@ void gemm64(const Gemm64 &g, cudaStream_t st) {
   if (part) {   // batch <= kSplitTarget here: one launch
     nsplit = (int)cdiv(g.K, kper);
     gemm64_kernel<<<dim3((unsigned)(tiles * nsplit), (unsigned)g.batch), NT, 0, st>>>(g, mtiles, ntiles, kper, part);
-    gemm64_sum<<<(unsigned)std::min<int64_t>(cdiv((int64_t)g.batch * g.M * g.N, 128), 1216), 128, 0, st>>>(g, nsplit, part);
+    gemm64_sum<<<(unsigned)std::min<int64_t>(cdiv((int64_t)g.batch * g.M * g.N, 32), 1216), 256, 0, st>>>(g, nsplit, part);
     dfree(part, st);
     return;
   }

@@ -22,6 +22,7 @@ namespace esmp2 {
 namespace {
 
 constexpr double WT = 0.5, WS = 1.0, WX = 0.5, WY = 0.5, WZ = 2.0;
+static_assert(WT == WX && WT == WY, "T, X and Y share one density product");
 
 struct GCtx {
   int No, Nv, N;
@@ -131,11 +132,11 @@ __global__ void kg_F2(GCtx c, double *Gf) {
   if (threadIdx.x == 0) Gf[No + cc] += s;
 }
 
-// F3: d/dF_ov(k,0), one block per k
+// F3: d/dF_ov(k,0), blocks (k, one of gridDim.y ranges of the sum over (j, a, b))
 __global__ void kg_F3(GCtx c, double *Gf) {
   const int No = c.No, Nv = c.Nv, k = blockIdx.x;
   double s = 0;
-  for (int64_t r = threadIdx.x; r < (int64_t)No * Nv * Nv; r += blockDim.x) {
+  for (int64_t r = blockIdx.y * (int64_t)blockDim.x + threadIdx.x; r < (int64_t)No * Nv * Nv; r += (int64_t)gridDim.y * blockDim.x) {
     const int b = (int)(r % Nv), a = (int)((r / Nv) % Nv), j = (int)(r / ((int64_t)Nv * Nv));
     s += -2.0 * WT * c.X(BT, 0, j, a, b) * c.X(BX, k, j, a, b)
          - WS * c.X(BS, j, 0, a, b) * c.X(BZ, j, k, a, b)
@@ -144,7 +145,7 @@ __global__ void kg_F3(GCtx c, double *Gf) {
          - WZ * c.X(BZ, j, k, a, b) * c.X(BS, j, 0, a, b);
   }
   s = block_sum(s);
-  if (threadIdx.x == 0) Gf[(int64_t)k * c.N + No] += s;
+  if (threadIdx.x == 0) atomicAdd(&Gf[(int64_t)k * c.N + No], s);
 }
 
 // F4: d/dF_ov(k,c), one block per (k,c)
@@ -250,6 +251,17 @@ __device__ void flush_diag(const SG &g, double *sdiag) {
     if (sdiag[k] != 0.0) atomicAdd(&g.Gdiag[k], sdiag[k]);
 }
 
+// 1 / x: a float32 reciprocal and two Newton steps (four float64 operations; the division takes some
+// twenty of the pipe that bounds these kernels), the division outside the range of float32.  Error below
+// 2 ulp; No=12 Nv=120, kg_s_ab + kg_s_cm with the division 1.6 ms, so 1.0 ms.
+__device__ __forceinline__ double recip(double x) {
+  const double ax = fabs(x);
+  if (!(ax > 1e-30 && ax < 1e30)) return 1.0 / x;
+  double y = (double)(1.0f / (float)x);
+  y = fma(y, fma(-x, y, 1.0), y);
+  return fma(y, fma(-x, y, 1.0), y);
+}
+
 // S-space derivative, the triples with exactly one transition pair (the energy's k_e2s_ab and
 // k_e2s_cm enumerate the same ones): b_I is lambda_u times one antisymmetrised integral, so a
 // thread that owns the integral sums over the pair u itself, adds its own two (ov|ov) elements
@@ -317,7 +329,7 @@ __global__ void __launch_bounds__(kST) kg_s_ab(SG g, int nchunk) {
         double q1 = 0.0;
         for (int u = 1; u < No; ++u) {
           const double m = (u != j && u != k && u != b && u != cc) ? 2.0 : 1.0;   // sectors A and B, or B alone
-          const double r = 1.0 / (s.du[u] + e), q = m * s.lu2[u] * r, d = 2.0 * dg * dg * q * r;
+          const double r = recip(s.du[u] + e), q = m * s.lu2[u] * r, d = 2.0 * dg * dg * q * r;
           q1 += q;
           su[u * kST] += d;
           gd += d;
@@ -363,7 +375,7 @@ __global__ void __launch_bounds__(kST) kg_s_cm(SG g, int nchunk) {
         double q1 = 0.0;
         for (int u = 1; u < No; ++u) {
           if (u == k || u == cc) continue;
-          const double r = 1.0 / (s.du[u] + e), q = s.lu2[u] * r, d = 2.0 * gv * gv * q * r;
+          const double r = recip(s.du[u] + e), q = s.lu2[u] * r, d = 2.0 * gv * gv * q * r;
           q1 += q;
           su[u * kST] += d;
           gd += d;
@@ -461,42 +473,51 @@ __global__ void kg_transpose(const double *A, double *At, int n) {
 
 }  // namespace
 
-// One-body densities of x (the N^5 part of <x, dA x>), accumulated into Gf (N x N).
-static void densities(esmp2_handle *h, const double *x, double *Gf) {
-  const int No = h->d.No, Nv = h->d.Nv, N = h->d.N;
+// One-body densities of x (the N^5 part of <x, dA x>), accumulated into Gf (N x N).  T, X and Y are
+// antisymmetric in both index pairs and S_ij^ab = S_ji^ba, so their sums over rows and over columns are
+// the same, and the slices i < j of the first three count twice: a product over the listed slices of the
+// three blocks (equal weights) takes 1.5 units of work in place of six, S one in place of two, Z two.
+// The float64 pipe bounds them: No=12 Nv=120, all float64 GEMMs of the gradient 7.2 -> 3.8 ms.
+static esmp2_status densities(esmp2_handle *h, const double *x, double *Gf) {
+  const int No = h->d.No, Nv = h->d.Nv, N = h->d.N, NN = No * No, half = No * (No - 1) / 2;
   const int64_t B = h->d.B, NvNv = (int64_t)Nv * Nv;
-  const double W[5] = {WT, WS, WX, WY, WZ};
-  for (int blk = 0; blk < 5; ++blk) {
-    const double *X = x + blk * B;
+  if (esmp2_status s = ensure_slist(h)) return s;
+  double *Gv = Gf + (int64_t)No * N + No;
+  // virtual: sum over (s, a) of X_s[a][p] X_s[a][q], and (by columns) over (s, b) of X_s[p][b] X_s[q][b]
+  auto virt = [&](const double *X, const int *list, int ns, double w, bool cols) {
     Gemm64 g{};
-    // virtual: sum over rows (s,a) of X[s][a][p] X[s][a][q]
-    g.M = Nv; g.N = Nv; g.K = No * No * Nv; g.batch = 1; g.alpha = W[blk]; g.beta = 1.0; g.sym = 1;
-    g.A = X; g.sAm = 1; g.sAk = Nv; g.B = X; g.sBk = Nv; g.sBn = 1;
-    g.C = Gf + (int64_t)No * N + No; g.sCm = N; g.sCn = 1;
-    gemm64(g, h->stream);
-    // virtual: sum over (s,b) of X[s][p][b] X[s][q][b]
-    g = Gemm64{};
-    g.M = Nv; g.N = Nv; g.K = No * No * Nv; g.batch = 1; g.alpha = W[blk]; g.beta = 1.0; g.sym = 1;
+    g.M = Nv; g.N = Nv; g.K = ns * Nv; g.batch = 1; g.alpha = w; g.beta = 1.0; g.sym = 1;
     g.Kin = Nv;
-    g.A = X; g.sAm = Nv; g.sAk = 1; g.sAk1 = NvNv;
-    g.B = X; g.sBk = 1; g.sBk1 = NvNv; g.sBn = Nv;
-    g.C = Gf + (int64_t)No * N + No; g.sCm = N; g.sCn = 1;
+    g.klist = list;
+    g.A = X; g.sAm = cols ? Nv : 1; g.sAk = cols ? 1 : Nv; g.sAk1 = NvNv;
+    g.B = X; g.sBn = cols ? Nv : 1; g.sBk = cols ? 1 : Nv; g.sBk1 = NvNv;
+    g.C = Gv; g.sCm = N; g.sCn = 1;
     gemm64(g, h->stream);
-    // occupied: -(sum over (j,ab) of X[l][j][ab] X[i][j][ab]) - (sum over (i',ab) of X[i'][l][ab] X[i'][i][ab])
-    g = Gemm64{};
-    g.M = No; g.N = No; g.K = (int)((int64_t)No * NvNv); g.batch = 1; g.alpha = -W[blk]; g.beta = 1.0; g.sym = 1;
-    g.A = X; g.sAm = (int64_t)No * NvNv; g.sAk = 1; g.B = X; g.sBk = 1; g.sBn = (int64_t)No * NvNv;
+    h->launches += 1;
+  };
+  // occupied: minus the sum over (j, ab) of X[l][j][ab] X[i][j][ab], and over (i', ab) of X[i'][l][ab] X[i'][i][ab]
+  auto occ = [&](const double *X, double w, bool second) {
+    Gemm64 g{};
+    g.M = No; g.N = No; g.K = (int)(No * NvNv); g.batch = 1; g.alpha = -w; g.beta = 1.0; g.sym = 1;
+    if (second) {
+      g.Kin = (int)NvNv;
+      g.sAk1 = g.sBk1 = (int64_t)No * NvNv;
+    }
+    g.A = X; g.sAm = second ? NvNv : (int64_t)No * NvNv; g.sAk = 1;
+    g.B = X; g.sBn = g.sAm; g.sBk = 1;
     g.C = Gf; g.sCm = N; g.sCn = 1;
     gemm64(g, h->stream);
-    g = Gemm64{};
-    g.M = No; g.N = No; g.K = (int)((int64_t)No * NvNv); g.batch = 1; g.alpha = -W[blk]; g.beta = 1.0; g.sym = 1;
-    g.Kin = (int)NvNv;
-    g.A = X; g.sAm = NvNv; g.sAk = 1; g.sAk1 = (int64_t)No * NvNv;
-    g.B = X; g.sBk = 1; g.sBk1 = (int64_t)No * NvNv; g.sBn = NvNv;
-    g.C = Gf; g.sCm = N; g.sCn = 1;
-    gemm64(g, h->stream);
-    h->launches += 4;
-  }
+    h->launches += 1;
+  };
+  if (half) virt(x, h->slist, 3 * half, 4.0 * WT, false);
+  virt(x + BS * B, nullptr, NN, 2.0 * WS, false);
+  virt(x + BZ * B, nullptr, NN, WZ, false);
+  virt(x + BZ * B, nullptr, NN, WZ, true);
+  for (int blk : {BT, BX, BY}) occ(x + blk * B, 2.0 * WT, false);
+  occ(x + BS * B, 2.0 * WS, false);
+  occ(x + BZ * B, WZ, false);
+  occ(x + BZ * B, WZ, true);
+  return ESMP2_OK;
 }
 
 esmp2_status gradient(esmp2_handle *h, double *dF_host, double *dOVOV_host, int adjoint, double *adj_diff) {
@@ -551,12 +572,12 @@ esmp2_status gradient(esmp2_handle *h, double *dF_host, double *dOVOV_host, int 
   GCtx c;
   c.No = No; c.Nv = Nv; c.N = N; c.B = h->d.B; c.x = h->s64.x; c.lam = h->lam; c.ovov = h->ovov; c.F = h->F;
   c.omega = h->omega_op;
-  densities(h, h->s64.x, Gf);
+  if (esmp2_status sd = densities(h, h->s64.x, Gf)) { release(); return sd; }
   kg_ovov_L<<<1216, 256, 0, st>>>(c, Gov);
   kg_small<<<(unsigned)cdiv((int64_t)No * Nv, 128), 128, 0, st>>>(c, Gov, Gf);
   kg_scalars<<<1216, 256, 0, st>>>(c, acc);
   kg_F2<<<Nv, 256, 0, st>>>(c, Gf);
-  kg_F3<<<No, 256, 0, st>>>(c, Gf);
+  kg_F3<<<dim3((unsigned)No, (unsigned)std::max<int64_t>(1, std::min<int64_t>(cdiv(1216, No), (int64_t)No * Nv * Nv / 2048))), 256, 0, st>>>(c, Gf);
   kg_F4<<<No * Nv, 128, 0, st>>>(c, Gf);
   kg_F5to8<<<2 * (No + Nv), 128, 0, st>>>(c, Gf);
   kg_finish_scalars<<<1, 32, 0, st>>>(c, acc, Gf);

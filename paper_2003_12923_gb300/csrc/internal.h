@@ -36,6 +36,7 @@ struct Gemm64 {
   double *C; int64_t sCm, sCn, sCb;
   int Kin;
   int64_t sAk1, sBk1;
+  const int *klist;       // Kin > 0: k1 counts the entries of this list (slices) instead of 0, 1, ...
   int sym;                // C is symmetric (M = N, B(k, n) = A(n, k)): tiles above the diagonal only, mirrored
 };
 void gemm64(const Gemm64 &g, cudaStream_t st);
