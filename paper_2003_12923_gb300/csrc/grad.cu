@@ -251,23 +251,13 @@ __device__ void flush_diag(const SG &g, double *sdiag) {
     if (sdiag[k] != 0.0) atomicAdd(&g.Gdiag[k], sdiag[k]);
 }
 
-// 1 / x: a float32 reciprocal and two Newton steps (four float64 operations; the division takes some
-// twenty of the pipe that bounds these kernels), the division outside the range of float32.  Error below
-// 2 ulp; No=12 Nv=120, kg_s_ab + kg_s_cm with the division 1.6 ms, so 1.0 ms.
-__device__ __forceinline__ double recip(double x) {
-  const double ax = fabs(x);
-  if (!(ax > 1e-30 && ax < 1e30)) return 1.0 / x;
-  double y = (double)(1.0f / (float)x);
-  y = fma(y, fma(-x, y, 1.0), y);
-  return fma(y, fma(-x, y, 1.0), y);
-}
-
 // S-space derivative, the triples with exactly one transition pair (the energy's k_e2s_ab and
 // k_e2s_cm enumerate the same ones): b_I is lambda_u times one antisymmetrised integral, so a
 // thread that owns the integral sums over the pair u itself, adds its own two (ov|ov) elements
 // without atomics (no other thread writes them) and keeps the diagonal sums in registers and
 // private shared-memory slots.  One triple at a time with nine scattered float64 atomics each took
-// 17.5 ms at No=12 Nv=120, this form 1.0 ms.
+// 17.5 ms at No=12 Nv=120, this form 1.0 ms.  (A float32 reciprocal with two Newton steps in place of the
+// division was slower: 0.96 ms against 0.76 ms for the two kernels, the conversions share the pipe.)
 constexpr int kST = 128;   // threads of the S-space gradient kernels
 
 // shared memory: lu2[No], du[No], sdiag[N + 1], private per-u sums [No][kST]
@@ -329,7 +319,7 @@ __global__ void __launch_bounds__(kST) kg_s_ab(SG g, int nchunk) {
         double q1 = 0.0;
         for (int u = 1; u < No; ++u) {
           const double m = (u != j && u != k && u != b && u != cc) ? 2.0 : 1.0;   // sectors A and B, or B alone
-          const double r = recip(s.du[u] + e), q = m * s.lu2[u] * r, d = 2.0 * dg * dg * q * r;
+          const double r = 1.0 / (s.du[u] + e), q = m * s.lu2[u] * r, d = 2.0 * dg * dg * q * r;
           q1 += q;
           su[u * kST] += d;
           gd += d;
@@ -375,7 +365,7 @@ __global__ void __launch_bounds__(kST) kg_s_cm(SG g, int nchunk) {
         double q1 = 0.0;
         for (int u = 1; u < No; ++u) {
           if (u == k || u == cc) continue;
-          const double r = recip(s.du[u] + e), q = s.lu2[u] * r, d = 2.0 * gv * gv * q * r;
+          const double r = 1.0 / (s.du[u] + e), q = s.lu2[u] * r, d = 2.0 * gv * gv * q * r;
           q1 += q;
           su[u * kST] += d;
           gd += d;
@@ -477,7 +467,7 @@ __global__ void kg_transpose(const double *A, double *At, int n) {
 // antisymmetric in both index pairs and S_ij^ab = S_ji^ba, so their sums over rows and over columns are
 // the same, and the slices i < j of the first three count twice: a product over the listed slices of the
 // three blocks (equal weights) takes 1.5 units of work in place of six, S one in place of two, Z two.
-// The float64 pipe bounds them: No=12 Nv=120, all float64 GEMMs of the gradient 7.2 -> 3.8 ms.
+// The float64 pipe bounds them: No=12 Nv=120, all float64 GEMMs of the gradient 6.3 -> 3.8 ms.
 static esmp2_status densities(esmp2_handle *h, const double *x, double *Gf) {
   const int No = h->d.No, Nv = h->d.Nv, N = h->d.N, NN = No * No, half = No * (No - 1) / 2;
   const int64_t B = h->d.B, NvNv = (int64_t)Nv * Nv;
