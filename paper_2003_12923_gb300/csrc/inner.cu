@@ -156,6 +156,21 @@ __device__ __forceinline__ void cta_partials(double (&v)[NQ], double *red) {
   }
 }
 
+// (float)x by integer operations: the conversion runs on the float64 pipe (two a clock and SM) and bound
+// the pass that uses this.  The significand is rounded to nearest even; what does not land on a normal
+// float32 is converted.
+__device__ __forceinline__ float to_f32(double x) {
+  const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+  const int ef = (int)(hi >> 20) & 0x7FF;
+  uint32_t t = 0;                                    // below 2^-150: a zero
+  if (ef >= 870) {
+    if (ef < 897 || ef > 1149) return (float)x;
+    t = __funnelshift_l(lo, hi, 3) - (0x180u << 23);   // exponent field ef - 896, upper 23 bits
+    t += (lo << 3) + (t & 1u) > 0x80000000u ? 1u : 0u;
+  }
+  return __uint_as_float(t | (hi & 0x80000000u));
+}
+
 __device__ __forceinline__ float blk_w(int blk) { return blk == BZ ? 2.f : 1.f; }
 
 // ---------------------------------------------------------------- layout conversions
@@ -189,25 +204,48 @@ __global__ void kp_init(PV pv, const double *r64, const __half *dinv, float *r, 
   cta_partials<2>(v, red);
 }
 
+constexpr int kRowChunk = 32;   // rows of a slice per CTA iteration of the conversions below
+__host__ __device__ __forceinline__ int row_chunks(int Nv) { return (Nv + kRowChunk - 1) / kRowChunk; }
+
 // x64 (full storage) += d (packed); T, X, Y slices also update their (j, i) partner with -d.
-// One warp per packed row (slice, a); consecutive lanes take consecutive b, so every load and
-// every read-modify-write of the float64 rows is one contiguous segment per warp.
-__global__ void __launch_bounds__(256) kp_acc64(PV pv, double *x, const float *d) {
+// slots (rotated preconditioner): the last step alpha p is not in d yet, and d holds nothing before the
+// second direction.  A CTA takes kRowChunk rows of one slice, a warp one row at a time, VW consecutive b
+// per lane (two where rows of x64 start on 16-byte boundaries).  Memory-bound: 4.7 TB/s over its five
+// streams at No=30 Nv=400 (3.2 ms; the pass over d alone took 3.1 ms, and the separate update of d that
+// the second stream replaces 1.2 ms).
+template <int VW>
+__global__ void __launch_bounds__(256) kp_acc64(PV pv, double *x, const float *d, const float *p, const double *slots) {
+  using D = std::conditional_t<VW == 2, double2, double>;
+  using S = std::conditional_t<VW == 2, float2, float>;
   const Packed &L = pv.L;
-  const int64_t rows = (int64_t)L.nslices * L.Nv, NvNv = (int64_t)L.Nv * L.Nv, B = (int64_t)L.NN * NvNv;
-  const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5, Nv = L.Nv;
-  for (int64_t row = (int64_t)blockIdx.x * wpb + (threadIdx.x >> 5); row < rows; row += (int64_t)gridDim.x * wpb) {
-    const int s = (int)(row / Nv), a = (int)(row % Nv);
-    int blk, i, j;
-    pv.decode(s, blk, i, j);
-    const float *src = d + (int64_t)s * L.SL + (int64_t)a * L.Nvp;
-    double *x1 = x + blk * B + ((int64_t)i * L.No + j) * NvNv + (int64_t)a * Nv;
-    double *x2 = x + blk * B + ((int64_t)j * L.No + i) * NvNv + (int64_t)a * Nv;
-    const bool anti = !(blk == BS || blk == BZ);
-    for (int b = lane; b < Nv; b += 32) {
-      const double v = (double)src[b];
-      x1[b] += v;
-      if (anti) x2[b] -= v;
+  const int64_t NvNv = (int64_t)L.Nv * L.Nv, B = (int64_t)L.NN * NvNv;
+  const int lane = threadIdx.x & 31, Nv = L.Nv, nc = row_chunks(Nv);
+  const float alpha = slots ? (float)slots[4] : 0.f;
+  const bool with_d = !slots || slots[22] > 1.0;
+  const int s = blockIdx.x / nc, a0 = (blockIdx.x % nc) * kRowChunk, a1 = min(Nv, a0 + kRowChunk);
+  int blk, i, j;
+  pv.decode(s, blk, i, j);
+  const bool anti = !(blk == BS || blk == BZ);
+  double *xa = x + blk * B + ((int64_t)i * L.No + j) * NvNv, *xb = x + blk * B + ((int64_t)j * L.No + i) * NvNv;
+  for (int a = a0 + (threadIdx.x >> 5); a < a1; a += 8) {
+    const int64_t e0 = (int64_t)s * L.SL + (int64_t)a * L.Nvp;
+    double *x1 = xa + (int64_t)a * Nv, *x2 = xb + (int64_t)a * Nv;
+#pragma unroll 2
+    for (int b = VW * lane; b < Nv; b += VW * 32) {
+      S dv{}, sv{};
+      if (with_d) dv = *reinterpret_cast<const S *>(d + e0 + b);
+      if (slots) sv = *reinterpret_cast<const S *>(p + e0 + b);
+      D u = *reinterpret_cast<D *>(x1 + b), w{};
+      if (anti) w = *reinterpret_cast<D *>(x2 + b);
+      if constexpr (VW == 2) {
+        const double vx = (double)fmaf(alpha, sv.x, dv.x), vy = (double)fmaf(alpha, sv.y, dv.y);
+        u.x += vx; u.y += vy; w.x -= vx; w.y -= vy;
+      } else {
+        const double v = (double)fmaf(alpha, sv, dv);
+        u += v; w -= v;
+      }
+      *reinterpret_cast<D *>(x1 + b) = u;
+      if (anti) *reinterpret_cast<D *>(x2 + b) = w;
     }
   }
 }
@@ -911,32 +949,48 @@ __device__ __forceinline__ void st_bf4(__nv_bfloat16 *p4, float4 v) {
   *reinterpret_cast<uint2 *>(p4) = u;
 }
 
-// start of an inner solve: r = r64 on the packed slots, rb = bf16(r), d = 0; partials <r, r>_w.
-// One warp per packed row (slice, a), four consecutive b per lane.
-__global__ void __launch_bounds__(256) kp_init_rj(PV pv, const double *r64, float *r, __nv_bfloat16 *rb, float *d,
-                                                  double *red) {
+// start of an inner solve: r = r64 on the packed slots, rb = bf16(r); partials <r, r>_w.
+// A CTA iteration takes kRowChunk rows of one slice, a warp one row at a time, four consecutive b per
+// lane (two 16-byte loads where rows of r64 start on 16-byte boundaries).  No=30 Nv=400: 1.85 ms with
+// d = 0 written too, 1.57 ms without, 1.11 ms with integer rounding (6.2 TB/s).
+template <bool VEC>
+__global__ void __launch_bounds__(256) kp_init_rj(PV pv, const double *r64, float *r, __nv_bfloat16 *rb, double *red) {
   const Packed &L = pv.L;
-  const int64_t rows = (int64_t)L.nslices * L.Nv, NvNv = (int64_t)L.Nv * L.Nv, B = (int64_t)L.NN * NvNv;
-  const int lane = threadIdx.x & 31, wpb = blockDim.x >> 5, q4 = L.Nvp >> 2, Nv = L.Nv;
+  const int64_t NvNv = (int64_t)L.Nv * L.Nv, B = (int64_t)L.NN * NvNv;
+  const int lane = threadIdx.x & 31, q4 = L.Nvp >> 2, Nv = L.Nv, nc = row_chunks(Nv), items = L.nslices * nc;
   float a1 = 0.f;
-  for (int64_t row = (int64_t)blockIdx.x * wpb + (threadIdx.x >> 5); row < rows; row += (int64_t)gridDim.x * wpb) {
-    const int s = (int)(row / Nv), a = (int)(row % Nv);
+  for (int it = blockIdx.x; it < items; it += gridDim.x) {
+    const int s = it / nc, a0 = (it % nc) * kRowChunk, a1r = min(Nv, a0 + kRowChunk);
     int blk, i, j;
     pv.decode(s, blk, i, j);
-    const double *src = r64 + blk * B + ((int64_t)i * L.No + j) * NvNv + (int64_t)a * Nv;
-    const int64_t e0 = (int64_t)s * L.SL + (int64_t)a * L.Nvp;
+    const double *slice = r64 + blk * B + ((int64_t)i * L.No + j) * NvNv;
     const float w = blk_w(blk);
-    for (int c = lane; c < q4; c += 32) {
-      const int b = 4 * c;
-      float4 v;
-      v.x = b < Nv ? (float)src[b] : 0.f;
-      v.y = b + 1 < Nv ? (float)src[b + 1] : 0.f;
-      v.z = b + 2 < Nv ? (float)src[b + 2] : 0.f;
-      v.w = b + 3 < Nv ? (float)src[b + 3] : 0.f;
-      *reinterpret_cast<float4 *>(r + e0 + b) = v;
-      st_bf4(rb + e0 + b, v);
-      *reinterpret_cast<float4 *>(d + e0 + b) = make_float4(0.f, 0.f, 0.f, 0.f);
-      a1 += w * (v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w);
+    for (int a = a0 + (threadIdx.x >> 5); a < a1r; a += 8) {
+      const double *src = slice + (int64_t)a * Nv;
+      const int64_t e0 = (int64_t)s * L.SL + (int64_t)a * L.Nvp;
+#pragma unroll 2
+      for (int c = lane; c < q4; c += 32) {
+        const int b = 4 * c;
+        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (VEC) {   // Nv even: a pair is inside the row or outside it
+          if (b < Nv) {
+            const double2 t = *reinterpret_cast<const double2 *>(src + b);
+            v.x = to_f32(t.x); v.y = to_f32(t.y);
+          }
+          if (b + 2 < Nv) {
+            const double2 t = *reinterpret_cast<const double2 *>(src + b + 2);
+            v.z = to_f32(t.x); v.w = to_f32(t.y);
+          }
+        } else {
+          v.x = b < Nv ? to_f32(src[b]) : 0.f;
+          v.y = b + 1 < Nv ? to_f32(src[b + 1]) : 0.f;
+          v.z = b + 2 < Nv ? to_f32(src[b + 2]) : 0.f;
+          v.w = b + 3 < Nv ? to_f32(src[b + 3]) : 0.f;
+        }
+        *reinterpret_cast<float4 *>(r + e0 + b) = v;
+        st_bf4(rb + e0 + b, v);
+        a1 += w * (v.x * v.x + v.y * v.y + v.z * v.z + v.w * v.w);
+      }
     }
   }
   double v[1] = {(double)a1};
@@ -963,19 +1017,25 @@ __global__ void kp_update_rj(PV pv, const double *slots, float *r, const float *
   cta_partials<1>(v, red);
 }
 
-// d += alpha p; p = z + beta p; pb = bf16(p) (if kept)
+// d += alpha p; p = z + beta p; pb = bf16(p) (if kept).  The first direction of a solve (slot 22 = 1)
+// reads neither p nor d, the second one starts d: 10 and 18 of the 22 bytes per element.
 __global__ void kp_p_rj(PV pv, const double *slots, const float *z, float *p, float *d, __nv_bfloat16 *pb) {
   const Packed &L = pv.L;
   const float alpha = (float)slots[4], beta = (float)slots[5];
+  const int dir = (int)slots[22];
   const int64_t n4 = L.n >> 2;
   const float4 *z4 = reinterpret_cast<const float4 *>(z);
   float4 *p4 = reinterpret_cast<float4 *>(p), *d4 = reinterpret_cast<float4 *>(d);
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n4; e += (int64_t)gridDim.x * blockDim.x) {
-    const float4 pv4 = p4[e], zv = __ldg(z4 + e);
-    float4 dv = d4[e];
-    dv.x += alpha * pv4.x; dv.y += alpha * pv4.y; dv.z += alpha * pv4.z; dv.w += alpha * pv4.w;
-    d4[e] = dv;
-    const float4 pn = make_float4(zv.x + beta * pv4.x, zv.y + beta * pv4.y, zv.z + beta * pv4.z, zv.w + beta * pv4.w);
+    float4 pn = __ldg(z4 + e);
+    if (dir > 1) {
+      const float4 po = p4[e];
+      float4 dv = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (dir > 2) dv = d4[e];
+      dv.x += alpha * po.x; dv.y += alpha * po.y; dv.z += alpha * po.z; dv.w += alpha * po.w;
+      d4[e] = dv;
+      pn.x += beta * po.x; pn.y += beta * po.y; pn.z += beta * po.z; pn.w += beta * po.w;
+    }
     p4[e] = pn;
     if (pb) st_bf4(pb + 4 * e, pn);
   }
@@ -1346,8 +1406,11 @@ double packed_wdot(esmp2_handle *h, const float *u, const float *v) {
   return t;
 }
 
-void packed_accumulate(esmp2_handle *h, double *x64) {
-  kp_acc64<<<2432, 256, 0, h->stream>>>(PV{h->pk}, x64, h->pd);
+void packed_accumulate(esmp2_handle *h, double *x64, bool rj) {
+  const double *slots = rj ? h->red_out : nullptr;
+  const unsigned grid = (unsigned)(h->pk.nslices * row_chunks(h->d.Nv));
+  if (h->d.Nv & 1) kp_acc64<1><<<grid, 256, 0, h->stream>>>(PV{h->pk}, x64, h->pd, packed_p(h), slots);
+  else kp_acc64<2><<<grid, 256, 0, h->stream>>>(PV{h->pk}, x64, h->pd, packed_p(h), slots);
   h->launches += 1;
 }
 
@@ -1374,14 +1437,12 @@ esmp2_status packed_rj_setup(esmp2_handle *h) {
   A(reinterpret_cast<void **>(&h->pOcc), sizeof(float) * (size_t)L.nslices);
   A(reinterpret_cast<void **>(&h->pCode), sizeof(int) * (size_t)L.nslices);
   A(reinterpret_cast<void **>(&h->pdot2), sizeof(double) * 5 * (size_t)kCoupleGrid);
-  A(reinterpret_cast<void **>(&h->zero_slots), sizeof(double) * 32);
   if (e != cudaSuccess) return check_cuda(h, e, "rotated preconditioner buffers");
   // pad columns of the GEMM operands and of z start (and stay) zero: the transposed epilogue
   // writes columns < Nv only, and p = z + beta p must keep zero pads (they are K of the sigma GEMM)
   cudaMemsetAsync(h->pRbf, 0, sizeof(__nv_bfloat16) * (size_t)L.n, st);
   cudaMemsetAsync(h->pT1, 0, sizeof(__nv_bfloat16) * (size_t)L.n, st);
   cudaMemsetAsync(h->pZ, 0, sizeof(float) * (size_t)L.n, st);
-  cudaMemsetAsync(h->zero_slots, 0, sizeof(double) * 32, st);
   std::vector<double> R((size_t)Nv * Nv);
   std::vector<float> F((size_t)N * N), Fs((size_t)N * N);
   e = cudaMemcpyAsync(R.data(), h->Rv, sizeof(double) * R.size(), cudaMemcpyDeviceToHost, st);
@@ -1451,38 +1512,39 @@ static esmp2_status packed_precond(esmp2_handle *h) {
   return check_cuda(h, cudaGetLastError(), "packed_precond");
 }
 
-// start of a preconditioned inner solve: r (packed) from r64, d = 0, z = M^-1 r, p = z; slots:
-// rr (1) and rz (0)
+// start of a preconditioned inner solve: r (packed) from r64; slots: rr (1), no direction yet (22)
 esmp2_status packed_rj_init(esmp2_handle *h, const double *r64, int grid) {
-  const Packed &L = h->pk;
-  PV pv{L};
+  PV pv{h->pk};
   cudaStream_t st = h->stream;
-  kp_init_rj<<<grid, 256, 0, st>>>(pv, r64, h->pr, static_cast<__nv_bfloat16 *>(h->pRbf), h->pd, h->red);
-  k_finalize_ext(h->red, grid, h->red_out, 5, st);
-  h->launches += 2;
-  if (esmp2_status s = packed_precond(h)) return s;
-  k_finalize_ext(h->pdot2, 5 * kCoupleGrid, h->red_out, 7, st);
-  kp_p_rj<<<grid, 256, 0, st>>>(pv, h->zero_slots, h->pZ, packed_p(h), h->pd,
-                                h->tf32 ? nullptr : static_cast<__nv_bfloat16 *>(h->pop));
+  auto *rb = static_cast<__nv_bfloat16 *>(h->pRbf);
+  if (h->d.Nv & 1) kp_init_rj<false><<<grid, 256, 0, st>>>(pv, r64, h->pr, rb, h->red);
+  else kp_init_rj<true><<<grid, 256, 0, st>>>(pv, r64, h->pr, rb, h->red);
+  k_finalize_ext(h->red, grid, h->red_out, 7, st);
   h->launches += 2;
   return check_cuda(h, cudaGetLastError(), "packed_rj_init");
 }
 
-// the part of a preconditioned inner iteration after q = A p and alpha: r -= alpha q, z = M^-1 r,
-// beta, d += alpha p, p = z + beta p
-esmp2_status packed_rj_step(esmp2_handle *h, int grid) {
-  const Packed &L = h->pk;
-  PV pv{L};
+// the next direction (first in an iteration, so that the residual that ends the solve is not
+// preconditioned: No=20 Nv=200 57.9 -> 55.2 ms, No=30 Nv=400 338 -> 320 ms): z = M^-1 r, beta, d += alpha p (the previous step), p = z + beta p
+esmp2_status packed_rj_direction(esmp2_handle *h, int grid) {
+  PV pv{h->pk};
   cudaStream_t st = h->stream;
-  kp_update_rj<<<grid, 256, 0, st>>>(pv, h->red_out, h->pr, h->pq, static_cast<__nv_bfloat16 *>(h->pRbf), h->red);
-  k_finalize_ext(h->red, grid, h->red_out, 5, st);
-  h->launches += 2;
   if (esmp2_status s = packed_precond(h)) return s;
   k_finalize_ext(h->pdot2, 5 * kCoupleGrid, h->red_out, 6, st);
   kp_p_rj<<<grid, 256, 0, st>>>(pv, h->red_out, h->pZ, packed_p(h), h->pd,
                                 h->tf32 ? nullptr : static_cast<__nv_bfloat16 *>(h->pop));
   h->launches += 2;
-  return check_cuda(h, cudaGetLastError(), "packed_rj_step");
+  return check_cuda(h, cudaGetLastError(), "packed_rj_direction");
+}
+
+// after q = A p and alpha: r -= alpha q
+esmp2_status packed_rj_update(esmp2_handle *h, int grid) {
+  PV pv{h->pk};
+  cudaStream_t st = h->stream;
+  kp_update_rj<<<grid, 256, 0, st>>>(pv, h->red_out, h->pr, h->pq, static_cast<__nv_bfloat16 *>(h->pRbf), h->red);
+  k_finalize_ext(h->red, grid, h->red_out, 5, st);
+  h->launches += 2;
+  return check_cuda(h, cudaGetLastError(), "packed_rj_update");
 }
 
 // per-stage timing of `reps` packed inner sigma builds of the packed copy of x (CUDA events):

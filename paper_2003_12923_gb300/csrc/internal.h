@@ -163,7 +163,6 @@ struct esmp2_handle {
   float *pLam = nullptr, *pOcc = nullptr;  // diagonal of F_vv in that basis; per-slice occupied part
   int *pCode = nullptr;     // per-slice block | 8 (i == 0) | 16 (j == 0)
   double *pdot2 = nullptr;  // partials of <r, z>_w
-  double *zero_slots = nullptr;  // 32 zero doubles (alpha = beta = 0)
   cudaEvent_t ovvv_ready = nullptr;  // create: the OVVV input copy (side stream) has landed
   bool x_zero = true;       // s64.x is known to be zero (its sigma is zero, no build needed)
   bool r_true = false;      // s64.r holds the true residual -b - A x of s64.x (same basis)
@@ -248,10 +247,11 @@ void packed_init(esmp2_handle *h, const double *r64, int grid);
 esmp2_status packed_rj_setup(esmp2_handle *h);
 void k_finalize_ext(const double *red, int nparts, double *slots, int mode, cudaStream_t st);
 esmp2_status packed_rj_init(esmp2_handle *h, const double *r64, int grid);
-esmp2_status packed_rj_step(esmp2_handle *h, int grid);
+esmp2_status packed_rj_direction(esmp2_handle *h, int grid);
+esmp2_status packed_rj_update(esmp2_handle *h, int grid);
 esmp2_status ensure_vrot(esmp2_handle *h, bool exact);
 float *packed_p(esmp2_handle *h);
-void packed_accumulate(esmp2_handle *h, double *x64);
+void packed_accumulate(esmp2_handle *h, double *x64, bool rj);
 double packed_wdot(esmp2_handle *h, const float *u, const float *v);
 esmp2_status sigma_mixed_packed(esmp2_handle *h, const double *x, double *y);
 void antisym_project(esmp2_handle *h, double *v);

@@ -78,8 +78,8 @@ __device__ __forceinline__ void block_partials(double (&v)[NQ], double *red) {
 }
 
 // Sum the partials of nq quantities in fixed order; mode selects the scalar bookkeeping.
-// slots: 0 rz, 1 rr, 2 bb, 3 pq, 4 alpha, 5 beta, 8.. generic results (slots 4, 5 of a zeroed
-// slot array give alpha = beta = 0)
+// slots: 0 rz, 1 rr, 2 bb, 3 pq, 4 alpha, 5 beta, 8.. generic results (22 directions
+// formed in the preconditioned inner solve)
 // One CTA, every quantity in the same pass: it sits on the critical path of each iteration (a loop per
 // quantity on 256 threads took 7.5 us for 6080 partials).
 __global__ void __launch_bounds__(1024) k_finalize(const double *__restrict__ red, int nparts, int nq, double *slots, int mode) {
@@ -107,11 +107,13 @@ __global__ void __launch_bounds__(1024) k_finalize(const double *__restrict__ re
     else slots[1] = t;
   } else if (mode == 5) {     // rr alone
     slots[1] = t;
-  } else if (mode == 6) {     // rz_new alone -> beta
-    slots[5] = t / slots[0];
+  } else if (mode == 6) {     // rz_new alone -> beta (0 for the first direction)
+    slots[5] = slots[22] > 0.0 ? t / slots[0] : 0.0;
     slots[0] = t;
-  } else if (mode == 7) {     // rz alone (start)
-    slots[0] = t;
+    slots[22] += 1.0;
+  } else if (mode == 7) {     // rr at the start of an inner solve
+    slots[1] = t;
+    slots[22] = 0.0;
   } else if (mode == 8) {     // the S-space energy
     slots[20] = t;
   } else {                    // generic
@@ -1196,13 +1198,17 @@ esmp2_status solve_mixed(esmp2_handle *h, double tol, int maxit, esmp2_solve_inf
     const double target = std::max(eta * r0, 0.25 * tol * bn);
     int inner = 0, since_best = 0;
     double best = r0;
-    // one inner iteration: q = A p, alpha, x/r update, beta, p update (device scalars only)
+    // one inner iteration, device scalars only: q = A p, alpha, d/r update, beta, p update; with the
+    // rotated preconditioner z = M^-1 r, beta, d and p update, q = A p, alpha, r update, so that
+    // nothing is preconditioned after the last residual
     const bool dbg_dot = std::getenv("ESMP2_DEBUG") != nullptr && !use_graph;
     double fused_pq = 0.0, sep_pq = 0.0;
     auto inner_step = [&]() -> esmp2_status {
       const int64_t l0 = h->launches;
+      esmp2_status s2 = rj ? packed_rj_direction(h, kRedBlocks) : ESMP2_OK;
+      if (s2) return s2;
       // p.q partials from the coupling pass
-      esmp2_status s2 = packed ? sigma_packed(h, p32, q32, true, h->pdot) : sigma_inner(h, p32, q32, fused_bf16, h->red);
+      s2 = packed ? sigma_packed(h, p32, q32, true, h->pdot) : sigma_inner(h, p32, q32, fused_bf16, h->red);
       if (s2) return s2;
       if (packed && dbg_dot) {  // diagnostics (ESMP2_DEBUG, no graph capture): <p, A p> by a separate pass
         std::vector<double> part(h->pdot_n);
@@ -1215,8 +1221,8 @@ esmp2_status solve_mixed(esmp2_handle *h, double tol, int maxit, esmp2_solve_inf
       if (packed) k_finalize<<<1, 1024, 0, st>>>(h->pdot, h->pdot_n, 1, h->red_out, 1);
       else k_finalize<<<1, 1024, 0, st>>>(h->red, (int)couple_dot_parts(h), 1, h->red_out, 1);
       h->launches += 1;
-      if (rj) {   // r -= alpha q, z = M^-1 r (rotated Jacobi), beta, d and p
-        if ((s2 = packed_rj_step(h, kRedBlocks))) return s2;
+      if (rj) {   // r -= alpha q
+        if ((s2 = packed_rj_update(h, kRedBlocks))) return s2;
       } else {
         ki_update<<<kRedBlocks, kRedThreads, 0, st>>>(ic, h->red_out, r32, q32, h->red);
         k_finalize<<<1, 1024, 0, st>>>(h->red, kRedBlocks, 2, h->red_out, 2);
@@ -1280,7 +1286,7 @@ esmp2_status solve_mixed(esmp2_handle *h, double tol, int maxit, esmp2_solve_inf
       // x stays in the singlet subspace exactly: d is exactly antisymmetric in (a, b) and
       // spin-flip symmetric in S (the packed coupling pass writes both images from one value),
       // and kp_acc64 adds +d and -d to the two slices (negation commutes with rounding)
-      packed_accumulate(h, x);
+      packed_accumulate(h, x, rj);
     } else {
       kt_accumulate<float><<<kRedBlocks, kRedThreads, 0, st>>>(c, x, d32);
       h->launches += 1;
