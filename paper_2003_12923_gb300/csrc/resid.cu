@@ -370,86 +370,59 @@ struct ArrowW64 {
   double fl[32];  // F_l,t for 1 <= l < No, else 0
   double fk[32];  // F_l,t' for l < No, else 0
 };
-// T, X, Y from the slices i < j: OC1[q] = sum_{l>=1} F_lt x_lq (x_lq = -x_ql for l > q), X also OX[q] =
-// sum_l F_l,t' X_lq; one thread per element (a, b)
+// T, X, Y from the slices i < j: OC1[m] = sum_{l>=1} F_lt x_lm (x_lm = -x_ml for l > m), X also OX[m] =
+// sum_l F_l,t' X_lm
 template <int BLK>
-__device__ __forceinline__ void kr_arrow_anti(int No, int64_t NvNv, int64_t B, const double *__restrict__ x, double *oc1, double *ox,
-                                              const ArrowW64 &w) {
+__device__ __forceinline__ void kr_arrow_anti(int No, int m, int64_t NvNv, int64_t B, int64_t e, const double *__restrict__ x,
+                                              double *oc1, double *ox, const ArrowW64 &w) {
   constexpr bool WX = BLK == BX;
-  const double *xb = x + BLK * B;
-  double *o1 = oc1 + (int64_t)BLK * No * NvNv;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < NvNv; e += (int64_t)gridDim.x * blockDim.x) {
-    double c1[32], cx[WX ? 32 : 1];
-#pragma unroll
-    for (int q = 0; q < 32; ++q) c1[q] = 0.0;
-#pragma unroll
-    for (int q = 0; q < (WX ? 32 : 1); ++q) cx[q] = 0.0;
-    for (int p = 0; p < No; ++p) {
-      const double *row = xb + (int64_t)p * No * NvNv + e;
-      const double flp = w.fl[p], fkp = w.fk[p];
-      double r1 = 0.0, rx = 0.0;
-#pragma unroll
-      for (int q = 1; q < 32; ++q) {
-        if (q > p && q < No) {
-          const double v = row[(int64_t)q * NvNv];
-          c1[q] += flp * v;
-          r1 += w.fl[q] * v;
-          if constexpr (WX) {
-            cx[q] += fkp * v;
-            rx += w.fk[q] * v;
-          }
-        }
-      }
-      double cp = 0.0, cxp = 0.0;
-#pragma unroll
-      for (int m = 0; m < 32; ++m)
-        if (m == p) {
-          cp = c1[m];
-          if constexpr (WX) cxp = cx[m];
-        }
-      o1[(int64_t)p * NvNv + e] = cp - r1;
-      if constexpr (WX) ox[(int64_t)p * NvNv + e] = cxp - rx;
-    }
+  const double *xb = x + BLK * B + e;
+  double c = 0.0, r = 0.0, cx = 0.0, rx = 0.0;
+#pragma unroll 8
+  for (int l = 0; l < m; ++l) {
+    const double v = xb[(int64_t)(l * No + m) * NvNv];
+    c += w.fl[l] * v;
+    if (WX) cx += w.fk[l] * v;
   }
+#pragma unroll 8
+  for (int l = m + 1; l < No; ++l) {
+    const double v = xb[(int64_t)(m * No + l) * NvNv];
+    r += w.fl[l] * v;
+    if (WX) rx += w.fk[l] * v;
+  }
+  oc1[((int64_t)BLK * No + m) * NvNv + e] = c - r;
+  if (WX) ox[(int64_t)m * NvNv + e] = cx - rx;
 }
-// S, Z: OC1[m] = sum_{l>=1} F_lt x_lm; Z also OZ[l] = sum_m F_m,t' Z_lm
+// S, Z: OC1[m] = sum_{l>=1} F_lt x_lm; Z also OZ[m] = sum_l F_l,t' Z_ml
 template <int BLK>
-__device__ __forceinline__ void kr_arrow_full(int No, int64_t NvNv, int64_t B, const double *__restrict__ x, double *oc1, double *oz,
-                                              const ArrowW64 &w) {
-  const double *xb = x + BLK * B;
-  double *o1 = oc1 + (int64_t)BLK * No * NvNv;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < NvNv; e += (int64_t)gridDim.x * blockDim.x) {
-    double c1[32];
-#pragma unroll
-    for (int m = 0; m < 32; ++m) c1[m] = 0.0;
-    for (int l = 0; l < No; ++l) {
-      const double *row = xb + (int64_t)l * No * NvNv + e;
-      const double fll = w.fl[l];
-      double rz = 0.0;
-#pragma unroll
-      for (int m = 0; m < 32; ++m) {
-        if (m < No) {
-          const double v = row[(int64_t)m * NvNv];
-          c1[m] += fll * v;
-          if (BLK == BZ) rz += w.fk[m] * v;
-        }
-      }
-      if (BLK == BZ) oz[(int64_t)l * NvNv + e] = rz;
-    }
-#pragma unroll
-    for (int m = 0; m < 32; ++m)
-      if (m < No) o1[(int64_t)m * NvNv + e] = c1[m];
+__device__ __forceinline__ void kr_arrow_full(int No, int m, int64_t NvNv, int64_t B, int64_t e, const double *__restrict__ x,
+                                              double *oc1, double *oz, const ArrowW64 &w) {
+  const double *xb = x + BLK * B + e;
+  double c = 0.0, z = 0.0;
+#pragma unroll 8
+  for (int l = 0; l < No; ++l) {
+    c += w.fl[l] * xb[(int64_t)(l * No + m) * NvNv];
+    if (BLK == BZ) z += w.fk[l] * xb[(int64_t)(m * No + l) * NvNv];
   }
+  oc1[((int64_t)BLK * No + m) * NvNv + e] = c;
+  if (BLK == BZ) oz[(int64_t)m * NvNv + e] = z;
 }
 
+// One thread per sum: the CTAs of one range of elements (a, b) and all m run side by side, so the second
+// read of an amplitude (as x_lm and as -x_ml) hits L2.  Bound by float64 (two to four operations per
+// amplitude).  A thread that kept every sum of an element in registers had No times fewer threads:
+// No=20 Nv=200 0.57 ms, No=30 Nv=400 3.1 ms; this form 1.8 ms at the latter, 1.7 ms of float64 work.
 __global__ void __launch_bounds__(128) k_arrow_sums(int No, int64_t NvNv, int64_t B, const double *__restrict__ x, double *oc1,
                                                     double *ox, double *oz, const __grid_constant__ ArrowW64 w) {
+  const int m = blockIdx.x % No;
+  const int64_t e = (int64_t)(blockIdx.x / No) * 128 + threadIdx.x;
+  if (e >= NvNv) return;
   switch (blockIdx.y) {   // X first: it does the most
-    case 0: kr_arrow_anti<BX>(No, NvNv, B, x, oc1, ox, w); break;
-    case 1: kr_arrow_full<BZ>(No, NvNv, B, x, oc1, oz, w); break;
-    case 2: kr_arrow_full<BS>(No, NvNv, B, x, oc1, oz, w); break;
-    case 3: kr_arrow_anti<BT>(No, NvNv, B, x, oc1, ox, w); break;
-    default: kr_arrow_anti<BY>(No, NvNv, B, x, oc1, ox, w); break;
+    case 0: kr_arrow_anti<BX>(No, m, NvNv, B, e, x, oc1, ox, w); break;
+    case 1: kr_arrow_full<BZ>(No, m, NvNv, B, e, x, oc1, oz, w); break;
+    case 2: kr_arrow_full<BS>(No, m, NvNv, B, e, x, oc1, oz, w); break;
+    case 3: kr_arrow_anti<BT>(No, m, NvNv, B, e, x, oc1, ox, w); break;
+    default: kr_arrow_anti<BY>(No, m, NvNv, B, e, x, oc1, ox, w); break;
   }
 }
 
@@ -536,7 +509,7 @@ esmp2_status residual_sym(esmp2_handle *h, const double *x, const double *b, dou
   }
   ArrowW64 w;
   for (int l = 0; l < 32; ++l) { w.fl[l] = h->arrow_w64[l]; w.fk[l] = h->arrow_w64[32 + l]; }
-  const unsigned ga = (unsigned)std::min<int64_t>(cdiv(NvNv, 128), 4096);
+  const unsigned ga = (unsigned)(No * cdiv(NvNv, 128));
   k_arrow_sums<<<dim3(ga, 5), 128, 0, st>>>(No, NvNv, B, x, h->cp.OC1, h->cp.OX, h->cp.OZ, w);
   launch_intermediates64(h, F, 2, x);
   fill(h, c, F, x);
