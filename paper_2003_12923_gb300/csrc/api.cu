@@ -306,6 +306,7 @@ esmp2_status esmp2_set_solution(esmp2_handle *h, const double *x) {
   cudaMemcpyAsync(h->s64.x, x, sizeof(double) * h->d.n, cudaMemcpyDeviceToDevice, h->stream);
   h->x_basis = 0;
   h->x_zero = false;
+  h->x_sym = false;
   h->r_true = false;
   return check_cuda(h, cudaGetLastError(), "set_solution");
 }

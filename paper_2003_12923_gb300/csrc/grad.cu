@@ -499,6 +499,15 @@ static esmp2_status densities(esmp2_handle *h, const double *x, double *Gf) {
     gemm64(g, h->stream);
     h->launches += 1;
   };
+  if (!h->x_sym) {   // a vector set by the caller: every sum as it stands
+    const double w[5] = {WT, WS, WX, WY, WZ};
+    for (int blk = 0; blk < 5; ++blk)
+      for (bool second : {false, true}) {
+        virt(x + blk * B, nullptr, NN, w[blk], second);
+        occ(x + blk * B, w[blk], second);
+      }
+    return ESMP2_OK;
+  }
   if (half) virt(x, h->slist, 3 * half, 4.0 * WT, false);
   virt(x + BS * B, nullptr, NN, 2.0 * WS, false);
   virt(x + BZ * B, nullptr, NN, WZ, false);
@@ -525,6 +534,7 @@ esmp2_status gradient(esmp2_handle *h, double *dF_host, double *dOVOV_host, int 
     cudaMemsetAsync(h->s64.x, 0, sizeof(double) * n, st);
     h->x_zero = true;
     h->r_true = false;
+    const bool xsym = h->x_sym;
     esmp2_solve_info info{};
     esmp2_status s = solve64(h, 1e-12, 5000, &info);
     if (s != ESMP2_OK && s != ESMP2_ERR_NOT_CONVERGED) { cudaFree(xs); return s; }
@@ -537,6 +547,7 @@ esmp2_status gradient(esmp2_handle *h, double *dF_host, double *dOVOV_host, int 
     if (adj_diff) *adj_diff = xx > 0 ? std::sqrt(dd / xx) : 0.0;
     cudaMemcpyAsync(h->s64.x, xs, sizeof(double) * n, cudaMemcpyDeviceToDevice, st);
     h->x_zero = false;
+    h->x_sym = xsym;
     h->r_true = false;
     cudaStreamSynchronize(st);
     cudaFree(xs);

@@ -121,6 +121,7 @@ struct esmp2_handle {
   double *red = nullptr;    // reduction partials
   double *red_out = nullptr;// reduction results (device)
   double *hred = nullptr;   // pinned host copy of reduction results
+  bool x_sym = true;       // x has the singlet symmetries (every solve makes it so; a vector set by the caller may not)
   bool solved = false;
   bool e2s_done = false;
   double e2s = 0;

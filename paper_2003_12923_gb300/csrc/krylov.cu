@@ -789,6 +789,7 @@ esmp2_status solve64(esmp2_handle *h, double tol, int maxit, esmp2_solve_info *i
     h->launches += 1;
   }
   if (!h->x_zero) singlet_project(h, x);
+  h->x_sym = true;
   int nsig = 0;
   double sl[32], bnorm = -1.0;
   // r = -b - A x (projected), p = M^-1 r, the slots rz and rr
@@ -940,6 +941,7 @@ esmp2_status solve_minres(esmp2_handle *h, double tol, int maxit, esmp2_solve_in
     if (e != cudaSuccess) return check_cuda(h, e, "MINRES vectors");
   }
   singlet_project(h, h->s64.x);
+  h->x_sym = true;
   const VCtx c = vctx(h, h->Farr);
   double *x = h->s64.x, *q = h->s64.q, *r1 = h->s64.r, *r2 = h->s64.p, *v = h->mr_v, *w1 = h->mr_a, *w2 = h->mr_b;
   if (!x || !q || !r1 || !r2 || !v || !w1 || !w2 || !h->barr || !h->Farr) {
@@ -1072,6 +1074,7 @@ esmp2_status solve_mixed(esmp2_handle *h, double tol, int maxit, esmp2_solve_inf
   // S_ji^ba); the packed inner solve acts on that subspace only, so x and every residual
   // handed to it are projected onto it (removing the rounding-level components outside)
   if (!h->x_zero) singlet_project(h, h->s64.x);
+  h->x_sym = true;
   const VCtx c = vctx(h, arrowv ? h->Farr : h->Fsemi);
   const double *bsel = arrowv ? h->barr : h->bsemi;
   debug_phase(h, "solve: x rotation + projection");
