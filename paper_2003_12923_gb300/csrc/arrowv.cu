@@ -14,7 +14,7 @@
 // exact digit-split products per slice.
 //
 // The eigenvectors of the virtual block come from the one-sided (Hestenes) Jacobi method with
-// the round-robin ordering of disjoint pairs: one launch per round, one warp per pair rotating
+// the round-robin ordering of disjoint pairs: one launch per round, one CTA per pair rotating
 // two rows of B and of the accumulated rotation (all accesses along contiguous rows).
 #include <cuda_runtime.h>
 

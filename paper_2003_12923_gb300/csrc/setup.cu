@@ -383,86 +383,128 @@ __global__ void k_f0vo(const double *F, const double *lam, const double *ooov, c
   f0[e] = v;
 }
 
-__device__ __forceinline__ bool valid_elem(int blk, int i, int j, int a, int b) {
-  if ((blk == BT || blk == BX || blk == BY) && (i == j || a == b)) return false;
-  if (blk == BX && (i == 0 || j == 0 || a == 0 || b == 0)) return false;
-  if (blk == BZ && (j == 0 || b == 0 || (i == 0 && a == 0))) return false;
-  return true;
-}
-
 // b = Q H Psi0 on the stored blocks (Slater-Condon rules with Psi0 = sum_u lam_u (u -> u')):
 //  doubles: P(ij)P(ab)[s_ia f0_bj] + P(ij) sum_c <ab||cj> s_ic - P(ab) sum_k <kb||ij> s_ka
 //  triples: P(k/ij)P(c/ab)[<ab||ij> s_kc]  (disconnected product of the double and the single)
 //  Q[i][u][b][a] = (ia|bu'): the OVVT integrals with the last two index pairs moved so
 //  that one of the two OVVT terms of every T/S element runs along b; the other (a and b
-//  exchanged) is staged through shared memory.  One CTA per (block, i, j, 32-row strip of
-//  a), b in tiles of 32.
+//  exchanged) is staged through shared memory.  One CTA per (pair i <= j, 32-row strip of a, T and S
+//  or X, Y and Z), b in tiles of 32: both slices (i, j) and (j, i) of every block come from the same
+//  two integrals, so each is read once (T, S: twice) for up to six results.  One CTA per block
+//  and slice took 11.3 ms at No=30 Nv=400, this form 7.7 ms (9 GB; row segments of 256 bytes in ten
+//  streams keep it well below the copy rate).
 __global__ void __launch_bounds__(256) k_rhs(const double *lam, const double *f0, const double *ovov,
                                              const double *ooov, const double *Q, double *out, int No, int Nv) {
   __shared__ double tji[32][33], tij[32][33];
-  const int64_t sNv = Nv, NvNv = (int64_t)Nv * Nv;
-  const int blk = blockIdx.z, i = blockIdx.y / No, j = blockIdx.y % No, a0 = blockIdx.x * 32;
-  const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const int64_t sNv = Nv, NvNv = (int64_t)Nv * Nv, B = (int64_t)No * No * NvNv;
+  int i = 0, j = blockIdx.y;
+  while (j >= No - i) { j -= No - i; ++i; }
+  j += i;
+  const int a0 = blockIdx.x * 32, tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
+  const bool eq = i == j;
 #define OVOV(i, a, j, b) ovov[(((int64_t)(i) * sNv + (a)) * No + (j)) * sNv + (b)]
 #define OOOV(i, j, k, a) ooov[(((int64_t)(i) * No + (j)) * No + (k)) * sNv + (a)]
 #define F0(a, j) f0[(int64_t)(a) * No + (j)]
-  const double *Qji = Q + ((int64_t)j * No + i) * NvNv;  // Qji[a][b] = OVVT(j, b, a, i)
-  const double *Qij = Q + ((int64_t)i * No + j) * NvNv;  // Qij[a][b] = OVVT(i, b, a, j)
-  double *ys = out + (((int64_t)blk * No + i) * No + j) * NvNv;
+  double *oij = out + ((int64_t)i * No + j) * NvNv, *oji = out + ((int64_t)j * No + i) * NvNv;
   const double li = lam[i], lj = lam[j], l0 = lam[0];
-  for (int b0 = 0; b0 < Nv; b0 += 32) {
-    if (blk == BT || blk == BS) {  // tji[bb][aa] = OVVT(j, a, b, i), tij[bb][aa] = OVVT(i, a, b, j)
+  if (blockIdx.z == 0) {   // T, S
+    const double *Qji = Q + ((int64_t)j * No + i) * NvNv;  // Qji[a][b] = OVVT(j, b, a, i)
+    const double *Qij = Q + ((int64_t)i * No + j) * NvNv;  // Qij[a][b] = OVVT(i, b, a, j)
+    for (int b0 = 0; b0 < Nv; b0 += 32) {
+      const int b = b0 + tx;
+      double p[4], q[4];
       __syncthreads();
-      for (int r = ty; r < 32; r += 8) {
-        const int bb = b0 + r, aa = a0 + tx;
-        const bool in = bb < Nv && aa < Nv;
+#pragma unroll
+      for (int rr = 0; rr < 4; ++rr) {   // tji[bb][aa] = OVVT(j, a, b, i), tij[bb][aa] = OVVT(i, a, b, j)
+        const int r = ty + 8 * rr, a = a0 + r, bb = b0 + r, aa = a0 + tx;
+        const bool in = bb < Nv && aa < Nv, on = a < Nv && b < Nv;
         tji[r][tx] = in ? Qji[(int64_t)bb * Nv + aa] : 0.0;
         tij[r][tx] = in ? Qij[(int64_t)bb * Nv + aa] : 0.0;
+        p[rr] = on ? Qji[(int64_t)a * Nv + b] : 0.0;
+        q[rr] = on ? Qij[(int64_t)a * Nv + b] : 0.0;
       }
       __syncthreads();
-    }
-    const int b = b0 + tx;
-    if (b >= Nv) continue;
 #pragma unroll
-    for (int rr = 0; rr < 4; ++rr) {
-      const int ar = ty + 8 * rr, a = a0 + ar;
-      if (a >= Nv) break;
-      double v = 0.0;
-      if (valid_elem(blk, i, j, a, b)) {
-        if (blk == BT) {
-          if (a == i) v += li * F0(b, j);
-          if (a == j) v -= lj * F0(b, i);
-          if (b == i) v -= li * F0(a, j);
-          if (b == j) v += lj * F0(a, i);
-          v += li * (Qji[(int64_t)a * Nv + b] - tji[tx][ar]) - lj * (Qij[(int64_t)a * Nv + b] - tij[tx][ar]);
-          if (a < No) v -= lam[a] * (OOOV(a, i, j, b) - OOOV(a, j, i, b));
-          if (b < No) v += lam[b] * (OOOV(b, i, j, a) - OOOV(b, j, i, a));
-        } else if (blk == BS) {
-          if (a == i) v += li * F0(b, j);
-          if (b == j) v += lj * F0(a, i);
-          v += li * Qji[(int64_t)a * Nv + b] + lj * tij[tx][ar];
-          if (a < No) v -= lam[a] * OOOV(a, i, j, b);
-          if (b < No) v -= lam[b] * OOOV(b, j, i, a);
-        } else if (blk == BX || blk == BY) {
-          // t j k -> t' b c  (here j,k,b,c = i,j,a,b):  lam_t <bc||jk> + P(jk)P(bc)[lam_k d_ck q(j,b)]
-          v = l0 * (OVOV(i, a, j, b) - OVOV(j, a, i, b));
-          // X: q(j,b) = <t'b||tj> = (t't|bj) - (t'j|bt);  Y: q(j,b) = (t't|bj) (opposite spins)
-          auto q = [&](int jj, int bb) {
-            double r = OVOV(0, 0, jj, bb);
-            if (blk == BX) r -= OVOV(jj, 0, 0, bb);
-            return r;
-          };
-          if (b == j) v += lj * q(i, a);
-          if (b == i) v -= li * q(j, a);
-          if (a == j) v -= lj * q(i, b);
-          if (a == i) v += li * q(j, b);
-        } else {  // BZ: i t k -> a t' c  (here k,c = j,b)
-          v = l0 * OVOV(i, a, j, b);
-          if (b == j) v += lj * OVOV(i, a, 0, 0);
-          if (a == i) v += li * (OVOV(j, b, 0, 0) - OVOV(0, b, j, 0));
+      for (int rr = 0; rr < 4; ++rr) {
+        const int ar = ty + 8 * rr, a = a0 + ar;
+        if (a >= Nv || b >= Nv) continue;
+        const int64_t ab = (int64_t)a * Nv + b;
+        double t = 0.0, s1 = 0.0, s2 = 0.0;   // T_ij, S_ij, S_ji
+        if (!eq && a != b) {
+          if (a == i) t += li * F0(b, j);
+          if (a == j) t -= lj * F0(b, i);
+          if (b == i) t -= li * F0(a, j);
+          if (b == j) t += lj * F0(a, i);
+          t += li * (p[rr] - tji[tx][ar]) - lj * (q[rr] - tij[tx][ar]);
+          if (a < No) t -= lam[a] * (OOOV(a, i, j, b) - OOOV(a, j, i, b));
+          if (b < No) t += lam[b] * (OOOV(b, i, j, a) - OOOV(b, j, i, a));
+        }
+        if (a == i) s1 += li * F0(b, j);
+        if (b == j) s1 += lj * F0(a, i);
+        s1 += li * p[rr] + lj * tij[tx][ar];
+        if (a < No) s1 -= lam[a] * OOOV(a, i, j, b);
+        if (b < No) s1 -= lam[b] * OOOV(b, j, i, a);
+        oij[ab] = t;
+        oij[B + ab] = s1;
+        if (!eq) {
+          if (a == j) s2 += lj * F0(b, i);
+          if (b == i) s2 += li * F0(a, j);
+          s2 += lj * q[rr] + li * tji[tx][ar];
+          if (a < No) s2 -= lam[a] * OOOV(a, j, i, b);
+          if (b < No) s2 -= lam[b] * OOOV(b, i, j, a);
+          oji[ab] = -t;
+          oji[B + ab] = s2;
         }
       }
-      ys[(int64_t)a * Nv + b] = v;
+    }
+  } else {   // X, Y: t j k -> t' b c (here j,k,b,c = i,j,a,b);  Z: i t k -> a t' c (here k,c = j,b)
+    for (int b = tx; b < Nv; b += 32) {
+      double p[4], q[4];
+#pragma unroll
+      for (int rr = 0; rr < 4; ++rr) {
+        const int a = a0 + ty + 8 * rr;
+        p[rr] = a < Nv ? OVOV(i, a, j, b) : 0.0;
+        q[rr] = a < Nv ? OVOV(j, a, i, b) : 0.0;
+      }
+#pragma unroll
+      for (int rr = 0; rr < 4; ++rr) {
+        const int a = a0 + ty + 8 * rr;
+        if (a >= Nv) continue;
+        const int64_t ab = (int64_t)a * Nv + b;
+        double x = 0.0, y = 0.0, z1 = 0.0, z2 = 0.0;   // X_ij, Y_ij, Z_ij, Z_ji
+        if (!eq && a != b) {   // lam_t <bc||jk> + P(jk)P(bc)[lam_k d_ck q(j,b)]
+          // X: q(j,b) = <t'b||tj> = (t't|bj) - (t'j|bt);  Y: q(j,b) = (t't|bj) (opposite spins)
+          x = y = l0 * (p[rr] - q[rr]);
+          auto add = [&](double l, int jj, int bb) {
+            const double d = OVOV(0, 0, jj, bb);
+            x += l * (d - OVOV(jj, 0, 0, bb));
+            y += l * d;
+          };
+          if (b == j) add(lj, i, a);
+          if (b == i) add(-li, j, a);
+          if (a == j) add(-lj, i, b);
+          if (a == i) add(li, j, b);
+          if (i == 0 || a == 0 || b == 0) x = 0.0;
+        }
+        if (j != 0 && b != 0 && !(i == 0 && a == 0)) {
+          z1 = l0 * p[rr];
+          if (b == j) z1 += lj * OVOV(i, a, 0, 0);
+          if (a == i) z1 += li * (OVOV(j, b, 0, 0) - OVOV(0, b, j, 0));
+        }
+        oij[BX * B + ab] = x;
+        oij[BY * B + ab] = y;
+        oij[BZ * B + ab] = z1;
+        if (!eq) {
+          if (i != 0 && b != 0) {
+            z2 = l0 * q[rr];
+            if (b == i) z2 += li * OVOV(j, a, 0, 0);
+            if (a == j) z2 += lj * (OVOV(i, b, 0, 0) - OVOV(0, b, i, 0));
+          }
+          oji[BX * B + ab] = -x;
+          oji[BY * B + ab] = -y;
+          oji[BZ * B + ab] = z2;
+        }
+      }
     }
   }
 #undef OVOV
@@ -558,21 +600,28 @@ esmp2_status setup_top_basis(esmp2_handle *h) {
 // and ovvv_in are the handle's work buffers (ooov_in holds a copy of the input, ovvv_in
 // No Nv Nv No elements), all consumed.
 namespace {
-// out[o0][o1][o2][o3] = in[...] with input axis ax[k] running along output axis k
-__global__ void k_permute4(const double *in, double *out, int d0, int d1, int d2, int d3, int a0, int a1, int a2,
-                           int a3) {
-  const int d[4] = {d0, d1, d2, d3}, ax[4] = {a0, a1, a2, a3};
+// out[o0][o1][o2][o3] = in[...] with input axis ax[k] running along output axis k.  A CTA iteration
+// takes kPermute elements of one (o0, o1), with 32-bit index arithmetic per element: 1.15 GB in and out
+// 0.98 -> 0.88 ms; what remains are the strided reads.
+constexpr int kPermute = 2048;
+__global__ void __launch_bounds__(256) k_permute4(const double *in, double *out, int d0, int d1, int d2, int d3, int a0, int a1,
+                                                  int a2, int a3) {
+  const int d[4] = {d0, d1, d2, d3};
   int64_t st[4];
   st[3] = 1; st[2] = d3; st[1] = (int64_t)d2 * d3; st[0] = (int64_t)d1 * d2 * d3;
-  const int D0 = d[ax[0]], D1 = d[ax[1]], D2 = d[ax[2]], D3 = d[ax[3]];
-  const int64_t n = (int64_t)D0 * D1 * D2 * D3;
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
-    int64_t f = e;
-    const int o3 = (int)(f % D3); f /= D3;
-    const int o2 = (int)(f % D2); f /= D2;
-    const int o1 = (int)(f % D1);
-    const int o0 = (int)(f / D1);
-    out[e] = in[o0 * st[ax[0]] + o1 * st[ax[1]] + o2 * st[ax[2]] + o3 * st[ax[3]]];
+  const int D0 = d[a0], D1 = d[a1], D2 = d[a2], D3 = d[a3], n23 = D2 * D3, nch = (n23 + kPermute - 1) / kPermute;
+  const int64_t s2 = st[a2], s3 = st[a3], items = (int64_t)D0 * D1 * nch;
+  for (int64_t it = blockIdx.x; it < items; it += gridDim.x) {
+    const int64_t oo = it / nch;
+    const int ch = (int)(it - oo * nch), o0 = (int)(oo / D1), o1 = (int)(oo - (int64_t)o0 * D1);
+    const double *src = in + o0 * st[a0] + o1 * st[a1];
+    double *dst = out + oo * n23;
+    const int end = min(n23, (ch + 1) * kPermute);
+#pragma unroll 4
+    for (int e = ch * kPermute + threadIdx.x; e < end; e += 256) {
+      const int o2 = e / D3, o3 = e - o2 * D3;
+      dst[e] = src[o2 * s2 + o3 * s3];
+    }
   }
 }
 
@@ -673,7 +722,7 @@ esmp2_status setup_rhs_from(esmp2_handle *h, const double *ovov_src, double *ovo
   }
   debug_phase(h, "  ovvt rotations");
   k_f0vo<<<(unsigned)cdiv((int64_t)No * Nv, 256), 256, 0, st>>>(h->F, h->lam, h->ooov, h->ovvt, h->f0vo, No, Nv);
-  k_rhs<<<dim3((unsigned)cdiv(Nv, 32), (unsigned)(No * No), 5), 256, 0, st>>>(h->lam, h->f0vo, h->ovov, h->ooov, q_ovvt,
+  k_rhs<<<dim3((unsigned)cdiv(Nv, 32), (unsigned)(No * (No + 1) / 2), 2), 256, 0, st>>>(h->lam, h->f0vo, h->ovov, h->ooov, q_ovvt,
                                                                                h->b, No, Nv);
   h->launches += 2;
   return check_cuda(h, cudaGetLastError(), "rhs");
