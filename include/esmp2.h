@@ -190,9 +190,9 @@ esmp2_status esmp2_rhs(esmp2_handle *h, double *b);
  * ESMP2_REDUCED_MINRES: preconditioned MINRES (Paige-Saunders) in float64 in that basis, for
  * operators that are not positive definite; restarted from x until the true residual meets tol.
  * Stops when the TRUE relative residual ||b + A x|| / ||b|| (fp64) <= tol.
- * (Mixed: intermediate true residuals far from tol take fewer exact digit levels and a
- * float32 coupling pass, accurate relative to their own size; the residual that stops
- * the solve, and that the energy reuses, is float64-accurate throughout.)
+ * (Mixed: intermediate true residuals far from tol take fewer exact digit levels, accurate
+ * relative to their own size; the residual that stops the solve, and that the energy reuses,
+ * is float64-accurate throughout.)
  * Errors: NOT_CONVERGED (maxit CG iterations in total), INDEFINITE, CUDA.
  * The solution stays on the device (esmp2_get_solution); a later solve warm-starts
  * from it. */
@@ -293,9 +293,9 @@ esmp2_status esmp2_kernel_times(esmp2_kernel_time *out);
  * another framework owns the whole device heap through its own caching allocator, and
  * latency-critical loops where a cudaMalloc/cudaFree pair would synchronise the device.
  * It calls no cudaMalloc, cudaFree or allocating library routine: its scratch (bf16 copies
- * of x and F, the fp32 accumulator, an error flag) is one file-scope device array of
- * ESMP2_NOALLOC_MAX_BYTES that every GPU loading this library holds until process exit.
- * The scratch needed is 256 + (2 Nv Nvp) + (2 S Nv Nvp) + (4 S Nv Nv) bytes (each term
+ * of x and F) is one file-scope device array of ESMP2_NOALLOC_MAX_BYTES that every GPU loading
+ * this library holds until process exit, its error flag a file-scope managed word per device.
+ * The limit counts 256 + (2 Nv Nvp) + (2 S Nv Nvp) + (4 S Nv Nv) bytes (each term
  * rounded up to 256, Nvp = Nv rounded up to 8); larger requests return
  * ESMP2_ERR_UNSUPPORTED without touching the device.
  * The first call on a device looks up the array's device address (cudaGetSymbolAddress)

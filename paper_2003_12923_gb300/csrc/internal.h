@@ -269,8 +269,8 @@ esmp2_status ensure_p64(esmp2_handle *h);
 esmp2_status virt_split(esmp2_handle *h, const double *x, double *y, double *p64, int sym, int levels, bool join = true);
 // float64 residual of the refinement on the independent slices (resid.cu)
 int residual_parts();
-esmp2_status sigma_sym_tail(esmp2_handle *h, const double *x, double *y, bool s_sym);
-esmp2_status sigma64_finish(esmp2_handle *h, const double *x, double *y, bool s_sym);
+esmp2_status sigma_sym_tail(esmp2_handle *h, const double *x, double *y, bool s_sym, cudaEvent_t after_inter = nullptr);
+esmp2_status sigma64_finish(esmp2_handle *h, const double *x, double *y, bool s_sym, cudaEvent_t after_inter = nullptr);
 esmp2_status residual_sym(esmp2_handle *h, const double *x, const double *b, double *r, int levels);
 int hyll_parts();
 void hylleraas_sym(esmp2_handle *h, const double *b, const double *x, const double *r);

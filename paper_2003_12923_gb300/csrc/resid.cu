@@ -528,9 +528,10 @@ esmp2_status residual_sym(esmp2_handle *h, const double *x, const double *b, dou
 // The last stage of the float64 sigma in the TOP basis (No <= 32): y from the products P64 with the
 // occupied sums folded in (T, X, Y; with s_sym also S) and the Z part already in y; the partials of
 // <x, y> over these blocks go to h->red (T, X, Y, Z and, with s_sym, S: residual_parts() in all).
-esmp2_status sigma_sym_tail(esmp2_handle *h, const double *x, double *y, bool s_sym) {
+esmp2_status sigma_sym_tail(esmp2_handle *h, const double *x, double *y, bool s_sym, cudaEvent_t after_inter) {
   RC c{};
   launch_intermediates64(h, h->F, 0, x);
+  if (after_inter) cudaEventRecord(after_inter, h->stream);
   fill(h, c, h->F, x);
   c.P = h->P64;
   c.yz = y + BZ * h->d.B;

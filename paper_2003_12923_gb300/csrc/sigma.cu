@@ -622,8 +622,8 @@ esmp2_status index_terms64(esmp2_handle *h, const double *F, const double *x, do
 
 // couplings, shift and masks after index_terms64 (TOP basis, No <= 32): the symmetric pass, and the
 // element-wise pass for an S without the spin-flip symmetry
-esmp2_status sigma64_finish(esmp2_handle *h, const double *x, double *y, bool s_sym) {
-  esmp2_status s = sigma_sym_tail(h, x, y, s_sym);
+esmp2_status sigma64_finish(esmp2_handle *h, const double *x, double *y, bool s_sym, cudaEvent_t after_inter) {
+  esmp2_status s = sigma_sym_tail(h, x, y, s_sym, after_inter);
   if (s || s_sym) return s;
   launch_couple_s(make_ctx<double>(h, h->F, 0), x, y, h->cp, h->stream);
   h->launches += 1;
@@ -646,8 +646,7 @@ esmp2_status profile64(esmp2_handle *h, const double *x, double *y, int reps, do
       cudaEventRecord(ev[3], h->stream);
       launch_couple64(h, h->F, 0, x, y);
     } else {
-      cudaEventRecord(ev[3], h->stream);   // the intermediates are part of the last stage
-      if (esmp2_status s = sigma64_finish(h, x, y, false)) return s;
+      if (esmp2_status s = sigma64_finish(h, x, y, false, ev[3])) return s;
     }
     cudaEventRecord(ev[4], h->stream);
     cudaEventSynchronize(ev[4]);
