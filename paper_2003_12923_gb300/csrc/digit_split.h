@@ -19,20 +19,22 @@ __device__ __forceinline__ double scale_i64(long long V, int e) {
   return __longlong_as_double((long long)bits);
 }
 
-// Digits of one element.  The magnitude is split, U = |Z| + sum_k 32 64^k over the lower P - 1 digits, so
-// that digit p >= 2 of |Z| is field - 32 and digit 1 the rest; the sign goes to every digit, so -v has
+// Digits of one element, W = 6 bits each (7 where few products are summed: bf16 holds them exactly).  The
+// magnitude is split, U = |Z| + sum_k 32 64^k over the lower P - 1 digits, so
+// that digit p >= 2 of |Z| is field - 32 and digit 1 the rest (64 and 128 for W = 7); the sign goes to every digit, so -v has
 // the negated digits and its products (with the dropped pairs of low weight) are exactly the
 // negated ones.  |Z| by shifts of the significand (round half up): float64 arithmetic would cost two
 // operations of its slow pipe.
-template <int P>
+template <int P, int W = 6>
 __device__ __forceinline__ long long digit_word(double v, int es) {
-  constexpr long long bias = (((1ll << (6 * (P - 1))) - 1) / 63) * 32;
+  constexpr long long bias = (((1ll << (W * (P - 1))) - 1) / ((1 << W) - 1)) * (1 << (W - 1));
   const unsigned long long u = (unsigned long long)__double_as_longlong(v);
   const int ef = (int)(u >> 52) & 0x7FF;
-  const int sh = 1075 - ef + es - 6 * P;   // >= 0 for every finite |v| < 2^(es - 1)
+  const int sh = 1075 - ef + es - W * P;   // >= 54 - W P for every finite |v| < 2^(es - 1)
   unsigned long long m = (u & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull;
   if (sh > 0) m = sh < 55 && ef != 0 ? ((m >> (sh - 1)) + 1) >> 1 : 0;
-  if (ef == 0x7FF) m = 1ull << (6 * P - 1);   // an infinity or NaN saturates
+  else if (W * P > 54) m <<= min(-sh, W * P - 54);
+  if (ef == 0x7FF) m = 1ull << (W * P - 1);   // an infinity or NaN saturates
   return (long long)m + bias;
 }
 // The signs of two elements as bf16 factors +-1.0, packed.
@@ -41,11 +43,13 @@ __device__ __forceinline__ uint32_t sign_pair(double v0, double v1) {
 }
 // Digit p (1-based) of two elements as packed bf16: 128 + field is the bf16 with the field in its low
 // mantissa bits, so one packed fused multiply-add gives sign (field - 32) (digit 1: sign field) exactly.
-template <int P>
+template <int P, int W = 6>
 __device__ __forceinline__ uint32_t digit_pair(long long U0, long long U1, uint32_t sg, int p) {
-  const int sh = 6 * (P - p);
-  const uint32_t w = (__byte_perm((uint32_t)(U0 >> sh), (uint32_t)(U1 >> sh), 0x5410) & 0x003F003Fu) | 0x43004300u;
-  const uint32_t c = (p == 1 ? 0xC300C300u : 0xC320C320u) ^ (sg & 0x80008000u);   // -128 or -160 times the sign
+  static_assert(W == 6 || W == 7, "a field fits the mantissa of 128 + field");
+  const int sh = W * (P - p);
+  const uint32_t w = (__byte_perm((uint32_t)(U0 >> sh), (uint32_t)(U1 >> sh), 0x5410) & (W == 6 ? 0x003F003Fu : 0x007F007Fu)) | 0x43004300u;
+  // -128, or -160 (W = 7: -192), times the sign
+  const uint32_t c = (p == 1 ? 0xC300C300u : W == 6 ? 0xC320C320u : 0xC340C340u) ^ (sg & 0x80008000u);
   uint32_t r;
   asm("fma.rn.bf16x2 %0, %1, %2, %3;" : "=r"(r) : "r"(w), "r"(sg), "r"(c));
   return r;
@@ -55,22 +59,23 @@ __device__ __forceinline__ uint32_t digit_pair(long long U0, long long U1, uint3
 // the last one, for NL <= 8: sum_l v[l] 64^(NL-1-l).  SMALL: every |v| < 2^22, so that the integer is
 // read off the bits of v + 1.5 2^23 (two full-rate operations; conversions run at an eighth of the rate);
 // else |v| < 2^23, converted.
-template <int NL, bool SMALL>
-__device__ __forceinline__ long long join_levels(const float (&v)[NL]) {
+template <int NL, bool SMALL, int W = 6, int NV = NL>
+__device__ __forceinline__ long long join_levels(const float (&v)[NV]) {
   constexpr uint32_t C = 0x4B400000u;   // bits of 1.5 2^23
   auto bits = [&](int l) -> uint32_t {
     return SMALL ? __float_as_uint(v[l] + 12582912.0f) : (uint32_t)__float2int_rn(v[l]);
   };
   auto pair = [&](int l) -> int {       // two levels fit 32 bits
-    return (int)(bits(l) * 64u + bits(l + 1) - (SMALL ? C * 65u : 0u));
+    return (int)(bits(l) * (1u << W) + bits(l + 1) - (SMALL ? C * ((1u << W) + 1u) : 0u));
   };
   long long V = pair(0);
 #pragma unroll
-  for (int l = 2; l + 1 < NL; l += 2) V = V * 4096 + pair(l);
-  if constexpr (NL & 1) V = V * 64 + (int)(bits(NL - 1) - (SMALL ? C : 0u));
+  for (int l = 2; l + 1 < NL; l += 2) V = V * (1 << (2 * W)) + pair(l);
+  if constexpr (NL & 1) V = V * (1 << W) + (int)(bits(NL - 1) - (SMALL ? C : 0u));
   return V;
 }
-// v / 64 rounded half away from zero (odd in v)
+// v / 64 and v / 128 rounded half away from zero (odd in v)
 __device__ __forceinline__ int round64(int v) { return (v + 31 + (v >= 0 ? 1 : 0)) >> 6; }
+__device__ __forceinline__ int round128(int v) { return (v + 63 + (v >= 0 ? 1 : 0)) >> 7; }
 
 }  // namespace esmp2

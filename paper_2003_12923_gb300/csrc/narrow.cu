@@ -5,7 +5,8 @@
 // Both have only No multiply-adds per element, too few to hide double-float arithmetic on the float32
 // pipes (13 operations per multiply-add bound them) and far too many for the float64 pipe.  Here the
 // operand is split into eight exact bf16 digit planes (digits.cu) on its way through shared memory,
-// tcgen05 forms the level sums (levels 2 .. 9, exact in fp32; 2^-48 of the row's largest element), and the levels are joined as integers
+// tcgen05 forms the level sums (levels 2 .. 9, exact in fp32; 2^-55 of the row's largest element for the
+// rotations, 2^-48 for OVVV), and the levels are joined as integers
 // and rounded once: one read and one write of HBM, no digit planes in memory.
 // No=30 Nv=400: the rotations of a solve 44 -> 14.6 ms against double-float arithmetic, the OVVV
 // contraction 27.4 -> 7.8 ms (and 2 ms for its row exponents); No=16 Nv=160 rotations 3.7 -> 1.2 ms.
@@ -57,10 +58,11 @@ struct Args {
 __device__ __forceinline__ uint32_t sw64(int r, int c) { return (uint32_t)(r * 64 + ((c ^ ((r >> 1) & 3)) << 4)); }
 
 // digits of eight consecutive K elements of one row, one 16-byte store per plane
+template <int W>
 __device__ __forceinline__ void store_digits(uint8_t *tile, int plane_bytes, int row, int c, const double (&v)[8], int e) {
   long long U[8];
 #pragma unroll
-  for (int k = 0; k < 8; ++k) U[k] = digit_word<P>(v[k], e);
+  for (int k = 0; k < 8; ++k) U[k] = digit_word<P, W>(v[k], e);
   uint32_t sg[4];
 #pragma unroll
   for (int k = 0; k < 4; ++k) sg[k] = sign_pair(v[2 * k], v[2 * k + 1]);
@@ -68,8 +70,8 @@ __device__ __forceinline__ void store_digits(uint8_t *tile, int plane_bytes, int
 #pragma unroll
   for (int p = 1; p <= P; ++p)
     *reinterpret_cast<uint4 *>(dst + (p - 1) * plane_bytes) =
-        make_uint4(digit_pair<P>(U[0], U[1], sg[0], p), digit_pair<P>(U[2], U[3], sg[1], p),
-                   digit_pair<P>(U[4], U[5], sg[2], p), digit_pair<P>(U[6], U[7], sg[3], p));
+        make_uint4(digit_pair<P, W>(U[0], U[1], sg[0], p), digit_pair<P, W>(U[2], U[3], sg[1], p),
+                   digit_pair<P, W>(U[4], U[5], sg[2], p), digit_pair<P, W>(U[6], U[7], sg[3], p));
 }
 __device__ __forceinline__ int hi_abs(double v) {   // high word of |v|; infinities and NaN do not take part in a scale
   const int h = __double2hiint(v) & 0x7FFFFFFF;
@@ -84,6 +86,9 @@ template <bool ROW, int BN, bool SMALL>
 __global__ void __launch_bounds__(NTHREADS, 1) k_narrow(const __grid_constant__ CUtensorMap tB, const __grid_constant__ Args g) {
   constexpr int B_PLANE = b_plane<BN>(), B_STAGE = P * B_PLANE, ACC = 256;   // TMEM columns per accumulator set
   constexpr bool HALF = !ROW && BN == 16;
+  // bits per digit: 7 for the occupied form (K <= 32: every level sum is below 2^20), so that the right
+  // factor, the same in every row, carries no truncation above 2^-55; the time is the same as with 6 bits
+  constexpr int W = ROW ? 6 : 7;
   constexpr int CW = HALF ? 8 : 16;   // conversion warps per chunk
   extern __shared__ uint8_t smem_raw[];
   uint8_t *sA = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -116,7 +121,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_narrow(const __grid_constant__ 
       double v[8];
 #pragma unroll
       for (int k = 0; k < 8; ++k) v[k] = (n < g.N && c * 8 + k < g.K) ? g.R[(c * 8 + k) * g.N + n] : 0.0;
-      store_digits(sB, B_PLANE, n, c, v, eR);
+      store_digits<W>(sB, B_PLANE, n, c, v, eR);
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
@@ -242,7 +247,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_narrow(const __grid_constant__ 
         // every warp waits for itself: a wait that runs out ends the conversion for good
         ok = __all_sync(0xffffffffu, mbar_wait(&a_empty[st], ph));
         if (!ok) break;
-        store_digits(sA + st * A_STAGE, A_PLANE, row, kg, w, e);
+        store_digits<W>(sA + st * A_STAGE, A_PLANE, row, kg, w, e);
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncwarp();
         if (lane == 0) mbar_arrive(&a_full[st]);
@@ -266,7 +271,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_narrow(const __grid_constant__ 
       tc_after();
       const int row = quarter * 32 + lane;
       const int64_t r = t * BM + row;
-      const int e = (ROW ? (r < g.rows ? __ldg(g.es + r / g.per) : 0) : exp_of(rexp[lt & 7][row])) + eR - 54;
+      const int e = (ROW ? (r < g.rows ? __ldg(g.es + r / g.per) : 0) : exp_of(rexp[lt & 7][row])) + eR - (W == 6 ? 54 : 56);
       const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(ab * ACC + chalf * (BN / 2));
       double *dst = nullptr;
       int64_t pitch = 1;
@@ -298,7 +303,9 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_narrow(const __grid_constant__ 
             keep(q[l][c]);
             f[l] = __uint_as_float(q[l][c]);
           }
-          const long long V = join_levels<P, SMALL>(f);
+          long long V;   // W = 7: in units of the level before the last one, to stay within 64 bits
+          if constexpr (W == 6) V = join_levels<P, SMALL>(f);
+          else V = join_levels<P - 1, SMALL, W, P>(f) + round128(__float2int_rn(f[P - 1]));
           const int n = chalf * (BN / 2) + c4 * 4 + c;
           if (dst && n < g.N) dst[n * pitch] = scale_i64(V, e);
         }
