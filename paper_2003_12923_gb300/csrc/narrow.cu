@@ -63,15 +63,18 @@ __device__ __forceinline__ void store_digits(uint8_t *tile, int plane_bytes, int
   long long U[8];
 #pragma unroll
   for (int k = 0; k < 8; ++k) U[k] = digit_word<P, W>(v[k], e);
-  uint32_t sg[4];
+  uint32_t sg[4], rg[4];
 #pragma unroll
-  for (int k = 0; k < 4; ++k) sg[k] = sign_pair(v[2 * k], v[2 * k + 1]);
+  for (int k = 0; k < 4; ++k) {
+    sg[k] = sign_pair(v[2 * k], v[2 * k + 1]);
+    rg[k] = range_pair(v[2 * k], v[2 * k + 1]);
+  }
   uint8_t *dst = tile + sw64(row, c);
 #pragma unroll
   for (int p = 1; p <= P; ++p)
     *reinterpret_cast<uint4 *>(dst + (p - 1) * plane_bytes) =
-        make_uint4(digit_pair<P, W>(U[0], U[1], sg[0], p), digit_pair<P, W>(U[2], U[3], sg[1], p),
-                   digit_pair<P, W>(U[4], U[5], sg[2], p), digit_pair<P, W>(U[6], U[7], sg[3], p));
+        make_uint4(digit_pair<P, W>(U[0], U[1], sg[0], rg[0], p), digit_pair<P, W>(U[2], U[3], sg[1], rg[1], p),
+                   digit_pair<P, W>(U[4], U[5], sg[2], rg[2], p), digit_pair<P, W>(U[6], U[7], sg[3], rg[3], p));
 }
 __device__ __forceinline__ int hi_abs(double v) {   // high word of |v|; infinities and NaN do not take part in a scale
   const int h = __double2hiint(v) & 0x7FFFFFFF;
