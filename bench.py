@@ -491,12 +491,12 @@ def family_roofline(name, kt, peaks, peak_src, fp64_peak, steps):
         out["kernel"] = ("vg::k_vgemm, bf16 (or tf32) operands, the packed inner sigma's virtual-index GEMM: achieved = "
                          "the method's flops 4 n_unique Nv per build"
                          if name == "contraction" else
-                         "k_virt, exact bf16 digit products (float64-accurate residual, energy, rotations): "
+                         "dg::k_levels, exact bf16 digit products (float64-accurate residual, energy, rotations): "
                          "achieved = the method's flops of each contraction once; achieved_executed = every "
                          "digit pair the tensor cores run")
     elif name == "coupling":
         out.update({"bound": "hbm", "unit": "GB/s", "peak": peaks["hbm_gbs"], "achieved": kt["alg_units"] / sec / 1e9,
-                    "kernel": "kp_couple_anti/s/z (packed float32 inner coupling pass) and k_couple (float64 true "
+                    "kernel": "kp_couple_anti/s/z (packed float32 inner coupling pass) and k_sym_pass (float64 true "
                               "residual): algorithmic bytes = one read of x and of the products, one write of y",
                     "peak_source": f"copy bandwidth, {peak_src} (MEASURED_PEAKS.json)"})
     elif name == "gemm64":
