@@ -130,7 +130,9 @@ typedef struct {
  * SVD of C, Householder completion of the virtual space; Sec. II.A), transforms F and
  * the integrals, builds the right-hand side b = Q H Psi0 on D+L and the diagonal.
  * Inputs are copied; the caller keeps ownership.  Stream: the default stream until
- * esmp2_set_stream().  Errors: INVALID_ARG, UNSUPPORTED, OOM, CUDA. */
+ * esmp2_set_stream().  Host F and C are searched for non-finite elements (INVALID_ARG), the integrals
+ * are not: a NaN or infinity there makes b, and what is solved from it, NaN.
+ * Errors: INVALID_ARG, UNSUPPORTED, OOM, CUDA. */
 esmp2_status esmp2_create(esmp2_handle **h, const esmp2_desc *d);
 void esmp2_destroy(esmp2_handle *h);
 const char *esmp2_last_error(const esmp2_handle *h);

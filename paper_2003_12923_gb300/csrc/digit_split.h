@@ -4,7 +4,10 @@
 
 namespace esmp2 {
 
-// V 2^e as float64, V rounded to 53 bits; integer operations only
+// A joined sum that has no value (a NaN or infinity among the operands); sums stay above -2^63.
+constexpr long long kNoValue = (long long)(1ull << 63);
+
+// V 2^e as float64, V rounded to 53 bits (NaN for kNoValue); integer operations only
 __device__ __forceinline__ double scale_i64(long long V, int e) {
   if (V == 0) return 0.0;
   unsigned long long u = V < 0 ? 0ull - (unsigned long long)V : (unsigned long long)V;
@@ -16,6 +19,7 @@ __device__ __forceinline__ double scale_i64(long long V, int e) {
   if (eb <= 0) bits = 0;
   if (eb >= 2047) bits = 0x7FF0000000000000ull;
   if (V < 0) bits |= 0x8000000000000000ull;
+  if (V == kNoValue) bits = 0x7FF8000000000000ull;
   return __longlong_as_double((long long)bits);
 }
 
@@ -41,13 +45,20 @@ __device__ __forceinline__ long long digit_word(double v, int es) {
   unsigned long long m = (u & 0xFFFFFFFFFFFFFull) | 0x10000000000000ull;
   if (sh > 0) m = sh < 55 && ef != 0 ? ((m >> (sh - 1)) + 1) >> 1 : 0;
   else if (W * P > 54) m <<= min(-sh, W * P - 54);
-  if (ef == 0x7FF) m = 1ull << (W * P - 1);   // an infinity or NaN saturates
   return (long long)m + bias;
 }
-// The signs of two elements as bf16 factors +-1.0, packed.
+__device__ __forceinline__ bool non_finite(double v) { return (~(uint32_t)__double2hiint(v) & 0x7FF00000u) == 0; }
+// The signs of two elements as bf16 factors +-1.0, packed.  For a NaN or infinity the factor is NaN: all its
+// digits become NaN, the tensor cores carry it into every level sum of its row (or, in the right factor,
+// column), and no_value finds it there, so that such an element spoils the results that depend on it
+// and never passes for a number.  (It takes no part in a scale: k_slice_exp, hi_abs.)
 __device__ __forceinline__ uint32_t sign_pair(double v0, double v1) {
-  return (((uint32_t)__double2hiint(v0) >> 16) & 0x8000u) | ((uint32_t)__double2hiint(v1) & 0x80000000u) | 0x3F803F80u;
+  uint32_t s = (((uint32_t)__double2hiint(v0) >> 16) & 0x8000u) | ((uint32_t)__double2hiint(v1) & 0x80000000u) | 0x3F803F80u;
+  if (non_finite(v0)) s |= 0x7FC0u;
+  if (non_finite(v1)) s |= 0x7FC00000u;
+  return s;
 }
+__device__ __forceinline__ bool no_value(float leading_sum) { return leading_sum != leading_sum; }
 // The ranges of two elements, packed as the difference of their constants in digit_pair.
 __device__ __forceinline__ uint32_t range_pair(double v0, double v1) { return digit_range(v0) | (digit_range(v1) << 16); }
 // Digit p (1-based) of two elements as packed bf16: 128 + field is the bf16 with the field in its low

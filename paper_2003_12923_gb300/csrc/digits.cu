@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           for (int l = 0; l < NI; ++l) f[l] = __uint_as_float(r[l][c]);
           long long v = join_levels<NI, SMALL>(f);
           if constexpr (NLEV > 8) v += round64(__float2int_rn(__uint_as_float(r[8][c])));
-          V[c8 * 8 + c] = v;
+          V[c8 * 8 + c] = no_value(f[0]) ? kNoValue : v;
         }
       }
       tc_before();
@@ -258,11 +258,14 @@ __global__ void __launch_bounds__(NTHREADS, 1)
 }
 
 // ---------------------------------------------------------------------------- digit splits
-// Exponent of one Nv x Nv matrix, element (r, c) at r ld + c cs (one CTA).
+// Exponent of one Nv x Nv matrix, element (r, c) at r ld + c cs (one CTA); infinities and NaN do not take part.
 __global__ void k_mat_exp(const double *x, int n, int64_t ld, int64_t cs, int *es) {
   __shared__ double red[32];
   double m = 0.0;
-  for (int64_t e = threadIdx.x; e < (int64_t)n * n; e += blockDim.x) m = fmax(m, fabs(x[(e / n) * ld + (e % n) * cs]));
+  for (int64_t e = threadIdx.x; e < (int64_t)n * n; e += blockDim.x) {
+    const double v = x[(e / n) * ld + (e % n) * cs];
+    if (!non_finite(v)) m = fmax(m, fabs(v));
+  }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) m = fmax(m, __shfl_xor_sync(0xffffffffu, m, o));
   if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = m;
@@ -278,15 +281,20 @@ __global__ void k_mat_exp(const double *x, int n, int64_t ld, int64_t cs, int *e
     }
   }
 }
-// its P digit planes, out[p][r][c] with row pitch Nvp, pad columns zero
+// its P digit planes, out[p][r][c] with row pitch Nvp, pad columns zero; NaN digits for an infinity or NaN
 __global__ void k_mat_digits(const double *x, int n, int Nvp, int64_t ld, int64_t cs, const int *es, int P,
                              __nv_bfloat16 *out) {
   const int64_t plane = (int64_t)n * Nvp;
   const double scale = ldexp(1.0, 6 * P - *es);
   for (int r = blockIdx.x; r < n; r += gridDim.x) {
     for (int c = threadIdx.x; c < Nvp; c += blockDim.x) {
-      long long Z = c < n ? __double2ll_rn(x[r * ld + c * cs] * scale) : 0;
+      const double v = c < n ? x[r * ld + c * cs] : 0.0;
       __nv_bfloat16 *dst = out + (int64_t)r * Nvp + c;
+      if (non_finite(v)) {
+        for (int p = 0; p < P; ++p) dst[p * plane] = __ushort_as_bfloat16(0x7FFF);
+        continue;
+      }
+      long long Z = __double2ll_rn(v * scale);
       for (int p = P - 1; p > 0; --p) {   // least significant digit first
         const long long d = ((Z + 32) & 63) - 32;
         Z = (Z - d) >> 6;                 // exact: Z - d is a multiple of 64

@@ -309,6 +309,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_narrow(const __grid_constant__ 
           long long V;   // W = 7: in units of the level before the last one, to stay within 64 bits
           if constexpr (W == 6) V = join_levels<P, SMALL>(f);
           else V = join_levels<P - 1, SMALL, W, P>(f) + round128(__float2int_rn(f[P - 1]));
+          if (no_value(f[0])) V = kNoValue;
           const int n = chalf * (BN / 2) + c4 * 4 + c;
           if (dst && n < g.N) dst[n * pitch] = scale_i64(V, e);
         }
