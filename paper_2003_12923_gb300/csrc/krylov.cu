@@ -814,7 +814,7 @@ esmp2_status solve64(esmp2_handle *h, double tol, int maxit, esmp2_solve_info *i
   double rr = sl[1];
   int it = 0;
   esmp2_status result = ESMP2_ERR_NOT_CONVERGED;
-  double relres = bnorm > 0 ? std::sqrt(rr) / bnorm : 0.0;
+  double relres = bnorm != 0.0 ? std::sqrt(rr) / bnorm : 0.0;
   if (bnorm == 0.0) { result = ESMP2_OK; h->r_true = true; }
   while (result != ESMP2_OK && it < maxit) {
     if (std::sqrt(rr) <= tol * bnorm) {  // confirm with the true residual
@@ -975,7 +975,7 @@ esmp2_status solve_minres(esmp2_handle *h, double tol, int maxit, esmp2_solve_in
       bn = std::sqrt(sb[8]);
     }
     const double beta1 = std::sqrt(std::max(sl[8], 0.0));
-    relres = bn > 0 ? std::sqrt(std::max(sl[9], 0.0)) / bn : 0.0;
+    relres = bn != 0.0 ? std::sqrt(std::max(sl[9], 0.0)) / bn : 0.0;   // NaN stays NaN: not converged
     if (std::getenv("ESMP2_DEBUG"))
       std::fprintf(stderr, "esmp2 minres: restart %d relres %.3e iterations %d\n", restarts, relres, iters);
     if (relres <= tol) {
@@ -1172,7 +1172,8 @@ esmp2_status solve_mixed(esmp2_handle *h, double tol, int maxit, esmp2_solve_inf
     if ((s = read_slots(h, sl, 32))) return s;
     if (bb < 0.0) bb = sl[9];
     const double rn = std::sqrt(sl[8]), bn = std::sqrt(bb);
-    relres = bn > 0 ? rn / bn : 0.0;
+    relres = bn != 0.0 ? rn / bn : 0.0;
+    if (std::isnan(relres)) { h->err = "non-finite right-hand side or residual"; break; }
     if (std::getenv("ESMP2_DEBUG"))
       std::fprintf(stderr, "esmp2 refine: outer %d relres %.3e inner_total %d levels %d\n", outer, relres, inner_total, lv_k);
     if (relres <= 1e1 * tol && approx) { rho_next = 0.0; continue; }  // confirm at full accuracy
@@ -1299,7 +1300,7 @@ esmp2_status solve_mixed(esmp2_handle *h, double tol, int maxit, esmp2_solve_inf
     ++outer;
     if ((s = check_device_flag(h))) return s;
   }
-  if (result == ESMP2_ERR_NOT_CONVERGED && stalled < 3)
+  if (result == ESMP2_ERR_NOT_CONVERGED && stalled < 3 && !std::isnan(relres))
     h->err = "refinement did not reach the tolerance within maxit inner iterations";
   if (info) {
     info->iterations = inner_total;

@@ -35,6 +35,23 @@ def test_non_finite_integral_reaches_the_result(No, Nv, seed, block, idx, bad):
     h.close()
 
 
+@pytest.mark.parametrize("No,Nv,seed", SIZES)
+def test_non_finite_right_hand_side_is_not_converged(No, Nv, seed):
+    from paper_2003_12923_gb300 import esmp2
+    inst = dict(synth.make_instance(No, Nv, seed))
+    inst["ooov"] = inst["ooov"].copy()
+    inst["ooov"][1, 0, 2, 3] = math.nan
+    h = handle_for(inst)
+    precs = [esmp2.FP64, esmp2.MIXED_BF16]
+    if No <= 32:
+        precs += [esmp2.MIXED_TF32, esmp2.REDUCED_MIXED, esmp2.REDUCED_MINRES]
+    for prec in precs:
+        r = h.solve(tol=1e-8, maxit=20, precision=prec, raise_on_error=False)
+        assert r["status"] in (esmp2.ERR_INDEFINITE, esmp2.ERR_NOT_CONVERGED), (prec, r)
+        assert r["iterations"] <= 20 and not r["rel_residual"] <= 1e-8, (prec, r)
+    h.close()
+
+
 @pytest.mark.parametrize("bad", [math.nan, -math.inf])
 @pytest.mark.parametrize("No,Nv,seed", SIZES)
 def test_non_finite_vector_reaches_sigma(No, Nv, seed, bad):
