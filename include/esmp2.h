@@ -132,7 +132,7 @@ typedef struct {
  * Inputs are copied; the caller keeps ownership.  Stream: the default stream until
  * esmp2_set_stream().  Host F and C are searched for non-finite elements (INVALID_ARG), the integrals
  * are not: a NaN or infinity there makes b, and what is solved from it, NaN.
- * Errors: INVALID_ARG, UNSUPPORTED, OOM, CUDA. */
+ * Errors: INVALID_ARG, UNSUPPORTED, OOM, CUDA, TIMEOUT. */
 esmp2_status esmp2_create(esmp2_handle **h, const esmp2_desc *d);
 void esmp2_destroy(esmp2_handle *h);
 const char *esmp2_last_error(const esmp2_handle *h);
@@ -195,7 +195,7 @@ esmp2_status esmp2_rhs(esmp2_handle *h, double *b);
  * (Mixed: intermediate true residuals far from tol take fewer exact digit levels, accurate
  * relative to their own size; the residual that stops the solve, and that the energy reuses,
  * is float64-accurate throughout.)
- * Errors: NOT_CONVERGED (maxit CG iterations in total), INDEFINITE, CUDA.
+ * Errors: NOT_CONVERGED (maxit CG iterations in total), INDEFINITE, CUDA, TIMEOUT.
  * The solution stays on the device (esmp2_get_solution); a later solve warm-starts
  * from it. */
 esmp2_status esmp2_solve(esmp2_handle *h, double tol, int maxit, esmp2_precision p, esmp2_solve_info *info);
@@ -322,6 +322,14 @@ esmp2_status esmp2_virtual_contraction_noalloc(const double *x, const double *Fv
  * the scratch array of esmp2_virtual_contraction_noalloc (so it must not overlap such a call
  * on the GPU) and synchronises `stream` (a cudaStream_t, NULL = legacy default). */
 esmp2_status esmp2_selftest_bounded_wait(int wait_ms, void *stream);
+
+/* Self-test of the report of such a wait by the calls that work on a handle: raises the handle's
+ * error flag, as a wait that runs out does (in stream order, nothing is waited for).  The next call
+ * that depends on a kernel with bounded waits (the mixed, FP64_TC and MINRES solves,
+ * esmp2_get_solution of a solution held in another basis, esmp2_energy where it builds a sigma,
+ * low-precision esmp2_sigma for No <= 32) returns ESMP2_ERR_TIMEOUT and clears the flag.
+ * Errors: INVALID_ARG, OOM, CUDA. */
+esmp2_status esmp2_selftest_raise_timeout(esmp2_handle *h);
 
 #ifdef __cplusplus
 }

@@ -172,6 +172,7 @@ esmp2_status esmp2::create_impl(esmp2_handle **out, const esmp2_desc *d, cudaStr
   h->omega_op = h->omega - h->level_shift;
   debug_phase(h, "create: TOP basis");
   if (!s) s = setup_rhs_from(h, ovov_src, ovov_in, ooov_in, ovvv_src, ovvv_in, scratch);
+  if (!s) s = check_device_flag(h);   // the transforms' kernels have bounded waits
   if (h->ovvv_ready) {   // whatever happened above, the handle's stream is ordered after the copy
     cudaStreamWaitEvent(h->stream, h->ovvv_ready, 0);
     cudaEventDestroy(h->ovvv_ready);
@@ -297,6 +298,12 @@ esmp2_status esmp2_get_solution(esmp2_handle *h, double *x) {
       src = x;
     }
     if (esmp2_status s = rotate_occ(h, src, x, h->s64.p, false)) return s;
+    // a wait of the rotation that ran out leaves parts of x unwritten (while the stream is captured the
+    // flag waits for the next call that reads it)
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusActive;
+    if (cudaStreamIsCapturing(h->stream, &cap) != cudaSuccess) cudaGetLastError();
+    if (cap == cudaStreamCaptureStatusNone)
+      if (esmp2_status s = check_device_flag(h)) return s;
   }
   return check_cuda(h, cudaGetLastError(), "get_solution");
 }
@@ -314,6 +321,12 @@ esmp2_status esmp2_set_solution(esmp2_handle *h, const double *x) {
 esmp2_status esmp2_grad(esmp2_handle *h, double *dF, double *dOVOV, int adjoint_solve, double *adjoint_rel_diff) {
   if (!h) return ESMP2_ERR_INVALID_ARG;
   return gradient(h, dF, dOVOV, adjoint_solve, adjoint_rel_diff);
+}
+
+esmp2_status esmp2_selftest_raise_timeout(esmp2_handle *h) {
+  if (!h) return ESMP2_ERR_INVALID_ARG;
+  if (esmp2_status s = ensure_dflag(h)) return s;
+  return check_cuda(h, cudaMemsetAsync(h->dflag, 1, sizeof(int), h->stream), "device flag");
 }
 
 esmp2_status esmp2_energy(esmp2_handle *h, esmp2_energy_parts *parts) {

@@ -433,6 +433,7 @@ esmp2_status x_to_basis(esmp2_handle *h, int target) {
     if ((s = rotate_virt(h, x, x, tmp, true))) return s;
     h->x_basis = 2;
   }
+  if ((s = check_device_flag(h))) return s;
   return check_cuda(h, cudaGetLastError(), "x_to_basis");
 }
 

@@ -806,6 +806,8 @@ esmp2_status solve64(esmp2_handle *h, double tol, int maxit, esmp2_solve_info *i
     k_finalize<<<1, 1024, 0, st>>>(h->red, 5 * kRowCtas, 2, h->red_out, 0);
     h->launches += 4;
     if (esmp2_status s2 = read_slots(h, sl, 32)) return s2;
+    if (virt_tc && !zero)   // before this residual is taken for a converged one
+      if (esmp2_status s2 = check_device_flag(h)) return s2;
     if (bnorm < 0.0) bnorm = std::sqrt(sl[9]);
     return ESMP2_OK;
   };
@@ -907,6 +909,7 @@ esmp2_status energy(esmp2_handle *h, esmp2_energy_parts *parts) {
   }
   double sl[32];
   if ((s = read_slots(h, sl, 32))) return s;
+  if (!h->r_true && (s = check_device_flag(h))) return s;   // of the sigma build above
   double e_blk[5];
   for (int k = 0; k < 5; ++k) e_blk[k] = kWeights[k] * (2.0 * sl[8 + 2 * k] + sl[9 + 2 * k]);
   if (small_pairs) {
@@ -1170,6 +1173,7 @@ esmp2_status solve_mixed(esmp2_handle *h, double tol, int maxit, esmp2_solve_inf
     }
     if (!cold) ++nsig64;
     if ((s = read_slots(h, sl, 32))) return s;
+    if (!cold && (s = check_device_flag(h))) return s;   // the inner solve before it and this residual
     if (bb < 0.0) bb = sl[9];
     const double rn = std::sqrt(sl[8]), bn = std::sqrt(bb);
     relres = bn != 0.0 ? rn / bn : 0.0;
@@ -1283,7 +1287,10 @@ esmp2_status solve_mixed(esmp2_handle *h, double tol, int maxit, esmp2_solve_inf
       if (rn_in < 0.99 * best) { best = rn_in; since_best = 0; } else ++since_best;
       if (rn_in <= target || inner >= 200 || since_best >= 8) break;  // converged or stagnating
     }
-    if (result == ESMP2_ERR_INDEFINITE) break;
+    if (result == ESMP2_ERR_INDEFINITE) {
+      if ((s = check_device_flag(h))) return s;   // a wait that ran out, not the operator
+      break;
+    }
     if (std::getenv("ESMP2_DEBUG")) std::fprintf(stderr, "esmp2 refine:   inner %d  |r_in|/|r0| %.3e\n", inner, std::sqrt(sl[1]) / r0);
     rho_next = relres * std::max(r0 > 0 ? std::sqrt(sl[1]) / r0 : 0.0, 1e-4);
     if (packed) {
@@ -1298,7 +1305,6 @@ esmp2_status solve_mixed(esmp2_handle *h, double tol, int maxit, esmp2_solve_inf
     }
     h->x_zero = false;
     ++outer;
-    if ((s = check_device_flag(h))) return s;
   }
   if (result == ESMP2_ERR_NOT_CONVERGED && stalled < 3 && !std::isnan(relres))
     h->err = "refinement did not reach the tolerance within maxit inner iterations";

@@ -97,8 +97,8 @@ esmp2_status ensure_mixed(esmp2_handle *h, bool semi) {
   const int No = h->d.No, Nv = h->d.Nv, N = h->d.N, m = No - 1;
   const size_t n = (size_t)h->d.n;
   cudaError_t e = cudaSuccess;
-  auto A = [&](void **p, size_t bytes) {
-    if (e == cudaSuccess) e = dmalloc(p, bytes ? bytes : 1, h->stream);
+  auto A = [&](void **p, size_t bytes) {   // (kept from an earlier call that failed further on)
+    if (e == cudaSuccess && !*p) e = dmalloc(p, bytes ? bytes : 1, h->stream);
   };
   A(reinterpret_cast<void **>(&h->Rocc), sizeof(double) * No * No);
   A(reinterpret_cast<void **>(&h->Rocct), sizeof(double) * No * No);
@@ -153,9 +153,10 @@ esmp2_status ensure_mixed(esmp2_handle *h, bool semi) {
     std::vector<double> rows((size_t)No * N);
     e = cudaMemcpyAsync(rows.data(), h->Fsemi, sizeof(double) * rows.size(), cudaMemcpyDeviceToHost, h->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
-    if (e != cudaSuccess) {
+    s = e == cudaSuccess ? check_device_flag(h) : check_cuda(h, e, "mixed set-up");   // of the rotation of b
+    if (s) {
       dfree(V, h->stream); dfree(W2, h->stream); dfree(T1, h->stream);
-      return check_cuda(h, e, "mixed set-up");
+      return s;
     }
     for (int l = 0; l < 32; ++l) {
       h->arrow_w[l] = (l >= 1 && l < No) ? (float)rows[(size_t)l * N] : 0.f;
@@ -170,6 +171,7 @@ esmp2_status ensure_mixed(esmp2_handle *h, bool semi) {
 }
 
 esmp2_status check_device_flag(esmp2_handle *h) {
+  if (!h->dflag) return ESMP2_OK;   // no kernel with bounded waits has run
   int f = 0;
   cudaMemcpyAsync(&f, h->dflag, sizeof(int), cudaMemcpyDeviceToHost, h->stream);
   cudaError_t e = cudaStreamSynchronize(h->stream);

@@ -66,7 +66,8 @@ EXPORTS = ("esmp2_create", "esmp2_destroy", "esmp2_last_error", "esmp2_set_strea
            "esmp2_top_basis", "esmp2_sigma", "esmp2_rhs", "esmp2_solve", "esmp2_get_solution",
            "esmp2_set_solution", "esmp2_energy", "esmp2_kernel_launches", "esmp2_profile_sigma",
            "esmp2_virtual_contraction", "esmp2_virtual_contraction_noalloc", "esmp2_batch_solve", "esmp2_grad",
-           "esmp2_kernel_timing", "esmp2_kernel_times", "esmp2_selftest_bounded_wait")
+           "esmp2_kernel_timing", "esmp2_kernel_times", "esmp2_selftest_bounded_wait",
+           "esmp2_selftest_raise_timeout")
 MIXED_READY = True
 
 
@@ -127,6 +128,8 @@ def load(path: str | None = None):
         L.esmp2_kernel_times.argtypes = [ctypes.POINTER(KernelTime)]
         L.esmp2_selftest_bounded_wait.restype = I
         L.esmp2_selftest_bounded_wait.argtypes = [I, P]
+        L.esmp2_selftest_raise_timeout.restype = I
+        L.esmp2_selftest_raise_timeout.argtypes = [P]
         if path is None:
             _lib = L
         return L
@@ -316,6 +319,10 @@ class Handle:
         self._check(self.L.esmp2_grad(self._h, dF.ctypes.data, dov.ctypes.data, 1 if adjoint_solve else 0,
                                       ctypes.byref(diff)))
         return dF, dov, diff.value
+
+    def selftest_raise_timeout(self):
+        """Raise the handle's error flag as a bounded wait that ran out does (see include/esmp2.h)."""
+        self._check(self.L.esmp2_selftest_raise_timeout(self._h))
 
     @property
     def kernel_launches(self) -> int:
