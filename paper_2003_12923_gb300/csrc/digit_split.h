@@ -78,7 +78,8 @@ __device__ __forceinline__ uint32_t digit_pair(long long U0, long long U1, uint3
 // Integer-valued accumulators v[0 .. NL-1] (levels 2 .. NL + 1 of one element) joined at the weight of
 // the last one, for NL <= 8: sum_l v[l] 64^(NL-1-l).  SMALL: every |v| < 2^22, so that the integer is
 // read off the bits of v + 1.5 2^23 (two full-rate operations; conversions run at an eighth of the rate);
-// else |v| < 2^23, converted.
+// else |v| <= 2^24 (exact in fp32), converted.  Level l holds l + 1 digit products a step of K, so a pair
+// stays within K 2^(2W-2) ((l + 1) 2^W + l + 2) < 2^31 for W = 6, l <= 6, K <= 1820 and W = 7, l <= 4, K <= 480.
 template <int NL, bool SMALL, int W = 6, int NV = NL>
 __device__ __forceinline__ long long join_levels(const float (&v)[NV]) {
   constexpr uint32_t C = 0x4B400000u;   // bits of 1.5 2^23

@@ -527,12 +527,6 @@ bool split_supported(const esmp2_handle *h, int levels) {
   return 2LL * h->d.Nv * (levels - 1) * 1024 < (1LL << 24);
 }
 
-// binary exponents of n contiguous Nv x Nv slices
-void slice_exponents(esmp2_handle *h, const double *x, int n, int *es) {
-  dg::k_slice_exp<<<n, 256, 0, h->stream>>>(x, h->d.Nv * h->d.Nv, es, nullptr);
-  h->launches += 1;
-}
-
 // device error flag of the bounded waits
 esmp2_status ensure_dflag(esmp2_handle *h) {
   if (h->dflag) return ESMP2_OK;
@@ -669,12 +663,6 @@ esmp2_status xwm_split(esmp2_handle *h, const double *X, int64_t rows, double *Y
   g.err = h->dflag;
   const double fl = 2.0 * (double)rows * Nv * Nv;   // one float64-accurate rotation
   return run_digits(h, X, nullptr, S, S, *dig, g, levels, fl, fl);
-}
-
-// digit planes of W_v^T
-esmp2_status ensure_wv_digits(esmp2_handle *h) {
-  if (esmp2_status s = ensure_split(h)) return s;
-  return ensure_matrix_digits(h, h->Wv, &h->Rdig, &h->eR, 1);
 }
 
 esmp2_status xwv_split(esmp2_handle *h, const double *X, int64_t rows, double *Y) {

@@ -286,10 +286,8 @@ esmp2_status sigma64_arrow(esmp2_handle *h, const double *x, double *y);
 void virt_arrow64(esmp2_handle *h, const double *x, double *y);
 esmp2_status rotate_occ(esmp2_handle *h, const double *in, double *out, double *tmp, bool to_semi);
 esmp2_status mode_product_small(esmp2_handle *h, const double *in, double *out, int64_t P, int K, int64_t Q, const double *R);
-esmp2_status rows_times_narrow(esmp2_handle *h, const double *in, double *out, int64_t M, int N, const void *dig, int eR);
-void slice_exponents(esmp2_handle *h, const double *x, int n, int *es);
+esmp2_status rows_times_narrow(esmp2_handle *h, const double *in, double *out, int64_t M, int N, const double *Mat);
 esmp2_status ensure_dflag(esmp2_handle *h);
-esmp2_status ensure_wv_digits(esmp2_handle *h);
 esmp2_status eigvecs_occ(esmp2_handle *h, double *Vt);
 void complement_basis(esmp2_handle *h, const double *W, int n, double *J0);
 inline int64_t cdiv(int64_t a, int64_t b) { return (a + b - 1) / b; }

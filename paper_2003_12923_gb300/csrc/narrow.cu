@@ -4,12 +4,14 @@
 //
 // Both have only No multiply-adds per element, too few to hide double-float arithmetic on the float32
 // pipes (13 operations per multiply-add bound them) and far too many for the float64 pipe.  Here the
-// operand is split into eight exact bf16 digit planes (digits.cu) on its way through shared memory,
-// tcgen05 forms the level sums (levels 2 .. 9, exact in fp32; 2^-55 of the row's largest element for the
-// rotations, 2^-48 for OVVV), and the levels are joined as integers
+// operand is split into eight exact bf16 digit planes of seven bits (digits.cu) on its way through shared
+// memory, tcgen05 forms the level sums (levels 2 .. 9, exact in fp32; 2^-55 of the row's largest element
+// times the right factor's), and the levels are joined as integers
 // and rounded once: one read and one write of HBM, no digit planes in memory.
 // No=30 Nv=400: the rotations of a solve 44 -> 14.6 ms against double-float arithmetic, the OVVV
-// contraction 27.4 -> 7.8 ms (and 2 ms for its row exponents); No=16 Nv=160 rotations 3.7 -> 1.2 ms.
+// contraction 27.4 -> 10.9 ms, 2 of them for its row exponents (10.3 ms with six-bit digits and one scale
+// per Nv x Nv slice, which lost a row's last bits by as much as it was smaller than its slice: an element
+// 2^-30 of it kept 11 bits); No=16 Nv=160 rotations 3.7 -> 1.2 ms.
 //
 // A tile is 128 result rows; persistent CTAs of 28 warps:
 //   warps 0, 1   MMA issuer; TMA of the right factor's digit chunks (OVVV form)
@@ -35,6 +37,11 @@ using namespace ptx;
 
 constexpr int P = 8;                    // digit planes of both operands
 constexpr int BM = 128, BK = 32;
+// Longest sum over K of one launch: every level sum stays below 2^24 (8 pairs x 2^12 x 480) and the joined
+// integer below 2^63 (480 / 4 x 2^56).  The OVVV product of a larger Nv runs in K ranges of equal length,
+// added in float64.
+constexpr int K_MAX = 480;
+constexpr int W = 7;                    // bits per digit
 constexpr int A_PLANE = BM * 64, A_STAGE = P * A_PLANE;   // 64 KB
 // result columns of a tile, 32 or 16 (No <= 16)
 template <int BN> constexpr int b_plane() { return BN * 64; }
@@ -45,11 +52,12 @@ struct Args {
   const double *in;
   double *out;
   int64_t rows, tiles;
-  int K, N, nk;
+  int K, N, nk;      // K: length of the sum of this launch
   int64_t Q;         // occupied form: row c = p Q + q reads in[(p K + k) Q + q], writes out[(p N + n) Q + q]
   const double *R;   // occupied form: right factor, K x N row-major
-  const int *es;     // OVVV form: binary exponents, row r belongs to slice r / per
-  int per, eR;
+  const int *es;     // OVVV form: binary exponent of every row, ...
+  const int *eR;     // ... that of the right factor,
+  int ld, k0, add;   // ... row pitch, first K element, and whether out is added to
   int vec;           // OVVV form: 16-byte loads
   int *err;
 };
@@ -57,9 +65,8 @@ struct Args {
 // byte offset of 16-byte group c of row r in a K-major tile of 64-byte rows, 64-byte swizzle
 __device__ __forceinline__ uint32_t sw64(int r, int c) { return (uint32_t)(r * 64 + ((c ^ ((r >> 1) & 3)) << 4)); }
 
-// digits of eight consecutive K elements of one row, one 16-byte store per plane
-template <int W>
-__device__ __forceinline__ void store_digits(uint8_t *tile, int plane_bytes, int row, int c, const double (&v)[8], int e) {
+// digits of eight consecutive K elements of one row, 16 bytes per plane, to dst + (p - 1) pitch
+__device__ __forceinline__ void put_digits(uint8_t *dst, int64_t pitch, const double (&v)[8], int e) {
   long long U[8];
 #pragma unroll
   for (int k = 0; k < 8; ++k) U[k] = digit_word<P, W>(v[k], e);
@@ -69,12 +76,14 @@ __device__ __forceinline__ void store_digits(uint8_t *tile, int plane_bytes, int
     sg[k] = sign_pair(v[2 * k], v[2 * k + 1]);
     rg[k] = range_pair(v[2 * k], v[2 * k + 1]);
   }
-  uint8_t *dst = tile + sw64(row, c);
 #pragma unroll
   for (int p = 1; p <= P; ++p)
-    *reinterpret_cast<uint4 *>(dst + (p - 1) * plane_bytes) =
+    *reinterpret_cast<uint4 *>(dst + (p - 1) * pitch) =
         make_uint4(digit_pair<P, W>(U[0], U[1], sg[0], rg[0], p), digit_pair<P, W>(U[2], U[3], sg[1], rg[1], p),
                    digit_pair<P, W>(U[4], U[5], sg[2], rg[2], p), digit_pair<P, W>(U[6], U[7], sg[3], rg[3], p));
+}
+__device__ __forceinline__ void store_digits(uint8_t *tile, int plane_bytes, int row, int c, const double (&v)[8], int e) {
+  put_digits(tile + sw64(row, c), plane_bytes, v, e);
 }
 __device__ __forceinline__ int hi_abs(double v) {   // high word of |v|; infinities and NaN do not take part in a scale
   const int h = __double2hiint(v) & 0x7FFFFFFF;
@@ -82,16 +91,52 @@ __device__ __forceinline__ int hi_abs(double v) {   // high word of |v|; infinit
 }
 __device__ __forceinline__ int exp_of(int hi) { return hi >> 20 ? (hi >> 20) - 1021 : 0; }   // as k_slice_exp
 
-// ROW: OVVV form; BN: result columns; SMALL: every level sum below 2^22.  A conversion thread takes
+// OVVV form: binary exponent of every row (length n, pitch n), a warp per row; as k_slice_exp, one row
+// at a time: the scale of the whole Nv x Nv slice would cost a small row the bits it is smaller by.
+// (No=30 Nv=400: the pass over 15.4 GB takes as long as one over slices, 2 ms.)
+__global__ void __launch_bounds__(256) k_row_exp(const double *x, int64_t rows, int n, int *es) {
+  const int lane = threadIdx.x & 31;
+  const int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+  if (r >= rows) return;
+  const double *src = x + r * n;
+  int m = 0;
+#pragma unroll 8
+  for (int c = lane; c < n; c += 32) m = max(m, hi_abs(src[c]));
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if (lane == 0) es[r] = exp_of(m);
+}
+
+// OVVV form: digit planes of the right factor, out[p][n][k] (row pitch Kp) from column n < N of M (K x ldM),
+// rows N .. bn and the pad columns zero; one CTA
+__global__ void __launch_bounds__(1024) k_factor_digits(const double *M, int ldM, int K, int N, int Kp, int bn,
+                                                        __nv_bfloat16 *out, int *eR) {
+  __shared__ int mx;
+  if (threadIdx.x == 0) mx = 0;
+  __syncthreads();
+  int m = 0;
+  for (int u = threadIdx.x; u < K * N; u += 1024) m = max(m, hi_abs(M[(int64_t)(u / N) * ldM + u % N]));
+  atomicMax(&mx, m);
+  __syncthreads();
+  const int e = exp_of(mx);
+  if (threadIdx.x == 0) *eR = e;
+  for (int u = threadIdx.x; u < bn * (Kp >> 3); u += 1024) {
+    const int n = u % bn, c = (u / bn) * 8;
+    double v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v[k] = (n < N && c + k < K) ? M[(int64_t)(c + k) * ldM + n] : 0.0;
+    put_digits(reinterpret_cast<uint8_t *>(out + (int64_t)n * Kp + c), (int64_t)bn * Kp * 2, v, e);
+  }
+}
+
+// ROW: OVVV form; BN: result columns.  A conversion thread takes
 // eight K elements of a row; the occupied form with BN = 16 has K <= 16 and half as many of these per
 // tile, so its two halves of the conversion warps take turns.
-template <bool ROW, int BN, bool SMALL>
+template <bool ROW, int BN>
 __global__ void __launch_bounds__(NTHREADS, 1) k_narrow(const __grid_constant__ CUtensorMap tB, const __grid_constant__ Args g) {
   constexpr int B_PLANE = b_plane<BN>(), B_STAGE = P * B_PLANE, ACC = 256;   // TMEM columns per accumulator set
   constexpr bool HALF = !ROW && BN == 16;
-  // bits per digit: 7 for the occupied form (K <= 32: every level sum is below 2^20), so that the right
-  // factor, the same in every row, carries no truncation above 2^-55; the time is the same as with 6 bits
-  constexpr int W = ROW ? 6 : 7;
+  constexpr bool SMALL = !ROW;   // occupied form (K <= 32): every level sum is below 2^20
   constexpr int CW = HALF ? 8 : 16;   // conversion warps per chunk
   extern __shared__ uint8_t smem_raw[];
   uint8_t *sA = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -111,8 +156,10 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_narrow(const __grid_constant__ 
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_base)), "r"(512) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
-  int eR = g.eR;
-  if constexpr (!ROW) {   // the right factor's digits, row n = column n of R, once per CTA
+  int eR = 0;
+  if constexpr (ROW) {
+    eR = __ldg(g.eR);
+  } else {   // the right factor's digits, row n = column n of R, once per CTA
     __syncthreads();
     int m = 0;
     for (int e = threadIdx.x; e < g.K * g.N; e += NTHREADS) m = max(m, hi_abs(g.R[e]));
@@ -124,7 +171,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_narrow(const __grid_constant__ 
       double v[8];
 #pragma unroll
       for (int k = 0; k < 8; ++k) v[k] = (n < g.N && c * 8 + k < g.K) ? g.R[(c * 8 + k) * g.N + n] : 0.0;
-      store_digits<W>(sB, B_PLANE, n, c, v, eR);
+      store_digits(sB, B_PLANE, n, c, v, eR);
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   }
@@ -182,7 +229,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_narrow(const __grid_constant__ 
           if (!mbar_wait(&a_empty[st], ph)) { ok = false; break; }
           mbar_expect_tx(&b_full[st], (uint32_t)B_STAGE);
 #pragma unroll
-          for (int p = 0; p < P; ++p) tma_3d(sB + st * B_STAGE + p * B_PLANE, &tB, &b_full[st], kc * BK, 0, p);
+          for (int p = 0; p < P; ++p) tma_3d(sB + st * B_STAGE + p * B_PLANE, &tB, &b_full[st], g.k0 + kc * BK, 0, p);
           st ^= 1;
           ph ^= (uint32_t)(st == 0);
         }
@@ -205,7 +252,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_narrow(const __grid_constant__ 
         for (int k = 0; k < 8; ++k) v[k] = (r < g.rows && kg * 8 + k < g.K) ? src[(int64_t)k * g.Q] : 0.0;
       } else {
         const int k0 = kc * BK + kg * 8;
-        const double *src = g.in + r * g.K + k0;
+        const double *src = g.in + r * g.ld + g.k0 + k0;
         if (g.vec) {
 #pragma unroll
           for (int k = 0; k < 8; k += 2) {
@@ -245,12 +292,12 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_narrow(const __grid_constant__ 
           if (kg == 0) rexp[slot][row] = m;
         } else {
           const int64_t r = t * BM + row;
-          e = r < g.rows ? __ldg(g.es + r / g.per) : 0;
+          e = r < g.rows ? __ldg(g.es + r) : 0;
         }
         // every warp waits for itself: a wait that runs out ends the conversion for good
         ok = __all_sync(0xffffffffu, mbar_wait(&a_empty[st], ph));
         if (!ok) break;
-        store_digits<W>(sA + st * A_STAGE, A_PLANE, row, kg, w, e);
+        store_digits(sA + st * A_STAGE, A_PLANE, row, kg, w, e);
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncwarp();
         if (lane == 0) mbar_arrive(&a_full[st]);
@@ -274,7 +321,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_narrow(const __grid_constant__ 
       tc_after();
       const int row = quarter * 32 + lane;
       const int64_t r = t * BM + row;
-      const int e = (ROW ? (r < g.rows ? __ldg(g.es + r / g.per) : 0) : exp_of(rexp[lt & 7][row])) + eR - (W == 6 ? 54 : 56);
+      const int e = (ROW ? (r < g.rows ? __ldg(g.es + r) : 0) : exp_of(rexp[lt & 7][row])) + eR - 56;
       const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(ab * ACC + chalf * (BN / 2));
       double *dst = nullptr;
       int64_t pitch = 1;
@@ -306,12 +353,14 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_narrow(const __grid_constant__ 
             keep(q[l][c]);
             f[l] = __uint_as_float(q[l][c]);
           }
-          long long V;   // W = 7: in units of the level before the last one, to stay within 64 bits
-          if constexpr (W == 6) V = join_levels<P, SMALL>(f);
-          else V = join_levels<P - 1, SMALL, W, P>(f) + round128(__float2int_rn(f[P - 1]));
+          // in units of the level before the last one, to stay within 64 bits
+          long long V = join_levels<P - 1, SMALL, W, P>(f) + round128(__float2int_rn(f[P - 1]));
           if (no_value(f[0])) V = kNoValue;
           const int n = chalf * (BN / 2) + c4 * 4 + c;
-          if (dst && n < g.N) dst[n * pitch] = scale_i64(V, e);
+          if (dst && n < g.N) {
+            const double v = scale_i64(V, e);
+            dst[n * pitch] = ROW && g.add ? dst[n * pitch] + v : v;
+          }
         }
       }
       __syncwarp();
@@ -326,11 +375,11 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_narrow(const __grid_constant__ 
   if (threadIdx.x == 0 && fail) atomicOr(g.err, 1);
 }
 
-template <bool ROW, int BN, bool SMALL>
+template <bool ROW, int BN>
 esmp2_status launch(esmp2_handle *h, const CUtensorMap &mB, nr::Args &g) {
   if (g.rows <= 0) return ESMP2_OK;
   constexpr int smem = smem_bytes<BN>();
-  if (cudaError_t e = smem_limit_once(reinterpret_cast<const void *>(k_narrow<ROW, BN, SMALL>), smem))
+  if (cudaError_t e = smem_limit_once(reinterpret_cast<const void *>(k_narrow<ROW, BN>), smem))
     return check_cuda(h, e, "k_narrow shared-memory limit");
   g.tiles = cdiv(g.rows, BM);
   g.nk = (g.K + BK - 1) / BK;
@@ -338,7 +387,7 @@ esmp2_status launch(esmp2_handle *h, const CUtensorMap &mB, nr::Args &g) {
   int dev = 0, sms = 148;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  k_narrow<ROW, BN, SMALL><<<(unsigned)std::min<int64_t>(g.tiles, sms), NTHREADS, smem, h->stream>>>(mB, g);
+  k_narrow<ROW, BN><<<(unsigned)std::min<int64_t>(g.tiles, sms), NTHREADS, smem, h->stream>>>(mB, g);
   h->launches += 1;
   return check_cuda(h, cudaGetLastError(), "k_narrow");
 }
@@ -355,7 +404,7 @@ esmp2_status mode_product_small(esmp2_handle *h, const double *in, double *out, 
     g.rows = P * Q;
     g.K = K; g.N = K; g.Q = Q;
     g.R = R;
-    return K <= 16 ? nr::launch<false, 16, true>(h, CUtensorMap{}, g) : nr::launch<false, 32, true>(h, CUtensorMap{}, g);
+    return K <= 16 ? nr::launch<false, 16>(h, CUtensorMap{}, g) : nr::launch<false, 32>(h, CUtensorMap{}, g);
   }
   Gemm64 g{};
   g.alpha = 1.0; g.beta = 0.0;
@@ -368,38 +417,48 @@ esmp2_status mode_product_small(esmp2_handle *h, const double *in, double *out, 
   return ESMP2_OK;
 }
 
-// out[m][n] = sum_k in[m][k] W[k][n], n < N <= 32, for M rows of length Nv (M a multiple of Nv): the first N
-// columns of the matrix whose transposed digit planes are `dig` (exponent eR).  in is read twice, for
-// the power-of-two scale of each Nv x Nv slice and for the product.
-esmp2_status rows_times_narrow(esmp2_handle *h, const double *in, double *out, int64_t M, int N, const void *dig, int eR) {
-  const int Nv = h->d.Nv, Nvp = (Nv + 7) & ~7;
+// out[m][n] = sum_k in[m][k] M[k][n], n < N <= 32, for M rows of length Nv: the first N columns of the
+// Nv x Nv matrix Mat.  in is read twice, for the power-of-two scale of each row and for the product.
+esmp2_status rows_times_narrow(esmp2_handle *h, const double *in, double *out, int64_t M, int N, const double *Mat) {
+  const int Nv = h->d.Nv, Nvp = (Nv + 7) & ~7, bn = N <= 16 ? 16 : 32;
   if (esmp2_status s = ensure_dflag(h)) return s;
-  int *es = nullptr;
-  cudaError_t e = dmalloc(reinterpret_cast<void **>(&es), sizeof(int) * (size_t)(M / Nv), h->stream);
-  if (e != cudaSuccess) return check_cuda(h, e, "slice exponents");
-  slice_exponents(h, in, (int)(M / Nv), es);
+  // the factor's digit planes, its exponent, the rows' exponents
+  const size_t dig_bytes = sizeof(__nv_bfloat16) * (size_t)nr::P * bn * Nvp;   // a multiple of 256
+  uint8_t *ws = nullptr;
+  cudaError_t e = dmalloc(reinterpret_cast<void **>(&ws), dig_bytes + sizeof(int) * (size_t)(M + 4), h->stream);
+  if (e != cudaSuccess) return check_cuda(h, e, "row exponents");
+  int *eR = reinterpret_cast<int *>(ws + dig_bytes), *es = eR + 4;
+  nr::k_factor_digits<<<1, 1024, 0, h->stream>>>(Mat, Nv, Nv, N, Nvp, bn, reinterpret_cast<__nv_bfloat16 *>(ws), eR);
+  nr::k_row_exp<<<(unsigned)cdiv(M, 8), 256, 0, h->stream>>>(in, M, Nv, es);
+  h->launches += 2;
   CUtensorMap mB;
-  const uint64_t dims[3] = {(uint64_t)Nvp, (uint64_t)Nv, (uint64_t)kDigitPlanes};
-  const uint64_t str[2] = {(uint64_t)Nvp * 2, (uint64_t)Nvp * Nv * 2};
-  const int bn = N <= 16 ? 16 : 32;
+  const uint64_t dims[3] = {(uint64_t)Nvp, (uint64_t)bn, (uint64_t)nr::P};
+  const uint64_t str[2] = {(uint64_t)Nvp * 2, (uint64_t)Nvp * bn * 2};
   const uint32_t box[3] = {nr::BK, (uint32_t)bn, 1};
-  if (!tma_map_bf16(&mB, dig, 3, dims, str, box, 64)) {
-    dfree(es, h->stream);
+  if (!tma_map_bf16(&mB, ws, 3, dims, str, box, 64)) {
+    dfree(ws, h->stream);
     h->err = "tensor map encoding failed";
     return ESMP2_ERR_CUDA;
   }
   nr::Args g{};
   g.in = in; g.out = out;
   g.rows = M;
-  g.K = Nv; g.N = N; g.Q = 1;
+  g.N = N; g.Q = 1;
   g.es = es;
-  g.per = Nv;
   g.eR = eR;
+  g.ld = Nv;
   g.vec = (Nv % 2) == 0 && reinterpret_cast<uintptr_t>(in) % 16 == 0;
-  const bool small = (int64_t)Nv * nr::P * 1024 < (1 << 22);
-  const esmp2_status s = bn == 16 ? (small ? nr::launch<true, 16, true>(h, mB, g) : nr::launch<true, 16, false>(h, mB, g))
-                                  : (small ? nr::launch<true, 32, true>(h, mB, g) : nr::launch<true, 32, false>(h, mB, g));
-  dfree(es, h->stream);
+  const int parts = (Nv + nr::K_MAX - 1) / nr::K_MAX;
+  const int kper = ((Nv + parts - 1) / parts + nr::BK - 1) / nr::BK * nr::BK;   // <= K_MAX, a multiple of BK
+  static_assert(nr::K_MAX % nr::BK == 0, "a K range ends on a chunk");
+  esmp2_status s = ESMP2_OK;
+  for (int k0 = 0; k0 < Nv && !s; k0 += kper) {
+    g.k0 = k0;
+    g.K = std::min(kper, Nv - k0);
+    g.add = k0 > 0;
+    s = bn == 16 ? nr::launch<true, 16>(h, mB, g) : nr::launch<true, 32>(h, mB, g);
+  }
+  dfree(ws, h->stream);
   return s;
 }
 

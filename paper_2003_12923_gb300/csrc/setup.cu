@@ -690,8 +690,7 @@ esmp2_status setup_rhs_from(esmp2_handle *h, const double *ovov_src, double *ovo
     if (h->ovvv_ready) cudaStreamWaitEvent(st, h->ovvv_ready, 0);   // host OVVV copied on a side stream
     int dims[4] = {No, Nv, Nv, Nv};
     if (No <= 32 && tc) {  // c -> u' (first No columns of Wv)
-      if ((s = ensure_wv_digits(h))) return s;
-      if ((s = rows_times_narrow(h, ovvv_src, scratch, (int64_t)No * Nv * Nv, No, h->Rdig, h->eR))) return s;
+      if ((s = rows_times_narrow(h, ovvv_src, scratch, (int64_t)No * Nv * Nv, No, h->Wv))) return s;
     } else {
       mode_product(ovvv_src, scratch, dims, 3, h->Wv, No, Nv, st);
     }
