@@ -489,11 +489,11 @@ esmp2_status residual_sym(esmp2_handle *h, const double *x, const double *b, dou
   const bool av = h->arrowv;
   const double *F = av ? h->Farr : h->Fsemi;
   double *q = h->s64.q;
-  esmp2_status s = ensure_p64(h);
-  if (!s) s = ensure_slist(h);
+  esmp2_status s = ensure_slist(h);
+  if (!s && !av) s = ensure_p64(h);   // the element-wise form has no products to hold
   if (s) return s;
   RC c{};
-  c.P = h->P64;
+  c.P = av ? x : h->P64;   // (av: not read)
   if (av) {
     virt_arrow_sums(h, x);
     c.rho = h->rho64;

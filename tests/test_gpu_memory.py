@@ -1,0 +1,42 @@
+"""Device memory a solve holds, from the counters of the device's memory pool."""
+import ctypes
+
+import pytest
+
+import synth
+from tests.gpu_util import handle_for
+
+pytestmark = pytest.mark.gpu
+
+
+class _Pool:
+    def __init__(self):
+        import torch
+        torch.cuda.synchronize()
+        try:
+            self.rt = ctypes.CDLL("libcudart.so.%s" % torch.version.cuda.split(".")[0])
+        except OSError:
+            self.rt = ctypes.CDLL("/usr/local/cuda/lib64/libcudart.so")
+        self.pool = ctypes.c_void_p()
+        assert self.rt.cudaDeviceGetDefaultMemPool(ctypes.byref(self.pool), torch.cuda.current_device()) == 0
+
+    def used(self):
+        import torch
+        torch.cuda.synchronize()
+        v = ctypes.c_uint64()
+        assert self.rt.cudaMemPoolGetAttribute(self.pool, 7, ctypes.byref(v)) == 0   # cudaMemPoolAttrUsedMemCurrent
+        return v.value
+
+
+def test_reduced_solve_holds_no_product_vector():
+    from paper_2003_12923_gb300 import esmp2
+    No, Nv = 8, 80
+    vec = 8 * 5 * No * No * Nv * Nv
+    h = handle_for(synth.make_instance(No, Nv, 1))
+    pool = _Pool()
+    h.solve(tol=1e-8, maxit=500, precision=esmp2.REDUCED_MIXED)
+    u = pool.used()
+    h.sigma(h.rhs(), esmp2.FP64)
+    # the float64 sigma is the first call to need the products, four blocks of a vector at least
+    assert pool.used() - u >= 0.79 * vec
+    h.close()
