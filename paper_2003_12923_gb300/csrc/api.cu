@@ -30,7 +30,7 @@ bool finite_host(const double *p, size_t n) {
 void free_handle(esmp2_handle *h) {
   void *ptrs[] = {h->C, h->U, h->lam, h->Wv, h->W, h->F, h->f0vo, h->scal, h->ovov, h->ooov, h->ovvt, h->b,
                   h->s64.x, h->s64.r, h->s64.p, h->s64.q, h->s64.w, h->cp.VX, h->cp.OX, h->cp.WZ, h->cp.OZ,
-                  h->cp.G, h->cp.H, h->cp.CYZ, h->cp.GP, h->cp.HP, h->P64, h->dinv64, h->F32, h->dinv32, h->cp32.VX, h->cp32.GP, h->cp32.WZ, h->cp32.HP,
+                  h->cp.G, h->cp.H, h->cp.CYZ, h->cp.GP, h->cp.HP, h->P64, h->F32, h->dinv32, h->cp32.VX, h->cp32.GP, h->cp32.WZ, h->cp32.HP,
                   h->cp32.OX, h->cp32.OZ, h->cp32.OC1, h->cp32.OC2, h->cp32.G, h->cp32.H, h->cp32.CYZ, h->red, h->red_out, h->xlp, h->Fvlp, h->ylp, h->r32, h->p32,
                   h->q32, h->x32, h->dflag, h->Rocc, h->Rocct, h->Fsemi, h->bsemi, h->cp.OC1, h->cp.OC2,
                   h->xdig, h->Fdig, h->es, h->slist, h->Rdig, h->pr, h->pp, h->pq, h->pd, h->pdinv, h->pop, h->pW, h->pop32, h->pW32, h->pRbf, h->pT1, h->pZ, h->pWR, h->pWRt, h->pLam, h->pOcc, h->pCode, h->pdot2, h->Rv, h->Rvt, h->Rvdig, h->Rvtdig, h->Farr, h->barr, h->F32arr, h->rho64, h->kap64, h->pRho, h->pKap, h->jB, h->jJ, h->jflag, h->mr_a, h->mr_b, h->mr_v,

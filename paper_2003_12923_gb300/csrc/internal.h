@@ -116,8 +116,8 @@ struct esmp2_handle {
   float arrow_w[64] = {};   // host copy of F32[l][0] (1 <= l < No) and F32[l][No] (l < No)
   double arrow_w64[64] = {}; // the same in float64
   __half *dinv32 = nullptr; // Jacobi preconditioner in that basis (n halves)
-  double *dinv64 = nullptr; // Jacobi preconditioner of the float64 solve (n)
-  double *P64 = nullptr;    // products of the virtual-index pass (float64 sigma workspace, n)
+  double *P64 = nullptr;    // products of the virtual-index pass (float64 sigma workspace, p64_blocks B)
+  int p64_blocks = 0;       // 4 (T, S, X, Y), with digit products also Z
   double *red = nullptr;    // reduction partials
   double *red_out = nullptr;// reduction results (device)
   double *hred = nullptr;   // pinned host copy of reduction results
@@ -265,7 +265,7 @@ int split_levels_for(double tol);
 bool split_supported(const esmp2_handle *h, int levels);
 esmp2_status ensure_split(esmp2_handle *h);
 esmp2_status ensure_slist(esmp2_handle *h);
-esmp2_status ensure_p64(esmp2_handle *h);
+esmp2_status ensure_p64(esmp2_handle *h, int blocks);
 esmp2_status virt_split(esmp2_handle *h, const double *x, double *y, double *p64, int sym, int levels, bool join = true);
 // float64 residual of the refinement on the independent slices (resid.cu)
 int residual_parts();

@@ -44,6 +44,27 @@ struct VCtx {
     if (blk >= BX) d += F[(int64_t)No * N + No] - F[0];
     return 1.0 / d;
   }
+  // 1 / diag(A) where A acts (dinv's masks), (F_aa + F_bb) - (F_ii + F_jj): the same rounding for every
+  // image of an amplitude
+  __device__ __forceinline__ double occ_part(int blk, int i, int j) const {
+    const double shift = F[(int64_t)No * N + No] - F[0];
+    return (F[(int64_t)i * N + i] + F[(int64_t)j * N + j]) + omega - (blk >= BX ? shift : 0.0);
+  }
+  __device__ __forceinline__ double dinv_sym(int blk, int i, int j, int a, int b, double occ) const {
+    bool zero = false;
+    if ((blk == BT || blk == BX || blk == BY) && (i == j || a == b)) zero = true;
+    if (blk == BX && (i == 0 || j == 0 || a == 0 || b == 0)) zero = true;
+    if (blk == BZ && (j == 0 || b == 0 || (i == 0 && a == 0))) zero = true;
+    return zero ? 0.0 : 1.0 / ((F[(int64_t)(No + a) * N + No + a] + F[(int64_t)(No + b) * N + No + b]) - occ);
+  }
+  __device__ __forceinline__ double dinv_sym(int64_t e) const {
+    int64_t f = e;
+    const int b = (int)(f % Nv); f /= Nv;
+    const int a = (int)(f % Nv); f /= Nv;
+    const int j = (int)(f % No); f /= No;
+    const int i = (int)(f % No), blk = (int)(f / No);
+    return dinv_sym(blk, i, j, a, b, occ_part(blk, i, j));
+  }
   __device__ __forceinline__ double w(int64_t e) const {
     const int blk = (int)(e / B);
     return blk == 1 ? 1.0 : (blk == 4 ? 2.0 : 0.5);
@@ -121,27 +142,18 @@ __global__ void __launch_bounds__(1024) k_finalize(const double *__restrict__ re
   }
 }
 
-// M^-1 = 1 / diag(A), zero on the slots that are not amplitudes; a CTA iteration per row (blk, i, j, a).
-// (F_aa + F_bb) - (F_ii + F_jj): the same rounding for every image of an amplitude.
+// M^-1 = 1 / diag(A), zero on the slots that are not amplitudes; a CTA iteration per row (blk, i, j, a)
 __global__ void __launch_bounds__(128) k_dinv64(VCtx c, double *dinv) {
-  const int No = c.No, Nv = c.Nv, N = c.N;
+  const int No = c.No, Nv = c.Nv;
   const int64_t rows = 5LL * No * No * Nv;
-  const double shift = c.F[(int64_t)No * N + No] - c.F[0];
   for (int64_t row = blockIdx.x; row < rows; row += gridDim.x) {
     int64_t f = row;
     const int a = (int)(f % Nv); f /= Nv;
     const int j = (int)(f % No); f /= No;
     const int i = (int)(f % No), blk = (int)(f / No);
-    const double occ = (c.F[(int64_t)i * N + i] + c.F[(int64_t)j * N + j]) + c.omega - (blk >= BX ? shift : 0.0);
-    const double fa = c.F[(int64_t)(No + a) * N + No + a];
+    const double occ = c.occ_part(blk, i, j);
     double *out = dinv + row * Nv;
-    for (int b = threadIdx.x; b < Nv; b += blockDim.x) {
-      bool zero = false;
-      if ((blk == BT || blk == BX || blk == BY) && (i == j || a == b)) zero = true;
-      if (blk == BX && (i == 0 || j == 0 || a == 0 || b == 0)) zero = true;
-      if (blk == BZ && (j == 0 || b == 0 || (i == 0 && a == 0))) zero = true;
-      out[b] = zero ? 0.0 : 1.0 / ((fa + c.F[(int64_t)(No + b) * N + No + b]) - occ);
-    }
+    for (int b = threadIdx.x; b < Nv; b += blockDim.x) out[b] = c.dinv_sym(blk, i, j, a, b, occ);
   }
 }
 
@@ -171,12 +183,14 @@ __device__ __forceinline__ double blk_weight(int blk) { return blk == 1 ? 1.0 : 
 
 // p = M^-1 r; partials <r, M^-1 r>_w, <r, r>_w.  Block by block, weights on the block sums; M^-1 is read
 // (8 bytes) instead of formed (an index decode and a float64 division, some 20 operations of the
-// float64 pipe per element: 72 us against 20 at No=8 Nv=80).
+// float64 pipe per element: 72 us against 20 at No=8 Nv=80).  STORED = false, here and below: formed after
+// all, in a solve that finds no room for one more vector.
+template <bool STORED>
 __global__ void k_pcg_start(VCtx c, const double *dinv, const double *r, double *p, double *red) {
   const int blk = blockIdx.y;
   double s0 = 0.0, s1 = 0.0;
   for (int64_t e = blk * c.B + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < (blk + 1) * c.B; e += (int64_t)gridDim.x * blockDim.x) {
-    const double ri = r[e], z = dinv[e] * ri;
+    const double ri = r[e], z = (STORED ? dinv[e] : c.dinv_sym(e)) * ri;
     p[e] = z;
     s0 = fma(ri, z, s0);
     s1 = fma(ri, ri, s1);
@@ -193,6 +207,7 @@ __global__ void k_dot_w(VCtx c, const double *u, const double *v_, double *red) 
 }
 
 // x += alpha p; r -= alpha q; partials <r,M^-1 r>, <r,r>
+template <bool STORED>
 __global__ void k_pcg_update(VCtx c, const double *slots, const double *dinv, double *x, double *r, const double *p,
                              const double *q, double *red) {
   const double alpha = slots[4];
@@ -200,7 +215,7 @@ __global__ void k_pcg_update(VCtx c, const double *slots, const double *dinv, do
   double s0 = 0.0, s1 = 0.0;
 #pragma unroll 2
   for (int64_t e = blk * c.B + blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < (blk + 1) * c.B; e += (int64_t)gridDim.x * blockDim.x) {
-    const double pe = p[e], qe = q[e], xe = x[e], re = r[e], de = dinv[e];
+    const double pe = p[e], qe = q[e], xe = x[e], re = r[e], de = STORED ? dinv[e] : c.dinv_sym(e);
     x[e] = fma(alpha, pe, xe);
     const double ri = fma(-alpha, qe, re);
     r[e] = ri;
@@ -212,10 +227,11 @@ __global__ void k_pcg_update(VCtx c, const double *slots, const double *dinv, do
 }
 
 // p = M^-1 r + beta p
+template <bool STORED>
 __global__ void k_pcg_p(VCtx c, const double *slots, const double *dinv, const double *r, double *p) {
   const double beta = slots[5];
   for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < 5 * c.B; e += (int64_t)gridDim.x * blockDim.x)
-    p[e] = fma(beta, p[e], dinv[e] * r[e]);
+    p[e] = fma(beta, p[e], (STORED ? dinv[e] : c.dinv_sym(e)) * r[e]);
 }
 
 // ---- low-precision inner PCG (vectors of type T, float64 reductions)
@@ -781,13 +797,25 @@ esmp2_status solve64(esmp2_handle *h, double tol, int maxit, esmp2_solve_info *i
   // every vector stays on the singlet symmetries bit for bit: x and the first residual are projected,
   // A keeps them (No <= 32; larger No takes the general sigma and projects p), and M^-1 has them
   const bool sym = h->d.No <= 32;
-  esmp2_status s = ESMP2_OK;
-  if (!h->dinv64) {
-    cudaError_t e = dmalloc(reinterpret_cast<void **>(&h->dinv64), sizeof(double) * (size_t)h->d.n, st);
-    if (e != cudaSuccess) return check_cuda(h, e, "preconditioner");
-    k_dinv64<<<2432, 128, 0, st>>>(c, h->dinv64);
+  // what the sigma builds need comes first, then M^-1 for the length of this solve if there is room for
+  // it (a vector; without it the kernels form M^-1 as they go)
+  esmp2_status s = ensure_p64(h, virt_tc ? 5 : 4);
+  if (!s) s = ensure_slist(h);
+  if (!s && virt_tc) s = ensure_split(h);
+  if (s) return s;
+  struct Scratch {
+    double *p = nullptr;
+    cudaStream_t st;
+    ~Scratch() { dfree(p, st); }
+  } minv{nullptr, st};
+  if (dmalloc(reinterpret_cast<void **>(&minv.p), sizeof(double) * (size_t)h->d.n, st) == cudaSuccess) {
+    k_dinv64<<<2432, 128, 0, st>>>(c, minv.p);
     h->launches += 1;
+  } else {
+    cudaGetLastError();
+    minv.p = nullptr;
   }
+  const double *dinv = minv.p;
   if (!h->x_zero) singlet_project(h, x);
   h->x_sym = true;
   int nsig = 0;
@@ -802,7 +830,7 @@ esmp2_status solve64(esmp2_handle *h, double tol, int maxit, esmp2_solve_info *i
     k_residual<<<dim3(kRowCtas, 5), kRedThreads, 0, st>>>(c, h->b, zero ? nullptr : q, r, h->red, bnorm < 0.0 ? 1 : 0);
     k_finalize<<<1, 1024, 0, st>>>(h->red, 5 * kRowCtas, 2, h->red_out, 3);
     singlet_project(h, r);
-    k_pcg_start<<<dim3(kRowCtas, 5), kRedThreads, 0, st>>>(c, h->dinv64, r, p, h->red);
+    (dinv ? k_pcg_start<true> : k_pcg_start<false>)<<<dim3(kRowCtas, 5), kRedThreads, 0, st>>>(c, dinv, r, p, h->red);
     k_finalize<<<1, 1024, 0, st>>>(h->red, 5 * kRowCtas, 2, h->red_out, 0);
     h->launches += 4;
     if (esmp2_status s2 = read_slots(h, sl, 32)) return s2;
@@ -836,9 +864,10 @@ esmp2_status solve64(esmp2_handle *h, double tol, int maxit, esmp2_solve_info *i
       k_finalize<<<1, 1024, 0, st>>>(h->red, kRedBlocks, 1, h->red_out, 1);
       h->launches += 2;
     }
-    k_pcg_update<<<dim3(kRowCtas, 5), kRedThreads, 0, st>>>(c, h->red_out, h->dinv64, x, r, p, q, h->red);
+    (dinv ? k_pcg_update<true> : k_pcg_update<false>)<<<dim3(kRowCtas, 5), kRedThreads, 0, st>>>(c, h->red_out, dinv, x, r, p, q,
+                                                                                             h->red);
     k_finalize<<<1, 1024, 0, st>>>(h->red, 5 * kRowCtas, 2, h->red_out, 2);
-    k_pcg_p<<<kRedBlocks, kRedThreads, 0, st>>>(c, h->red_out, h->dinv64, r, p);
+    (dinv ? k_pcg_p<true> : k_pcg_p<false>)<<<kRedBlocks, kRedThreads, 0, st>>>(c, h->red_out, dinv, r, p);
     h->launches += 3;
     if (!sym) antisym_project(h, p);
     if ((s = read_slots(h, sl, 32))) return s;

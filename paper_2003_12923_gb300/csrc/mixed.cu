@@ -229,7 +229,7 @@ esmp2_status virtual_contraction(esmp2_handle *h, const double *x, double *y, in
     return check_cuda(h, cudaGetLastError(), "virtual contraction");
   }
   if (mode == 2) {
-    esmp2_status s = ensure_p64(h);
+    esmp2_status s = ensure_p64(h, 5);
     if (!s) s = virt_split(h, x, y, h->P64, 0, kFp64TcLevels);
     if (!s) s = check_device_flag(h);
     return s ? s : check_cuda(h, cudaGetLastError(), "virtual contraction");

@@ -490,7 +490,7 @@ esmp2_status residual_sym(esmp2_handle *h, const double *x, const double *b, dou
   const double *F = av ? h->Farr : h->Fsemi;
   double *q = h->s64.q;
   esmp2_status s = ensure_slist(h);
-  if (!s && !av) s = ensure_p64(h);   // the element-wise form has no products to hold
+  if (!s && !av) s = ensure_p64(h, levels ? 5 : 4);   // the element-wise form has no products to hold
   if (s) return s;
   RC c{};
   c.P = av ? x : h->P64;   // (av: not read)

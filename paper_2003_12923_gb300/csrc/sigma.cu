@@ -599,7 +599,7 @@ esmp2_status index_terms64(esmp2_handle *h, const double *F, const double *x, do
                            cudaEvent_t mid = nullptr) {
   const int No = h->d.No, Nv = h->d.Nv, N = h->d.N;
   const bool fused = No <= 32;
-  esmp2_status s = ensure_p64(h);
+  esmp2_status s = ensure_p64(h, tc_levels ? 5 : 4);
   if (!s) s = ensure_slist(h);
   if (s) return s;
   s_sym = s_sym && fused;
@@ -854,10 +854,21 @@ esmp2_status virt64_sym(esmp2_handle *h, const double *F, const double *x, doubl
   return ESMP2_OK;
 }
 
-esmp2_status ensure_p64(esmp2_handle *h) {
-  if (h->P64) return ESMP2_OK;
-  cudaError_t e = dmalloc(reinterpret_cast<void **>(&h->P64), sizeof(double) * (size_t)h->d.n, h->stream);
+// products of at least `blocks` blocks: five, so that the buffer stays where it is for the life of the
+// handle (a caller may have captured a sigma), fewer only where there is no room
+esmp2_status ensure_p64(esmp2_handle *h, int blocks) {
+  if (h->P64 && h->p64_blocks >= blocks) return ESMP2_OK;
+  dfree(h->P64, h->stream);
+  cudaError_t e = cudaErrorMemoryAllocation;
+  int got = 5;
+  for (; e != cudaSuccess && got >= blocks; --got) {
+    h->P64 = nullptr;
+    e = dmalloc(reinterpret_cast<void **>(&h->P64), sizeof(double) * (size_t)got * h->d.B, h->stream);
+    if (e == cudaSuccess) break;
+    cudaGetLastError();
+  }
   if (e != cudaSuccess) h->P64 = nullptr;
+  h->p64_blocks = e == cudaSuccess ? got : 0;
   return e == cudaSuccess ? ESMP2_OK : check_cuda(h, e, "sigma64 workspace");
 }
 
@@ -888,7 +899,7 @@ esmp2_status sigma64_F(esmp2_handle *h, const double *F, int arrow, const double
     if (esmp2_status s = index_terms64(h, F, x, y, tc_levels, s_sym)) return s;
     if (h->d.No <= 32) return sigma64_finish(h, x, y, s_sym);
   } else {
-    if (esmp2_status s0 = ensure_p64(h)) return s0;
+    if (esmp2_status s0 = ensure_p64(h, tc_levels ? 5 : 4)) return s0;
     if (tc_levels) {
       esmp2_status s = virt_split(h, x, y, h->P64, s_sym ? 2 : 1, tc_levels);
       if (s) return s;
