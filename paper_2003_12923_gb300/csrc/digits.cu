@@ -471,9 +471,9 @@ const char *run_levels(esmp2_handle *h, const double *x, const int *jobs, int np
   const int64_t plane = (int64_t)njobs * Nv * Nvp;
   __nv_bfloat16 *xd = static_cast<__nv_bfloat16 *>(h->xdig);
   const int vec = (Nv % 2) == 0 && reinterpret_cast<uintptr_t>(x) % 16 == 0;
-  dg::k_digits<NLEV><<<1216, 256, 0, h->stream>>>(x, Nv, Nvp, h->es, jobs, nplain, plane, xd, vec);
+  dg::k_digits<NLEV><<<1216, 256, 0, h->stream>>>(x, Nv, Nvp, g.es, jobs, nplain, plane, xd, vec);
   if (njobs > nplain) {
-    dg::k_digits_t<NLEV><<<1216, 256, 0, h->stream>>>(x, Nv, Nvp, h->es, jobs, nplain, njobs, plane, xd);
+    dg::k_digits_t<NLEV><<<1216, 256, 0, h->stream>>>(x, Nv, Nvp, g.es, jobs, nplain, njobs, plane, xd);
     h->launches += 1;
   }
   KScope ks(h->stream, ESMP2_KT_DIGITS, alg, exec);
@@ -485,30 +485,54 @@ esmp2_status run_digits(esmp2_handle *h, const double *x, const int *jobs, int n
                         int levels, double alg, double per_pair) {
   const int Nvp = (g.Nv + 7) & ~7;
   levels = std::max(levels, 5);   // fewer levels than five would gain nothing
-  const size_t need = sizeof(__nv_bfloat16) * (size_t)(levels - 1) * njobs * g.Nv * Nvp;
-  if (need > h->xdig_bytes) {     // stream-ordered: the old planes are released after their last use
-    // the first contraction of a block vector takes room for nine levels of it, so that the growing
-    // level counts of a refinement do not allocate again
-    const size_t room = jobs ? std::max(need, sizeof(__nv_bfloat16) * (size_t)8 * njobs * g.Nv * Nvp) : need;
+  const size_t plane = sizeof(__nv_bfloat16) * (size_t)g.Nv * Nvp;   // one digit plane of a slice
+  const size_t one = plane * (levels - 1), need = one * njobs;
+  if (need > h->xdig_bytes && !h->xdig_final) {   // stream-ordered: the old planes are released after their last use
+    // The transforms of the set-up take what they need.  The first call on a whole block vector takes nine
+    // planes of the job list of sym = 1, and that stays: a caller may have captured what works on it.
+    // Calls that need more, or all of them where there was less room, work in passes.
+    const int NN = h->d.No * h->d.No;
+    h->xdig_final = jobs || njobs > NN;
+    size_t room = h->xdig_final ? plane * kDigitPlanes * h->njobs[1] : need;
+    const size_t least = plane * kDigitPlanes;
     dfree(h->xdig, h->stream);
     h->xdig = nullptr;
     h->xdig_bytes = 0;
     cudaError_t e = dmalloc(&h->xdig, room, h->stream);
-    if (e != cudaSuccess) { h->xdig = nullptr; return check_cuda(h, e, "digit planes"); }
+    while (e != cudaSuccess && room > least) {
+      cudaGetLastError();
+      e = dmalloc(&h->xdig, room = std::max(least, room / 2), h->stream);
+    }
+    if (e != cudaSuccess) {
+      h->xdig = nullptr;
+      h->xdig_final = false;
+      return check_cuda(h, e, "digit planes");
+    }
     h->xdig_bytes = room;
   }
-  g.R = (int64_t)njobs * g.Nv;
+  const int per = (int)std::min<size_t>(njobs, h->xdig_bytes / one);   // jobs of one pass
   g.vec2 = (g.Nv % 2) == 0 && (reinterpret_cast<uintptr_t>(g.y) | reinterpret_cast<uintptr_t>(g.P)) % 16 == 0;
-  g.jobs = jobs;
-  const double exec = 0.5 * levels * (levels - 1) * per_pair;
   const char *m = nullptr;
-  switch (levels) {
-    case 5: m = run_levels<4>(h, x, jobs, nplain, njobs, Fd, g, alg, exec); break;
-    case 6: m = run_levels<5>(h, x, jobs, nplain, njobs, Fd, g, alg, exec); break;
-    case 7: m = run_levels<6>(h, x, jobs, nplain, njobs, Fd, g, alg, exec); break;
-    case 8: m = run_levels<7>(h, x, jobs, nplain, njobs, Fd, g, alg, exec); break;
-    case 9: m = run_levels<8>(h, x, jobs, nplain, njobs, Fd, g, alg, exec); break;
-    default: m = run_levels<9>(h, x, jobs, nplain, njobs, Fd, g, alg, exec); break;
+  double *const y0 = g.y;
+  const int *const es0 = g.es;
+  for (int j0 = 0; j0 < njobs && !m; j0 += per) {
+    const int nj = std::min(per, njobs - j0), np = std::max(0, std::min(nj, nplain - j0));
+    const double part = (double)nj / njobs, a = part * alg, e = part * 0.5 * levels * (levels - 1) * per_pair;
+    const int *jl = jobs ? jobs + j0 : nullptr;
+    g.R = (int64_t)nj * g.Nv;
+    g.jobs = jl;
+    const int64_t off = jobs ? 0 : (int64_t)j0 * g.Nv * g.Nv;   // without a list, job k of the pass is slice k
+    const double *xp = x + off;
+    g.y = y0 + off;
+    g.es = es0 + (jobs ? 0 : j0);
+    switch (levels) {
+      case 5: m = run_levels<4>(h, xp, jl, np, nj, Fd, g, a, e); break;
+      case 6: m = run_levels<5>(h, xp, jl, np, nj, Fd, g, a, e); break;
+      case 7: m = run_levels<6>(h, xp, jl, np, nj, Fd, g, a, e); break;
+      case 8: m = run_levels<7>(h, xp, jl, np, nj, Fd, g, a, e); break;
+      case 9: m = run_levels<8>(h, xp, jl, np, nj, Fd, g, a, e); break;
+      default: m = run_levels<9>(h, xp, jl, np, nj, Fd, g, a, e); break;
+    }
   }
   if (m) { h->err = m; return ESMP2_ERR_CUDA; }
   return check_cuda(h, cudaGetLastError(), "digit levels");

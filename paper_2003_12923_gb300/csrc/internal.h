@@ -171,6 +171,7 @@ struct esmp2_handle {
   // float64-accurate virtual-index terms from exact bf16 digit products (tcgen05)
   void *xdig = nullptr;     // digit planes of the stacked rows [levels-1][jobs][Nv][Nvp] bf16
   size_t xdig_bytes = 0;
+  bool xdig_final = false;  // sized for whole block vectors: stays where it is
   void *Fdig = nullptr;     // digit planes of F_vv [levels-1][Nv][Nvp] bf16
   int *es = nullptr;        // per-slice exponents (5 No^2) and that of F_vv (last entry)
   int *slist = nullptr;     // slices of the symmetric form (T, X, Y with i < j; all S, Z)

@@ -90,3 +90,29 @@ def test_float64_solve_without_room_for_its_preconditioner():
     torch.cuda.empty_cache()
     assert torch.equal(h.solution(), x)
     h.close()
+
+
+def test_digit_products_in_passes_where_the_planes_find_no_room():
+    import torch
+    from paper_2003_12923_gb300 import esmp2
+    No, Nv = 12, 160
+    vec = 8 * 5 * No * No * Nv * Nv
+    inst = synth.make_instance(No, Nv, 1)
+    h = handle_for(inst)
+    x = h.rhs()
+    ref = h.sigma(x, esmp2.FP64_TC)
+    h.solve(tol=1e-8, maxit=500, precision=esmp2.REDUCED_MIXED)
+    sol = h.solution()   # rotated back by products without a job list
+    h.close()
+    h = handle_for(inst)
+    pool = _Pool()
+    y = torch.empty_like(x)
+    hog = pool.leave(1.6 * vec)   # the products' vector and less than a quarter of the planes
+    h.sigma(x, esmp2.FP64_TC, out=y)
+    torch.cuda.synchronize()
+    del hog
+    torch.cuda.empty_cache()
+    assert torch.equal(y, ref)    # sums of integers: the same whatever the passes
+    h.solve(tol=1e-8, maxit=500, precision=esmp2.REDUCED_MIXED)
+    assert torch.equal(h.solution(), sol)
+    h.close()
