@@ -296,7 +296,8 @@ esmp2_status esmp2_kernel_times(esmp2_kernel_time *out);
  * latency-critical loops where a cudaMalloc/cudaFree pair would synchronise the device.
  * It calls no cudaMalloc, cudaFree or allocating library routine: its scratch (bf16 copies
  * of x and F) is one file-scope device array of ESMP2_NOALLOC_MAX_BYTES that every GPU loading
- * this library holds until process exit, its error flag a file-scope managed word per device.
+ * this library holds until process exit, its error flag a file-scope managed word per device, which
+ * the host reads and writes while other streams may run (concurrent managed access, as on GB300).
  * The limit counts 256 + (2 Nv Nvp) + (2 S Nv Nvp) + (4 S Nv Nv) bytes (each term
  * rounded up to 256, Nvp = Nv rounded up to 8); larger requests return
  * ESMP2_ERR_UNSUPPORTED without touching the device.

@@ -247,7 +247,7 @@ esmp2_status ensure_vrot(esmp2_handle *h, bool exact) {
     A(reinterpret_cast<void **>(&h->jflag), sizeof(unsigned) * 4);
     if (e != cudaSuccess) return check_cuda(h, e, "virtual rotation buffers");
     if (m >= 1) {
-      // B = Jt A from the complement of t' next to the input orbitals (2 sweeps to 1e-2 at No=30
+      // B = Jt A from the complement of t' next to the input orbitals (3 sweeps to 1e-2 at No=30
       // Nv=400 from there, 8 from the identity in the TOP basis)
       complement_basis(h, h->Wv, Nv, h->jJ);
       Gemm64 g{};
@@ -309,7 +309,7 @@ esmp2_status ensure_vrot(esmp2_handle *h, bool exact) {
     }
     // a sweep whose rotations were all below the target: 1e-14 (none rotated) for the exact
     // basis; for the preconditioner every pair of rows orthogonal to 1e-2 (the inner iteration
-    // count at No=30 Nv=400 is the same as with 1e-6, and the sweeps fall from 9 to 8)
+    // count at No=30 Nv=400 is the same as with 1e-6)
     const float target = exact ? 0.f : 1e-4f;
     bool done = false;
     int sweeps = 0;

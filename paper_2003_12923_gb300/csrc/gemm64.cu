@@ -10,10 +10,10 @@
 //     same scheduler;
 //   * too few tiles for the chip and a long K: K is cut into slices of at least 64 with their own
 //     CTAs, the partial results are summed in a fixed order by a second kernel.
-// Measured at start / now (64 x 64 x 16 tiles padded in M, N and K; no K slices): one-body densities
-// of No=12 Nv=120 1948 / 7.2 ms
-// (20 launches, half of the tiles by symmetry); float64 sigma of No=6 Nv=30 0.90 / 0.14 ms (21 GEMM
-// launches of one under-filled wave each, now one), of No=13 Nv=113 10.7 / 4.1 ms.
+// Measured against 64 x 64 x 16 tiles padded in M, N and K and no K slices: the GEMMs of a gradient of
+// No=12 Nv=120 1948 -> 3.8 ms (densities on half of the tiles by symmetry, each sum once); a float64 sigma
+// of No=6 Nv=30 0.90 -> 0.094 ms (21 launches of one under-filled wave each, now k_virt64 and the passes of
+// sigma.cu and resid.cu), of No=13 Nv=113 10.7 -> 3.65 ms.
 #include <algorithm>
 
 #include "internal.h"

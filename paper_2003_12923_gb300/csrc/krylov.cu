@@ -234,53 +234,6 @@ __global__ void k_pcg_p(VCtx c, const double *slots, const double *dinv, const d
     p[e] = fma(beta, p[e], (STORED ? dinv[e] : c.dinv_sym(e)) * r[e]);
 }
 
-// ---- low-precision inner PCG (vectors of type T, float64 reductions)
-// r = r64 (the fp64 outer residual); d = 0; p = M^-1 r; partials <r,M^-1 r>, <r,r>
-template <typename T>
-__global__ void kt_init(VCtx c, const double *r64, T *r, T *p, T *d, double *red) {
-  double v[2] = {0.0, 0.0};
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < 5 * c.B; e += (int64_t)gridDim.x * blockDim.x) {
-    const T ri = (T)r64[e];
-    const double z = c.dinv(e) * (double)ri, w = c.w(e);
-    r[e] = ri;
-    p[e] = (T)z;
-    d[e] = (T)0;
-    v[0] += w * (double)ri * z;
-    v[1] += w * (double)ri * (double)ri;
-  }
-  block_partials<2>(v, red);
-}
-
-template <typename T>
-__global__ void kt_dot(VCtx c, const T *u, const T *v_, double *red) {
-  double v[1] = {0.0};
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < 5 * c.B; e += (int64_t)gridDim.x * blockDim.x)
-    v[0] += c.w(e) * (double)u[e] * (double)v_[e];
-  block_partials<1>(v, red);
-}
-
-template <typename T>
-__global__ void kt_update(VCtx c, const double *slots, T *d, T *r, const T *p, const T *q, double *red) {
-  const double alpha = slots[4];
-  double v[2] = {0.0, 0.0};
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < 5 * c.B; e += (int64_t)gridDim.x * blockDim.x) {
-    d[e] = (T)((double)d[e] + alpha * (double)p[e]);
-    const double ri = (double)r[e] - alpha * (double)q[e];
-    r[e] = (T)ri;
-    const double w = c.w(e);
-    v[0] += w * ri * c.dinv(e) * ri;
-    v[1] += w * ri * ri;
-  }
-  block_partials<2>(v, red);
-}
-
-template <typename T>
-__global__ void kt_p(VCtx c, const double *slots, const T *r, T *p) {
-  const double beta = slots[5];
-  for (int64_t e = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; e < 5 * c.B; e += (int64_t)gridDim.x * blockDim.x)
-    p[e] = (T)(c.dinv(e) * (double)r[e] + beta * (double)p[e]);
-}
-
 // ---- float inner PCG: block-by-block streaming, float arithmetic, the Jacobi preconditioner
 // read from a half-precision vector (a fixed diagonal SPD preconditioner: rounding it only
 // perturbs the preconditioner), per-thread float partial sums combined in float64.  With

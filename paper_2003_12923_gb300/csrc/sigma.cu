@@ -9,9 +9,10 @@
 //      Table 1, and the mixed-spin L-triple cross terms), plus the constant shift
 //      -omega and the pair energy F_t't' - F_tt of the L-triples;
 //  (3) zeroing of slots that are not amplitudes (Pauli-forbidden or duplicated).
-// Part (1) runs as four float64 GEMM passes here (the mixed-precision path replaces
-// them with tcgen05 contractions), parts (2)-(3) as one element-wise pass fed by
-// small intermediates.
+// Part (1): the virtual-index terms of every listed slice in one launch (k_virt64, or digit
+// products on the tensor cores), the occupied-index terms in one pass from shared memory (k_occ64;
+// No > 32: two batched float64 GEMMs).  Parts (2)-(3): one element-wise pass fed by small intermediates,
+// on the independent amplitudes where the symmetries allow it (resid.cu).
 #include <algorithm>
 
 #include "internal.h"

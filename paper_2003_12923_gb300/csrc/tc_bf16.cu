@@ -608,8 +608,9 @@ void fvv_bf16(esmp2_handle *h, const double *F, void *dst) {
 // contraction: code that runs while another framework owns the whole device heap through
 // its own caching allocator (a cudaMalloc there fails or fragments that allocator's
 // budget), and latency-critical loops where a cudaMalloc/cudaFree pair would synchronise
-// the device.  For them the scratch (bf16 copies of x and F, the fp32 accumulator output
-// and an error flag) lives in one file-scope device array of ESMP2_NOALLOC_MAX_BYTES.
+// the device.  For them the scratch (bf16 copies of x and F) lives in one file-scope device array
+// of ESMP2_NOALLOC_MAX_BYTES.  The size limit of a request also counts a float32 product, which the
+// epilogue no longer writes: the limit is part of the call's contract.
 // Every GPU that loads this library holds that array until the process exits.
 namespace esmp2 {
 namespace {
@@ -621,6 +622,8 @@ unsigned char *g_noalloc_ptr[kMaxDevices] = {nullptr};
 
 // Error flag of the allocation-free contraction, one cache line per device.  Managed: the host clears
 // and reads it without a launch or a copy, and the kernel touches it only when a wait has run out.
+// The host may touch it while kernels of other streams run (cudaDevAttrConcurrentManagedAccess, which
+// every GB300 has).
 __managed__ int g_noalloc_flag[kMaxDevices][32];
 
 inline size_t align256(size_t v) { return (v + 255) & ~(size_t)255; }

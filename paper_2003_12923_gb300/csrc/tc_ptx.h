@@ -1,4 +1,4 @@
-// tcgen05 / TMA / mbarrier primitives of the digit-level kernel (inline PTX for sm_103a).
+// tcgen05 / TMA / mbarrier primitives of the digit-product kernels (digits.cu, narrow.cu; inline PTX for sm_103a).
 #pragma once
 #include <cuda.h>
 #include <cstdint>
