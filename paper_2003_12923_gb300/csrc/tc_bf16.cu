@@ -32,9 +32,12 @@
 #include <cstdlib>
 
 #include "internal.h"
+#include "tc_ptx.h"
 
 namespace esmp2 {
 namespace tc {
+
+using namespace ptx;
 
 constexpr int BM = 128;           // accumulator rows (TMEM lanes)
 constexpr int BN_MAX = 256;       // accumulator columns per tile
@@ -45,59 +48,6 @@ constexpr int B_BYTES = BN_MAX * BK * 2;      // 32 KB
 constexpr int STAGE_BYTES = A_BYTES + B_BYTES;
 constexpr int SMEM_BYTES = STAGES * STAGE_BYTES + 1024;
 constexpr int NTHREADS = 320;     // producer warp, MMA warp, 8 epilogue warps
-constexpr uint64_t WAIT_NS = 2000000000ull;   // 2 s per wait
-
-__device__ __forceinline__ uint32_t smem_u32(const void *p) {
-  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-__device__ __forceinline__ uint64_t gtimer() {
-  uint64_t t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-__device__ __forceinline__ void mbar_init(uint64_t *b, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(b)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint64_t *b, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(b)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint64_t *b) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(b)) : "memory");
-}
-__device__ __forceinline__ bool mbar_test(uint32_t addr, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-      : "=r"(ok)
-      : "r"(addr), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// Bounded wait: true when the phase of the given parity has completed.
-__device__ __forceinline__ bool mbar_wait(uint64_t *b, uint32_t parity, uint64_t limit = WAIT_NS) {
-  const uint32_t a = smem_u32(b);
-  if (mbar_test(a, parity)) return true;
-  const uint64_t t0 = gtimer();
-  while (!mbar_test(a, parity))
-    if (gtimer() - t0 > limit) return false;
-  return true;
-}
-__device__ __forceinline__ void tma_3d(void *dst, const CUtensorMap *m, uint64_t *bar, int x, int y, int z) {
-  asm volatile(
-      "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::
-          "r"(smem_u32(dst)),
-      "l"(reinterpret_cast<uint64_t>(m)), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar))
-      : "memory");
-}
-__device__ __forceinline__ void tma_2d(void *dst, const CUtensorMap *m, uint64_t *bar, int x, int y) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
-          smem_u32(dst)),
-      "l"(reinterpret_cast<uint64_t>(m)), "r"(x), "r"(y), "r"(smem_u32(bar))
-      : "memory");
-}
-__device__ __forceinline__ void tc_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
 // Shared-memory matrix descriptor (tcgen05): start >> 4, LBO >> 4 at bit 16, SBO >> 4 at
 // bit 32, descriptor version 1 at bit 46, layout type at bit 61 (2 = 128-byte swizzle).
@@ -110,16 +60,6 @@ __device__ __forceinline__ uint64_t sdesc(uint32_t addr, uint32_t lbo, uint32_t 
 __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N, int b_mn_major) {
   return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)b_mn_major << 16) | ((uint32_t)(N >> 3) << 17) |
          ((uint32_t)(M >> 4) << 24);
-}
-__device__ __forceinline__ void umma(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
-  asm volatile(
-      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d),
-      "l"(a), "l"(b), "r"(idesc), "r"(acc)
-      : "memory");
-}
-__device__ __forceinline__ void umma_commit(uint64_t *bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-               : "memory");
 }
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float (&v)[16]) {
   uint32_t r[16];
@@ -150,7 +90,7 @@ struct Args {
   int mirror;        // slices of T, X, Y (i < j listed) also write -y into slice (j, i)
   int No;
   int *err;          // error flag (device)
-  uint64_t wait_ns;  // limit of every mbarrier wait (0: WAIT_NS)
+  uint64_t wait_ns;  // limit of every mbarrier wait (0: kWaitNs)
   int no_copies;     // failure-detection self-test only: the producer issues no copies, so the
                      // first wait on a full slot runs out with nothing in flight
 };
@@ -188,7 +128,7 @@ __global__ void __launch_bounds__(NTHREADS, 1)
   // operands are complete from here on (returns at once for an ordinary launch)
   asm volatile("griddepcontrol.wait;" ::: "memory");
   const uint32_t tmem = tmem_base;
-  const uint64_t lim = g.wait_ns ? g.wait_ns : WAIT_NS;
+  const uint64_t lim = g.wait_ns ? g.wait_ns : kWaitNs;
   const int per_slice = g.a_tiles * g.b_tiles;
 
   if (warp == 0) {
@@ -258,9 +198,9 @@ __global__ void __launch_bounds__(NTHREADS, 1)
             const uint32_t A = smem_u32(smem + st * STAGE_BYTES), B = A + A_BYTES;
             for (int k = 0; k < ksteps; ++k) {
               if (term == 1)   // X_s[a][c] F[c][b]
-                umma(d, sdesc(A + 32 * k, 16, 1024), sdesc(B + 32 * k, 16, 1024), id2, first ? 0u : 1u);
+                umma_bf16(d, sdesc(A + 32 * k, 16, 1024), sdesc(B + 32 * k, 16, 1024), id2, first ? 0u : 1u);
               else             // F[a][c] X_s[c][b]
-                umma(d, sdesc(A + 32 * k, 16, 1024), sdesc(B + 2048 * k, BK * 128, 1024), id1, first ? 0u : 1u);
+                umma_bf16(d, sdesc(A + 32 * k, 16, 1024), sdesc(B + 2048 * k, BK * 128, 1024), id1, first ? 0u : 1u);
               first = false;
             }
             umma_commit(&empty[st]);

@@ -1,4 +1,4 @@
-// tcgen05 / TMA / mbarrier primitives of the digit-product kernels (digits.cu, narrow.cu; inline PTX for sm_103a).
+// tcgen05 / TMA / mbarrier primitives of the tensor-core kernels (inline PTX for sm_103a).
 #pragma once
 #include <cuda.h>
 #include <cstdint>
@@ -46,6 +46,13 @@ __device__ __forceinline__ void tma_3d(void *dst, const CUtensorMap *m, uint64_t
       "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];" ::
           "r"(smem_u32(dst)),
       "l"(reinterpret_cast<uint64_t>(m)), "r"(x), "r"(y), "r"(z), "r"(smem_u32(bar))
+      : "memory");
+}
+__device__ __forceinline__ void tma_2d(void *dst, const CUtensorMap *m, uint64_t *bar, int x, int y) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
+          smem_u32(dst)),
+      "l"(reinterpret_cast<uint64_t>(m)), "r"(x), "r"(y), "r"(smem_u32(bar))
       : "memory");
 }
 __device__ __forceinline__ void tc_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }

@@ -35,9 +35,12 @@
 #include <algorithm>
 
 #include "internal.h"
+#include "tc_ptx.h"
 
 namespace esmp2 {
 namespace vg {
+
+using namespace ptx;
 
 constexpr int BM = 128;                 // accumulator rows (TMEM lanes)
 constexpr int CHUNK_B = 64;             // bytes of one operand row per K chunk (the swizzle span)
@@ -54,61 +57,6 @@ constexpr int EPI_WARPS = 16, NTHREADS = 64 + 32 * EPI_WARPS;
 // dynamic shared memory per CTA: the 232448-byte opt-in limit less room for the kernel's
 // static shared memory (barriers, TMEM address, flags, the epilogue's 10 KB staging tile and 1 KB table)
 constexpr int SMEM_MAX = 232448 - 2048 - 11264;
-constexpr uint64_t WAIT_NS = 2000000000ull;
-
-__device__ __forceinline__ uint32_t smem_u32(const void *p) {
-  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-__device__ __forceinline__ uint64_t gtimer() {
-  uint64_t t;
-  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-  return t;
-}
-__device__ __forceinline__ void mbar_init(uint64_t *b, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(b)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(uint64_t *b, uint32_t bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_u32(b)), "r"(bytes) : "memory");
-}
-__device__ __forceinline__ void mbar_arrive(uint64_t *b) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(b)) : "memory");
-}
-__device__ __forceinline__ bool mbar_test(uint32_t addr, uint32_t parity) {
-  uint32_t ok;
-  asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}\n"
-      : "=r"(ok)
-      : "r"(addr), "r"(parity)
-      : "memory");
-  return ok != 0;
-}
-// bounded wait: true when the phase of the given parity has completed
-__device__ __forceinline__ bool mbar_wait(uint64_t *b, uint32_t parity, uint64_t limit = WAIT_NS) {
-  const uint32_t a = smem_u32(b);
-  if (mbar_test(a, parity)) return true;
-  const uint64_t t0 = gtimer();
-  while (!mbar_test(a, parity))
-    if (gtimer() - t0 > limit) return false;
-  return true;
-}
-__device__ __forceinline__ void tma_2d(void *dst, const CUtensorMap *m, uint64_t *bar, int x, int y) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::"r"(
-          smem_u32(dst)),
-      "l"(reinterpret_cast<uint64_t>(m)), "r"(x), "r"(y), "r"(smem_u32(bar))
-      : "memory");
-}
-__device__ __forceinline__ void tc_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
-__device__ __forceinline__ void tc_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
-
-// Shared-memory matrix descriptor (tcgen05), K-major operand with 64-byte swizzle: start >> 4,
-// leading byte offset 16 >> 4 (unused by swizzled K-major layouts), stride byte offset = one
-// group of 8 rows of 64 bytes (512 >> 4), descriptor version 1 at bit 46, layout type 4
-// (64-byte swizzle) at bit 61.
-__device__ __forceinline__ uint64_t sdesc64(uint32_t addr) {
-  return (uint64_t)((addr >> 4) & 0x3FFFu) | ((uint64_t)1 << 16) | ((uint64_t)(512 >> 4) << 32) | (1ull << 46) |
-         (4ull << 61);
-}
 // Instruction descriptor: D fp32 (bits 4-5 = 1); A and B format (bits 7-9, 10-12) bf16 = 1 of
 // kind::f16 or tf32 = 2 of kind::tf32; both K-major; N >> 3 at bit 17, M >> 4 at bit 24.
 template <bool TF32>
@@ -131,18 +79,6 @@ __device__ __forceinline__ void umma(uint32_t d, uint64_t a, uint64_t b, uint32_
         "l"(a), "l"(b), "r"(idesc), "r"(acc)
         : "memory");
 }
-__device__ __forceinline__ void umma_commit(uint64_t *bar) {
-  asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(smem_u32(bar))
-               : "memory");
-}
-// eight consecutive accumulator columns of the warp's 32 lanes; valid after tmem_wait and keep
-__device__ __forceinline__ void tmem_ld8(uint32_t taddr, uint32_t (&r)[8]) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7])
-               : "r"(taddr));
-}
-__device__ __forceinline__ void tmem_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
-__device__ __forceinline__ void keep(uint32_t &r) { asm volatile("" : "+r"(r)); }
 __device__ __forceinline__ float rcp_approx(float x) {
   float r;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
