@@ -4,10 +4,7 @@
 
 namespace esmp2 {
 
-// A joined sum that has no value (a NaN or infinity among the operands); sums stay above -2^63.
-constexpr long long kNoValue = (long long)(1ull << 63);
-
-// V 2^e as float64, V rounded to 53 bits (NaN for kNoValue); integer operations only
+// V 2^e as float64, V rounded to 53 bits; integer operations only
 __device__ __forceinline__ double scale_i64(long long V, int e) {
   if (V == 0) return 0.0;
   unsigned long long u = V < 0 ? 0ull - (unsigned long long)V : (unsigned long long)V;
@@ -19,8 +16,13 @@ __device__ __forceinline__ double scale_i64(long long V, int e) {
   if (eb <= 0) bits = 0;
   if (eb >= 2047) bits = 0x7FF0000000000000ull;
   if (V < 0) bits |= 0x8000000000000000ull;
-  if (V == kNoValue) bits = 0x7FF8000000000000ull;
   return __longlong_as_double((long long)bits);
+}
+
+// A joined sum that has no value (a NaN or infinity among the operands); sums stay above -2^63.
+constexpr long long kNoValue = (long long)(1ull << 63);
+__device__ __forceinline__ double scale_or_nan(long long V, int e) {
+  return V == kNoValue ? __longlong_as_double(0x7FF8000000000000ll) : scale_i64(V, e);
 }
 
 // Digits of one element, W = 6 bits each (7 where few products are summed: bf16 holds them exactly).  The
@@ -48,12 +50,16 @@ __device__ __forceinline__ long long digit_word(double v, int es) {
   return (long long)m + bias;
 }
 __device__ __forceinline__ bool non_finite(double v) { return (~(uint32_t)__double2hiint(v) & 0x7FF00000u) == 0; }
-// The signs of two elements as bf16 factors +-1.0, packed.  For a NaN or infinity the factor is NaN: all its
-// digits become NaN, the tensor cores carry it into every level sum of its row (or, in the right factor,
-// column), and no_value finds it there, so that such an element spoils the results that depend on it
-// and never passes for a number.  (It takes no part in a scale: k_slice_exp, hi_abs.)
+// The signs of two elements as bf16 factors +-1.0, packed.
 __device__ __forceinline__ uint32_t sign_pair(double v0, double v1) {
-  uint32_t s = (((uint32_t)__double2hiint(v0) >> 16) & 0x8000u) | ((uint32_t)__double2hiint(v1) & 0x80000000u) | 0x3F803F80u;
+  return (((uint32_t)__double2hiint(v0) >> 16) & 0x8000u) | ((uint32_t)__double2hiint(v1) & 0x80000000u) | 0x3F803F80u;
+}
+// The same with a NaN factor for a NaN or infinity: all its digits become NaN, the tensor cores carry it
+// into every level sum of its row (or, in the right factor, column), and no_value finds it there, so that
+// such an element spoils the results that depend on it and never passes for a number.  (It takes no
+// part in the scale of its slice, k_slice_exp: the other rows are what they would be without it.)
+__device__ __forceinline__ uint32_t sign_pair_nan(double v0, double v1) {
+  uint32_t s = sign_pair(v0, v1);
   if (non_finite(v0)) s |= 0x7FC0u;
   if (non_finite(v1)) s |= 0x7FC00000u;
   return s;

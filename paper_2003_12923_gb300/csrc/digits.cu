@@ -230,18 +230,18 @@ __global__ void __launch_bounds__(NTHREADS, 1)
           double *dst = g.P + off + a;
 #pragma unroll
           for (int c = 0; c < HC; ++c)
-            if (b0 + c < g.Nv) dst[(int64_t)(b0 + c) * g.Nv] = scale_i64(V[c], e);
+            if (b0 + c < g.Nv) dst[(int64_t)(b0 + c) * g.Nv] = scale_or_nan(V[c], e);
         } else {
           double *dst = (g.one[s / g.per_block] ? g.P : g.y) + off + (int64_t)a * g.Nv + b0;
           if (g.vec2) {
 #pragma unroll
             for (int c = 0; c < HC; c += 2)
               if (b0 + c < g.Nv)
-                *reinterpret_cast<double2 *>(dst + c) = make_double2(scale_i64(V[c], e), scale_i64(V[c + 1], e));
+                *reinterpret_cast<double2 *>(dst + c) = make_double2(scale_or_nan(V[c], e), scale_or_nan(V[c + 1], e));
           } else {
 #pragma unroll
             for (int c = 0; c < HC; ++c)
-              if (b0 + c < g.Nv) dst[c] = scale_i64(V[c], e);
+              if (b0 + c < g.Nv) dst[c] = scale_or_nan(V[c], e);
           }
         }
       }
@@ -352,7 +352,7 @@ __global__ void __launch_bounds__(256) k_digits(const double *x, int Nv, int Nvp
         if (c + 1 < Nv) v.y = src[c + 1];
       }
       const long long U0 = digit_word<P>(v.x, e), U1 = digit_word<P>(v.y, e);
-      const uint32_t sg = sign_pair(v.x, v.y), rg = range_pair(v.x, v.y);
+      const uint32_t sg = sign_pair_nan(v.x, v.y), rg = range_pair(v.x, v.y);
 #pragma unroll
       for (int p = 1; p <= P; ++p)
         *reinterpret_cast<uint32_t *>(dst + (p - 1) * plane + c) = digit_pair<P>(U0, U1, sg, rg, p);
@@ -380,7 +380,7 @@ __global__ void __launch_bounds__(256) k_digits_t(const double *x, int Nv, int N
     if (c0 + c >= Nvp) continue;
     for (int q = w; q < 32 && a0 + q < Nv; q += 8) {
       const long long U0 = digit_word<P>(t[c][q], e), U1 = digit_word<P>(t[c + 1][q], e);
-      const uint32_t sg = sign_pair(t[c][q], t[c + 1][q]), rg = range_pair(t[c][q], t[c + 1][q]);
+      const uint32_t sg = sign_pair_nan(t[c][q], t[c + 1][q]), rg = range_pair(t[c][q], t[c + 1][q]);
       __nv_bfloat16 *dst = out + ((int64_t)job * Nv + a0 + q) * Nvp + c0 + c;
 #pragma unroll
       for (int p = 1; p <= P; ++p)

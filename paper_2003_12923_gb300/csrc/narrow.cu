@@ -8,10 +8,10 @@
 // memory, tcgen05 forms the level sums (levels 2 .. 9, exact in fp32; 2^-55 of the row's largest element
 // times the right factor's), and the levels are joined as integers
 // and rounded once: one read and one write of HBM, no digit planes in memory.
-// No=30 Nv=400: the rotations of a solve 44 -> 14.6 ms against double-float arithmetic, the OVVV
-// contraction 27.4 -> 10.9 ms, 2 of them for its row exponents (10.3 ms with six-bit digits and one scale
-// per Nv x Nv slice, which lost a row's last bits by as much as it was smaller than its slice: an element
-// 2^-30 of it kept 11 bits); No=16 Nv=160 rotations 3.7 -> 1.2 ms.
+// No=30 Nv=400: the rotations of a solve 44 -> 16.2 ms against double-float arithmetic, the OVVV
+// contraction 27.4 -> 10.6 ms, 2.4 of them for its row exponents (10.3 ms with six-bit digits and one
+// scale per Nv x Nv slice, which lost a row's last bits by as much as it was smaller than its slice: an
+// element 2^-30 of it kept 11 bits); No=16 Nv=160 rotations 3.7 -> 1.4 ms.
 //
 // A tile is 128 result rows; persistent CTAs of 28 warps:
 //   warps 0, 1   MMA issuer; TMA of the right factor's digit chunks (OVVV form)
@@ -21,6 +21,10 @@
 // Digit p of the operand meets the digits 1 .. 9 - p of the right factor, stacked along N (their
 // levels are neighbouring accumulators): eight MMAs per K step instead of 36.  Two sets of
 // accumulators (2 x 8 levels x 32 columns fill TMEM): the epilogue of a tile runs beside the next one.
+//
+// A row with a NaN or infinity has the exponent field 0x7FF as its scale (kBadExp) and gets NaN results, so
+// does a column of the right factor with one.  Found once per row, not per element: with NaN digits and a
+// look at every result (as in digits.cu) the rotations of No=30 Nv=400 took 16.9 ms.
 #include <cuda.h>
 #include <cuda_bf16.h>
 
@@ -56,7 +60,7 @@ struct Args {
   int64_t Q;         // occupied form: row c = p Q + q reads in[(p K + k) Q + q], writes out[(p N + n) Q + q]
   const double *R;   // occupied form: right factor, K x N row-major
   const int *es;     // OVVV form: binary exponent of every row, ...
-  const int *eR;     // ... that of the right factor,
+  const int *eR;     // ... that of the right factor, a mask of its columns with a NaN or infinity,
   int ld, k0, add;   // ... row pitch, first K element, and whether out is added to
   int vec;           // OVVV form: 16-byte loads
   int *err;
@@ -85,15 +89,14 @@ __device__ __forceinline__ void put_digits(uint8_t *dst, int64_t pitch, const do
 __device__ __forceinline__ void store_digits(uint8_t *tile, int plane_bytes, int row, int c, const double (&v)[8], int e) {
   put_digits(tile + sw64(row, c), plane_bytes, v, e);
 }
-__device__ __forceinline__ int hi_abs(double v) {   // high word of |v|; infinities and NaN do not take part in a scale
-  const int h = __double2hiint(v) & 0x7FFFFFFF;
-  return h < 0x7FF00000 ? h : 0;
-}
-__device__ __forceinline__ int exp_of(int hi) { return hi >> 20 ? (hi >> 20) - 1021 : 0; }   // as k_slice_exp
+__device__ __forceinline__ int hi_abs(double v) { return __double2hiint(v) & 0x7FFFFFFF; }   // high word of |v|
+__device__ __forceinline__ int hi_finite(double v) { return non_finite(v) ? 0 : hi_abs(v); }
+// binary exponent of a row whose largest hi_abs is hi (as k_slice_exp; kBadExp: it is not finite)
+constexpr int kBadExp = 2047 - 1021;
+__device__ __forceinline__ int exp_of(int hi) { return hi >> 20 ? (hi >> 20) - 1021 : 0; }
 
-// OVVV form: binary exponent of every row (length n, pitch n), a warp per row; as k_slice_exp, one row
-// at a time: the scale of the whole Nv x Nv slice would cost a small row the bits it is smaller by.
-// (No=30 Nv=400: the pass over 15.4 GB takes as long as one over slices, 2 ms.)
+// OVVV form: binary exponent of every row (length n, pitch n), a warp per row.  The scale of the whole Nv x Nv slice would cost a small row the bits it is smaller by.
+// (No=30 Nv=400: the pass over 15.4 GB takes 2.4 ms, one CTA per slice took 2.0.)
 __global__ void __launch_bounds__(256) k_row_exp(const double *x, int64_t rows, int n, int *es) {
   const int lane = threadIdx.x & 31;
   const int64_t r = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
@@ -108,18 +111,23 @@ __global__ void __launch_bounds__(256) k_row_exp(const double *x, int64_t rows, 
 }
 
 // OVVV form: digit planes of the right factor, out[p][n][k] (row pitch Kp) from column n < N of M (K x ldM),
-// rows N .. bn and the pad columns zero; one CTA
+// rows N .. bn and the pad columns zero; eR: its exponent and the mask of its non-finite columns; one CTA
 __global__ void __launch_bounds__(1024) k_factor_digits(const double *M, int ldM, int K, int N, int Kp, int bn,
                                                         __nv_bfloat16 *out, int *eR) {
   __shared__ int mx;
-  if (threadIdx.x == 0) mx = 0;
+  __shared__ unsigned bad;
+  if (threadIdx.x == 0) { mx = 0; bad = 0; }
   __syncthreads();
   int m = 0;
-  for (int u = threadIdx.x; u < K * N; u += 1024) m = max(m, hi_abs(M[(int64_t)(u / N) * ldM + u % N]));
+  for (int u = threadIdx.x; u < K * N; u += 1024) {
+    const double v = M[(int64_t)(u / N) * ldM + u % N];
+    m = max(m, hi_finite(v));
+    if (non_finite(v)) atomicOr(&bad, 1u << (u % N));
+  }
   atomicMax(&mx, m);
   __syncthreads();
   const int e = exp_of(mx);
-  if (threadIdx.x == 0) *eR = e;
+  if (threadIdx.x == 0) { eR[0] = e; eR[1] = (int)bad; }
   for (int u = threadIdx.x; u < bn * (Kp >> 3); u += 1024) {
     const int n = u % bn, c = (u / bn) * 8;
     double v[8];
@@ -144,11 +152,13 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_narrow(const __grid_constant__ 
   __shared__ uint64_t a_full[2], a_empty[2], b_full[2], acc_full[2], acc_empty[2];
   __shared__ uint32_t tmem_base;
   __shared__ int fail, rmax, rexp[8][BM];
+  __shared__ unsigned rbad;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   if (threadIdx.x == 0) {
     for (int s = 0; s < 2; ++s) { mbar_init(&a_full[s], CW); mbar_init(&a_empty[s], 1); mbar_init(&b_full[s], 1); mbar_init(&acc_full[s], 1); mbar_init(&acc_empty[s], 8); }
     fail = 0;
     rmax = 0;
+    rbad = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   for (int k = threadIdx.x; k < 8 * BM; k += NTHREADS) (&rexp[0][0])[k] = 0;
@@ -162,7 +172,10 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_narrow(const __grid_constant__ 
   } else {   // the right factor's digits, row n = column n of R, once per CTA
     __syncthreads();
     int m = 0;
-    for (int e = threadIdx.x; e < g.K * g.N; e += NTHREADS) m = max(m, hi_abs(g.R[e]));
+    for (int e = threadIdx.x; e < g.K * g.N; e += NTHREADS) {
+      m = max(m, hi_finite(g.R[e]));
+      if (non_finite(g.R[e])) atomicOr(&rbad, 1u << (e % g.N));
+    }
     atomicMax(&rmax, m);
     __syncthreads();
     eR = exp_of(rmax);
@@ -321,7 +334,7 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_narrow(const __grid_constant__ 
       tc_after();
       const int row = quarter * 32 + lane;
       const int64_t r = t * BM + row;
-      const int e = (ROW ? (r < g.rows ? __ldg(g.es + r) : 0) : exp_of(rexp[lt & 7][row])) + eR - 56;
+      const int er = ROW ? (r < g.rows ? __ldg(g.es + r) : 0) : exp_of(rexp[lt & 7][row]), e = er + eR - 56;
       const uint32_t taddr = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(ab * ACC + chalf * (BN / 2));
       double *dst = nullptr;
       int64_t pitch = 1;
@@ -354,14 +367,18 @@ __global__ void __launch_bounds__(NTHREADS, 1) k_narrow(const __grid_constant__ 
             f[l] = __uint_as_float(q[l][c]);
           }
           // in units of the level before the last one, to stay within 64 bits
-          long long V = join_levels<P - 1, SMALL, W, P>(f) + round128(__float2int_rn(f[P - 1]));
-          if (no_value(f[0])) V = kNoValue;
+          const long long V = join_levels<P - 1, SMALL, W, P>(f) + round128(__float2int_rn(f[P - 1]));
           const int n = chalf * (BN / 2) + c4 * 4 + c;
           if (dst && n < g.N) {
             const double v = scale_i64(V, e);
             dst[n * pitch] = ROW && g.add ? dst[n * pitch] + v : v;
           }
         }
+      }
+      const unsigned bad = er == kBadExp ? ~0u : ROW ? (unsigned)__ldg(g.eR + 1) : rbad;
+      if (bad && dst) {
+        for (int n = chalf * (BN / 2); n < min(g.N, (chalf + 1) * (BN / 2)); ++n)
+          if ((bad >> n) & 1) dst[n * pitch] = __longlong_as_double(0x7FF8000000000000ll);
       }
       __syncwarp();
     }
