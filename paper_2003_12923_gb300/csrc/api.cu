@@ -116,7 +116,7 @@ esmp2_status esmp2::create_impl(esmp2_handle **out, const esmp2_desc *d, cudaStr
     ALLOC(h->red, nred);
   }
   ALLOC(h->red_out, (size_t)32);
-  if ((ce = cudaMallocHost(reinterpret_cast<void **>(&h->hred), sizeof(double) * 32)) != cudaSuccess)
+  if ((ce = cudaMallocHost(reinterpret_cast<void **>(&h->hred), sizeof(double) * 33)) != cudaSuccess)
     return check_cuda(h, ce, "pinned alloc");
   debug_phase(h, "create: allocations");
   // inputs -> device; device-resident OVOV and OVVV are read in place by the first pass of

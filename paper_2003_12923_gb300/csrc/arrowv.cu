@@ -379,6 +379,7 @@ esmp2_status ensure_arrow(esmp2_handle *h) {
   if (e != cudaSuccess) return check_cuda(h, e, "reduced-cost basis buffers");
   // the right-hand side in the reduced-cost basis (float64-exact digit-split rotations)
   s = rotate_virt(h, h->bsemi, h->barr, h->s64.w ? h->s64.w : h->s64.p, true);
+  if (!s) s = check_device_flag(h);
   if (s) return s;
   debug_phase(h, "  reduced basis: rhs rotation");
   h->arrow_ready = true;
@@ -386,7 +387,8 @@ esmp2_status ensure_arrow(esmp2_handle *h) {
 }
 
 // out = R~^T X R~ (to_arrow) or R~ X R~^T for every slice X of a full-storage block vector:
-// X R (digit-split product), transpose, X R again, transpose.  in may equal out; tmp: n doubles.
+// X R (digit-split product), transpose, X R again, transpose.  in may equal out; tmp: n doubles.  The
+// caller reads the error flag of the bounded waits.
 esmp2_status rotate_virt(esmp2_handle *h, const double *in, double *out, double *tmp, bool to_arrow) {
   const int No = h->d.No, Nv = h->d.Nv;
   const int64_t S = 5LL * No * No, rows = S * Nv;
@@ -401,12 +403,12 @@ esmp2_status rotate_virt(esmp2_handle *h, const double *in, double *out, double 
   if ((s = xwm_split(h, out, rows, tmp, M, dig, eM, slot))) return s;
   k_tr64<<<gt, 256, 0, h->stream>>>(tmp, out, S, Nv);
   h->launches += 2;
-  if ((s = check_device_flag(h))) return s;
   return check_cuda(h, cudaGetLastError(), "rotate_virt");
 }
 
-// Move the stored solution to `target` (0 TOP, 1 semicanonical-occupied, 2 reduced-cost basis).
-esmp2_status x_to_basis(esmp2_handle *h, int target) {
+// Move the stored solution to `target` (0 TOP, 1 semicanonical-occupied, 2 reduced-cost basis).  check =
+// false: the caller reads the error flag of the bounded waits itself before it uses a result.
+esmp2_status x_to_basis(esmp2_handle *h, int target, bool check) {
   if (h->x_basis == target) return ESMP2_OK;
   if (h->x_zero) {   // zero in every basis
     h->x_basis = target;
@@ -433,7 +435,7 @@ esmp2_status x_to_basis(esmp2_handle *h, int target) {
     if ((s = rotate_virt(h, x, x, tmp, true))) return s;
     h->x_basis = 2;
   }
-  if ((s = check_device_flag(h))) return s;
+  if (check && (s = check_device_flag(h))) return s;
   return check_cuda(h, cudaGetLastError(), "x_to_basis");
 }
 

@@ -489,12 +489,13 @@ esmp2_status run_digits(esmp2_handle *h, const double *x, const int *jobs, int n
   const size_t one = plane * (levels - 1), need = one * njobs;
   if (need > h->xdig_bytes && !h->xdig_final) {   // stream-ordered: the old planes are released after their last use
     // The transforms of the set-up take what they need.  The first call on a whole block vector takes nine
-    // planes of the job list of sym = 1, and that stays: a caller may have captured what works on it.
+    // planes of the job list of sym = 1 (of the longest, sym = 0, where that is small: a second pass would
+    // cost No=1 Nv=40 a third of its 60 us), and that stays: a caller may have captured what works on it.
     // Calls that need more, or all of them where there was less room, work in passes.
     const int NN = h->d.No * h->d.No;
     h->xdig_final = jobs || njobs > NN;
-    size_t room = h->xdig_final ? plane * kDigitPlanes * h->njobs[1] : need;
-    const size_t least = plane * kDigitPlanes;
+    const size_t least = plane * kDigitPlanes, full = least * h->njobs[0];
+    size_t room = !h->xdig_final ? need : full <= (size_t)256 << 20 ? full : least * h->njobs[1];
     dfree(h->xdig, h->stream);
     h->xdig = nullptr;
     h->xdig_bytes = 0;

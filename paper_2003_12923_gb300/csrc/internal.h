@@ -120,7 +120,7 @@ struct esmp2_handle {
   int p64_blocks = 0;       // 4 (T, S, X, Y), with digit products also Z
   double *red = nullptr;    // reduction partials
   double *red_out = nullptr;// reduction results (device)
-  double *hred = nullptr;   // pinned host copy of reduction results
+  double *hred = nullptr;   // pinned host copy of reduction results (32) and of the device error flag
   bool x_sym = true;       // x has the singlet symmetries (every solve makes it so; a vector set by the caller may not)
   bool solved = false;
   bool e2s_done = false;
@@ -241,6 +241,9 @@ esmp2_status check_cuda(esmp2_handle *h, cudaError_t e, const char *what);
 esmp2_status ensure_mixed(esmp2_handle *h, bool semi);
 esmp2_status sigma_inner(esmp2_handle *h, const float *p, float *q, bool p_bf16_ready = false, double *dot = nullptr);
 esmp2_status check_device_flag(esmp2_handle *h);
+// its two halves, for a caller that synchronises anyway: the copy to hred[32], and the look at it after that
+void copy_device_flag(esmp2_handle *h);
+esmp2_status device_flag_status(esmp2_handle *h);
 // packed inner solve (inner.cu)
 esmp2_status packed_setup(esmp2_handle *h);
 esmp2_status sigma_packed(esmp2_handle *h, const float *p, float *q, bool pb_ready, double *dot, int stages = 7);
@@ -282,7 +285,7 @@ esmp2_status xwm_split(esmp2_handle *h, const double *X, int64_t rows, double *Y
 // reduced-cost basis (arrowv.cu)
 esmp2_status ensure_arrow(esmp2_handle *h);
 esmp2_status rotate_virt(esmp2_handle *h, const double *in, double *out, double *tmp, bool to_arrow);
-esmp2_status x_to_basis(esmp2_handle *h, int target);
+esmp2_status x_to_basis(esmp2_handle *h, int target, bool check = true);
 esmp2_status sigma64_arrow(esmp2_handle *h, const double *x, double *y);
 void virt_arrow64(esmp2_handle *h, const double *x, double *y);
 esmp2_status rotate_occ(esmp2_handle *h, const double *in, double *out, double *tmp, bool to_semi);

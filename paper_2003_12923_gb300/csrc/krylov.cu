@@ -718,12 +718,14 @@ static VCtx vctx(const esmp2_handle *h, const double *F = nullptr) {
   return c;
 }
 
-static esmp2_status read_slots(esmp2_handle *h, double *out, int n) {
+// flag: also the error flag of the bounded waits, behind the same synchronisation
+static esmp2_status read_slots(esmp2_handle *h, double *out, int n, bool flag = false) {
+  if (flag) copy_device_flag(h);
   cudaMemcpyAsync(h->hred, h->red_out, sizeof(double) * 32, cudaMemcpyDeviceToHost, h->stream);
   cudaError_t e = cudaStreamSynchronize(h->stream);
   if (e != cudaSuccess) return check_cuda(h, e, "sync");
   for (int k = 0; k < n; ++k) out[k] = h->hred[k];
-  return ESMP2_OK;
+  return flag ? device_flag_status(h) : ESMP2_OK;
 }
 
 double dot_w(esmp2_handle *h, const double *u, const double *v) {
@@ -786,9 +788,8 @@ esmp2_status solve64(esmp2_handle *h, double tol, int maxit, esmp2_solve_info *i
     (dinv ? k_pcg_start<true> : k_pcg_start<false>)<<<dim3(kRowCtas, 5), kRedThreads, 0, st>>>(c, dinv, r, p, h->red);
     k_finalize<<<1, 1024, 0, st>>>(h->red, 5 * kRowCtas, 2, h->red_out, 0);
     h->launches += 4;
-    if (esmp2_status s2 = read_slots(h, sl, 32)) return s2;
-    if (virt_tc && !zero)   // before this residual is taken for a converged one
-      if (esmp2_status s2 = check_device_flag(h)) return s2;
+    // (the flag before this residual is taken for a converged one)
+    if (esmp2_status s2 = read_slots(h, sl, 32, virt_tc && !zero)) return s2;
     if (bnorm < 0.0) bnorm = std::sqrt(sl[9]);
     return ESMP2_OK;
   };
@@ -890,8 +891,7 @@ esmp2_status energy(esmp2_handle *h, esmp2_energy_parts *parts) {
     dfree(gdf, st);
   }
   double sl[32];
-  if ((s = read_slots(h, sl, 32))) return s;
-  if (!h->r_true && (s = check_device_flag(h))) return s;   // of the sigma build above
+  if ((s = read_slots(h, sl, 32, !h->r_true))) return s;   // the flag: of the sigma build above
   double e_blk[5];
   for (int k = 0; k < 5; ++k) e_blk[k] = kWeights[k] * (2.0 * sl[8 + 2 * k] + sl[9 + 2 * k]);
   if (small_pairs) {
@@ -1053,7 +1053,7 @@ esmp2_status solve_mixed(esmp2_handle *h, double tol, int maxit, esmp2_solve_inf
   h->tf32 = tf32;
   h->arrowv = arrowv;
   debug_phase(h, "solve: basis set-up");
-  if ((s = x_to_basis(h, arrowv ? 2 : 1))) return s;
+  if ((s = x_to_basis(h, arrowv ? 2 : 1, false))) return s;   // (the first residual of a warm start reads the flag)
   cudaStream_t st = h->stream;
   // the singlet solution lies in the symmetric subspace (antisymmetric T, X, Y; S_ij^ab =
   // S_ji^ba); the packed inner solve acts on that subspace only, so x and every residual
@@ -1154,8 +1154,7 @@ esmp2_status solve_mixed(esmp2_handle *h, double tol, int maxit, esmp2_solve_inf
       h->launches += 2;
     }
     if (!cold) ++nsig64;
-    if ((s = read_slots(h, sl, 32))) return s;
-    if (!cold && (s = check_device_flag(h))) return s;   // the inner solve before it and this residual
+    if ((s = read_slots(h, sl, 32, !cold))) return s;   // the flag: of the inner solve before it and this residual
     if (bb < 0.0) bb = sl[9];
     const double rn = std::sqrt(sl[8]), bn = std::sqrt(bb);
     relres = bn != 0.0 ? rn / bn : 0.0;

@@ -170,18 +170,24 @@ esmp2_status ensure_mixed(esmp2_handle *h, bool semi) {
   return check_cuda(h, cudaGetLastError(), "mixed set-up");
 }
 
-esmp2_status check_device_flag(esmp2_handle *h) {
-  if (!h->dflag) return ESMP2_OK;   // no kernel with bounded waits has run
-  int f = 0;
-  cudaMemcpyAsync(&f, h->dflag, sizeof(int), cudaMemcpyDeviceToHost, h->stream);
-  cudaError_t e = cudaStreamSynchronize(h->stream);
-  if (e != cudaSuccess) return check_cuda(h, e, "device flag");
-  if (f) {
+void copy_device_flag(esmp2_handle *h) {
+  if (h->dflag) cudaMemcpyAsync(h->hred + 32, h->dflag, sizeof(int), cudaMemcpyDeviceToHost, h->stream);
+}
+
+esmp2_status device_flag_status(esmp2_handle *h) {
+  if (h->dflag && *reinterpret_cast<volatile int *>(h->hred + 32)) {
     h->err = "a bounded device-side wait timed out in the tensor-core kernel";
     cudaMemsetAsync(h->dflag, 0, sizeof(int), h->stream);
     return ESMP2_ERR_TIMEOUT;
   }
   return ESMP2_OK;
+}
+
+esmp2_status check_device_flag(esmp2_handle *h) {
+  if (!h->dflag) return ESMP2_OK;   // no kernel with bounded waits has run
+  copy_device_flag(h);
+  cudaError_t e = cudaStreamSynchronize(h->stream);
+  return e != cudaSuccess ? check_cuda(h, e, "device flag") : device_flag_status(h);
 }
 
 // Inner (low-precision) sigma in the semicanonical-occupied basis: q = A p with the
